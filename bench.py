@@ -99,7 +99,7 @@ def workload(args, rank):
 
 
 PROFILE = os.path.join(ROOT, "profiles", "batch_kernel_mixed_d7-21_p003.md")
-KERNEL_SOURCES = ["decoder.cu", "qec_internal.h", "capi.cpp"]
+KERNEL_SOURCES = ["decoder.cu", "balls.cu", "qec_internal.h", "capi.cpp"]
 
 
 _TOKENS = re.compile(r'"(?:\\.|[^"\\])*"|//[^\n]*|/\*.*?\*/', re.S)

@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libqec.so")
-SOURCES = ["decoder.cu", "capi.cpp", "noalloc.cu", "serve.cpp"]
+SOURCES = ["decoder.cu", "balls.cu", "capi.cpp", "noalloc.cu", "serve.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

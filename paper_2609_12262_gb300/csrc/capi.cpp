@@ -38,6 +38,10 @@ struct qec_graph {
     unsigned long long *d_eobs = nullptr;
     int2 *d_eend = nullptr;
     unsigned *d_commit = nullptr;   // commit-region bitmap (sliding windows)
+    int *d_seam = nullptr;          // distances to its border
+    unsigned long long *d_vbnd = nullptr;
+    int4 *d_bhdr = nullptr;         // ball table
+    int2 *d_ball = nullptr;
     int components = 0;             // connected components of the detector graph
     long long diam_ub = 0;          // upper bound on detector-detector distances (internal units)
     int upper_single = 0;           // every event above level 1 forms one processing cluster
@@ -200,29 +204,114 @@ struct PhysKey {
     int lo, hi, w, idx;
 };
 
-// Exact single-source distances over detector-detector slots (boundary
-// vertices are leaves, so no path passes through them).
-void dijkstra_host(const std::vector<int> &row, const std::vector<Slot> &slots, int src, std::vector<long long> &dist) {
-    const long long INF = LLONG_MAX;
-    std::fill(dist.begin(), dist.end(), INF);
-    using Item = std::pair<long long, int>;
-    std::priority_queue<Item, std::vector<Item>, std::greater<Item>> pq;
-    dist[(size_t)src] = 0;
-    pq.push({0, src});
-    while (!pq.empty()) {
-        const Item it = pq.top();
-        pq.pop();
-        if (it.first != dist[(size_t)it.second]) continue;
-        for (int j = row[(size_t)it.second]; j < row[(size_t)it.second + 1]; j++) {
+// Exact distances over detector-detector slots (boundary vertices are leaves,
+// so no path passes through them) from a set of start distances.  Weights are
+// bounded, so the queue is a ring of buckets, one per distance modulo
+// (largest weight + 1); a heap where that ring would be large.
+struct Distances {
+    const std::vector<int> &row;
+    const std::vector<Slot> &slots;
+    const int wmax;
+    std::vector<std::vector<int>> ring;
+    std::vector<int> order;   // vertices settled by the last run, by distance
+
+    Distances(const std::vector<int> &r, const std::vector<Slot> &s, int w) : row(r), slots(s), wmax(w) {
+        if (wmax < (1 << 16)) ring.resize((size_t)wmax + 1);
+    }
+
+    // dist: start distances (LLONG_MAX: none) in, distances out; starts: the
+    // vertices with a start distance
+    void run(std::vector<long long> &dist, const std::vector<int> &starts) {
+        order.clear();
+        if (!ring.empty()) run_ring(dist, starts);
+        else run_heap(dist, starts);
+    }
+
+    void from(int src, std::vector<long long> &dist) {
+        std::fill(dist.begin(), dist.end(), LLONG_MAX);
+        dist[(size_t)src] = 0;
+        run(dist, {src});
+    }
+
+  private:
+    template <class Push>
+    void relax(std::vector<long long> &dist, int x, Push push) {
+        order.push_back(x);
+        const long long d = dist[(size_t)x];
+        for (int j = row[(size_t)x]; j < row[(size_t)x + 1]; j++) {
             const Slot sl = slots[(size_t)j];
-            if (sl.code < 0) continue;
-            const long long nd = it.first + sl.w;
-            if (nd < dist[(size_t)sl.code]) {
-                dist[(size_t)sl.code] = nd;
-                pq.push({nd, sl.code});
-            }
+            if (sl.code < 0 || d + sl.w >= dist[(size_t)sl.code]) continue;
+            dist[(size_t)sl.code] = d + sl.w;
+            push(d + sl.w, sl.code);
         }
     }
+
+    void run_ring(std::vector<long long> &dist, const std::vector<int> &starts) {
+        // starts enter the ring when their distance comes up
+        std::vector<int> wait(starts);
+        std::sort(wait.begin(), wait.end(), [&](int a, int b) { return dist[(size_t)a] < dist[(size_t)b]; });
+        std::vector<long long> first(wait.size());
+        for (size_t i = 0; i < wait.size(); i++) first[i] = dist[(size_t)wait[i]];
+        const long long C = (long long)ring.size();
+        size_t next = 0, held = 0;
+        long long d = 0;
+        while (held || next < wait.size()) {
+            if (!held) d = first[next];
+            for (; next < wait.size() && first[next] == d; next++)
+                if (dist[(size_t)wait[next]] == d) { ring[(size_t)(d % C)].push_back(wait[next]); held++; }
+            auto &b = ring[(size_t)(d % C)];
+            for (size_t i = 0; i < b.size(); i++) {   // positive weights: no push into this bucket
+                const int x = b[i];
+                if (dist[(size_t)x] != d) continue;
+                relax(dist, x, [&](long long nd, int y) { ring[(size_t)(nd % C)].push_back(y); held++; });
+            }
+            held -= b.size();
+            b.clear();
+            d++;
+        }
+    }
+
+    void run_heap(std::vector<long long> &dist, const std::vector<int> &starts) {
+        using Item = std::pair<long long, int>;
+        std::priority_queue<Item, std::vector<Item>, std::greater<Item>> pq;
+        for (int s : starts) pq.push({dist[(size_t)s], s});
+        while (!pq.empty()) {
+            const Item it = pq.top();
+            pq.pop();
+            if (it.first != dist[(size_t)it.second]) continue;
+            relax(dist, it.second, [&](long long nd, int y) { pq.push({nd, y}); });
+        }
+    }
+};
+
+// Every vertex's canonical boundary candidate: distance to the nearest
+// boundary vertex << 32 | lowest merged id among the boundary edges at that
+// distance (all ones: none reachable).  A vertex at that distance holds the
+// edge itself or has it through a neighbour nearer to the boundary.
+std::vector<unsigned long long> boundary_candidates(int n, Distances &D) {
+    std::vector<long long> dist((size_t)n, LLONG_MAX);
+    std::vector<int> starts;
+    for (int x = 0; x < n; x++) {
+        for (int j = D.row[(size_t)x]; j < D.row[(size_t)x + 1]; j++)
+            if (D.slots[(size_t)j].code < 0) dist[(size_t)x] = std::min<long long>(dist[(size_t)x], D.slots[(size_t)j].w);
+        if (dist[(size_t)x] != LLONG_MAX) starts.push_back(x);
+    }
+    D.run(dist, starts);
+    std::vector<unsigned long long> out((size_t)n, ~0ull);
+    for (int x : D.order) {
+        const long long d = dist[(size_t)x];
+        unsigned eid = ~0u;
+        for (int j = D.row[(size_t)x]; j < D.row[(size_t)x + 1]; j++) {
+            const Slot sl = D.slots[(size_t)j];
+            if (sl.code < 0) {
+                if (sl.w == d) eid = std::min(eid, (unsigned)(-1 - sl.code));
+            } else if (dist[(size_t)sl.code] != LLONG_MAX && dist[(size_t)sl.code] + sl.w == d) {
+                eid = std::min(eid, (unsigned)out[(size_t)sl.code]);
+            }
+        }
+        out[(size_t)x] = ((unsigned long long)d << 32) | eid;
+    }
+    return out;
 }
 
 // Connected components of the detector graph and an upper bound on the
@@ -230,22 +319,21 @@ void dijkstra_host(const std::vector<int> &row, const std::vector<Slot> &slots, 
 // central vertex (triangle inequality through it).  Three Dijkstra runs per
 // component: from its first vertex v, from the vertex x farthest from v, and
 // from the vertex c minimising max(d(v, c), d(x, c)).
-void graph_extent(int n, const std::vector<int> &row, const std::vector<Slot> &slots, int &components,
-                  long long &diam_ub) {
+void graph_extent(int n, Distances &D, int &components, long long &diam_ub) {
     std::vector<int> comp((size_t)n, -1);
     std::vector<long long> dv((size_t)n), dx((size_t)n), dc((size_t)n);
     components = 0;
     diam_ub = 0;
     for (int v = 0; v < n; v++) {
         if (comp[(size_t)v] >= 0) continue;
-        dijkstra_host(row, slots, v, dv);
+        D.from(v, dv);
         int x = v;
         for (int y = 0; y < n; y++)
             if (dv[(size_t)y] != LLONG_MAX) {
                 comp[(size_t)y] = components;
                 if (dv[(size_t)y] > dv[(size_t)x]) x = y;
             }
-        dijkstra_host(row, slots, x, dx);
+        D.from(x, dx);
         int c = v;
         long long best = LLONG_MAX;
         for (int y = 0; y < n; y++)
@@ -253,7 +341,7 @@ void graph_extent(int n, const std::vector<int> &row, const std::vector<Slot> &s
                 const long long m = std::max(dv[(size_t)y], dx[(size_t)y]);
                 if (m < best) { best = m; c = y; }
             }
-        dijkstra_host(row, slots, c, dc);
+        D.from(c, dc);
         long long ecc_v = 0, ecc_c = 0;
         for (int y = 0; y < n; y++)
             if (comp[(size_t)y] == components) {
@@ -592,7 +680,8 @@ int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) {
     // be met).  Then the events left after level 1 form exactly one processing
     // cluster.  b_2 is taken as b_1 when the schedule stored only one level
     // (b_k increases with k, so this only errs on the safe side).
-    graph_extent(n, row, slots, g->components, g->diam_ub);
+    Distances D(row, slots, g->wmax);
+    graph_extent(n, D, g->components, g->diam_ub);
     {
         const long long b2 = g->num_levels >= 2 ? g->bk[1] : g->bk[0];
         g->upper_single = (g->components == 1 && b2 >= g->diam_ub) ? 1 : 0;
@@ -602,6 +691,14 @@ int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) {
     d.eobs = g->d_eobs;
     d.eend = g->d_eend;
     d.seid = g->d_seid;
+    const std::vector<unsigned long long> vb = boundary_candidates(n, D);
+    ce = cudaMalloc(&g->d_vbnd, sizeof(unsigned long long) * (size_t)n);
+    if (ce == cudaSuccess)
+        ce = cudaMemcpy(g->d_vbnd, vb.data(), sizeof(unsigned long long) * (size_t)n, cudaMemcpyHostToDevice);
+    d.vbnd = g->d_vbnd;
+    if (ce == cudaSuccess) ce = qec::build_ball_table(d, &g->d_bhdr, &g->d_ball);
+    if (ce == cudaErrorMemoryAllocation) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
+    if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "graph tables"); }
     *out = g;
     return QEC_OK;
 }
@@ -648,6 +745,10 @@ int qec_graph_destroy(qec_graph *g) {
     if (g->d_eend) cudaFree(g->d_eend);
     if (g->d_seid) cudaFree(g->d_seid);
     if (g->d_commit) cudaFree(g->d_commit);
+    if (g->d_seam) cudaFree(g->d_seam);
+    if (g->d_vbnd) cudaFree(g->d_vbnd);
+    if (g->d_bhdr) cudaFree(g->d_bhdr);
+    if (g->d_ball) cudaFree(g->d_ball);
     delete g;
     return QEC_OK;
 }
@@ -661,8 +762,11 @@ int qec_graph_set_commit_region(qec_graph *g, const uint32_t *detector_bitmap) {
             if (ce != cudaSuccess) return cuda_fail(ce, "cudaDeviceSynchronize");
             cudaFree(g->d_commit);
         }
+        if (g->d_seam) cudaFree(g->d_seam);
         g->d_commit = nullptr;
+        g->d_seam = nullptr;
         g->dg.commit = nullptr;
+        g->dg.seam = nullptr;
         return QEC_OK;
     }
     std::vector<unsigned> bits((size_t)g->words, 0u);
@@ -675,6 +779,13 @@ int qec_graph_set_commit_region(qec_graph *g, const uint32_t *detector_bitmap) {
     }
     ce = cudaMemcpy(g->d_commit, bits.data(), sizeof(unsigned) * (size_t)g->words, cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaMemcpy");
+    if (!g->d_seam) {
+        ce = cudaMalloc(&g->d_seam, sizeof(int) * (size_t)g->n);
+        if (ce != cudaSuccess) { g->d_seam = nullptr; return fail(QEC_ENOMEM, "cudaMalloc"); }
+    }
+    ce = qec::build_seam(g->dg, g->d_commit, g->d_seam);
+    if (ce != cudaSuccess) return cuda_fail(ce, "commit region tables");
+    g->dg.seam = g->d_seam;
     g->dg.commit = g->d_commit;
     return QEC_OK;
 }

@@ -9,34 +9,39 @@
 //   1. defect compaction: the shot's syndrome bitmap is read with 16-byte
 //      vector loads and compacted by a warp prefix sum (input D of the paper's
 //      "Decoding task"; Alg. 1 input).
-//   2. flooder: every detection event s owns an explored ball {x : dist(s,x) <=
-//      R_s} with exact graph distances (hash table keyed by (vertex, event)),
-//      explored once its region starts growing and kept at R_s >= Rad(s) + L
-//      (L above the largest weight).  A ball is grown band by band (band >=
-//      largest weight) by team-parallel label-correcting relaxation from the
-//      previous band; each new entry is checked against the other events'
-//      balls holding the same vertex, and against events sitting on it, which
-//      records the exact distance of every pair of events whose balls touch.
-//      The graph-fill region of s (SI S1) is the ball of radius Rad(s) <= R_s,
-//      so two regions are found touching exactly when their pair distance
-//      equals Rad(a) + Rad(b) (ARRIVE = a band extension, COLLIDE = a tight
-//      pair, boundary COLLIDE = Rad(s) reaching the nearest boundary, IMPLODE =
-//      an inner blossom's dual reaching 0).
-//   3. Algorithm 1, level 1: each event's neighbourhood within b_1 (paths of
-//      one or two edges when three smallest weights exceed b_1, else a bounded
-//      search) gives every pair within b_1 and every boundary contact; min-label
-//      components, the diameter <= d_1 test and the parity condition decide the
-//      level-1 processing clusters.
+//   2. neighbourhoods: every pair of events within b_1 is read off the graph's
+//      ball table (balls.cu: for each detector the detectors near it with exact
+//      distances), by testing the entries of each event's list against the
+//      syndrome row; every event's nearest boundary is read off a second table.
+//      A growing region keeps an explored radius R_s >= Rad(s) + L (L above the
+//      largest weight); when it falls due (EXTEND) the events it can touch until
+//      the next time come from the pairs already listed or from the farther
+//      entries of its list, so the ball itself stays virtual.  Only a region
+//      that outgrows the table's radius (about 1 shot in 1,000 at d = 21,
+//      p = 0.003, 1 in 60 at d = 51, p = 0.005) makes its shot explore balls
+//      {x : dist(s,x) <= R_s} (hash table keyed by (vertex, event), grown band
+//      by band by team-parallel label-correcting relaxation; each new entry is
+//      checked against the other events' balls holding the same vertex, and
+//      against events sitting on it).  Either way the exact distance of two
+//      events is known before their regions touch.  The graph-fill region of s
+//      (SI S1) is the ball of radius Rad(s) <= R_s, so two regions are found
+//      touching exactly when their pair distance equals Rad(a) + Rad(b) (ARRIVE =
+//      an extension, COLLIDE = a tight pair, boundary COLLIDE = Rad(s) reaching
+//      the nearest boundary, IMPLODE = an inner blossom's dual reaching 0).
+//   3. Algorithm 1, level 1: with every pair within b_1 and every boundary
+//      contact, min-label components, the diameter <= d_1 test and the parity
+//      condition decide the level-1 processing clusters.
 //   4. Algorithm 2: level-1 clusters are solved independently (closed form for
 //      the isolated pair and boundary singleton, the event loop otherwise), then
 //      every remaining event runs from t = 0 with the stopped level-1
 //      configurations present as frozen regions (hierarchical execution rule).
 //      Global mode runs every event in one execution instead.
-//   5. Tracing: blossoms are expanded into matched event pairs and boundary
-//      matches; the weight is the sum of the tight pair / boundary distances and
-//      the observable mask the XOR of the canonical paths' masks.  The
-//      sliding-window instantiations (batch_kernel<true, *>) also walk every
-//      path and commit the edges that touch the window's commit region.
+//   5. Result: the weight is the sum of the duals (every matched edge is tight),
+//      the observable mask that of the boundary matches' edges.  Only where
+//      detector-detector edges carry observables, and in the sliding-window
+//      instantiations (batch_kernel<true, *>), blossoms are expanded into matched
+//      event pairs and their canonical paths walked: a window commits the edges
+//      that touch its commit region.
 //
 // Simultaneous events are applied in the canonical order (t, kind, lo, hi) with
 // kind EXTEND < IMPLODE < COLLIDE < BOUNDARY and lo, hi the ranks of the events
@@ -50,11 +55,18 @@
 // thread writes between the barrier before the read and the barrier after it,
 // so all threads of a team always take the same path.
 //
-// The rarely taken matcher steps (augment, blossom, shatter), the tracing and
-// the level-1 neighbourhood searches are kept out of line (__noinline__): the
-// event loop and the flooder stay inlined, and the kernel's hot code stays
-// small enough for the instruction cache (each choice measured on the full
-// batch; inlining the flooder or moving it out of line are both slower).
+// The rarely taken matcher steps (augment, blossom, shatter), the path walks and
+// the explored balls are kept out of line (__noinline__), so that the kernel's
+// hot code stays small enough for the instruction cache.
+//
+// What bounds it: dependent loads of per-shot state and of the tables (no
+// contraction, and the algorithmic bytes take a thousandth of the time).  The
+// ball table replaced, per event, ~25 hash insertions with their contact walks
+// and two enumerations of two-edge paths by ~13 coalesced list entries: a
+// million shots of d = 7 .. 21 at p = 0.003 from 88.7 to 21.5 ms, 100,000 of
+// d = 11 with own weights from 6.1 to 1.46 ms, 1,024 circuit-level d = 13 shots
+// (whose two-edge rule does not hold) from 7.4 to 0.16 ms, one d = 51 window
+// from 1.42 to 0.92 ms.
 
 #include <algorithm>
 #include <climits>
@@ -86,7 +98,7 @@ constexpr long long T_MAX = (1LL << 26) - 1;
 enum { MATE_NONE = -1, MATE_BOUNDARY = -2 };
 
 // slab counters (C_R0 .. C_NEXT: work-list counters of multi-warp teams)
-enum { C_ECOUNT = 0, C_WL = 1, C_NPAIRS = 2, C_CCOUNT = 3, C_NFREE = 4, C_ERR = 5, C_FRESH = 6, C_NHI = 7,
+enum { C_ECOUNT = 0, C_WL = 1, C_NPAIRS = 2, C_CCOUNT = 3, C_NFREE = 4, C_ERR = 5, C_NHI = 7,
        C_TL = 8, C_CHANGED = 9, C_TNP = 10, C_TNX = 11, C_R0 = 12, C_NEXT = 15, C_TOTAL = 16 };
 enum { ERR_CAP = 1, ERR_INTERNAL = 2 };
 
@@ -362,11 +374,9 @@ struct __align__(16) NRec {
 };
 __device__ __forceinline__ int4 ld_nd(const NRec *p) { return *reinterpret_cast<const int4 *>(p); }
 
-// A pair of events whose balls met, as a block-wide team keeps it: ranks
-// lo < hi, exact distance (equal to the hash entry's value after every
-// barrier), hash slot.  All ones (lo = -1) is an unused record: a record
-// reserved by an insert that lost the race for its slot to the same pair
-// stays so.  A one-warp team lists the pairs' hash slots instead (plist).
+// A pair of events and their exact distance: ranks lo < hi (lo = -1: an unused
+// record), the distance, and the pair's hash slot (-1 while the pair is only
+// listed; set once the shot explores balls, see go_real).
 struct __align__(16) PRec {
     int lo, hi;
     unsigned val;
@@ -387,11 +397,9 @@ struct Slab {
     int *xsrc, *xR, *xcnt, *xcur;         // sources being extended, target radii, band counts
     int *xidx;                            // position of a source in xsrc during an extension
     int *wcum;                            // detection events in syndrome words before word w
-    // pairs: key (lo << 32 | hi), value distance; one-warp teams list the
-    // used slots (plist), block-wide teams keep pair records (pr, carved
-    // last) whose index the hash entry's upper word holds
+    // pair records, and once the shot explores balls their hash (key lo << 32
+    // | hi, value distance, the record's index in the upper word)
     HEnt *pt;
-    int *plist;
     PRec *pr;
     // matcher nodes (leaf s = node s, blossoms above K)
     NRec *nd;
@@ -422,7 +430,8 @@ __host__ __device__ inline long long carve(char *base, const SlabCaps &c, Slab &
     S.xsrc = bump<int>(p, c.kc); S.xR = bump<int>(p, c.kc); S.xcnt = bump<int>(p, c.kc); S.xcur = bump<int>(p, c.kc);
     S.xidx = bump<int>(p, c.kc);
     S.wcum = bump<int>(p, c.wcap);
-    S.pt = bump<HEnt>(p, c.phc); S.plist = bump<int>(p, c.phc);
+    S.pt = bump<HEnt>(p, c.phc);
+    S.pr = bump<PRec>(p, (c.phc >> 1) + 1);
     S.nd = bump<NRec>(p, c.nc);
     S.tpar = bump<int>(p, c.nc); S.tps = bump<int>(p, c.nc); S.tpo = bump<int>(p, c.nc);
     S.mate = bump<int>(p, c.nc); S.ms = bump<int>(p, c.nc); S.mo = bump<int>(p, c.nc);
@@ -432,7 +441,6 @@ __host__ __device__ inline long long carve(char *base, const SlabCaps &c, Slab &
     S.stk = bump<int>(p, 4 * c.nc + 64);
     S.cnode = bump<int>(p, c.cc); S.cs = bump<int>(p, c.cc); S.co = bump<int>(p, c.cc);
     S.ctr = bump<int>(p, C_TOTAL);
-    S.pr = bump<PRec>(p, (c.phc >> 1) + 1);   // last: the one-warp layout above is unchanged
     return (long long)(p - base) + 16;
 }
 
@@ -449,6 +457,9 @@ struct Shot {
     unsigned hmask;   // explored-entry hash mask
     unsigned pmask;   // pair hash mask
     int ec, wc, nc, cc;
+    int pcap;         // pair records the slab holds
+    int real;         // balls are explored (else every ball is virtual, see extend_due)
+    int paths;        // a path was walked through an explored ball
     int band;
     int L;                 // lookahead: explored radius >= Rad + L for every growing region
     const unsigned *row;   // the shot's syndrome row (defect test)
@@ -516,94 +527,42 @@ __device__ int ht_upsert(const Slab &S, const Shot &C, int v, int s, int d, unsi
     return -1;
 }
 
-// Insert-or-decrease the pair (a, b) with distance d.  REC (block-wide
-// teams): a new pair reserves the next pair record before claiming its slot,
-// and every value written to the hash entry is also applied to the record by
-// the thread that wrote it, so both hold the minimum after the next barrier.
-// Otherwise the claimed slot is appended to the pair list.
-template <bool REC>
+// Insert-or-decrease the pair (a, b) with distance d (shots that explore
+// balls): a new pair reserves the next record, complete but for its slot,
+// before claiming its hash slot, and every smaller value goes to the entry and
+// to the record, so both hold the minimum after the next barrier.
 __device__ void pair_upsert(const Slab &S, const Shot &C, int a, int b, int d) {
-    int lo = a < b ? a : b, hi = a < b ? b : a;
+    const int lo = a < b ? a : b, hi = a < b ? b : a;
     const unsigned long long key = ((unsigned long long)(unsigned)lo << 32) | (unsigned)hi;
     unsigned i = pslot(lo, hi, C.pmask);
-    if constexpr (REC) {
-        int idx = -1;
-        for (unsigned n = 0; n <= C.pmask; n++) {
-            unsigned long long k, w;
-            asm volatile("ld.relaxed.cta.v2.b64 {%0, %1}, [%2];" : "=l"(k), "=l"(w) : "l"(&S.pt[i]) : "memory");
-            if (k == EMPTY64) {
-                if (idx < 0) {
-                    idx = atomicAdd(&S.ctr[C_NPAIRS], 1);
-                    if ((unsigned)idx * 2u > C.pmask) { set_err(S, ERR_CAP); return; }
-                }
-                if (claim_pair(&S.pt[i], key, d, idx, k, w)) {
-                    S.pr[idx].lo = lo; S.pr[idx].hi = hi; S.pr[idx].slot = (int)i;
-                    atomicMin(&S.pr[idx].val, (unsigned)d);
-                    return;
-                }
+    int idx = -1;
+    for (unsigned n = 0; n <= C.pmask; n++) {
+        unsigned long long k, w;
+        asm volatile("ld.relaxed.cta.v2.b64 {%0, %1}, [%2];" : "=l"(k), "=l"(w) : "l"(&S.pt[i]) : "memory");
+        if (k == EMPTY64) {
+            if (idx < 0) {
+                idx = atomicAdd(&S.ctr[C_NPAIRS], 1);
+                if ((unsigned)idx * 2u > C.pmask || idx >= C.pcap) { set_err(S, ERR_CAP); return; }
+                S.pr[idx] = PRec{lo, hi, (unsigned)d, -1};
+                __threadfence_block();
             }
-            if (k == key) {
-                const int v = (int)(unsigned)(w & 0xffffffffu), j = (int)(w >> 32);
-                if (d < v) {
-                    atomicMin(&S.pt[i].val, d);
-                    atomicMin(&S.pr[j].val, (unsigned)d);
-                }
-                return;   // a reserved record stays unused
-            }
-            i = (i + 1) & C.pmask;
-        }
-    } else {
-        for (unsigned n = 0; n <= C.pmask; n++) {
-            unsigned long long k;
-            int v;
-            ld_ent(&S.pt[i], k, v);
-            if (k == EMPTY64) {
-                if (claim_ent(&S.pt[i], key, d, k)) {
-                    int idx = atomicAdd(&S.ctr[C_NPAIRS], 1);
-                    if ((unsigned)idx * 2u > C.pmask) set_err(S, ERR_CAP);
-                    else S.plist[idx] = (int)i;
-                    return;
-                }
-                v = INF32;
-            }
-            if (k == key) {
-                if (d < v) atomicMin(&S.pt[i].val, d);
+            if (claim_pair(&S.pt[i], key, d, idx, k, w)) {
+                S.pr[idx].slot = (int)i;
                 return;
             }
-            i = (i + 1) & C.pmask;
         }
-    }
-    set_err(S, ERR_CAP);
-}
-
-__device__ int pair_get(const Slab &S, const Shot &C, int a, int b) {
-    int lo = a < b ? a : b, hi = a < b ? b : a;
-    const unsigned long long key = ((unsigned long long)(unsigned)lo << 32) | (unsigned)hi;
-    unsigned i = pslot(lo, hi, C.pmask);
-    for (unsigned n = 0; n <= C.pmask; n++) {
-        unsigned long long k;
-        int v;
-        ld_ent(&S.pt[i], k, v);
-        if (k == key) return v;
-        if (k == EMPTY64) return INF32;
+        if (k == key) {
+            const int v = (int)(unsigned)(w & 0xffffffffu), j = (int)(w >> 32);
+            if (d < v) {
+                atomicMin(&S.pt[i].val, d);
+                atomicMin(&S.pr[j].val, (unsigned)d);
+            }
+            if (idx >= 0) S.pr[idx].lo = -1;   // reserved, lost the slot to the same pair
+            return;
+        }
         i = (i + 1) & C.pmask;
     }
-    return INF32;
-}
-
-// The i-th pair found (ranks a < b, distance pv); false for an unused record.
-template <int NW>
-__device__ __forceinline__ bool pair_at(const Slab &S, int i, int &a, int &b, int &pv) {
-    if constexpr (NW == 1) {
-        unsigned long long k;
-        ld_ent(&S.pt[S.plist[i]], k, pv);
-        a = (int)(k >> 32); b = (int)(unsigned)(k & 0xffffffffu);
-        return true;
-    } else {
-        const int4 pq = ld_pr(&S.pr[i]);
-        a = pq.x; b = pq.y; pv = pq.z;
-        return a >= 0;
-    }
+    set_err(S, ERR_CAP);
 }
 
 struct SlotV {
@@ -632,44 +591,31 @@ __device__ __forceinline__ int rank_of(const Slab &S, const Shot &C, int v) {
     return S.wcum[v >> 5] + __popc(w & ((1u << (v & 31)) - 1u));
 }
 
-__device__ __forceinline__ void bnd_update(const Slab &S, int s, int d, int eid) {
-    unsigned long long v = ((unsigned long long)(unsigned)d << 32) | (unsigned)eid;
-    atomicMin(&S.sbnd[s], v);
-}
-
 // Grow the explored balls of the sources xsrc[0 .. nx) from radius sR[s] to
 // xR[i] (xR[i] - sR[s] >= largest weight), all at once: the previous band of
-// each source is the frontier, label-correcting relaxation runs on work lists
-// of table slots (a slot's key names the vertex and source, its value the
-// current distance) until no distance changes, every new entry is checked for
-// contacts with the other sources' balls, and each source's new band is stored
-// contiguously in `ent` as its next frontier.  Every thread of the team calls
-// with the same nx.
-template <int NW>
-__device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
+// each source is the frontier (its own vertex when never explored),
+// label-correcting relaxation runs on work lists of table slots (a slot's key
+// names the vertex and source, its value the current distance) until no
+// distance changes, with CONTACTS every new entry is checked for contacts with
+// the other sources' balls, and each source's new band is stored contiguously
+// in `ent` as its next frontier.  Every thread of the team calls with the same
+// nx.  Only shots with a region too large for the ball table get here, so it
+// stays out of line.
+template <bool CONTACTS, int NW>
+__device__ __noinline__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> T) {
     const DGraph &g = C.g;
     if (nx <= 0) return;
     const int lane = T.lane;
     T.sync();
     if (T.tid() == 0) {
-        S.ctr[C_TL] = 0; S.ctr[C_WL] = 0; S.ctr[C_FRESH] = 0;
+        S.ctr[C_TL] = 0; S.ctr[C_WL] = 0;
         if constexpr (NW > 1) { S.ctr[C_R0] = 0; S.ctr[C_R0 + 1] = 0; }
     }
     for (int i = T.tid(); i < nx; i += T.NT) { S.xcnt[i] = 0; S.xidx[S.xsrc[i]] = i; }
     T.sync();
     unsigned *F = reinterpret_cast<unsigned *>(S.wl0), *Wn = reinterpret_cast<unsigned *>(S.wl1);
-    // A source never explored whose target radius is below three smallest
-    // weights has a first ball made of paths of at most two edges: it is
-    // enumerated directly below (listed in xcur).  Initial frontier of the
-    // others: the previous band of every listed source; a source never
-    // explored so far starts from its own vertex at distance 0.
-    const int r3 = 3 * g.wmin;
     for (int i = T.tid(); i < nx; i += T.NT) {
         const int s = S.xsrc[i];
-        if (S.src[s].sR < 0 && S.xR[i] < r3) {
-            S.xcur[atomicAdd(&S.ctr[C_FRESH], 1)] = i;
-            continue;
-        }
         if (S.src[s].sR < 0) {
             unsigned hs;
             const int r = ht_upsert(S, C, S.svtx[s], s, 0, hs);
@@ -697,96 +643,6 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
     // three slots (a slot is cleared two rounds before its next use)
     int ntl = ldr(&S.ctr[C_TL]);
     const unsigned lt = (1u << lane) - 1u;
-    // new explored entry (table slot hs) of list position xi: one slot in `tl`
-    // per inserted entry, placed by ballot (one warp) or by one atomic per warp
-    auto append_tl = [&](bool ins, unsigned hs, int xi) {
-        const unsigned mt = __ballot_sync(FULL, ins);
-        int bt;
-        if constexpr (NW == 1) {
-            bt = ntl;
-            ntl += __popc(mt);
-        } else {
-            bt = 0;
-            if (lane == 0 && mt) bt = atomicAdd(&S.ctr[C_TL], __popc(mt));
-            bt = __shfl_sync(FULL, bt, 0);
-        }
-        if (ins) {
-            const int e = bt + __popc(mt & lt);
-            if (e < C.ec) S.tl[e] = ((unsigned long long)hs << 32) | (unsigned)xi; else set_err(S, ERR_CAP);
-        }
-    };
-    {
-        // first balls by enumeration: every vertex within radius R of the
-        // source is reached by a path of one or two edges, so the minimum over
-        // those paths is its exact distance; boundary candidates through the
-        // source and its neighbours (the band's farther vertices are the next
-        // extension's frontier, which adds theirs before a region can get
-        // there).  One lane per (source, adjacency slot), as in level1_2hop.
-        const int nfr = ldr(&S.ctr[C_FRESH]);
-        for (int base = T.warp() * WS; base < nfr; base += T.NT) {
-            const int idx = base + lane;
-            int src = -1, r0 = 0, deg = 0, xi = 0, s = 0, R = -1;
-            bool ins = false;
-            unsigned hs = 0;
-            if (idx < nfr) {
-                xi = S.xcur[idx];
-                s = S.xsrc[xi];
-                R = S.xR[xi];
-                src = S.svtx[s];
-                r0 = __ldg(g.row + src);
-                deg = __ldg(g.row + src + 1) - r0;
-                ins = ht_upsert(S, C, src, s, 0, hs) == 1;
-            }
-            append_tl(ins, hs, xi);
-            int incl = deg;
-            for (int o = 1; o < WS; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int total = __shfl_sync(FULL, incl, WS - 1);
-            const int excl = incl - deg;
-            for (int t0 = 0; t0 < total; t0 += WS) {
-                const int t = t0 + lane;
-                int ow = 0;
-                for (int step = WS / 2; step > 0; step >>= 1) {
-                    const int e = __shfl_sync(FULL, excl, ow + step);
-                    if (e <= t) ow += step;
-                }
-                const int osrc = __shfl_sync(FULL, src, ow);
-                const int oj = __shfl_sync(FULL, r0 - excl, ow) + t;
-                const int os = __shfl_sync(FULL, s, ow);
-                const int oR = __shfl_sync(FULL, R, ow);
-                const int oxi = __shfl_sync(FULL, xi, ow);
-                int an = -1, aw = 0;
-                bool ins1 = false;
-                unsigned h1 = 0;
-                if (t < total) {
-                    const SlotV a = load_slot(g, oj);
-                    aw = a.w;
-                    if (a.nbr < 0) bnd_update(S, os, a.w, a.eid);
-                    else if (a.w <= oR) {
-                        an = a.nbr;
-                        ins1 = ht_upsert(S, C, an, os, a.w, h1) == 1;
-                    }
-                }
-                append_tl(ins1, h1, oxi);
-                // second edges from the neighbour, one lane each
-                const int q0 = an >= 0 ? __ldg(g.row + an) : 0, q1 = an >= 0 ? __ldg(g.row + an + 1) : 0;
-                const int nq = __reduce_max_sync(FULL, (unsigned)(q1 - q0));
-                for (int k = 0; k < nq; k++) {
-                    bool ins2 = false;
-                    unsigned h2 = 0;
-                    if (k < q1 - q0) {
-                        const SlotV b = load_slot(g, q0 + k);
-                        const int nd = aw + b.w;
-                        if (b.nbr < 0) bnd_update(S, os, nd, b.eid);
-                        else if (nd <= oR && b.nbr != osrc) ins2 = ht_upsert(S, C, b.nbr, os, nd, h2) == 1;
-                    }
-                    append_tl(ins2, h2, oxi);
-                }
-            }
-        }
-    }
     for (int iter = 0;; iter++) {
         if (iter >= 4096) { if (T.tid() == 0) set_err(S, ERR_INTERNAL); break; }
         int nwl = 0;
@@ -837,8 +693,7 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
                     const int s = (int)(unsigned)(okey & 0xffffffffu);
                     const SlotV sl = load_slot(g, oj);
                     const int nd = odx + sl.w;
-                    if (sl.nbr < 0) bnd_update(S, s, nd, sl.eid);
-                    else if (nd <= oRn) r = ht_upsert(S, C, sl.nbr, s, nd, hs);
+                    if (sl.nbr >= 0 && nd <= oRn) r = ht_upsert(S, C, sl.nbr, s, nd, hs);
                 }
                 const unsigned mt = __ballot_sync(FULL, r == 1);
                 const unsigned mw = __ballot_sync(FULL, r >= 1);
@@ -959,7 +814,7 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
     // whose walk has ended takes the next unwalked entry, so the lanes stay busy
     // however the chain lengths vary (a warp of a larger team claims entries
     // from a shared counter).
-    {
+    if constexpr (CONTACTS) {
         int cur = -1, yv = 0, s = 0, dy = 0;
         unsigned pos = 0, nprobe = 0;
         int next = 0;
@@ -987,7 +842,7 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
                     nprobe = 0;
                     if (yv != S.svtx[s] && is_defect(C, yv)) {
                         const int f = rank_of(S, C, yv);
-                        if (f >= 0 && f != s) pair_upsert<(NW > 1)>(S, C, s, f, dy);
+                        if (f >= 0 && f != s) pair_upsert(S, C, s, f, dy);
                     }
                 }
             }
@@ -1001,7 +856,7 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
                 } else {
                     if ((int)(k >> 32) == yv) {
                         const int s2 = (int)(unsigned)(k & 0xffffffffu);
-                        if (s2 != s) pair_upsert<(NW > 1)>(S, C, s, s2, dy + v);
+                        if (s2 != s) pair_upsert(S, C, s, s2, dy + v);
                     }
                     pos = (pos + 1) & C.hmask;
                 }
@@ -1011,12 +866,148 @@ __device__ void extend_many(const Slab &S, const Shot &C, int nx, Team<NW> &T) {
     T.sync();
 }
 
-// Grow one source's ball by one band.  Every thread of the team calls.
+// Grow one source's ball by one band, without contacts (path tracing).  Every
+// thread of the team calls.
 template <int NW>
 __device__ void extend_one(const Slab &S, const Shot &C, int s, Team<NW> &T) {
     if (T.tid() == 0) { S.xsrc[0] = s; S.xR[0] = max(S.src[s].sR, 0) + C.band; }
     T.sync();
-    extend_many(S, C, 1, T);
+    extend_many<false>(S, C, 1, T);
+}
+
+// From here on the shot explores balls: the listed pairs enter the pair hash,
+// and every source with a virtual ball gets the ball of that radius.  Every
+// thread of the team calls.
+template <int NW>
+__device__ __noinline__ void go_real(const Slab &S, Shot &C, Team<NW> T) {
+    C.real = 1;
+    const int np = T.bcast(ldr(&S.ctr[C_NPAIRS]));
+    if (np > C.pcap || (unsigned)np * 2u > C.pmask) {
+        if (T.tid() == 0) set_err(S, ERR_CAP);
+        T.sync();
+        return;
+    }
+    T.sync();
+    if (T.tid() == 0) S.ctr[C_WL] = 0;
+    for (int i = T.tid(); i < np; i += T.NT) {
+        const int4 q = ld_pr(&S.pr[i]);
+        const unsigned long long key = ((unsigned long long)(unsigned)q.x << 32) | (unsigned)q.y;
+        unsigned h = pslot(q.x, q.y, C.pmask);
+        for (unsigned n = 0; n <= C.pmask; n++) {
+            unsigned long long k, w;
+            if (claim_pair(&S.pt[h], key, q.z, i, k, w)) { S.pr[i].slot = (int)h; break; }
+            if (k == key) { S.pr[i].lo = -1; break; }   // listed from both ends, at the same distance
+            h = (h + 1) & C.pmask;
+        }
+    }
+    T.sync();
+    for (int s = T.tid(); s < C.K; s += T.NT) {
+        const int r = S.src[s].sR;
+        if (r < 0) continue;
+        const int k = atomicAdd(&S.ctr[C_WL], 1);
+        S.xsrc[k] = s;
+        S.xR[k] = r;
+        S.src[s].sR = -1;
+    }
+    T.sync();
+    const int nx = T.bcast(ldr(&S.ctr[C_WL]));
+    T.sync();
+    extend_many<true>(S, C, nx, T);
+}
+
+// Radius within which every other detection event of source s has to be known
+// once its ball has radius R: no region with a smaller ball can be touched
+// farther away (Rad <= R - L for explored regions, Rad <= b1 / 2 for level-1
+// configurations never explored).
+__device__ __forceinline__ int reach_of(const Shot &C, int R) {
+    const int r = R - C.L;
+    return r + max(r, (C.g.b1 + 1) >> 1);
+}
+
+// EXTEND: every growing region whose radius has come within L of its explored
+// radius gets a larger ball.  While the ball table covers the radius that
+// matters (reach_of) the ball stays virtual: the events within that radius
+// are read off the table's list of the source's vertex (nothing at all when
+// the pairs within b1, listed at the start of the shot, already cover it).
+// Otherwise the shot goes over to explored balls.  The table's radius (balls.cu:
+// four largest weights) lets a region's radius grow to two edges before that;
+// a shot gains a band each time exactly when it would with explored balls, so
+// the diagnostics do not depend on which is used.  Returns the number of due
+// regions.  Every thread of the team calls; ends with a barrier.
+template <int NW>
+__device__ int extend_due(const Slab &S, Shot &C, Team<NW> &T) {
+    const DGraph &g = C.g;
+    for (;;) {
+        // the list counter is zero on entry (cleared ahead of the event
+        // search's barrier)
+        int any = 0;   // bit 0: a region is due, bit 1: one is beyond the table
+        for (int s = T.tid(); s < C.K; s += T.NT) {
+            const int4 r = ld_src(&S.src[s]);
+            const int rad = r.y, sR = r.z;
+            if (!rec_inplay(r) || rec_sexh(r) || sR - C.L + 1 - rad > 0 || S.nd[r.x].label != 1) continue;
+            const int R = max(sR + C.band, rad + C.L + C.band);
+            any |= 1;
+            if (!C.real) {
+                const int q = reach_of(C, R);
+                if (sR < 0 && q <= g.b1) { S.src[s].sR = R; continue; }
+                if (q > g.brad || sR > g.brad - g.wmax || __ldg(g.bhdr + S.svtx[s]).w < 0) { any |= 2; continue; }
+            }
+            const int k = atomicAdd(&S.ctr[C_WL], 1);
+            S.xsrc[k] = s;
+            S.xR[k] = R;
+        }
+        any = T.template red32<2>(any);
+        if constexpr (NW == 1) T.sync();
+        if (any & 2) {
+            go_real(S, C, T);
+            if (T.tid() == 0) S.ctr[C_WL] = 0;
+            T.sync();
+            if (T.bcast(ldr(&S.ctr[C_ERR]))) return any;
+            continue;
+        }
+        const int nx = T.bcast(ldr(&S.ctr[C_WL]));
+        if (C.real) {
+            T.sync();
+            extend_many<true>(S, C, nx, T);
+            return any;
+        }
+        for (int i = T.warp(); i < nx; i += NW) {
+            const int s = S.xsrc[i], R = S.xR[i], sR = S.src[s].sR;
+            const int v = S.svtx[s];
+            const int4 h = __ldg(g.bhdr + v);
+            const int q = reach_of(C, R), q0 = sR < 0 ? g.b1 : max(g.b1, reach_of(C, sR));
+            const int n = h.z + h.w;
+            bool more = false;
+            for (int k = 0; k < n; k += WS) {
+                bool hit = false;
+                int2 e = make_int2(0, 0);
+                if (k + T.lane < n) {
+                    e = __ldg(g.ball + (unsigned)h.x + k + T.lane);
+                    more |= e.y > sR;
+                    hit = e.y > q0 && e.y <= q && is_defect(C, e.x);
+                }
+                const unsigned m = __ballot_sync(FULL, hit);
+                if (!m) continue;
+                int b = 0;
+                if (T.lane == 0) b = atomicAdd(&S.ctr[C_NPAIRS], __popc(m));
+                b = __shfl_sync(FULL, b, 0);
+                if (hit) {
+                    const int j = b + __popc(m & ((1u << T.lane) - 1u));
+                    const int f = rank_of(S, C, e.x);
+                    if (j < C.pcap) S.pr[j] = PRec{min(s, f), max(s, f), (unsigned)e.y, -1};
+                    else set_err(S, ERR_CAP);
+                }
+            }
+            // a ball that gains no vertex has covered its component
+            more = __any_sync(FULL, more);
+            if (T.lane == 0) {
+                S.src[s].sR = R;
+                if (sR >= 0 && !more) S.src[s].sexh = 1;
+            }
+        }
+        T.sync();
+        return any;
+    }
 }
 
 // ---------------------------------------------------------------- matcher --
@@ -1301,16 +1292,9 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
             }
         };
         auto pair_item = [&](int i) {
-            int a, b, pv;
-            if constexpr (NW == 1) {
-                unsigned long long k;
-                ld_ent(&S.pt[S.plist[i]], k, pv);
-                a = (int)(k >> 32); b = (int)(unsigned)(k & 0xffffffffu);
-            } else {   // the pair's record: one round trip less
-                const int4 pq = ld_pr(&S.pr[i]);
-                a = pq.x; b = pq.y; pv = pq.z;
-                if (a < 0) return;
-            }
+            const int4 pq = ld_pr(&S.pr[i]);
+            const int a = pq.x, b = pq.y, pv = pq.z;
+            if (a < 0) return;
             const int4 qa = ld_src(&S.src[a]), qb = ld_src(&S.src[b]);
             const int ia = rec_inplay(qa), ib = rec_inplay(qb), A = qa.x, B = qb.x;
             const int ra = qa.y, rb = qb.y;
@@ -1345,11 +1329,9 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
                 else node_item(j - np);
             }
         }
-        // a block resets the EXTEND list counter ahead of the reduction's
-        // barrier (nothing uses it between ball extensions)
-        if constexpr (NW > 1) {
-            if (T.tid() == 0) S.ctr[C_WL] = 0;
-        }
+        // the EXTEND list counter is reset ahead of the reduction's barrier
+        // (nothing uses it between ball extensions)
+        if (T.tid() == 0) S.ctr[C_WL] = 0;
         T.reduce_ev(best, flags, inner_leaf_min);
         if (flags & 2) return RUN_INTERNAL;
         if (!(flags & 1)) return RUN_OK;
@@ -1390,27 +1372,7 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
         // one warp keeps its barrier here.
         if constexpr (NW == 1) T.sync();
         if (kind == EV_EXTEND) {
-            // every growing region that reached its explored radius now.  In a
-            // block the counter is already zero, and each thread reads only the
-            // radii it updated itself (same striding as the dual update)
-            if constexpr (NW == 1) {
-                if (T.tid() == 0) S.ctr[C_WL] = 0;
-                T.sync();
-            }
-            for (int s = T.tid(); s < C.K; s += T.NT) {
-                const int4 r = ld_src(&S.src[s]);
-                const int rad = r.y;
-                if (rec_inplay(r) && !rec_sexh(r) && S.nd[r.x].label == 1 && r.z - C.L + 1 - rad <= 0) {
-                    const int k = atomicAdd(&S.ctr[C_WL], 1);
-                    S.xsrc[k] = s;
-                    S.xR[k] = max(r.z + C.band, rad + C.L + C.band);
-                }
-            }
-            T.sync();
-            // after the barrier the counter stays unchanged until extend_many's
-            // own first barrier: every thread reads the same count
-            if constexpr (NW == 1) extend_many(S, C, T.bcast(ldr(&S.ctr[C_WL])), T);
-            else extend_many(S, C, ldr(&S.ctr[C_WL]), T);
+            extend_due(S, C, T);
         } else if (kind == EV_IMPLODE) {
             // the blossom is read by every thread before any thread's shatter
             // loop rewrites the stop pointers
@@ -1449,12 +1411,82 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
     }
 }
 
-// Canonical path observable from source s (its Dijkstra tree) to vertex x at
-// distance dx: predecessor = lowest edge id among tight edges.  Every thread
-// of the team calls.
-template <int NW>
-__device__ unsigned long long path_obs(const Slab &S, Shot &C, int s, int x, int dx, Team<NW> &T) {
+__device__ __forceinline__ bool in_commit(const DGraph &g, int v) {
+    return (__ldg(g.commit + (v >> 5)) >> (v & 31)) & 1u;
+}
+
+// One edge (cur, nxt, id e) of a path: its observables (COMMIT: only when the
+// edge touches the commit region, and an endpoint outside the region is
+// flipped in `carry`, by the calling thread).
+template <bool COMMIT>
+__device__ __forceinline__ unsigned long long path_edge(const DGraph &g, int cur, int nxt, int e, bool writer,
+                                                        unsigned *carry) {
+    if constexpr (COMMIT) {
+        const bool ci = in_commit(g, cur), ni = in_commit(g, nxt);
+        if (!ci && !ni) return 0;
+        if (ci != ni && writer) {
+            const int out = ci ? nxt : cur;
+            atomicXor(&carry[out >> 5], 1u << (out & 31));
+        }
+    }
+    return __ldg(g.eobs + e);
+}
+
+// Canonical path from vertex src (its Dijkstra tree) to vertex x at distance
+// dx: predecessor = lowest edge id among tight edges.  Distances come from
+// src's list in the ball table, which must cover dx.  One warp; every lane
+// returns the XOR of the path's observables (path_edge).
+template <bool COMMIT>
+__device__ unsigned long long walk_table(const Slab &S, const DGraph &g, int src, int4 h, int x, int dx, int lane,
+                                         unsigned *carry) {
+    unsigned long long o = 0;
+    const int n = h.z + max(h.w, 0);
+    int cur = x, dcur = dx;
+    for (int step = 0; step < 1 << 22 && cur != src; step++) {
+        const int r0 = __ldg(g.row + cur), deg = __ldg(g.row + cur + 1) - r0;
+        unsigned long long best = EMPTY64;
+        int dbest = INF32;
+        for (int j0 = 0; j0 < deg; j0 += WS) {
+            const int j = j0 + lane, nq = min(WS, deg - j0);
+            SlotV sl;
+            sl.nbr = -1; sl.w = 0; sl.eid = -1;
+            if (j < deg) sl = load_slot(g, r0 + j);
+            int dy = sl.nbr == src ? 0 : INF32;
+            for (int k = 0; k < n; k += WS) {
+                int2 e = make_int2(-2, 0);
+                if (k + lane < n) e = __ldg(g.ball + (unsigned)h.x + k + lane);
+                for (int q = 0; q < nq; q++) {
+                    const int y = __shfl_sync(FULL, sl.nbr, q);
+                    const unsigned m = __ballot_sync(FULL, e.x == y);
+                    if (!m) continue;
+                    const int d = __shfl_sync(FULL, e.y, __ffs(m) - 1);
+                    if (lane == q) dy = d;
+                }
+            }
+            unsigned long long key = EMPTY64;
+            if (sl.nbr >= 0 && dy != INF32 && dy + sl.w == dcur)
+                key = ((unsigned long long)(unsigned)__ldg(g.seid + r0 + j) << 32) | (unsigned)sl.nbr;
+            const unsigned long long kb = warp_min64(key);
+            if (kb < best) {
+                best = kb;
+                dbest = __shfl_sync(FULL, dy, __ffs(__ballot_sync(FULL, key == kb)) - 1);
+            }
+        }
+        if (best == EMPTY64) { if (lane == 0) set_err(S, ERR_INTERNAL); break; }
+        const int nxt = (int)(unsigned)(best & 0xffffffffu);
+        o ^= path_edge<COMMIT>(g, cur, nxt, (int)(best >> 32), lane == 0, carry);
+        cur = nxt;
+        dcur = dbest;
+    }
+    return o;
+}
+
+// The same from source s through its explored ball, which grows until it holds
+// dx.  Every thread of the team calls.
+template <bool COMMIT, int NW>
+__device__ unsigned long long walk_ball(const Slab &S, Shot &C, int s, int x, int dx, Team<NW> &T, unsigned *carry) {
     const DGraph &g = C.g;
+    C.paths = 1;
     for (int n = 0; n < 1 << 16; n++) {
         const int more = S.src[s].sR < dx && !S.src[s].sexh && !ldr(&S.ctr[C_ERR]);
         if (!T.bcast(more)) break;
@@ -1477,20 +1509,57 @@ __device__ unsigned long long path_obs(const Slab &S, Shot &C, int s, int x, int
         }
         best = T.min64(best);
         if (best == EMPTY64) { if (T.tid() == 0) S.ctr[C_ERR] |= ERR_INTERNAL; break; }
-        const int e = (int)(best >> 32);
-        o ^= __ldg(g.eobs + e);
-        cur = (int)(unsigned)(best & 0xffffffffu);
+        const int nxt = (int)(unsigned)(best & 0xffffffffu);
+        o ^= path_edge<COMMIT>(g, cur, nxt, (int)(best >> 32), T.tid() == 0, carry);
+        cur = nxt;
         dcur = ht_get(S, C, cur, s);
     }
     T.sync();
     return o;
 }
 
-// Expand the final matching into leaf-level pairs (tmpa[i], tmpb[i]; tmpb = -1
-// for a boundary match) and accumulate weight (internal units) and obs.
+// Distance of two matched events: their edge is tight, so it is the sum of
+// their radii less twice the duals of the blossoms that hold both.
+__device__ int tight_dist(const Slab &S, int a, int b) {
+    int d = S.src[a].srad + S.src[b].srad;
+    for (int B = S.nd[a].bpar; B >= 0; B = S.nd[B].bpar) {
+        int x = S.nd[b].bpar;
+        while (x >= 0 && x != B) x = S.nd[x].bpar;
+        if (x == B) {
+            for (; B >= 0; B = S.nd[B].bpar) d -= 2 * S.nd[B].y;
+            break;
+        }
+    }
+    return d;
+}
+
+// Weight (internal units) and observable of the final matching.  Every matched
+// edge is tight and every set with a dual has exactly one matched edge leaving
+// it, so the weight is the sum of all duals; the observable is that of the
+// boundary matches' edges, which the matched top-level nodes name.
 template <int NW>
-__device__ __noinline__ void trace(const Slab &S, Shot &C, Team<NW> T, int nhi, long long &wint,
-                                   unsigned long long &obs) {
+__device__ __forceinline__ void total(const Slab &S, const Shot &C, Team<NW> &T, int nhi, long long &wint,
+                                      unsigned long long &obs) {
+    long long w = 0;
+    unsigned long long o = 0;
+    for (int v = T.tid(); v < nhi; v += T.NT) {
+        const int4 q = ld_nd(&S.nd[v]);
+        if (!q.w) continue;
+        w += q.x;
+        if (q.y < 0 && S.mate[v] == MATE_BOUNDARY) {
+            const unsigned long long bb = S.sbnd[S.ms[v]];
+            if (bb == EMPTY64) set_err(S, ERR_INTERNAL);
+            else o ^= __ldg(C.g.eobs + (int)(unsigned)(bb & 0xffffffffu));
+        }
+    }
+    wint = T.sum64(w);
+    obs = T.xor64(o);
+}
+
+// Expand the final matching into leaf-level pairs (tmpa[i], tmpb[i]; tmpb = -1
+// for a boundary match); returns their number.
+template <int NW>
+__device__ int expand(const Slab &S, Shot &C, Team<NW> &T, int nhi) {
     // matched top-level nodes, team-parallel: each match appends its leaf pair
     // and queues the blossoms on either side for expansion (stack seeds)
     if (T.tid() == 0) { S.ctr[C_TNP] = 0; S.ctr[C_TNX] = 0; }
@@ -1536,124 +1605,81 @@ __device__ __noinline__ void trace(const Slab &S, Shot &C, Team<NW> T, int nhi, 
                 stk[sp++] = S.cnode[cb + i2]; stk[sp++] = lz;
             }
         }
+        S.ctr[C_TNX] = 0;
     }
-    np = T.bcast(np);
-    T.sync();
-    if (T.tid() == 0) S.ctr[C_TNP] = np;   // leaf pairs in tmpa / tmpb, read by commit_trace
-    long long w = 0;
-    unsigned long long o = 0;
-    for (int i = T.tid(); i < np; i += T.NT) {
-        const int a = S.tmpa[i], b = S.tmpb[i];
-        if (a < 0 || a >= C.K || b >= C.K) { set_err(S, ERR_INTERNAL); continue; }
-        if (b < 0) {
-            const unsigned long long bb = ldr(&S.sbnd[a]);
-            if (bb == EMPTY64) { set_err(S, ERR_INTERNAL); continue; }
-            w += (long long)(bb >> 32);
-            o ^= __ldg(C.g.eobs + (int)(unsigned)(bb & 0xffffffffu));
-        } else {
-            const int d = pair_get(S, C, a, b);
-            if (d == INF32) { set_err(S, ERR_INTERNAL); continue; }
-            w += d;
-        }
-    }
-    w = T.sum64(w);
-    o = T.xor64(o);
-    if (C.g.internal_obs && !T.bcast(ldr(&S.ctr[C_ERR]))) {
-        // detector-detector edges carry observables: walk the canonical paths
-        for (int i = 0; i < np; i++) {
-            const int a = S.tmpa[i], b = S.tmpb[i];
-            if (b < 0) {
-                const unsigned long long bb = ldr(&S.sbnd[a]);
-                const int e = (int)(unsigned)(bb & 0xffffffffu);
-                const int2 ue = __ldg(C.g.eend + e);
-                o ^= path_obs(S, C, a, ue.x, (int)(bb >> 32) - ue.y, T);
-            } else {
-                const int lo = min(a, b), hi = max(a, b);
-                o ^= path_obs(S, C, lo, S.svtx[hi], pair_get(S, C, lo, hi), T);
-            }
-        }
-    }
-    wint = w;
-    obs = o;
-    T.sync();
+    return T.bcast(np);
 }
 
-__device__ __forceinline__ bool in_commit(const DGraph &g, int v) {
-    return (__ldg(g.commit + (v >> 5)) >> (v & 31)) & 1u;
-}
-
-// Canonical path from source s's vertex to vertex x at distance dx (the path
-// of path_obs): the XOR of the observables of its edges that touch the commit
-// region; each such edge with its other endpoint outside the region flips that
-// endpoint in `carry` (thread 0 writes).  Every thread of the team calls.
-template <int NW>
-__device__ unsigned long long path_commit(const Slab &S, Shot &C, int s, int x, int dx, Team<NW> &T,
-                                          unsigned *carry) {
+// Walk the canonical paths of the final matching.  COMMIT (sliding windows):
+// the correction is the union of those paths and of the boundary edges; every
+// edge that touches the graph's commit region is committed, and the shot's
+// carry row receives the detectors outside the region flipped by committed
+// edges.  Otherwise `obs` gains the observables of detector-detector edges.
+// A path within the ball table's reach is walked by one warp; one that cannot
+// leave its side of the region's border (g.seam) commits nothing but its
+// observables, and is not walked when those edges carry none.  Farther paths
+// are walked through explored balls.  Every thread of the team calls.
+template <bool COMMIT, int NW>
+__device__ __noinline__ unsigned long long walk_paths(const Slab &S, Shot &C, Team<NW> T, int nhi, unsigned *carry) {
     const DGraph &g = C.g;
-    for (int n = 0; n < 1 << 16; n++) {
-        const int more = S.src[s].sR < dx && !S.src[s].sexh && !ldr(&S.ctr[C_ERR]);
-        if (!T.bcast(more)) break;
-        extend_one(S, C, s, T);
-    }
-    // a ball that outgrew the tables: the attempt is retried with larger ones
+    const int np = expand(S, C, T, nhi);
+    if constexpr (COMMIT)
+        for (int w = T.tid(); w < g.words; w += T.NT) carry[w] = 0u;
+    if (!C.real)   // no ball is explored yet
+        for (int s = T.tid(); s < C.K; s += T.NT) { S.src[s].sR = -1; S.src[s].sexh = 0; }
+    T.sync();
     if (T.bcast(ldr(&S.ctr[C_ERR]))) return 0;
-    unsigned long long o = 0;
-    const int src = S.svtx[s];
-    int cur = x, dcur = dx;
-    for (int n = 0; n < 1 << 22 && cur != src; n++) {
-        const int r0 = __ldg(g.row + cur), r1 = __ldg(g.row + cur + 1);
-        unsigned long long best = EMPTY64;
-        for (int j = r0 + T.tid(); j < r1; j += T.NT) {
-            SlotV sl = load_slot(g, j);
-            if (sl.nbr < 0) continue;
-            const int dy = ht_get(S, C, sl.nbr, s);
-            if (dy != INF32 && dy + sl.w == dcur)
-                best = min(best, ((unsigned long long)(unsigned)__ldg(g.seid + j) << 32) | (unsigned)sl.nbr);
-        }
-        best = T.min64(best);
-        if (best == EMPTY64) { if (T.tid() == 0) S.ctr[C_ERR] |= ERR_INTERNAL; break; }
-        const int e = (int)(best >> 32);
-        const int nxt = (int)(unsigned)(best & 0xffffffffu);
-        const bool ci = in_commit(g, cur), ni = in_commit(g, nxt);
-        if (ci || ni) {
-            o ^= __ldg(g.eobs + e);
-            if (ci != ni && T.tid() == 0) {
-                const int out = ci ? nxt : cur;
-                carry[out >> 5] ^= 1u << (out & 31);
+    unsigned long long mine = 0, whole = 0;   // found by this lane / by this warp together
+    for (int base = T.warp() * WS; base < np; base += T.NT) {
+        const int i = base + T.lane;
+        int v = 0, x = 0, dx = 0;
+        int4 h = make_int4(0, 0, 0, 0);
+        bool walk = false;
+        if (i < np) {
+            const int a = S.tmpa[i], b = S.tmpb[i];
+            int s = a;
+            if (b < 0) {
+                const unsigned long long bb = S.sbnd[a];
+                const int e = (int)(unsigned)(bb & 0xffffffffu);
+                const int2 ue = __ldg(g.eend + e);
+                x = ue.x;
+                dx = (int)(bb >> 32) - ue.y;
+                if constexpr (COMMIT) if (in_commit(g, x)) mine ^= __ldg(g.eobs + e);   // the boundary edge itself
+            } else {
+                s = min(a, b);
+                x = S.svtx[max(a, b)];
+                dx = tight_dist(S, a, b);
+            }
+            v = S.svtx[s];
+            bool skip = false;
+            if constexpr (COMMIT) skip = dx < __ldg(g.seam + v) && (!g.internal_obs || !in_commit(g, v));
+            h = __ldg(g.bhdr + v);
+            const int cover = h.w >= 0 ? g.brad : (h.z >= 0 ? g.b1 : -1);
+            if (!skip && dx > 0) {
+                walk = dx <= cover;
+                if (!walk) S.stk[atomicAdd(&S.ctr[C_TNX], 1)] = i;
             }
         }
-        cur = nxt;
-        dcur = ht_get(S, C, cur, s);
+        for (unsigned m = __ballot_sync(FULL, walk); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const int4 hl = make_int4(__shfl_sync(FULL, h.x, l), 0, __shfl_sync(FULL, h.z, l), __shfl_sync(FULL, h.w, l));
+            whole ^= walk_table<COMMIT>(S, g, __shfl_sync(FULL, v, l), hl, __shfl_sync(FULL, x, l),
+                                        __shfl_sync(FULL, dx, l), T.lane, carry);
+        }
     }
     T.sync();
-    return o;
-}
-
-// Sliding-window commit of a decoded shot (the leaf pairs left by trace): the
-// correction is the union of the canonical matching paths (and boundary
-// edges); every edge that touches the graph's commit region is committed.
-// Returns the committed observable; the shot's carry row receives the
-// detectors outside the region flipped by committed edges.  Every thread of
-// the team calls.
-template <int NW>
-__device__ __noinline__ unsigned long long commit_trace(const Slab &S, Shot &C, Team<NW> T, unsigned *carry) {
-    const DGraph &g = C.g;
-    for (int w = T.tid(); w < g.words; w += T.NT) carry[w] = 0u;
-    T.sync();
-    const int np = T.bcast(ldr(&S.ctr[C_TNP]));
-    unsigned long long o = 0;
-    for (int i = 0; i < np; i++) {
+    unsigned long long o = T.xor64(mine ^ (T.lane == 0 ? whole : 0));
+    const int nfar = T.bcast(ldr(&S.ctr[C_TNX]));
+    for (int k = 0; k < nfar; k++) {
         if (T.bcast(ldr(&S.ctr[C_ERR]))) break;
+        const int i = S.stk[k];
         const int a = S.tmpa[i], b = S.tmpb[i];
         if (b < 0) {
-            const unsigned long long bb = ldr(&S.sbnd[a]);
-            const int e = (int)(unsigned)(bb & 0xffffffffu);
-            const int2 ue = __ldg(g.eend + e);
-            if (in_commit(g, ue.x)) o ^= __ldg(g.eobs + e);   // the boundary edge itself
-            o ^= path_commit(S, C, a, ue.x, (int)(bb >> 32) - ue.y, T, carry);
+            const unsigned long long bb = S.sbnd[a];
+            const int2 ue = __ldg(g.eend + (int)(unsigned)(bb & 0xffffffffu));
+            o ^= walk_ball<COMMIT>(S, C, a, ue.x, (int)(bb >> 32) - ue.y, T, carry);
         } else {
-            const int lo = min(a, b), hi = max(a, b);
-            o ^= path_commit(S, C, lo, S.svtx[hi], pair_get(S, C, lo, hi), T, carry);
+            o ^= walk_ball<COMMIT>(S, C, min(a, b), S.svtx[max(a, b)], tight_dist(S, a, b), T, carry);
         }
     }
     T.sync();
@@ -1674,23 +1700,15 @@ template <int NW>
 __device__ __noinline__ void release_tables(const Slab &S, const Shot &C, Team<NW> T, bool all) {
     T.sync();
     const HEnt e = HEnt{EMPTY64, -1, -1};
-    const PRec pe = PRec{-1, -1, ~0u, -1};
     if (all) {
         for (unsigned i = T.tid(); i <= C.hmask; i += T.NT) S.ht[i] = e;
         for (unsigned i = T.tid(); i <= C.pmask; i += T.NT) S.pt[i] = e;
-        if constexpr (NW > 1)
-            for (unsigned i = T.tid(); i <= (C.pmask >> 1); i += T.NT) S.pr[i] = pe;
     } else {
-        const int ne = ldr(&S.ctr[C_ECOUNT]), np = ldr(&S.ctr[C_NPAIRS]);
+        const int ne = ldr(&S.ctr[C_ECOUNT]), np = min(ldr(&S.ctr[C_NPAIRS]), C.pcap);
         for (int i = T.tid(); i < ne; i += T.NT) S.ht[S.ent[i] & C.hmask] = e;
-        if constexpr (NW == 1) {
-            for (int i = T.tid(); i < np; i += T.NT) S.pt[S.plist[i] & C.pmask] = e;
-        } else {
-            for (int i = T.tid(); i < np; i += T.NT) {
-                const int sl = S.pr[i].slot;
-                if (sl >= 0) S.pt[sl & C.pmask] = e;
-                S.pr[i] = pe;
-            }
+        for (int i = T.tid(); i < np; i += T.NT) {
+            const int sl = S.pr[i].slot;
+            if (sl >= 0) S.pt[sl & C.pmask] = e;
         }
     }
     T.sync();
@@ -1750,130 +1768,86 @@ __device__ int load_defects(const Slab &S, const DGraph &g, const unsigned *row,
     return K > kcap ? -1 : K;
 }
 
-constexpr int LB_CAP = 64;   // vertices one lane holds while exploring one event
-
-// Lane-local bounded Dijkstra from event s to radius Rb (one lane, no shared
-// tables): records every other event within Rb through pair_upsert (from the
-// lower-ranked end only) and the canonical boundary candidate of s.  Returns
-// the number of vertices settled, or -1 if more than LB_CAP lie within Rb.
-template <bool REC>
-__device__ __noinline__ int local_ball(const Slab &S, const Shot &C, int s, int Rb) {
-    const DGraph &g = C.g;
-    int vv[LB_CAP], dd[LB_CAP];
-    unsigned long long fin = 0;   // settled flags
-    const int src = S.svtx[s];
-    int n = 1;
-    vv[0] = src;
-    dd[0] = 0;
-    unsigned long long bbest = EMPTY64;
-    int settled = 0;
-    for (int it = 0; it < LB_CAP; it++) {
-        int bi = -1, bd = INT_MAX;
-        for (int i = 0; i < n; i++)
-            if (!((fin >> i) & 1ull) && dd[i] < bd) { bd = dd[i]; bi = i; }
-        if (bi < 0) break;
-        fin |= 1ull << bi;
-        settled++;
-        const int x = vv[bi], dx = bd;
-        if (x != src && is_defect(C, x)) {
-            const int f = rank_of(S, C, x);
-            if (f > s) pair_upsert<REC>(S, C, s, f, dx);
-        }
-        const int r0 = __ldg(g.row + x), r1 = __ldg(g.row + x + 1);
-        for (int j = r0; j < r1; j++) {
-            const SlotV sl = load_slot(g, j);
-            const int nd = dx + sl.w;
-            if (sl.nbr < 0) {
-                const unsigned long long c = ((unsigned long long)(unsigned)nd << 32) | (unsigned)sl.eid;
-                bbest = c < bbest ? c : bbest;
-                continue;
-            }
-            if (nd > Rb) continue;
-            int k = 0;
-            while (k < n && vv[k] != sl.nbr) k++;
-            if (k < n) {
-                if (!((fin >> k) & 1ull) && nd < dd[k]) dd[k] = nd;
-            } else {
-                if (n == LB_CAP) return -1;
-                vv[n] = sl.nbr;
-                dd[n] = nd;
-                n++;
-            }
-        }
-    }
-    atomicMin(&S.sbnd[s], bbest);
-    return settled;
-}
-
-// Level-1 neighbourhoods by enumeration, for graphs in which a path of length
-// <= Rb has at most two edges (DGraph::hop2): every event reached from event s
-// by a path of one or two edges of length <= Rb is recorded through
-// pair_upsert from the lower-ranked end (the minimum over those paths is the
-// exact distance, since the shortest path has at most two edges), and the
-// boundary candidates through s itself or a neighbour within Rb go to sbnd[s].
-// Same records as local_ball's for every use: pairs within Rb exactly, and the
-// canonical boundary contact whenever it lies within Rb / 2 (a longer contact
-// is only an upper bound, refined by the flooder before a region can reach
-// it).  One lane per (event, adjacency slot of the event), numbered by a warp
-// prefix sum of the degrees; the warps of a team take 32 events each in turn.
-// Every thread of the team calls (no team barrier inside).
+// Pairs of events within b_1, each once (from its lower-ranked end), read off
+// the ball table: one lane per (event, entry of its vertex's list of higher
+// vertices within b_1), numbered by a warp prefix sum of the list lengths; the
+// warps of a team take 32 events each in turn.  Numbering the entries keeps
+// every lane busy although the lists differ in length (12 on average, fewer at
+// the code's sides), and half of each neighbourhood is enough since a pair is
+// found from its lower end.  Also the events' boundary distances (canonical
+// boundary edge in the low word).  Returns (per thread) bit 0: an event's list
+// is not complete, bit 1: an event has more than LB_CAP vertices within b_1 on
+// a graph where b_1 spans more than two edges.  Every thread of the team
+// calls; ends with a barrier.
+constexpr int LB_CAP = 64;
 template <int NW>
-__device__ __noinline__ void level1_2hop(const Slab &S, const Shot &C, int Rb, const Team<NW> T) {
+__device__ __forceinline__ int near_pairs(const Slab &S, const Shot &C, Team<NW> &T) {
     const DGraph &g = C.g;
     const int lane = T.lane;
+    int flags = 0, np = 0;
     for (int base = T.warp() * WS; base < C.K; base += T.NT) {
         const int s = base + lane;
-        int src = -1, r0 = 0, deg = 0;
+        int beg = 0, len = 0;
         if (s < C.K) {
-            src = S.svtx[s];
-            r0 = __ldg(g.row + src);
-            deg = __ldg(g.row + src + 1) - r0;
+            const int v = S.svtx[s];
+            const int4 h = __ldg(g.bhdr + v);
+            S.sbnd[s] = __ldg(g.vbnd + v);
+            if (h.z < 0) {
+                flags |= 1;
+            } else {
+                beg = h.x;
+                len = h.y;
+                if (!g.hop2 && h.z >= LB_CAP) flags |= 2;
+            }
         }
-        int incl = deg;
+        int incl = len;
+#pragma unroll
         for (int o = 1; o < WS; o <<= 1) {
             const int v = __shfl_up_sync(FULL, incl, o);
             if (lane >= o) incl += v;
         }
         const int total = __shfl_sync(FULL, incl, WS - 1);
-        const int excl = incl - deg;
+        const int excl = incl - len;
         for (int t0 = 0; t0 < total; t0 += WS) {
             const int t = t0 + lane;
-            int ow = 0;
+            int ow = 0;   // owner: the last lane whose first entry number is <= t
+#pragma unroll
             for (int step = WS / 2; step > 0; step >>= 1) {
                 const int e = __shfl_sync(FULL, excl, ow + step);
                 if (e <= t) ow += step;
             }
-            const int osrc = __shfl_sync(FULL, src, ow);
-            const int oj = __shfl_sync(FULL, r0 - excl, ow) + t;
-            if (t >= total) continue;
-            const int os = base + ow;
-            const SlotV a = load_slot(g, oj);
-            if (a.nbr < 0) {
-                atomicMin(&S.sbnd[os], ((unsigned long long)(unsigned)a.w << 32) | (unsigned)a.eid);
-                continue;
+            const unsigned oj = (unsigned)__shfl_sync(FULL, beg - excl, ow) + (unsigned)t;
+            bool hit = false;
+            int2 e = make_int2(0, 0);
+            unsigned word = 0;
+            if (t < total) {
+                e = __ldg(g.ball + oj);
+                word = __ldg(C.row + (e.x >> 5));
+                hit = (word >> (e.x & 31)) & 1u;
             }
-            if (a.w > Rb) continue;
-            if (is_defect(C, a.nbr)) {
-                const int f = rank_of(S, C, a.nbr);
-                if (f > os) pair_upsert<(NW > 1)>(S, C, os, f, a.w);
+            const unsigned m = __ballot_sync(FULL, hit);
+            if (!m) continue;
+            int b;
+            if constexpr (NW == 1) {
+                b = np;
+                np += __popc(m);
+            } else {
+                b = 0;
+                if (lane == 0) b = atomicAdd(&S.ctr[C_NPAIRS], __popc(m));
+                b = __shfl_sync(FULL, b, 0);
             }
-            unsigned long long bbest = EMPTY64;
-            const int q0 = __ldg(g.row + a.nbr), q1 = __ldg(g.row + a.nbr + 1);
-            for (int k = q0; k < q1; k++) {
-                const SlotV b = load_slot(g, k);
-                const int nd = a.w + b.w;
-                if (b.nbr < 0) {
-                    const unsigned long long c = ((unsigned long long)(unsigned)nd << 32) | (unsigned)b.eid;
-                    bbest = c < bbest ? c : bbest;
-                    continue;
-                }
-                if (nd > Rb || b.nbr == osrc || !is_defect(C, b.nbr)) continue;
-                const int f = rank_of(S, C, b.nbr);
-                if (f > os) pair_upsert<(NW > 1)>(S, C, os, f, nd);
+            if (hit) {
+                const int j = b + __popc(m & ((1u << lane) - 1u));
+                const int f = S.wcum[e.x >> 5] + __popc(word & ((1u << (e.x & 31)) - 1u));
+                if (j < C.pcap) S.pr[j] = PRec{base + ow, f, (unsigned)e.y, -1};
+                else set_err(S, ERR_CAP);
             }
-            if (bbest != EMPTY64) atomicMin(&S.sbnd[os], bbest);
         }
     }
+    if constexpr (NW == 1)
+        if (lane == 0) S.ctr[C_NPAIRS] = np;
+    T.sync();
+    return flags;
 }
 
 // Decode one shot with hash tables scaled by `scale`; returns QEC_SHOT_* or -1
@@ -1893,6 +1867,8 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     C.row = row;
     C.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
     C.nm = 0; C.ncut = 0; C.tcut = 0; C.tlast = 0; C.nx = 0;
+    C.real = 0;
+    C.pcap = A.caps.phc >> 1;
     if (g.words > A.caps.wcap) return -2;
     int K = 0;
     if (T.warp() == 0) K = load_defects(S, g, row, A.caps.kc, A.caps.wcap, T.lane);
@@ -1922,7 +1898,6 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     int nhi = K;
     for (int s = T.tid(); s < K; s += T.NT) {
         S.src[s] = SRec{s, 0, -1, 0, 0, 0, 0}; S.scnt[s] = 0; S.sbeg[s] = 0;
-        S.sbnd[s] = EMPTY64;
         S.nd[s] = NRec{0, -1, 0, 0}; S.tpar[s] = -1;
         S.mate[s] = MATE_NONE; S.nroot[s] = -1; S.minleaf[s] = s; S.clen[s] = 0;
     }
@@ -1938,36 +1913,36 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     // resolved at level 1, events of all level-1 runs
     int t1 = 0, e1 = 0, ncl1 = 0, nres1 = 0, ntot = 0;
     int gr = K;   // next level-1 cluster (its lowest event) that needs the event loop
+    // every pair within b_1 and every boundary distance.  An event whose list
+    // is not complete needs explored balls from the start.
+    const int odd = T.template red32<2>(near_pairs(S, C, T));
+    const int Rbig = max(g.b1, C.band);   // level-1 ball of an event with many vertices within b_1
+    if ((odd & 1) || ((odd & 2) && reach_of(C, Rbig) > g.b1)) go_real(S, C, T);
     if (A.mode == QEC_MODE_HIERARCHICAL) {
-        // ---- Algorithm 1, level 1: every event's neighbourhood within b_1 by a
-        // lane-local Dijkstra (each lane its own events): pairs within b_1 with their
-        // exact distance (found by reaching the other event's vertex) and the
-        // canonical boundary candidate.  Events whose neighbourhood is too large for
-        // the lane go through the team-wide flooder instead.
-        bool any_big = false;
-        if (g.hop2) {
-            level1_2hop(S, C, g.b1, T);
-        } else {
+        // ---- Algorithm 1, level 1.  An event with more than LB_CAP vertices
+        // within b_1 gets its first ball here
+        if (odd) {
+            if (T.tid() == 0) S.ctr[C_WL] = 0;
+            T.sync();
             for (int s = T.tid(); s < K; s += T.NT) {
-                const int r = local_ball<(NW > 1)>(S, C, s, g.b1);
-                if (r < 0) { S.cst0[s] = 1; any_big = true; } else S.cst0[s] = 0;
-            }
-        }
-        T.sync();
-        if (T.any(any_big)) {
-            if (T.tid() == 0) {
-                int k = 0;
-                for (int s = 0; s < K; s++)
-                    if (S.cst0[s]) { S.xsrc[k] = s; S.xR[k] = max(g.b1, C.band); k++; }
-                S.ctr[C_WL] = k;
+                const int nb = __ldg(g.bhdr + S.svtx[s]).z;
+                if (nb >= 0 && (nb < LB_CAP || g.hop2)) continue;
+                if (!C.real) { S.src[s].sR = Rbig; continue; }
+                const int k = atomicAdd(&S.ctr[C_WL], 1);
+                S.xsrc[k] = s;
+                S.xR[k] = Rbig;
             }
             T.sync();
-            extend_many(S, C, T.bcast(ldr(&S.ctr[C_WL])), T);
+            const int nx = T.bcast(ldr(&S.ctr[C_WL]));
+            T.sync();
+            extend_many<true>(S, C, nx, T);
         }
-        {
-            const int err = T.bcast(ldr(&S.ctr[C_ERR]));
-            if (err) return (err & ERR_INTERNAL) ? QEC_SHOT_INTERNAL : -1;
-        }
+    }
+    {
+        const int err = T.bcast(ldr(&S.ctr[C_ERR]));
+        if (err) return (err & ERR_INTERNAL) ? QEC_SHOT_INTERNAL : -1;
+    }
+    if (A.mode == QEC_MODE_HIERARCHICAL) {
         const int npairs = T.bcast(ldr(&S.ctr[C_NPAIRS]));
         // connected components of pairs within b_1: min-label propagation
         for (int s = T.tid(); s < K; s += T.NT) { S.comp[s] = s; S.cst0[s] = 0; S.cst1[s] = 0; S.cst2[s] = 0; }
@@ -1975,8 +1950,9 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
         for (int round = 0; round <= K; round++) {
             bool changed = false;
             for (int i = T.tid(); i < npairs; i += T.NT) {
-                int a, b, pv;
-                if (!pair_at<NW>(S, i, a, b, pv) || pv > g.b1) continue;
+                const int4 pq = ld_pr(&S.pr[i]);
+                const int a = pq.x, b = pq.y;
+                if (a < 0 || pq.z > g.b1) continue;
                 const int la = ldr(&S.comp[a]), lb = ldr(&S.comp[b]);
                 if (la != lb) {
                     const int m = min(la, lb);
@@ -1995,16 +1971,17 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
             if (bb != EMPTY64 && 2LL * (long long)(bb >> 32) <= (long long)g.b1) atomicOr(&S.cst1[r], 1);
         }
         T.sync();
-        // pairs within d_1 inside a component; each such pair also names its
-        // two events as each other's partner (xcur is free until the flooder
-        // runs), which is the partner of an accepted two-event cluster
+        // pairs within d_1 inside a component; each such pair is also noted at
+        // its two events (xcur is free until the flooder runs): the pair of an
+        // accepted two-event cluster
         for (int i = T.tid(); i < npairs; i += T.NT) {
-            int a, b, pv;
-            if (!pair_at<NW>(S, i, a, b, pv) || pv > g.d1) continue;
+            const int4 pq = ld_pr(&S.pr[i]);
+            const int a = pq.x, b = pq.y;
+            if (a < 0 || pq.z > g.d1) continue;
             if (S.comp[a] == S.comp[b]) {
                 atomicAdd(&S.cst2[S.comp[a]], 1);
-                S.xcur[a] = b;
-                S.xcur[b] = a;
+                S.xcur[a] = i;
+                S.xcur[b] = i;
             }
         }
         T.sync();
@@ -2022,10 +1999,9 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
                 S.mate[s] = MATE_BOUNDARY; S.ms[s] = s; S.mo[s] = -1; S.src[s].stop = s; S.nroot[s] = -1;
                 t1 = max(t1, bd); ncl1++; nres1++;   // one boundary event at time bd
             } else if (size == 2) {
-                // partner: the other member (its pair is the cluster's one pair
-                // within d_1, recorded above)
-                const int other = S.xcur[s];
-                const int d = pair_get(S, C, s, other);
+                // the cluster's one pair within d_1
+                const int4 pq = ld_pr(&S.pr[S.xcur[s]]);
+                const int other = pq.x == s ? pq.y : pq.x, d = pq.z;
                 const long long ba = (long long)(S.sbnd[s] >> 32), bo = (long long)(S.sbnd[other] >> 32);
                 if (d / 2 <= ba && d / 2 <= bo) {
                     S.nd[s] = NRec{d / 2, -1, 0, 1}; S.src[s].srad = d / 2;
@@ -2087,9 +2063,11 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     }
     long long wint = 0;
     unsigned long long ob = 0;
-    trace(S, C, T, nhi, wint, ob);
+    total(S, C, T, nhi, wint, ob);
     if constexpr (WIN) {   // sliding window: the committed part
-        if (!T.bcast(ldr(&S.ctr[C_ERR]))) ob = commit_trace(S, C, T, A.carry + (row - A.syn));
+        ob = walk_paths<true>(S, C, T, nhi, A.carry + (row - A.syn));
+    } else if (g.internal_obs) {   // detector-detector edges carry observables
+        ob ^= walk_paths<false>(S, C, T, nhi, nullptr);
     }
     const int err = T.bcast(ldr(&S.ctr[C_ERR]));
     if (err) return (err & ERR_INTERNAL) ? QEC_SHOT_INTERNAL : -1;
@@ -2121,10 +2099,11 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
                               unsigned scale, unsigned long long deadline, long long &w_out,
                               unsigned long long &o_out, int *dg) {
     Shot C;
-    C.hmask = 0;
-    C.pmask = 0;
+    C.real = 0;
+    C.paths = 0;
     const int st = decode_attempt_body<WIN, NW>(A, S, g, row, T, scale, deadline, w_out, o_out, dg, C);
-    if (C.hmask) release_tables(S, C, T, st != QEC_SHOT_OK);
+    // (the tables are used by explored balls only)
+    if (C.real || C.paths) release_tables(S, C, T, st != QEC_SHOT_OK);
     return st;
 }
 

@@ -2,6 +2,7 @@
 // kernels (decoder.cu).  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -33,6 +34,17 @@ struct DGraph {
     const int2 *eend;                 // [merged edges]: (lower detector endpoint, internal weight)
     const int *seid;                  // [row[n]]: merged edge id of every slot
     const unsigned *commit;           // [words]: detectors of the commit region (sliding windows), or NULL
+    const int *seam;                  // [n]: bound on the distance to the other side of the region's border, or NULL
+    // [n]: canonical boundary candidate of a detector: distance to the nearest
+    // boundary vertex << 32 | lowest merged id among the boundary edges at that
+    // distance; all ones when no boundary is reachable
+    const unsigned long long *vbnd;
+    // ball table (balls.cu): header {first entry, higher detectors within b1,
+    // detectors within b1 (-1: list not complete), detectors beyond b1 within
+    // brad (-1: not complete)} of every detector, entries {detector, distance}
+    const int4 *bhdr;
+    const int2 *ball;
+    int brad;
 };
 
 // Capacities of one warp's slab (per-shot working set).
@@ -84,6 +96,13 @@ struct BatchArgs {
     // a system-wide fence, once a shot's final results are written, or NULL
     int *done;
 };
+
+// Build the ball table of g (row, slot, n, b1, wmax set) on the current device
+// and set g's bhdr, ball and brad; the arrays are the caller's to free, also
+// after an error.  Detectors whose ball is too large get an incomplete header.
+cudaError_t build_ball_table(DGraph &g, int4 **hdr, int2 **ball);
+// Seam distances of a commit region (device bitmap) into seam[n].
+cudaError_t build_seam(const DGraph &g, const unsigned *commit, int *seam);
 
 long long slab_bytes_for(const SlabCaps &c);
 // Slab capacities for `kcap` detection events; hash tables and entry lists get
