@@ -1556,8 +1556,8 @@ __device__ __forceinline__ void total(const Slab &S, const Shot &C, Team<NW> &T,
     obs = T.xor64(o);
 }
 
-// Expand the final matching into leaf-level pairs (tmpa[i], tmpb[i]; tmpb = -1
-// for a boundary match); returns their number.
+// Expand the final matching into leaf-level pairs (tmpa[i], tmpb[i] at distance
+// cst2[i]; tmpb = -1 for a boundary match); returns their number.
 template <int NW>
 __device__ int expand(const Slab &S, Shot &C, Team<NW> &T, int nhi) {
     // matched top-level nodes, team-parallel: each match appends its leaf pair
@@ -1605,30 +1605,51 @@ __device__ int expand(const Slab &S, Shot &C, Team<NW> &T, int nhi) {
                 stk[sp++] = S.cnode[cb + i2]; stk[sp++] = lz;
             }
         }
-        S.ctr[C_TNX] = 0;
     }
-    return T.bcast(np);
+    np = T.bcast(np);
+    T.sync();
+    for (int i = T.tid(); i < np; i += T.NT)   // boundary matches: the boundary distance
+        S.cst2[i] = S.tmpb[i] < 0 ? (int)(S.sbnd[S.tmpa[i]] >> 32) : tight_dist(S, S.tmpa[i], S.tmpb[i]);
+    T.sync();
+    return np;
 }
 
-// Walk the canonical paths of the final matching.  COMMIT (sliding windows):
-// the correction is the union of those paths and of the boundary edges; every
-// edge that touches the graph's commit region is committed, and the shot's
-// carry row receives the detectors outside the region flipped by committed
-// edges.  Otherwise `obs` gains the observables of detector-detector edges.
-// A path within the ball table's reach is walked by one warp; one that cannot
-// leave its side of the region's border (g.seam) commits nothing but its
-// observables, and is not walked when those edges carry none.  Farther paths
-// are walked through explored balls.  Every thread of the team calls.
+// Hash table sizes of a shot with C.K events: about 8 (rarely ~15) explored
+// entries and 1 (at most ~2) pair per event at the design point; the tables
+// stay at most half full or the shot is retried with larger ones.
+__device__ __forceinline__ unsigned next_pow2(unsigned x) {
+    x--; x |= x >> 1; x |= x >> 2; x |= x >> 4; x |= x >> 8; x |= x >> 16;
+    return x + 1;
+}
+__device__ __forceinline__ void set_tables(const BatchArgs &A, Shot &C, unsigned scale) {
+    C.ec = A.caps.ec; C.wc = A.caps.wc; C.cc = A.caps.cc;
+    C.pcap = A.caps.phc >> 1;
+    C.hmask = min(next_pow2(max(128u, (unsigned)QEC_HT_FACTOR * (unsigned)C.K * scale)), (unsigned)A.caps.hc) - 1;
+    C.pmask = min(next_pow2(max(64u, 4u * (unsigned)C.K * scale)), (unsigned)A.caps.phc) - 1;
+}
+
+// Walk the canonical paths of a matching: np pairs of events tmpa[i], tmpb[i]
+// (-1: boundary) at distance cst2[i].  COMMIT (sliding windows): the correction
+// is the union of those paths and of the boundary edges; every edge that
+// touches the graph's commit region is committed, and the shot's carry row
+// receives the detectors outside the region flipped by committed edges.
+// Otherwise the result is the observables of the paths' edges.  A path within
+// the ball table's reach is walked by one warp; one that cannot leave its side
+// of the region's border (g.seam) commits nothing but its observables, and is
+// not walked when those edges carry none.  Farther paths are walked through
+// explored balls, for which a fast-path shot (scale > 0) sets up its tables
+// first.  svtx: the events' vertices.  Every thread of the team calls.
 template <bool COMMIT, int NW>
-__device__ __noinline__ unsigned long long walk_paths(const Slab &S, Shot &C, Team<NW> T, int nhi, unsigned *carry) {
+__device__ __noinline__ unsigned long long walk_paths(const BatchArgs &A, const Slab &S, Shot &C, Team<NW> T,
+                                                      const int *svtx, int np, unsigned scale, unsigned *carry) {
     const DGraph &g = C.g;
-    const int np = expand(S, C, T, nhi);
     if constexpr (COMMIT)
         for (int w = T.tid(); w < g.words; w += T.NT) carry[w] = 0u;
-    if (!C.real)   // no ball is explored yet
-        for (int s = T.tid(); s < C.K; s += T.NT) { S.src[s].sR = -1; S.src[s].sexh = 0; }
+    if (T.tid() == 0) {
+        S.ctr[C_TNX] = 0;
+        if (scale) S.ctr[C_ERR] = 0;
+    }
     T.sync();
-    if (T.bcast(ldr(&S.ctr[C_ERR]))) return 0;
     unsigned long long mine = 0, whole = 0;   // found by this lane / by this warp together
     for (int base = T.warp() * WS; base < np; base += T.NT) {
         const int i = base + T.lane;
@@ -1638,19 +1659,18 @@ __device__ __noinline__ unsigned long long walk_paths(const Slab &S, Shot &C, Te
         if (i < np) {
             const int a = S.tmpa[i], b = S.tmpb[i];
             int s = a;
+            dx = S.cst2[i];
             if (b < 0) {
-                const unsigned long long bb = S.sbnd[a];
-                const int e = (int)(unsigned)(bb & 0xffffffffu);
+                const int e = (int)(unsigned)(__ldg(g.vbnd + svtx[a]) & 0xffffffffu);
                 const int2 ue = __ldg(g.eend + e);
                 x = ue.x;
-                dx = (int)(bb >> 32) - ue.y;
+                dx -= ue.y;
                 if constexpr (COMMIT) if (in_commit(g, x)) mine ^= __ldg(g.eobs + e);   // the boundary edge itself
             } else {
                 s = min(a, b);
-                x = S.svtx[max(a, b)];
-                dx = tight_dist(S, a, b);
+                x = svtx[max(a, b)];
             }
-            v = S.svtx[s];
+            v = svtx[s];
             bool skip = false;
             if constexpr (COMMIT) skip = dx < __ldg(g.seam + v) && (!g.internal_obs || !in_commit(g, v));
             h = __ldg(g.bhdr + v);
@@ -1670,16 +1690,29 @@ __device__ __noinline__ unsigned long long walk_paths(const Slab &S, Shot &C, Te
     T.sync();
     unsigned long long o = T.xor64(mine ^ (T.lane == 0 ? whole : 0));
     const int nfar = T.bcast(ldr(&S.ctr[C_TNX]));
+    if (nfar == 0 || T.bcast(ldr(&S.ctr[C_ERR]))) return o;
+    C.paths = 1;
+    if (!C.real) {   // no ball is explored yet
+        if (scale) {
+            set_tables(A, C, scale);
+            for (int i = T.tid(); i < C_TOTAL; i += T.NT) S.ctr[i] = 0;
+        }
+        for (int s = T.tid(); s < C.K; s += T.NT) {
+            S.src[s].sR = -1; S.src[s].sexh = 0;
+            S.scnt[s] = 0; S.sbeg[s] = 0;
+            S.svtx[s] = svtx[s];
+        }
+        T.sync();
+    }
     for (int k = 0; k < nfar; k++) {
         if (T.bcast(ldr(&S.ctr[C_ERR]))) break;
         const int i = S.stk[k];
-        const int a = S.tmpa[i], b = S.tmpb[i];
+        const int a = S.tmpa[i], b = S.tmpb[i], d = S.cst2[i];
         if (b < 0) {
-            const unsigned long long bb = S.sbnd[a];
-            const int2 ue = __ldg(g.eend + (int)(unsigned)(bb & 0xffffffffu));
-            o ^= walk_ball<COMMIT>(S, C, a, ue.x, (int)(bb >> 32) - ue.y, T, carry);
+            const int2 ue = __ldg(g.eend + (unsigned)(__ldg(g.vbnd + S.svtx[a]) & 0xffffffffu));
+            o ^= walk_ball<COMMIT>(S, C, a, ue.x, d - ue.y, T, carry);
         } else {
-            o ^= walk_ball<COMMIT>(S, C, min(a, b), S.svtx[max(a, b)], tight_dist(S, a, b), T, carry);
+            o ^= walk_ball<COMMIT>(S, C, min(a, b), S.svtx[max(a, b)], d, T, carry);
         }
     }
     T.sync();
@@ -1712,11 +1745,6 @@ __device__ __noinline__ void release_tables(const Slab &S, const Shot &C, Team<N
         }
     }
     T.sync();
-}
-
-__device__ __forceinline__ unsigned next_pow2(unsigned x) {
-    x--; x |= x >> 1; x |= x >> 2; x |= x >> 4; x |= x >> 8; x |= x >> 16;
-    return x + 1;
 }
 
 // Compact the set bits of the shot's syndrome row into S.svtx; returns K
@@ -1859,7 +1887,6 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
                                    Team<NW> &T, unsigned scale, unsigned long long deadline, long long &w_out,
                                    unsigned long long &o_out, int *dg, Shot &C) {
     C.g = g;
-    C.ec = A.caps.ec; C.wc = A.caps.wc; C.cc = A.caps.cc;
     C.band = max(g.wmax, 1) * max(A.band_factor, 1);
     C.events = 0;
     C.t = 0;
@@ -1868,7 +1895,6 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     C.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
     C.nm = 0; C.ncut = 0; C.tcut = 0; C.tlast = 0; C.nx = 0;
     C.real = 0;
-    C.pcap = A.caps.phc >> 1;
     if (g.words > A.caps.wcap) return -2;
     int K = 0;
     if (T.warp() == 0) K = load_defects(S, g, row, A.caps.kc, A.caps.wcap, T.lane);
@@ -1886,13 +1912,7 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     }
     if (K > ID_MAX - 1 || 2 * K + 8 > A.caps.nc) return -2;
     C.nc = min(A.caps.nc, 2 * K + 16);   // leaves + at most K blossoms alive at once
-    // about 8 (rarely ~15) explored entries and 1 (at most ~2) pair per
-    // detection event at the design point; the tables stay at most half full or
-    // the shot is retried with larger ones
-    const unsigned hs = min(next_pow2(max(128u, (unsigned)QEC_HT_FACTOR * (unsigned)K * scale)), (unsigned)A.caps.hc);
-    const unsigned ps = min(next_pow2(max(64u, 4u * (unsigned)K * scale)), (unsigned)A.caps.phc);
-    C.hmask = hs - 1;
-    C.pmask = ps - 1;
+    set_tables(A, C, scale);
     clear_tables(S, C, T);
     // sources, leaf nodes, free list
     int nhi = K;
@@ -2064,10 +2084,15 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     long long wint = 0;
     unsigned long long ob = 0;
     total(S, C, T, nhi, wint, ob);
-    if constexpr (WIN) {   // sliding window: the committed part
-        ob = walk_paths<true>(S, C, T, nhi, A.carry + (row - A.syn));
-    } else if (g.internal_obs) {   // detector-detector edges carry observables
-        ob ^= walk_paths<false>(S, C, T, nhi, nullptr);
+    if (WIN || g.internal_obs) {
+        // sliding window: the committed part; else the observables of
+        // detector-detector edges
+        const int npath = expand(S, C, T, nhi);
+        if (T.bcast(ldr(&S.ctr[C_ERR])) == 0) {
+            const unsigned long long po = walk_paths<WIN>(A, S, C, T, S.svtx, npath, 0,
+                                                          WIN ? A.carry + (row - A.syn) : nullptr);
+            ob = WIN ? po : ob ^ po;
+        }
     }
     const int err = T.bcast(ldr(&S.ctr[C_ERR]));
     if (err) return (err & ERR_INTERNAL) ? QEC_SHOT_INTERNAL : -1;
@@ -2107,6 +2132,1058 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
     return st;
 }
 
+// ---------------------------------------------------------------- islands --
+//
+// The events left after level 1 fall into islands: the components of Algorithm
+// 1's level-1 graph (pairs within b_1) that were not accepted.  Two islands,
+// or an island and a stopped level-1 cluster, are more than b_1 apart, so they
+// hardly ever touch, and what touches only in its own island runs the same
+// events in the same order alone as inside one run over everything: the state
+// changes are disjoint and the canonical order restricted to an island is the
+// order of its own events.  So each island is run by itself, one warp each with
+// the whole state in shared memory, and afterwards every recorded pair that
+// joins two of them is checked: if the largest radii reach its distance, the
+// shot is decoded again by the run over all events.
+//
+// A run over everything costs a scan of all events and pairs per event: a d =
+// 51 window at p = 0.003 (1,170 events, 250 matcher events in 88 islands of at
+// most ~12 events) spent 87 % of its time there, a d = 21 shot (6 islands) 67 %.
+// Islands or shots outside the limits below take that run.
+constexpr int IN = 32;    // events of an island (one lane each); blossoms are nodes IN .. 2 IN - 1
+constexpr int IP = 64;    // pairs
+constexpr int IC = 96;    // blossom cycle entries
+
+struct __align__(16) Isl {
+    int y[2 * IN], rad[IN], pd[IP], ev[IN];
+    unsigned char pa[IP], pb[IP];
+    signed char lab[2 * IN], bpar[2 * IN], tpar[2 * IN], tps[2 * IN], tpo[2 * IN];
+    signed char mate[2 * IN], ms[2 * IN], mo[2 * IN], root[2 * IN], minl[2 * IN], top[IN];
+    unsigned char cn[IC], cs[IC], co[IC], cb[IN], cl[IN];   // cycles: child, its leaf, the next child's leaf
+    signed char ta[2 * IN], tb[2 * IN];                     // tree paths / expansion stack
+    int nc, err;
+};
+
+// Shared memory of a team: per-event arrays of shots with at most KS events
+// (larger shots use the slab), and one island per warp.
+template <int NW>
+struct __align__(16) FastShared {
+    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + KS / 4;
+    unsigned long long pr[PS];
+    int svtx[KS], bd[KS], comp[KS], px[KS], st[KS];
+    unsigned cw[KS];
+    int cnt[8];
+    Isl isl[NW];
+};
+
+enum { ST_RUN = -3 };
+enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2 };
+constexpr unsigned ISL_ALONE = 1u << 31;
+enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6 };   // FastShared::cnt
+
+// Per-event arrays of the shot being decoded (shared memory or slab).
+//   pr: pairs, lo << 46 | hi << 28 | distance; svtx: vertex; bd: boundary
+//   distance (INT_MAX: none); comp: lowest event of the component; cw, at a
+//   component's lowest event: size | pairs within d_1 << 12 | boundary contact
+//   << 31; px: a pair within d_1, later the largest radius; st: level-1 state,
+//   the partner or MATE_BOUNDARY in a closed form, MATE_NONE: a growing root of
+//   the top level, ST_RUN: in a level-1 cluster that was run
+struct Fast {
+    unsigned long long *pr;
+    int *svtx, *bd, *comp, *px, *st;
+    unsigned *cw;
+    int *cnt;
+    int pcap;
+};
+
+__device__ __forceinline__ unsigned long long pk_pair(int a, int b, int d) {
+    return ((unsigned long long)(unsigned)a << 46) | ((unsigned long long)(unsigned)b << 28) | (unsigned)d;
+}
+__device__ __forceinline__ int pr_lo(unsigned long long p) { return (int)(p >> 46); }
+__device__ __forceinline__ int pr_hi(unsigned long long p) { return (int)(p >> 28) & 0x3ffff; }
+__device__ __forceinline__ int pr_val(unsigned long long p) { return (int)(p & 0xfffffffu); }
+
+// What one island, or several, add to the shot (w: internal units).
+struct __align__(16) IslRec {
+    unsigned long long o;
+    int w, size;
+    int nm, ncut, tlast, nx;   // matcher events, those at times <= tcut, time of the last, bands counted here
+};
+
+__device__ __forceinline__ int isl_child_of(const Isl &I, int B, int leaf) {
+    int v = leaf;
+#pragma unroll 1
+    while (v >= 0 && I.bpar[v] != B) v = I.bpar[v];
+    return v;
+}
+
+// flip matches along the tree path from outer A to its root (lane 0)
+__device__ __forceinline__ void isl_flip(Isl &I, int A) {
+    int v = A;
+#pragma unroll 1
+    while (I.tpar[v] >= 0) {
+        const int i = I.tpar[v], o = I.tpar[i];
+        I.mate[i] = (signed char)o; I.ms[i] = I.tps[i]; I.mo[i] = I.tpo[i];
+        I.mate[o] = (signed char)i; I.ms[o] = I.tpo[i]; I.mo[o] = I.tps[i];
+        v = o;
+    }
+}
+
+// Event (c) on lane 0: the new blossom N over outer A, B of one tree; false
+// when the cycle pool is full.
+__device__ __noinline__ bool isl_blossom(Isl &I, int N, int A, int a, int B, int b) {
+    int na = 0, nb = 0;
+#pragma unroll 1
+    for (int v = A; v >= 0; v = I.tpar[v]) I.ta[na++] = (signed char)v;
+#pragma unroll 1
+    for (int v = B; v >= 0; v = I.tpar[v]) I.tb[nb++] = (signed char)v;
+#pragma unroll 1
+    while (na > 1 && nb > 1 && I.ta[na - 2] == I.tb[nb - 2]) { na--; nb--; }
+    const int Lc = I.ta[na - 1], m = na + nb - 1, cb = I.nc;
+    if (cb + m > IC) return false;
+    I.nc = cb + m;
+    int i = 0;
+    I.cn[cb + i++] = (unsigned char)Lc;
+#pragma unroll 1
+    for (int j = na - 2; j >= 0; j--) I.cn[cb + i++] = (unsigned char)I.ta[j];
+#pragma unroll 1
+    for (int j = 0; j <= nb - 2; j++) I.cn[cb + i++] = (unsigned char)I.tb[j];
+    const int ia = na - 1;
+    int ml = IN;
+#pragma unroll 1
+    for (int j = 0; j < m; j++) {
+        const int x = I.cn[cb + j], z = I.cn[cb + (j + 1 < m ? j + 1 : 0)];
+        if (j < ia) { I.cs[cb + j] = I.tpo[z]; I.co[cb + j] = I.tps[z]; }
+        else if (j == ia) { I.cs[cb + j] = (unsigned char)a; I.co[cb + j] = (unsigned char)b; }
+        else { I.cs[cb + j] = I.tps[x]; I.co[cb + j] = I.tpo[x]; }
+        ml = min(ml, (int)I.minl[x]);
+        I.bpar[x] = (signed char)N;
+    }
+    I.y[N] = 0; I.lab[N] = 1; I.bpar[N] = -1;
+    I.tpar[N] = I.tpar[Lc]; I.tps[N] = I.tps[Lc]; I.tpo[N] = I.tpo[Lc];
+    I.mate[N] = I.mate[Lc]; I.ms[N] = I.ms[Lc]; I.mo[N] = I.mo[Lc];
+    I.root[N] = I.root[Lc] == Lc ? (signed char)N : I.root[Lc];
+    I.minl[N] = (signed char)ml;
+    I.cb[N - IN] = (unsigned char)cb; I.cl[N - IN] = (unsigned char)m;
+    return true;
+}
+
+// Event (d) on lane 0: inner blossom B shatters (tops are set by the caller).
+__device__ __noinline__ void isl_shatter(Isl &I, int B) {
+    const int m = I.cl[B - IN], cb = I.cb[B - IN];
+    const int P = I.tpar[B], Cn = I.mate[B];
+    const int xp = isl_child_of(I, B, I.tps[B]), xc = isl_child_of(I, B, I.ms[B]);
+    int ip = -1, ic = -1;
+#pragma unroll 1
+    for (int j = 0; j < m; j++) {
+        if (I.cn[cb + j] == xp) ip = j;
+        if (I.cn[cb + j] == xc) ic = j;
+    }
+    if (ip < 0 || ic < 0 || Cn < 0) { I.err = 1; return; }
+#pragma unroll 1
+    for (int j = 0; j < m; j++) I.bpar[I.cn[cb + j]] = -1;
+    auto wrap = [&](int j) { j %= m; return j < 0 ? j + m : j; };
+    const int fwd = wrap(ic - ip), dir = (fwd % 2 == 0) ? 1 : -1, Ln = dir > 0 ? fwd : m - fwd;
+    int prev = -1;
+#pragma unroll 1
+    for (int j = 0; j <= Ln; j++) {
+        const int idx = wrap(ip + dir * j), q = I.cn[cb + idx];
+        I.lab[q] = (j % 2 == 0) ? -1 : 1;
+        I.root[q] = I.root[B];
+        if (j == 0) {
+            I.tpar[q] = (signed char)P; I.tps[q] = I.tps[B]; I.tpo[q] = I.tpo[B];
+        } else {
+            const int pidx = wrap(ip + dir * (j - 1));
+            const int self = dir > 0 ? I.co[cb + pidx] : I.cs[cb + idx], other = dir > 0 ? I.cs[cb + pidx] : I.co[cb + idx];
+            I.tpar[q] = (signed char)prev; I.tps[q] = (signed char)self; I.tpo[q] = (signed char)other;
+            if (j % 2 == 1) {
+                I.mate[q] = (signed char)prev; I.ms[q] = (signed char)self; I.mo[q] = (signed char)other;
+                I.mate[prev] = (signed char)q; I.ms[prev] = (signed char)other; I.mo[prev] = (signed char)self;
+            }
+        }
+        prev = q;
+    }
+    I.mate[prev] = (signed char)Cn; I.ms[prev] = I.ms[B]; I.mo[prev] = I.mo[B];
+    I.mate[Cn] = (signed char)prev; I.tpar[Cn] = (signed char)prev;
+#pragma unroll 1
+    for (int j = 1; j <= m - 1 - Ln; j += 2) {
+        const int i1 = wrap(ic + dir * j), i2 = wrap(ic + dir * (j + 1));
+        const int x = I.cn[cb + i1], z = I.cn[cb + i2];
+        const int lx = dir > 0 ? I.cs[cb + i1] : I.co[cb + i2], lz = dir > 0 ? I.co[cb + i1] : I.cs[cb + i2];
+        I.lab[x] = 0; I.lab[z] = 0;
+        I.tpar[x] = -1; I.tpar[z] = -1;
+        I.root[x] = -1; I.root[z] = -1;
+        I.mate[x] = (signed char)z; I.ms[x] = (signed char)lx; I.mo[x] = (signed char)lz;
+        I.mate[z] = (signed char)x; I.ms[z] = (signed char)lz; I.mo[z] = (signed char)lx;
+    }
+    I.lab[B] = 0; I.y[B] = 0;
+}
+
+// Distance of two matched events of an island (as tight_dist).
+__device__ __forceinline__ int isl_dist(const Isl &I, int a, int b) {
+    int d = I.rad[a] + I.rad[b];
+#pragma unroll 1
+    for (int B = I.bpar[a]; B >= 0; B = I.bpar[B]) {
+        int x = I.bpar[b];
+#pragma unroll 1
+        while (x >= 0 && x != B) x = I.bpar[x];
+        if (x == B) {
+#pragma unroll 1
+            for (; B >= 0; B = I.bpar[B]) d -= 2 * I.y[B];
+            break;
+        }
+    }
+    return d;
+}
+
+// A matched pair of the shot (b = -1: boundary) at distance d, for the path walks.
+__device__ __forceinline__ void put_path(const Slab &S, int *cnt, int a, int b, int d) {
+    const int k = atomicAdd(cnt, 1);   // at most one per event
+    S.tmpa[k] = a; S.tmpb[k] = b; S.cst2[k] = d;
+}
+
+// The matched pairs inside blossom `node` whose leaf ext is matched outside, and so on down (lane 0).
+__device__ __noinline__ void isl_expand(Isl &I, const Slab &S, int *cnt, int node, int ext) {
+    int sp = 0;
+    I.ta[sp] = (signed char)node; I.tb[sp++] = (signed char)ext;
+#pragma unroll 1
+    while (sp > 0) {
+        const int v = I.ta[--sp], e = I.tb[sp];
+        if (v < IN) continue;
+        const int m = I.cl[v - IN], cb = I.cb[v - IN], c0 = isl_child_of(I, v, e);
+        int i0 = 0;
+#pragma unroll 1
+        for (int j = 0; j < m; j++) if (I.cn[cb + j] == c0) i0 = j;
+        I.ta[sp] = (signed char)c0; I.tb[sp++] = (signed char)e;
+#pragma unroll 1
+        for (int j = 1; j < m; j += 2) {
+            const int i1 = (i0 + j) % m, i2 = (i0 + j + 1) % m;
+            const int lx = I.cs[cb + i1], lz = I.co[cb + i1];
+            put_path(S, cnt, I.ev[lx], I.ev[lz], isl_dist(I, lx, lz));
+            I.ta[sp] = (signed char)I.cn[cb + i1]; I.tb[sp++] = (signed char)lx;
+            I.ta[sp] = (signed char)I.cn[cb + i2]; I.tb[sp++] = (signed char)lz;
+        }
+    }
+}
+
+// Events farther from vertex v than the ball table's radius, up to q <= 2 brad -
+// 2 wmax: the shortest path to such an event passes a detector y at a distance
+// in (r - wmax, r] from v, r = q - brad + wmax <= brad, and the rest of it is
+// shorter than brad, so the event is in the list of one of those y.  Lane j gets
+// the j-th event found (rank f, exact distance d); returns their number, or -1
+// when a list is not complete or more than 32 are found.  One warp.
+__device__ __noinline__ int far_events(const Slab &S, const Shot &C, int v, int q, int lane, int &f, int &d) {
+    const DGraph &g = C.g;
+    const int4 h = __ldg(g.bhdr + v);
+    const int n = h.z + max(h.w, 0), r = q - g.brad + g.wmax;
+    int found = 0;
+    f = -1;
+    d = INT_MAX;
+#pragma unroll 1
+    for (int k = 0; k < n; k += WS) {
+        int2 e = make_int2(0, 0);
+        int4 he = make_int4(0, 0, 0, 0);
+        bool use = false;
+        if (k + lane < n) {
+            e = __ldg(g.ball + (unsigned)h.x + k + lane);
+            use = e.y > r - g.wmax && e.y <= r;
+            if (use) he = __ldg(g.bhdr + e.x);
+        }
+        if (__any_sync(FULL, he.w < 0)) return -1;
+        const int beg = he.x, len = he.z + he.w;
+#pragma unroll 1
+        for (unsigned m = __ballot_sync(FULL, use); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const int dy = __shfl_sync(FULL, e.y, l), ly = __shfl_sync(FULL, len, l);
+            const int2 *const list = g.ball + (unsigned)__shfl_sync(FULL, beg, l);
+#pragma unroll 1
+            for (int j = 0; j < ly; j += 4 * WS) {   // four loads in flight
+                int2 x[4];
+                unsigned hit = 0;
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    x[u] = make_int2(v, 0);
+                    if (j + u * WS + lane < ly) x[u] = __ldg(list + j + u * WS + lane);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (dy + x[u].y > g.brad && dy + x[u].y <= q && x[u].x != v && is_defect(C, x[u].x)) hit |= 1u << u;
+                if (!__any_sync(FULL, hit)) continue;
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+#pragma unroll 1
+                    for (unsigned mh = __ballot_sync(FULL, (hit >> u) & 1u); mh; mh &= mh - 1) {
+                        const int o = __ffs(mh) - 1;
+                        const int ro = rank_of(S, C, __shfl_sync(FULL, x[u].x, o)), dr = dy + __shfl_sync(FULL, x[u].y, o);
+                        const unsigned same = __ballot_sync(FULL, f == ro);
+                        if (!same) {
+                            if (found == WS) return -1;
+                            if (lane == found) { f = ro; d = dr; }
+                            found++;
+                        } else if (f == ro) {
+                            d = min(d, dr);
+                        }
+                    }
+                }
+            }
+        }
+    }
+    return found;
+}
+
+// Run the island of the component with lowest event c and `size` events from t
+// = 0 (SI S1, events as in run_matcher): growing roots and, in an island that
+// was joined with level-1 clusters, their events frozen as level 1 left them.
+// One warp.  np0: pairs within b_1.  tcut as in Shot.  level1: a level-1 cluster (its
+// bands are counted here; the top level's aged bands are collected in xR, since
+// regions due at the same time share one).  paths: the matched pairs are wanted.
+// Returns ISL_FAIL when the island is outside the limits, ISL_STOP when a region
+// touched a level-1 cluster outside or outgrew the ball table (the radii so far
+// are in px, cw[c] is ISL_ALONE).
+__device__ __forceinline__ int run_island(const Slab &S, const Shot &C, const Fast &F, Isl &I, int c, int size, int np0,
+                                           int tcut, bool level1, bool paths, int lane, IslRec &rec) {
+    const DGraph &g = C.g;
+    if (size > IN) return ISL_FAIL;
+    // members in rank order: the first is c, the others are near it
+    int n = 0;
+#pragma unroll 1
+    for (int base = c; base < C.K && n < size; base += WS) {
+        const int s = base + lane;
+        const bool in = s < C.K && F.comp[s] == c;
+        const unsigned m = __ballot_sync(FULL, in);
+        if (in) {
+            const int k = n + __popc(m & ((1u << lane) - 1u));
+            I.ev[k] = s;
+            F.cw[s] = (unsigned)k;   // its lane
+        }
+        n += __popc(m);
+    }
+    __syncwarp();
+    n = size;
+    int ev = 0, bd = INT_MAX, sR = -1, mrad = 0;
+    int meet = INT_MAX;   // radius at which this region touches a level-1 cluster
+    bool exh = false, bad = false;
+    if (lane < n) {
+        ev = I.ev[lane];
+        bd = F.bd[ev];
+        const int st = level1 ? MATE_NONE : F.st[ev];
+        const bool frozen = st != MATE_NONE;
+        if (st == ST_RUN) bad = true;
+        mrad = st == MATE_BOUNDARY ? bd : 0;   // of a frozen pair: set with its pair below
+        sR = frozen ? -1 : C.L + C.band;   // first extension, due at t = 0: within the listed pairs
+        I.rad[lane] = mrad; I.y[lane] = mrad;
+        I.lab[lane] = frozen ? 0 : 1; I.bpar[lane] = -1; I.tpar[lane] = -1;
+        I.mate[lane] = frozen ? MATE_BOUNDARY : MATE_NONE; I.ms[lane] = (signed char)lane; I.mo[lane] = -1;
+        I.root[lane] = frozen ? -1 : (signed char)lane; I.minl[lane] = (signed char)lane; I.top[lane] = (signed char)lane;
+    }
+    if (__any_sync(FULL, bad)) return ISL_FAIL;
+    __syncwarp();
+    if (lane == 0) { I.nc = 0; I.err = 0; }
+    int np = 0;
+#pragma unroll 1
+    for (int base = 0; base < np0; base += WS) {
+        const int i = base + lane;
+        unsigned long long p = 0;
+        bool in = false;
+        if (i < np0) {
+            p = F.pr[i];
+            in = F.comp[pr_lo(p)] == c;
+        }
+        const unsigned m = __ballot_sync(FULL, in);
+        if (!m) continue;
+        const int k = np + __popc(m & ((1u << lane) - 1u));
+        if (in && k < IP) {
+            const int a = (int)F.cw[pr_lo(p)], b = (int)F.cw[pr_hi(p)], d = pr_val(p);
+            I.pa[k] = (unsigned char)a;
+            I.pb[k] = (unsigned char)b;
+            I.pd[k] = d;
+            if (!level1 && F.st[pr_lo(p)] == pr_hi(p)) {   // a level-1 pair: frozen, matched at d / 2
+                I.rad[a] = I.rad[b] = I.y[a] = I.y[b] = d / 2;
+                I.mate[a] = (signed char)b; I.mo[a] = (signed char)b;
+                I.mate[b] = (signed char)a; I.mo[b] = (signed char)a;
+            }
+        }
+        np += __popc(m);
+    }
+    if (np > IP) return ISL_FAIL;
+    __syncwarp();
+    if (lane < n) mrad = I.rad[lane];
+    unsigned bal = 0;   // blossoms alive
+    auto stop = [&]() {
+        if (lane < n) F.px[ev] = mrad;
+        if (lane == 0) { F.cw[c] = ISL_ALONE; atomicAdd(&F.cnt[F_STOP], 1); }
+        __syncwarp();
+        return ISL_STOP;
+    };
+    int t = 0, nm = 0, ncut = 0, tlast = 0, nx = level1 ? 1 : 0;
+#pragma unroll 1
+    for (int it = 0;; it++) {
+        if (it > 200 * n) return ISL_FAIL;   // far below the shot's event budget
+        // next event: key dt << 12 | kind << 10 | lo << 5 | hi, dt < 2^20
+        unsigned key = ~0u;
+        bool grows = false;
+        auto cand = [&](int dt, int kind, int lo, int hi) {
+            bad |= dt < 0;
+            key = min(key, dt >= 0xfffff ? ~1u : ((unsigned)dt << 12) | (unsigned)(kind << 10 | lo << 5 | hi));
+        };
+        int lab = 0, rad = 0;
+        if (lane < n) {
+            lab = I.lab[I.top[lane]];
+            rad = I.rad[lane];
+            if (lab == 1) {
+                grows = true;
+                if (!exh) cand(max(0, sR - C.L + 1 - rad), EV_EXTEND, lane, 0);
+                if (bd != INT_MAX) cand(bd - rad, EV_BOUNDARY, lane, 0);
+            }
+        }
+#pragma unroll 1
+        for (int p = lane; p < np; p += WS) {
+            const int a = I.pa[p], b = I.pb[p], A = I.top[a], B = I.top[b];
+            const int r = I.lab[A] + I.lab[B];
+            if (A == B || r <= 0) continue;
+            const int gap = I.pd[p] - I.rad[a] - I.rad[b];
+            bad |= (gap & (r - 1)) != 0;
+            cand(r == 2 ? gap >> 1 : gap, EV_COLLIDE, min(a, b), max(a, b));
+        }
+        if ((bal >> lane) & 1u) {
+            const int v = IN + lane;
+            if (I.bpar[v] < 0 && I.lab[v] == -1) cand(I.y[v], EV_IMPLODE, I.minl[v], 0);
+        }
+        if (__any_sync(FULL, bad)) return ISL_FAIL;
+        if (!__any_sync(FULL, grows)) break;
+        key = __reduce_min_sync(FULL, key);
+        if (key >= ~1u) return ISL_FAIL;   // no event left (no solution), or far away
+        const int dt = (int)(key >> 12), kind = (int)(key >> 10) & 3, lo = (int)(key >> 5) & 31, hi = (int)key & 31;
+        t += dt;
+        if (t >= (1 << 25)) return ISL_FAIL;
+        if (__any_sync(FULL, lab == 1 && meet <= rad + dt)) {
+            mrad = max(mrad, rad + lab * dt);
+            return stop();
+        }
+        if (dt > 0) {
+            if (lane < n) {
+                rad += lab * dt;
+                I.rad[lane] = rad;
+                mrad = max(mrad, rad);
+                if (I.top[lane] == lane) I.y[lane] += lab * dt;
+            }
+            if ((bal >> lane) & 1u) {
+                const int v = IN + lane;
+                if (I.bpar[v] < 0) I.y[v] += I.lab[v] * dt;
+            }
+        }
+        __syncwarp();
+        if (kind == EV_EXTEND) {
+            // regions that came within L of their explored radius
+            const bool due = lab == 1 && !exh && sR - C.L + 1 - rad <= 0;
+            int R = 0, q = 0;
+            bool scan = false, far = false;
+            if (due) {
+                R = max(sR + C.band, rad + C.L + C.band);
+                q = reach_of(C, R);
+                scan = sR >= 0 || q > g.b1;
+                if (!scan) sR = R;
+                far = scan && (q > 2 * g.brad - 2 * g.wmax || sR > g.brad - g.wmax || __ldg(g.bhdr + F.svtx[ev]).w < 0);
+            }
+            if (__any_sync(FULL, far)) return stop();
+#pragma unroll 1
+            for (unsigned m = __ballot_sync(FULL, scan); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const int s = __shfl_sync(FULL, ev, l), ql = __shfl_sync(FULL, q, l), sRl = __shfl_sync(FULL, sR, l);
+                const int q0 = sRl < 0 ? g.b1 : max(g.b1, reach_of(C, sRl));
+                const int4 h = __ldg(g.bhdr + F.svtx[s]);
+                const int len = h.z + h.w;
+                bool more = false;
+                // the list's own events, then those beyond it
+                int nfar = 0, ff = 0, fd = 0;
+                if (ql > g.brad) nfar = far_events(S, C, F.svtx[s], ql, lane, ff, fd);
+                if (nfar < 0) return ISL_FAIL;
+#pragma unroll 1
+                for (int k = 0; k < len + (nfar ? WS : 0); k += WS) {
+                    bool hit = false;
+                    int f = 0, d = 0;
+                    if (k < len) {
+                        if (k + lane < len) {
+                            const int2 e = __ldg(g.ball + (unsigned)h.x + k + lane);
+                            more |= e.y > sRl;
+                            hit = e.y > q0 && e.y <= ql && is_defect(C, e.x);
+                            d = e.y;
+                            if (hit) f = rank_of(S, C, e.x);
+                        }
+                    } else {
+                        hit = lane < nfar && fd > q0;
+                        f = ff;
+                        d = fd;
+                    }
+                    const unsigned mh = __ballot_sync(FULL, hit);
+                    if (!mh) continue;
+                    const bool in = hit && F.comp[f] == c;
+                    // a level-1 cluster stands still unless it is touched
+                    const int mt = hit && !in && F.st[f] != MATE_NONE ? d - F.px[f] : INT_MAX;
+                    const int ml = __reduce_min_sync(FULL, mt);
+                    if (lane == l) meet = min(meet, ml);
+                    int b = 0;
+                    if (lane == 0) b = atomicAdd(&F.cnt[F_NP], __popc(mh));
+                    b = __shfl_sync(FULL, b, 0) + __popc(mh & ((1u << lane) - 1u));
+                    if (hit && b < F.pcap) F.pr[b] = pk_pair(min(s, f), max(s, f), d);
+                    const unsigned mi = __ballot_sync(FULL, in);
+                    const int j = np + __popc(mi & ((1u << lane) - 1u));
+                    if (in && j < IP) { I.pa[j] = (unsigned char)l; I.pb[j] = (unsigned char)F.cw[f]; I.pd[j] = d; }
+                    np += __popc(mi);
+                    if (np > IP || __any_sync(FULL, hit && b >= F.pcap)) return ISL_FAIL;
+                }
+                more = __any_sync(FULL, more);
+                if (lane == l) { exh = sR >= 0 && !more; sR = R; }
+            }
+            // a band: counted at once, except that at the top level regions of
+            // several islands coming of age at one time share it
+            if (level1 || dt == 0) {
+                nx++;
+            } else if (lane == 0) {
+                const int k = atomicAdd(&F.cnt[F_AGED], 1);
+                if (k < C.K) { S.xR[k] = t; S.sbeg[k] = c; S.scnt[k] = n; }
+            }
+            __syncwarp();
+            continue;
+        }
+        nm++;
+        if (t <= tcut) ncut++;
+        tlast = t;
+        if (kind == EV_IMPLODE) {
+            const int B = I.top[lo];
+            if (lane < n && I.top[lane] == B) I.top[lane] = (signed char)isl_child_of(I, B, lane);
+            __syncwarp();
+            if (lane == 0) isl_shatter(I, B);
+            bal &= ~(1u << (B - IN));
+            __syncwarp();
+            if (I.err) return ISL_FAIL;
+            continue;
+        }
+        int a = lo, b = hi, A = I.top[a], B = -1;
+        if (kind == EV_COLLIDE) {
+            B = I.top[b];
+            if (I.lab[A] != 1) { int x = A; A = B; B = x; x = a; a = b; b = x; }
+        }
+        const int lb = B >= 0 ? I.lab[B] : 0, mb = B >= 0 ? I.mate[B] : MATE_BOUNDARY;
+        const int rA = I.root[A], rB = lb == 1 ? I.root[B] : -3;
+        __syncwarp();
+        if (lb == 1 && rA == rB) {
+            // blossom
+            if (bal == ~0u) return ISL_FAIL;
+            const int N = IN + __ffs(~bal) - 1;
+            int ok = 0;
+            if (lane == 0) ok = isl_blossom(I, N, A, a, B, b);
+            if (!__shfl_sync(FULL, ok, 0)) return ISL_FAIL;
+            __syncwarp();
+            const int L0 = I.cn[I.cb[N - IN]];   // its root becomes N's
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {
+                const int v = lane + h * IN;
+                if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+                if (I.bpar[v] >= 0) continue;
+                const int tp = I.tpar[v], mt = I.mate[v];
+                if (tp >= 0 && I.bpar[tp] == N) I.tpar[v] = (signed char)N;
+                if (mt >= 0 && I.bpar[mt] == N) I.mate[v] = (signed char)N;
+                if (I.root[v] == L0) I.root[v] = (signed char)N;
+            }
+            if (lane < n) {
+                const int tp = I.top[lane];
+                if (I.bpar[tp] == N) I.top[lane] = (signed char)N;
+            }
+            bal |= 1u << (N - IN);
+        } else if (lb == 1 || mb == MATE_BOUNDARY) {
+            // augment: the trees' nodes leave them while lane 0 rematches
+            // along the tree paths
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {
+                const int v = lane + h * IN;
+                if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+                if (I.bpar[v] < 0 && I.lab[v] != 0 && (I.root[v] == rA || I.root[v] == rB)) { I.lab[v] = 0; I.root[v] = -1; }
+            }
+            if (lane == 0) {
+                isl_flip(I, A);
+                if (lb == 1) isl_flip(I, B);
+                if (B >= 0) {
+                    I.mate[A] = (signed char)B; I.ms[A] = (signed char)a; I.mo[A] = (signed char)b;
+                    I.mate[B] = (signed char)A; I.ms[B] = (signed char)b; I.mo[B] = (signed char)a;
+                } else {
+                    I.mate[A] = MATE_BOUNDARY; I.ms[A] = (signed char)a; I.mo[A] = -1;
+                }
+            }
+        } else if (lb == 0 && mb >= 0) {
+            if (lane == 0) {   // grow
+                I.lab[B] = -1; I.tpar[B] = (signed char)A; I.tps[B] = (signed char)b; I.tpo[B] = (signed char)a;
+                I.root[B] = (signed char)rA;
+                I.lab[mb] = 1; I.tpar[mb] = (signed char)B; I.tps[mb] = I.ms[mb]; I.tpo[mb] = I.mo[mb];
+                I.root[mb] = (signed char)rA;
+            }
+        } else {
+            return ISL_FAIL;
+        }
+        __syncwarp();
+    }
+    // result: the duals' sum, the boundary matches' observables, largest radii
+    int w = 0;
+    unsigned long long o = 0;
+    if (lane < n) {
+        w = I.y[lane];
+        F.px[ev] = mrad;
+    }
+    if ((bal >> lane) & 1u) w += I.y[IN + lane];
+    for (int h = 0; h < 2; h++) {
+        const int v = lane + h * IN;
+        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+        if (I.bpar[v] >= 0) continue;
+        const int mt = I.mate[v];
+        if (mt == MATE_BOUNDARY) {
+            const int s = I.ev[I.ms[v]];
+            o ^= __ldg(g.eobs + (unsigned)(__ldg(g.vbnd + F.svtx[s]) & 0xffffffffu));
+            if (paths) put_path(S, &F.cnt[F_NPATH], s, -1, F.bd[s]);
+        } else if (paths && v < mt) {
+            put_path(S, &F.cnt[F_NPATH], I.ev[I.ms[v]], I.ev[I.mo[v]], isl_dist(I, I.ms[v], I.mo[v]));
+        }
+    }
+    if (paths) {
+        for (unsigned m = bal; m; m &= m - 1) {
+            const int v = IN + __ffs(m) - 1;
+            if (lane == 0 && I.bpar[v] < 0) isl_expand(I, S, &F.cnt[F_NPATH], v, I.ms[v]);
+        }
+    }
+    rec.w = (int)__reduce_add_sync(FULL, (unsigned)w);
+    rec.o = ((unsigned long long)__reduce_xor_sync(FULL, (unsigned)(o >> 32)) << 32) | __reduce_xor_sync(FULL, (unsigned)o);
+    rec.size = n; rec.nm = nm; rec.ncut = ncut; rec.tlast = tlast; rec.nx = nx;
+    __syncwarp();
+    return ISL_OK;
+}
+
+// Detection events of the row into svtx (those past cap dropped) and their
+// counts before each word into S.wcum; returns their number.  Every thread of
+// the team calls; ends with a barrier.
+template <int NW>
+__device__ __forceinline__ int load_events(const Slab &S, const DGraph &g, const unsigned *row, int *svtx, int cap,
+                                           Team<NW> &T) {
+    int K = 0;
+    const int nvec = g.words >> 2;
+    const uint4 *rv = reinterpret_cast<const uint4 *>(row);
+#pragma unroll 1
+    for (int base = 0; base < nvec; base += T.NT) {
+        const int i = base + T.tid();
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < nvec) v = __ldg(rv + i);
+        unsigned wv[4] = {v.x, v.y, v.z, v.w};
+        if (i * 128 + 128 > g.n) {   // drop padding bits beyond n
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int bit0 = (i * 4 + q) * 32;
+                if (bit0 >= g.n) wv[q] = 0;
+                else if (bit0 + 32 > g.n) wv[q] &= (1u << (g.n - bit0)) - 1u;
+            }
+        }
+        const int c0 = __popc(wv[0]), c1 = c0 + __popc(wv[1]), c2 = c1 + __popc(wv[2]), c = c2 + __popc(wv[3]);
+        int total;
+        int pos = K + T.excl_scan(c, total);
+        if (i < nvec) reinterpret_cast<int4 *>(S.wcum)[i] = make_int4(pos, pos + c0, pos + c1, pos + c2);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            unsigned bits = wv[q];
+#pragma unroll 1
+            while (bits) {
+                const int b = __ffs(bits) - 1;
+                bits &= bits - 1;
+                if (pos < cap) svtx[pos] = (i * 4 + q) * 32 + b;
+                pos++;
+            }
+        }
+        K += total;
+    }
+    T.sync();
+    return K;
+}
+
+constexpr int USE_GENERAL = -3;   // the shot is outside the fast path's limits
+
+// Decode one shot by level 1 and islands.  Same results and diagnostics as the
+// general path below, which takes what is outside the limits (USE_GENERAL).
+constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
+
+// Components of the events by min-label propagation with shortcuts over the
+// pairs within b_1, [0, np0), and those marked MET in [np0, np1); labels start
+// as they are.  Every thread of the team calls; ends with a barrier.
+template <int NW>
+__device__ __forceinline__ void fast_components(const Fast &F, int np0, int np1, int K, Team<NW> &T) {
+    volatile int *comp = F.comp;
+#pragma unroll 1
+    for (int round = 0; round <= K; round++) {
+        bool changed = false;
+#pragma unroll 1
+        for (int i = T.tid(); i < np1; i += T.NT) {
+            const unsigned long long p = F.pr[i];
+            if (i >= np0 && !(p & MET)) continue;
+            const int a = pr_lo(p), b = pr_hi(p), la = comp[a], lb = comp[b];
+            if (la != lb) {
+                const int m = min(la, lb), h = max(la, lb);
+                atomicMin(&F.comp[a], m);
+                atomicMin(&F.comp[b], m);
+                atomicMin(&F.comp[h], m);
+                changed = true;
+            }
+        }
+        T.sync();
+        if (!T.any(changed)) break;
+#pragma unroll 1
+        for (int s = T.tid(); s < K; s += T.NT) {
+            const int r = comp[s], rr = comp[r];
+            if (rr < r) comp[s] = rr;
+        }
+        T.sync();
+    }
+}
+
+template <bool WIN, int NW>
+__device__ __forceinline__ int decode_fast(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
+                                           Team<NW> &T, FastShared<NW> &M, long long &w_out, unsigned long long &o_out,
+                                           int *dg) {
+    Shot C;
+    C.g = g;
+    C.row = row;
+    C.band = max(g.wmax, 1) * max(A.band_factor, 1);
+    C.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
+    C.real = 0;
+    C.paths = 0;
+    // level 1 present, lists complete, first extensions within the listed pairs
+    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (1 << 27) || reach_of(C, C.L + C.band) > g.b1 ||
+        g.words > A.caps.wcap)
+        return USE_GENERAL;
+    Fast F;
+    F.cnt = M.cnt;
+    F.svtx = M.svtx; F.bd = M.bd; F.comp = M.comp; F.px = M.px; F.st = M.st; F.cw = M.cw;
+    F.pr = M.pr;
+    F.pcap = M.PS;
+    int K = load_events(S, g, row, M.svtx, M.KS, T);
+    C.K = K;
+    if (K == 0) {
+        w_out = 0; o_out = 0;
+        if (dg && T.tid() < QEC_DIAG_FIELDS) dg[T.tid()] = 0;   // no detection event: E_ideal = 0
+        if constexpr (WIN)
+#pragma unroll 1
+            for (int w = T.tid(); w < g.words; w += T.NT) A.carry[(row - A.syn) + w] = 0u;
+        return QEC_SHOT_OK;
+    }
+    if (K > A.caps.kc || K > 4000) return USE_GENERAL;
+    const bool paths = WIN || g.internal_obs;
+    int np0 = 0;
+#pragma unroll 1
+    for (bool small = K <= M.KS;; small = false) {
+        if (!small) {   // per-event arrays in the slab
+            F.svtx = S.svtx; F.bd = S.cst0; F.comp = S.comp; F.px = S.xcur; F.st = S.xidx;
+            F.cw = reinterpret_cast<unsigned *>(S.cst1);
+            F.pr = S.tl;
+            F.pcap = A.caps.ec;
+            load_events(S, g, row, S.svtx, A.caps.kc, T);
+        }
+        if (T.tid() < 8) M.cnt[T.tid()] = 0;
+        T.sync();
+        // pairs within b_1 (as near_pairs)
+        int flags = 0, np = 0;
+        const int lane = T.lane;
+#pragma unroll 1
+        for (int base = T.warp() * WS; base < K; base += T.NT) {
+            const int s = base + lane;
+            int beg = 0, len = 0;
+            if (s < K) {
+                const int v = F.svtx[s];
+                const int4 h = __ldg(g.bhdr + v);
+                const unsigned long long vb = __ldg(g.vbnd + v);
+                F.bd[s] = vb == EMPTY64 ? INT_MAX : (int)(vb >> 32);
+                F.comp[s] = s;
+                F.cw[s] = 0;
+                F.st[s] = MATE_NONE;
+                if (h.z < 0 || (!g.hop2 && h.z >= LB_CAP)) flags |= 1;
+                beg = h.x;
+                len = h.z < 0 ? 0 : h.y;
+            }
+            int incl = len;
+#pragma unroll
+            for (int o = 1; o < WS; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int total = __shfl_sync(FULL, incl, WS - 1);
+            const int excl = incl - len;
+#pragma unroll 1
+            for (int t0 = 0; t0 < total; t0 += WS) {
+                const int t = t0 + lane;
+                int ow = 0;   // owner: the last lane whose first entry number is <= t
+#pragma unroll
+                for (int step = WS / 2; step > 0; step >>= 1) {
+                    const int e = __shfl_sync(FULL, excl, ow + step);
+                    if (e <= t) ow += step;
+                }
+                const unsigned oj = (unsigned)__shfl_sync(FULL, beg - excl, ow) + (unsigned)t;
+                bool hit = false;
+                int2 e = make_int2(0, 0);
+                unsigned word = 0;
+                if (t < total) {
+                    e = __ldg(g.ball + oj);
+                    word = __ldg(row + (e.x >> 5));
+                    hit = (word >> (e.x & 31)) & 1u;
+                }
+                const unsigned m = __ballot_sync(FULL, hit);
+                if (!m) continue;
+                int b;
+                if constexpr (NW == 1) {
+                    b = np;
+                    np += __popc(m);
+                } else {
+                    b = 0;
+                    if (lane == 0) b = atomicAdd(&M.cnt[F_NP], __popc(m));
+                    b = __shfl_sync(FULL, b, 0);
+                }
+                if (hit) {
+                    const int j = b + __popc(m & ((1u << lane) - 1u));
+                    const int f = S.wcum[e.x >> 5] + __popc(word & ((1u << (e.x & 31)) - 1u));
+                    if (j < F.pcap) F.pr[j] = pk_pair(base + ow, f, e.y);
+                }
+            }
+        }
+        if constexpr (NW == 1)
+            if (lane == 0) M.cnt[F_NP] = np;
+        flags = T.template red32<2>(flags);
+        if constexpr (NW == 1) T.sync();
+        if (flags) return USE_GENERAL;
+        np0 = M.cnt[F_NP];
+        if (np0 <= F.pcap && np0 < (1 << 18)) break;
+        if (!small) return USE_GENERAL;
+        T.sync();
+    }
+    fast_components(F, np0, np0, K, T);
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) {
+        const int r = F.comp[s];
+        atomicAdd(&F.cw[r], 1u);
+        if (2LL * F.bd[s] <= (long long)g.b1) atomicOr(&F.cw[r], 1u << 31);
+    }
+    // pairs within d_1, each noted at its two events: the pair of an accepted
+    // two-event cluster
+#pragma unroll 1
+    for (int i = T.tid(); i < np0; i += T.NT) {
+        const unsigned long long p = F.pr[i];
+        if (pr_val(p) > g.d1) continue;
+        atomicAdd(&F.cw[F.comp[pr_lo(p)]], 1u << 12);
+        F.px[pr_lo(p)] = i;
+        F.px[pr_hi(p)] = i;
+    }
+    T.sync();
+    // level-1 clusters in closed form; the other clusters (from the front of
+    // xsrc) and the islands (from its back) are listed by their lowest event
+    long long wsum = 0;
+    unsigned long long osum = 0;
+    IslRec *const recs = reinterpret_cast<IslRec *>(S.wl0);   // of the islands, by their lowest event
+    // of the level-1 clusters run (lane 0 of each warp)
+    long long lw = 0;
+    unsigned long long lo = 0;
+    int lnm = 0, lmax = 0, ltlast = 0, lnx = 0;
+    // what a closed form adds to the result
+    auto closed = [&](int s, int st, int d) {
+        if (st == MATE_BOUNDARY) {
+            wsum += F.bd[s];
+            osum ^= __ldg(g.eobs + (unsigned)(__ldg(g.vbnd + F.svtx[s]) & 0xffffffffu));
+            if (paths) put_path(S, &M.cnt[F_NPATH], s, -1, F.bd[s]);
+        } else {
+            wsum += d / 2;
+            if (paths && s < st) put_path(S, &M.cnt[F_NPATH], s, st, d);
+        }
+    };
+    int t1 = 0, ncl1 = 0, nres1 = 0;
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) {
+        const int r = F.comp[s];
+        const unsigned cw = F.cw[r];
+        const int size = (int)(cw & 4095u), prs = (int)(cw >> 12) & 0x7ffff;
+        const bool ok = prs == size * (size - 1) / 2 && ((cw >> 31) || size % 2 == 0);
+        if (ok && size <= 2) {
+            int st = MATE_BOUNDARY, rad = F.bd[s], d = 0;   // one boundary event at time bd
+            bool fine = true;
+            if (size == 2) {
+                const unsigned long long p = F.pr[F.px[s]];
+                st = pr_lo(p) == s ? pr_hi(p) : pr_lo(p);
+                d = pr_val(p);
+                rad = d / 2;   // one collision at time d/2
+                fine = rad <= F.bd[s] && rad <= F.bd[st];
+            }
+            if (fine) {
+                F.st[s] = st;
+                F.px[s] = rad;
+                t1 = max(t1, rad); nres1++;
+                if (s == r) ncl1++;
+                closed(s, st, d);
+                continue;
+            }
+        }
+        if (ok) F.st[s] = ST_RUN;
+        if (s == r) {
+            if (ok) { S.xsrc[atomicAdd(&M.cnt[F_N1], 1)] = s; nres1 += size; ncl1++; }
+            else S.xsrc[K - 1 - atomicAdd(&M.cnt[F_N2], 1)] = s;
+        }
+    }
+    T.sync();
+    const int n1 = M.cnt[F_N1];
+    if (dg) t1 = T.maxi(t1);
+    // the remaining level-1 clusters
+    int fail = 0;
+    Isl &I = M.isl[T.warp()];
+    int n2 = M.cnt[F_N2], nall = n2, naged = 0;
+    const int *all = S.xsrc + (K - n2);   // the islands
+#pragma unroll 1
+    for (int round = 0;; round++) {
+        if (round == 0 && n1 > 0) {
+#pragma unroll 1
+            for (int i = T.warp(); i < n1 && !fail; i += NW) {
+                const int c = S.xsrc[i];
+                IslRec r;
+                fail = run_island(S, C, F, I, c, (int)(F.cw[c] & 4095u), np0, 0, true, paths, T.lane, r) != ISL_OK;
+                if (T.lane == 0 && !fail) {
+                    lw += r.w; lo ^= r.o;
+                    lnm += r.nm; lmax = max(lmax, r.nm); ltlast = max(ltlast, r.tlast); lnx += r.nx;
+                }
+            }
+            if (dg) t1 = max(t1, T.maxi(ltlast));
+        }
+#pragma unroll 1
+        for (int i = T.warp(); i < n2 && !fail; i += NW) {
+            const int c = S.xsrc[K - 1 - i];
+            IslRec r;
+            r.size = -1;
+            fail = run_island(S, C, F, I, c, (int)(F.cw[c] & 4095u), np0, t1, false, paths, T.lane, r) == ISL_FAIL;
+            if (T.lane == 0) recs[c] = r;
+        }
+        fail = T.template red32<2>(fail);
+        if constexpr (NW == 1) T.sync();
+        if (fail) return USE_GENERAL;
+        // pairs recorded by extensions join different islands or clusters when
+        // the radii reach their distance
+        const int np1 = M.cnt[F_NP];
+        naged = M.cnt[F_AGED];
+        if (naged > K) return USE_GENERAL;
+        const int nstop = M.cnt[F_STOP];
+        if (np1 == np0) {
+            if (nstop) return USE_GENERAL;
+            break;
+        }
+        bool met = false;
+#pragma unroll 1
+        for (int i = np0 + T.tid(); i < np1; i += T.NT) {
+            const unsigned long long p = F.pr[i];
+            const int a = pr_lo(p), b = pr_hi(p);
+            if (F.comp[a] != F.comp[b] && F.px[a] + F.px[b] >= pr_val(p)) {
+                met = true;
+                if (F.st[a] == ST_RUN || F.st[b] == ST_RUN) fail = 1;
+                F.pr[i] = p | MET;
+                F.cw[F.comp[a]] = 0;
+                F.cw[F.comp[b]] = 0;
+            }
+        }
+        T.sync();
+        // a stopped island that met nothing needs explored balls
+#pragma unroll 1
+        for (int i = nstop ? T.tid() : n2; i < n2; i += T.NT)
+            if (F.cw[S.xsrc[K - 1 - i]] == ISL_ALONE) fail = 1;
+        if (T.any(fail != 0)) return USE_GENERAL;
+        if (!T.any(met)) break;
+        if (round == 32) return USE_GENERAL;
+        // join what met and run what was joined (with paths: everything, since
+        // their list starts over)
+        if (paths && n1) return USE_GENERAL;
+        fast_components(F, np0, np1, K, T);
+#pragma unroll 1
+        for (int s = T.tid(); s < K; s += T.NT) {
+            F.cw[s] = 0;
+            if (round == 0 && F.st[s] != MATE_NONE) recs[s].size = 0;   // not an island so far
+        }
+        if (T.tid() == 0) {
+            M.cnt[F_NP] = np0; M.cnt[F_N2] = 0; M.cnt[F_NALL] = 0; M.cnt[F_NPATH] = 0; M.cnt[F_STOP] = 0;
+        }
+        T.sync();
+#pragma unroll 1
+        for (int s = T.tid(); s < K; s += T.NT) atomicAdd(&F.cw[F.comp[s]], 1u);
+        T.sync();
+        wsum = 0;
+        osum = 0;
+#pragma unroll 1
+        for (int s = T.tid(); s < K; s += T.NT) {
+            const int c = F.comp[s], size = (int)F.cw[c], st = F.st[s];
+            if ((st == MATE_BOUNDARY && size == 1) || (st >= 0 && size == 2)) {
+                closed(s, st, 2 * F.px[s]);
+            } else if (s == c && st != ST_RUN) {
+                S.xcnt[atomicAdd(&M.cnt[F_NALL], 1)] = s;
+                if (paths || recs[s].size != size) S.xsrc[K - 1 - atomicAdd(&M.cnt[F_N2], 1)] = s;
+            }
+        }
+        T.sync();
+        n2 = M.cnt[F_N2];
+        nall = M.cnt[F_NALL];
+        all = S.xcnt;
+    }
+    // the islands together
+    int ntop = 0, ncut = 0, tlast = 0, tnx = 0;
+#pragma unroll 1
+    for (int i = T.tid(); i < nall; i += T.NT) {
+        const IslRec r = recs[all[i]];
+        wsum += r.w;
+        osum ^= r.o;
+        ntop += r.nm; ncut += r.ncut; tlast = max(tlast, r.tlast); tnx += r.nx;
+    }
+    const long long budget = min(A.max_events, 256LL * K + 4096);
+    if (budget < 256LL * K + 4096) {   // a budget set lower: the run over everything counts exactly
+        if ((long long)T.add(lnm + lnx + ntop + tnx) + naged + n1 + 2 > budget) return USE_GENERAL;
+    }
+    int aged = 0;
+    if (dg) {   // bands: one per time at which regions of the top level came of age
+#pragma unroll 1
+        for (int i = T.tid(); i < naged; i += T.NT) {
+            // (entries of islands that were joined since don't count)
+            auto live = [&](int k) { return F.comp[S.sbeg[k]] == S.sbeg[k] && recs[S.sbeg[k]].size == S.scnt[k]; };
+            const int x = S.xR[i];
+            int first = live(i);
+#pragma unroll 1
+            for (int j = 0; j < i && first; j++) first = !(S.xR[j] == x && live(j));
+            aged += first;
+        }
+        aged = T.add(aged);
+    }
+    const long long wint = T.sum64(wsum + lw);
+    unsigned long long ob = T.xor64(osum ^ lo);
+    if (paths) {
+        const unsigned long long po = walk_paths<WIN>(A, S, C, T, F.svtx, M.cnt[F_NPATH], 1,
+                                                      WIN ? A.carry + (row - A.syn) : nullptr);
+        const int err = T.bcast(ldr(&S.ctr[C_ERR]));
+        if (C.paths) release_tables(S, C, T, err != 0);
+        if (err) return USE_GENERAL;
+        ob = WIN ? po : ob ^ po;
+    }
+    w_out = wint / 2;
+    o_out = ob;
+    if (dg) {
+        // parallel event count over level 1 and the top level (Methods,
+        // "Numerical evaluation")
+        const int ncl = T.add(ncl1), nres = T.add(nres1);
+        lnm = T.add(lnm); lnx = T.add(lnx); lmax = T.maxi(lmax);
+        ntop = T.add(ntop); ncut = T.add(ncut); tnx = T.add(tnx); tlast = T.maxi(tlast);
+        // closed forms have one event each
+        const int e1 = max(lmax, ncl > n1 ? 1 : 0), ntot = (ncl - n1) + lnm;
+        if (T.tid() == 0) {
+            dg[QEC_DIAG_E_IDEAL] = ntop > 0 ? max(e1, ncut) + ntop - ncut : e1;
+            dg[QEC_DIAG_T_IDEAL] = ntop > 0 ? max(t1, tlast) : t1;
+            dg[QEC_DIAG_EVENTS] = ntot + ntop;
+            dg[QEC_DIAG_L1_CLUSTERS] = ncl;
+            dg[QEC_DIAG_L1_DEFECTS] = nres;
+            dg[QEC_DIAG_TOP_EVENTS] = ntop;
+            dg[QEC_DIAG_BANDS] = lnx + tnx + aged + (nall > 0 ? 1 : 0);
+            dg[QEC_DIAG_DEFECTS] = K;
+        }
+    }
+    return QEC_SHOT_OK;
+}
+
 // Detection events of a syndrome row (padding bits beyond n ignored).  One warp.
 __device__ int count_defects(const DGraph &g, const unsigned *row, int lane) {
     int c = 0;
@@ -2120,8 +3197,19 @@ __device__ int count_defects(const DGraph &g, const unsigned *row, int lane) {
     return (int)__reduce_add_sync(FULL, (unsigned)c);
 }
 
+// The general path: attempts with larger and larger tables.
 template <bool WIN, int NW>
-__device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, Team<NW> &T,
+__device__ __noinline__ int decode_general(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
+                                           Team<NW> T, unsigned long long deadline, long long &w,
+                                           unsigned long long &o, int *dg) {
+    int status = -1;
+    for (unsigned scale = 1; scale <= 64 && status == -1; scale *= 4)
+        status = decode_attempt<WIN, NW>(A, S, g, row, T, scale, deadline, w, o, dg);
+    return status;
+}
+
+template <bool WIN, int NW>
+__device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, Team<NW> &T, FastShared<NW> &M,
                             unsigned long long deadline) {
     int gi = A.graph_of_shot ? A.graph_of_shot[shot] : 0;
     if (gi < 0 || gi >= A.num_graphs) gi = 0;
@@ -2139,19 +3227,21 @@ __device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, T
                 if (T.warp() == 0) {
                     Team<1> T1;
                     T1.lane = T.lane;
-                    decode_shot<WIN, 1>(A, S, shot, T1, deadline);
+                    decode_shot<WIN, 1>(A, S, shot, T1, reinterpret_cast<FastShared<1> &>(M), deadline);
                 }
                 T.sync();
                 return;
             }
         }
     }
-    int status = -1;
     long long w = 0;
     unsigned long long o = 0;
     int *dg = A.diag_out ? A.diag_out + shot * QEC_DIAG_FIELDS : nullptr;
-    for (unsigned scale = 1; scale <= 64 && status == -1; scale *= 4)
-        status = decode_attempt<WIN, NW>(A, S, g, row, T, scale, deadline, w, o, dg);
+    int status = decode_fast<WIN, NW>(A, S, g, row, T, M, w, o, dg);
+    if (status == USE_GENERAL) {
+        T.sync();
+        status = decode_general<WIN, NW>(A, S, g, row, T, deadline, w, o, dg);
+    }
     const bool retried = status < 0 && A.pass == 0 && A.single_shot < 0;   // goes to the overflow pass
     if (status < 0) {
         status = QEC_SHOT_CAPACITY;
@@ -2189,8 +3279,10 @@ __device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, T
 template <bool WIN, int NW>
 __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW, NW == 1 ? QEC_MIN_BLOCKS : (NW == 4 ? 4 : 1))
 batch_kernel(const __grid_constant__ BatchArgs a) {
+    extern __shared__ __align__(16) char dyn[];   // one FastShared per team
     Team<NW> T;
     T.lane = threadIdx.x & 31;
+    FastShared<NW> &M = reinterpret_cast<FastShared<NW> *>(dyn)[NW == 1 ? threadIdx.x >> 5 : 0];
     if constexpr (NW > 1) {
         __shared__ TeamShared tsh;
         T.sh = &tsh;
@@ -2207,7 +3299,7 @@ batch_kernel(const __grid_constant__ BatchArgs a) {
         deadline = T.bcast64(t0) + (unsigned long long)a.watchdog_ns;
     }
     if (a.single_shot >= 0) {
-        if (wid == 0) decode_shot<WIN, NW>(a, S, a.single_shot, T, deadline);
+        if (wid == 0) decode_shot<WIN, NW>(a, S, a.single_shot, T, M, deadline);
         return;
     }
     unsigned long long *counter = a.queue + (a.pass == 0 ? 0 : 2);
@@ -2219,7 +3311,7 @@ batch_kernel(const __grid_constant__ BatchArgs a) {
         if ((long long)item >= limit) break;
         const long long shot = a.pass == 0 ? (a.order ? (long long)a.order[item] : (long long)item)
                                            : (long long)a.overflow[item];
-        decode_shot<WIN, NW>(a, S, shot, T, deadline);
+        decode_shot<WIN, NW>(a, S, shot, T, M, deadline);
     }
 }
 
@@ -2296,18 +3388,39 @@ SlabCaps caps_for_kcap(int kcap, int table_factor) {
     return c;
 }
 
-cudaError_t launch_batch(const BatchArgs &a, int grid, int block, cudaStream_t s, int team) {
-    if (a.carry) {
-        if (team == TEAM_BIG) batch_kernel<true, TEAM_BIG><<<grid, 32 * TEAM_BIG, 0, s>>>(a);
-        else batch_kernel<true, 1><<<grid, block, 0, s>>>(a);
-    } else if (team == TEAM_BIG) {
-        batch_kernel<false, TEAM_BIG><<<grid, 32 * TEAM_BIG, 0, s>>>(a);
-    } else if (team == TEAM_MID) {
-        batch_kernel<false, TEAM_MID><<<grid, 32 * TEAM_MID, 0, s>>>(a);
-    } else {
-        batch_kernel<false, 1><<<grid, block, 0, s>>>(a);
+namespace {
+
+// Launch one instantiation with its teams' shared memory (above 48 KB a kernel
+// needs the attribute, set on every launch of the current device: it is per
+// device, and a microsecond).
+template <bool WIN, int NW>
+cudaError_t launch_as(const BatchArgs &a, int grid, int block, cudaStream_t s) {
+    const int smem = (int)sizeof(FastShared<NW>) * (NW == 1 ? block / 32 : 1);
+    if (smem + (int)sizeof(TeamShared) > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(batch_kernel<WIN, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
     }
+    batch_kernel<WIN, NW><<<grid, NW == 1 ? block : 32 * NW, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <int NW>
+int blocks_per_sm(int block) {
+    const int smem = (int)sizeof(FastShared<NW>) * (NW == 1 ? block / 32 : 1);
+    int nb = 0;
+    cudaError_t e = cudaFuncSetAttribute(batch_kernel<false, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, NW>, block, (size_t)smem);
+    return e == cudaSuccess && nb > 0 ? nb : 1;
+}
+
+}  // namespace
+
+cudaError_t launch_batch(const BatchArgs &a, int grid, int block, cudaStream_t s, int team) {
+    if (a.carry) return team == TEAM_BIG ? launch_as<true, TEAM_BIG>(a, grid, block, s) : launch_as<true, 1>(a, grid, block, s);
+    if (team == TEAM_BIG) return launch_as<false, TEAM_BIG>(a, grid, block, s);
+    if (team == TEAM_MID) return launch_as<false, TEAM_MID>(a, grid, block, s);
+    return launch_as<false, 1>(a, grid, block, s);
 }
 
 int max_block_threads() {
@@ -2316,20 +3429,9 @@ int max_block_threads() {
     return fa.maxThreadsPerBlock > 0 ? fa.maxThreadsPerBlock : 32;
 }
 
-int occupancy_blocks(int block_threads) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, 1>, block_threads, 0) != cudaSuccess) return 1;
-    return nb > 0 ? nb : 1;
-}
+int occupancy_blocks(int block_threads) { return blocks_per_sm<1>(block_threads); }
 
-int team_occupancy_blocks(int team) {
-    int nb = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-    if (team == TEAM_BIG) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, TEAM_BIG>, 32 * TEAM_BIG, 0);
-    else if (team == TEAM_MID) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, TEAM_MID>, 32 * TEAM_MID, 0);
-    if (e != cudaSuccess) return 1;
-    return nb > 0 ? nb : 1;
-}
+int team_occupancy_blocks(int team) { return team == TEAM_BIG ? blocks_per_sm<TEAM_BIG>(32 * TEAM_BIG) : blocks_per_sm<TEAM_MID>(32 * TEAM_MID); }
 
 namespace {
 
