@@ -376,7 +376,7 @@ struct Workspace {
 
 Workspace g_ws[64];
 std::mutex g_tune_mu;
-qec_tuning g_tune = {4, 0, 1, 0, 4000000, 0, 2048, 1};
+qec_tuning g_tune = {8, 0, 1, 0, 4000000, 0, 2048, 1};
 
 void ws_free(Workspace &w) {
     if (w.slabs) cudaFree(w.slabs);
@@ -691,11 +691,15 @@ int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) {
     d.eobs = g->d_eobs;
     d.eend = g->d_eend;
     d.seid = g->d_seid;
-    const std::vector<unsigned long long> vb = boundary_candidates(n, D);
-    ce = cudaMalloc(&g->d_vbnd, sizeof(unsigned long long) * (size_t)n);
+    std::vector<unsigned long long> vb = boundary_candidates(n, D);
+    vb.resize(2 * (size_t)n, 0);   // then the observable mask of every candidate's edge
+    for (int x = 0; x < n; x++)
+        if (vb[(size_t)x] != ~0ull) vb[(size_t)n + x] = g->eobs[(size_t)(unsigned)vb[(size_t)x]];
+    ce = cudaMalloc(&g->d_vbnd, sizeof(unsigned long long) * vb.size());
     if (ce == cudaSuccess)
-        ce = cudaMemcpy(g->d_vbnd, vb.data(), sizeof(unsigned long long) * (size_t)n, cudaMemcpyHostToDevice);
+        ce = cudaMemcpy(g->d_vbnd, vb.data(), sizeof(unsigned long long) * vb.size(), cudaMemcpyHostToDevice);
     d.vbnd = g->d_vbnd;
+    d.vobs = g->d_vbnd + n;
     if (ce == cudaSuccess) ce = qec::build_ball_table(d, &g->d_bhdr, &g->d_ball);
     if (ce == cudaErrorMemoryAllocation) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
     if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "graph tables"); }
@@ -824,7 +828,7 @@ int qec_set_tuning(const qec_tuning *t) {
         return fail(QEC_EINVAL, "tuning value out of range");
     if (t->team_warps > 0 && t->team_warps != 1 && t->team_warps != qec::TEAM_MID && t->team_warps != qec::TEAM_BIG)
         return fail(QEC_EINVAL, "team_warps must be 1, 4 or 16 (0 keeps, negative = automatic)");
-    static const qec_tuning defaults = {4, 0, 1, 0, 4000000, 0, 2048, 1};
+    static const qec_tuning defaults = {8, 0, 1, 0, 4000000, 0, 2048, 1};
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto pick = [](auto v, auto cur, auto def) { return v > 0 ? v : (v < 0 ? def : cur); };
     g_tune.warps_per_block = pick(t->warps_per_block, g_tune.warps_per_block, defaults.warps_per_block);

@@ -69,6 +69,7 @@
 // from 1.42 to 0.92 ms.
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cstdint>
 
@@ -78,8 +79,8 @@
 #ifndef QEC_HT_FACTOR
 #define QEC_HT_FACTOR 64   // explored-table slots per detection event (rounded up to a power of two)
 #endif
-#ifndef QEC_MIN_BLOCKS
-#define QEC_MIN_BLOCKS 6   // 128-thread blocks per SM the register budget must allow
+#ifndef QEC_MAX_WARPS
+#define QEC_MAX_WARPS 8   // warps of a block that decode a shot each; 24 of them fit an SM
 #endif
 
 namespace qec {
@@ -2142,65 +2143,24 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
 // changes are disjoint and the canonical order restricted to an island is the
 // order of its own events.  So each island is run by itself, one warp each with
 // the whole state in shared memory, and afterwards every recorded pair that
-// joins two of them is checked: if the largest radii reach its distance, the
-// shot is decoded again by the run over all events.
+// joins two of them is checked: where the largest radii reach its distance, the
+// two are joined (an accepted cluster's events frozen as level 1 left them) and
+// run again.  A pair that can become tight is always recorded: see reach_of.
 //
 // A run over everything costs a scan of all events and pairs per event: a d =
 // 51 window at p = 0.003 (1,170 events, 250 matcher events in 88 islands of at
 // most ~12 events) spent 87 % of its time there, a d = 21 shot (6 islands) 67 %.
-// Islands or shots outside the limits below take that run.
+// Something is joined in 0.5 % of d = 21 shots and 11 % of those windows.
+//
+// Shots outside the limits below take the run over everything (the general
+// path).  The phases are separate functions whose loops are not unrolled, and
+// what they share lies in shared memory: with everything inlined and unrolled
+// the million-shot batch was 40 % slower, waiting for instructions and spilled
+// registers.
 constexpr int IN = 32;    // events of an island (one lane each); blossoms are nodes IN .. 2 IN - 1
 constexpr int IP = 64;    // pairs
 constexpr int IC = 96;    // blossom cycle entries
-
-struct __align__(16) Isl {
-    int y[2 * IN], rad[IN], pd[IP], ev[IN];
-    unsigned char pa[IP], pb[IP];
-    signed char lab[2 * IN], bpar[2 * IN], tpar[2 * IN], tps[2 * IN], tpo[2 * IN];
-    signed char mate[2 * IN], ms[2 * IN], mo[2 * IN], root[2 * IN], minl[2 * IN], top[IN];
-    unsigned char cn[IC], cs[IC], co[IC], cb[IN], cl[IN];   // cycles: child, its leaf, the next child's leaf
-    signed char ta[2 * IN], tb[2 * IN];                     // tree paths / expansion stack
-    int nc, err;
-};
-
-// Shared memory of a team: per-event arrays of shots with at most KS events
-// (larger shots use the slab), and one island per warp.
-template <int NW>
-struct __align__(16) FastShared {
-    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + KS / 4;
-    unsigned long long pr[PS];
-    int svtx[KS], bd[KS], comp[KS], px[KS], st[KS];
-    unsigned cw[KS];
-    int cnt[8];
-    Isl isl[NW];
-};
-
-enum { ST_RUN = -3 };
-enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2 };
-constexpr unsigned ISL_ALONE = 1u << 31;
-enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6 };   // FastShared::cnt
-
-// Per-event arrays of the shot being decoded (shared memory or slab).
-//   pr: pairs, lo << 46 | hi << 28 | distance; svtx: vertex; bd: boundary
-//   distance (INT_MAX: none); comp: lowest event of the component; cw, at a
-//   component's lowest event: size | pairs within d_1 << 12 | boundary contact
-//   << 31; px: a pair within d_1, later the largest radius; st: level-1 state,
-//   the partner or MATE_BOUNDARY in a closed form, MATE_NONE: a growing root of
-//   the top level, ST_RUN: in a level-1 cluster that was run
-struct Fast {
-    unsigned long long *pr;
-    int *svtx, *bd, *comp, *px, *st;
-    unsigned *cw;
-    int *cnt;
-    int pcap;
-};
-
-__device__ __forceinline__ unsigned long long pk_pair(int a, int b, int d) {
-    return ((unsigned long long)(unsigned)a << 46) | ((unsigned long long)(unsigned)b << 28) | (unsigned)d;
-}
-__device__ __forceinline__ int pr_lo(unsigned long long p) { return (int)(p >> 46); }
-__device__ __forceinline__ int pr_hi(unsigned long long p) { return (int)(p >> 28) & 0x3ffff; }
-__device__ __forceinline__ int pr_val(unsigned long long p) { return (int)(p & 0xfffffffu); }
+constexpr int LAB1 = 1 << 6;
 
 // What one island, or several, add to the shot (w: internal units).
 struct __align__(16) IslRec {
@@ -2208,6 +2168,83 @@ struct __align__(16) IslRec {
     int w, size;
     int nm, ncut, tlast, nx;   // matcher events, those at times <= tcut, time of the last, bands counted here
 };
+
+struct __align__(16) Isl {
+    int2 pair[IP];        // distance, lower event | higher event << 8
+    int pk[IN];           // per event: radius << 8 | (label of its top node + 1) << 6 | top node
+    int y[2 * IN];        // duals (leaves: written at the end)
+    int ev[IN], bd[IN];   // event of the shot, boundary distance
+    int xt[IN];           // radius at which the explored radius falls due (INT_MAX: ball exhausted)
+    int meet[IN];         // radius at which the region touches a level-1 cluster outside
+    IslRec rec;           // result
+    signed char lab[2 * IN], bpar[2 * IN], tpar[2 * IN], tps[2 * IN], tpo[2 * IN];
+    signed char mate[2 * IN], ms[2 * IN], mo[2 * IN], root[2 * IN], minl[2 * IN];
+    unsigned char cn[IC], cs[IC], co[IC], cb[IN], cl[IN];   // cycles: child, its leaf, the next child's leaf
+    signed char ta[2 * IN], tb[2 * IN];                     // tree paths / expansion stack
+    int nc, err;
+    __device__ __forceinline__ int top(int e) const { return pk[e] & (LAB1 - 1); }
+};
+
+enum { ST_RUN = -3 };
+enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2 };
+constexpr unsigned ISL_ALONE = 1u << 31;
+constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
+enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6, F_FAIL = 7, F_TOTAL = 8 };   // Fast::cnt
+
+// The shot being decoded by a team.  Per-event arrays, `stride` ints each, in
+// shared memory or, for shots with more events than it holds, in the slab:
+//   svtx  vertex                      bd  boundary distance (INT_MAX: none)
+//   comp  lowest event of the component
+//   px    a pair within d_1, later the largest radius
+//   st    level-1 state: the partner or MATE_BOUNDARY in a closed form,
+//         MATE_NONE: a growing root of the top level, ST_RUN: in a level-1
+//         cluster that was run
+//   cw    at a component's lowest event: size | pairs within d_1 << 12 |
+//         boundary contact << 31; in an island, the event's lane
+// and the pairs, lo << 46 | hi << 28 | distance.
+struct __align__(16) Fast {
+    const DGraph *g;
+    const unsigned *row;
+    const int *wcum;
+    int *ev;
+    unsigned long long *pr;
+    IslRec *recs;                      // of the islands, by their lowest event
+    int *list, *all;                   // clusters and islands to run; all islands once some were joined
+    int *aged_t, *aged_c, *aged_n;     // bands of regions that came of age: time, island, its size
+    int *pa, *pb, *pd;                 // matched pairs for the path walks
+    int stride, pcap, K, np0, tcut, L, band, paths;
+    int cnt[F_TOTAL];
+    __device__ __forceinline__ int *svtx() const { return ev; }
+    __device__ __forceinline__ int *bd() const { return ev + stride; }
+    __device__ __forceinline__ int *comp() const { return ev + 2 * stride; }
+    __device__ __forceinline__ int *px() const { return ev + 3 * stride; }
+    __device__ __forceinline__ int *st() const { return ev + 4 * stride; }
+    __device__ __forceinline__ unsigned *cw() const { return reinterpret_cast<unsigned *>(ev + 5 * stride); }
+    __device__ __forceinline__ bool defect(int v) const { return (__ldg(row + (v >> 5)) >> (v & 31)) & 1u; }
+    __device__ __forceinline__ int rank(int v) const {
+        return wcum[v >> 5] + __popc(__ldg(row + (v >> 5)) & ((1u << (v & 31)) - 1u));
+    }
+    // as reach_of
+    __device__ __forceinline__ int reach(int b1, int R) const { return R - L + max(R - L, (b1 + 1) >> 1); }
+};
+
+// Shared memory of a team: the shot, per-event arrays of shots with at most KS
+// events, and one island per warp.
+template <int NW>
+struct __align__(16) FastShared {
+    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + KS / 4;
+    Fast f;
+    unsigned long long pr[PS];
+    int ev[6 * KS];
+    Isl isl[NW];
+};
+
+__device__ __forceinline__ unsigned long long pk_pair(int a, int b, int d) {
+    return ((unsigned long long)(unsigned)a << 46) | ((unsigned long long)(unsigned)b << 28) | (unsigned)d;
+}
+__device__ __forceinline__ int pr_lo(unsigned long long p) { return (int)(p >> 46); }
+__device__ __forceinline__ int pr_hi(unsigned long long p) { return (int)(p >> 28) & 0x3ffff; }
+__device__ __forceinline__ int pr_val(unsigned long long p) { return (int)(p & (MET - 1)); }
 
 __device__ __forceinline__ int isl_child_of(const Isl &I, int B, int leaf) {
     int v = leaf;
@@ -2228,99 +2265,140 @@ __device__ __forceinline__ void isl_flip(Isl &I, int A) {
     }
 }
 
-// Event (c) on lane 0: the new blossom N over outer A, B of one tree; false
-// when the cycle pool is full.
-__device__ __noinline__ bool isl_blossom(Isl &I, int N, int A, int a, int B, int b) {
-    int na = 0, nb = 0;
+// Event (c): the new blossom N over outer A, B of one tree.  `bal`: blossoms
+// alive before.  Returns the event's top node, or -1 when the cycle pool is
+// full.  One warp.
+__device__ __noinline__ int isl_blossom(Isl &I, int N, int A, int a, int B, int b, int n, unsigned bal, int lane) {
+    int ok = 1;
+    if (lane == 0) {
+        int na = 0, nb = 0;
 #pragma unroll 1
-    for (int v = A; v >= 0; v = I.tpar[v]) I.ta[na++] = (signed char)v;
+        for (int v = A; v >= 0; v = I.tpar[v]) I.ta[na++] = (signed char)v;
 #pragma unroll 1
-    for (int v = B; v >= 0; v = I.tpar[v]) I.tb[nb++] = (signed char)v;
+        for (int v = B; v >= 0; v = I.tpar[v]) I.tb[nb++] = (signed char)v;
 #pragma unroll 1
-    while (na > 1 && nb > 1 && I.ta[na - 2] == I.tb[nb - 2]) { na--; nb--; }
-    const int Lc = I.ta[na - 1], m = na + nb - 1, cb = I.nc;
-    if (cb + m > IC) return false;
-    I.nc = cb + m;
-    int i = 0;
-    I.cn[cb + i++] = (unsigned char)Lc;
+        while (na > 1 && nb > 1 && I.ta[na - 2] == I.tb[nb - 2]) { na--; nb--; }
+        const int Lc = I.ta[na - 1], m = na + nb - 1, cb = I.nc;
+        if (cb + m > IC) {
+            ok = 0;
+        } else {
+            I.nc = cb + m;
+            int i = 0;
+            I.cn[cb + i++] = (unsigned char)Lc;
 #pragma unroll 1
-    for (int j = na - 2; j >= 0; j--) I.cn[cb + i++] = (unsigned char)I.ta[j];
+            for (int j = na - 2; j >= 0; j--) I.cn[cb + i++] = (unsigned char)I.ta[j];
 #pragma unroll 1
-    for (int j = 0; j <= nb - 2; j++) I.cn[cb + i++] = (unsigned char)I.tb[j];
-    const int ia = na - 1;
-    int ml = IN;
+            for (int j = 0; j <= nb - 2; j++) I.cn[cb + i++] = (unsigned char)I.tb[j];
+            const int ia = na - 1;
+            int ml = IN;
 #pragma unroll 1
-    for (int j = 0; j < m; j++) {
-        const int x = I.cn[cb + j], z = I.cn[cb + (j + 1 < m ? j + 1 : 0)];
-        if (j < ia) { I.cs[cb + j] = I.tpo[z]; I.co[cb + j] = I.tps[z]; }
-        else if (j == ia) { I.cs[cb + j] = (unsigned char)a; I.co[cb + j] = (unsigned char)b; }
-        else { I.cs[cb + j] = I.tps[x]; I.co[cb + j] = I.tpo[x]; }
-        ml = min(ml, (int)I.minl[x]);
-        I.bpar[x] = (signed char)N;
+            for (int j = 0; j < m; j++) {
+                const int x = I.cn[cb + j], z = I.cn[cb + (j + 1 < m ? j + 1 : 0)];
+                if (j < ia) { I.cs[cb + j] = I.tpo[z]; I.co[cb + j] = I.tps[z]; }
+                else if (j == ia) { I.cs[cb + j] = (unsigned char)a; I.co[cb + j] = (unsigned char)b; }
+                else { I.cs[cb + j] = I.tps[x]; I.co[cb + j] = I.tpo[x]; }
+                ml = min(ml, (int)I.minl[x]);
+                I.bpar[x] = (signed char)N;
+            }
+            I.y[N] = 0; I.lab[N] = 1; I.bpar[N] = -1;
+            I.tpar[N] = I.tpar[Lc]; I.tps[N] = I.tps[Lc]; I.tpo[N] = I.tpo[Lc];
+            I.mate[N] = I.mate[Lc]; I.ms[N] = I.ms[Lc]; I.mo[N] = I.mo[Lc];
+            I.root[N] = I.root[Lc] == Lc ? (signed char)N : I.root[Lc];
+            I.minl[N] = (signed char)ml;
+            I.cb[N - IN] = (unsigned char)cb; I.cl[N - IN] = (unsigned char)m;
+        }
     }
-    I.y[N] = 0; I.lab[N] = 1; I.bpar[N] = -1;
-    I.tpar[N] = I.tpar[Lc]; I.tps[N] = I.tps[Lc]; I.tpo[N] = I.tpo[Lc];
-    I.mate[N] = I.mate[Lc]; I.ms[N] = I.ms[Lc]; I.mo[N] = I.mo[Lc];
-    I.root[N] = I.root[Lc] == Lc ? (signed char)N : I.root[Lc];
-    I.minl[N] = (signed char)ml;
-    I.cb[N - IN] = (unsigned char)cb; I.cl[N - IN] = (unsigned char)m;
-    return true;
+    if (!__shfl_sync(FULL, ok, 0)) return -1;
+    __syncwarp();
+    const int L0 = I.cn[I.cb[N - IN]];   // if it was its tree's root, N is now
+#pragma unroll 1
+    for (int h = 0; h < 2; h++) {
+        const int v = lane + h * IN;
+        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+        if (I.bpar[v] >= 0) continue;
+        const int tp = I.tpar[v], mt = I.mate[v];
+        if (tp >= 0 && I.bpar[tp] == N) I.tpar[v] = (signed char)N;
+        if (mt >= 0 && I.bpar[mt] == N) I.mate[v] = (signed char)N;
+        if (I.root[v] == L0) I.root[v] = (signed char)N;
+    }
+    int top = lane;
+    if (lane < n) {
+        top = I.top(lane);
+        if (I.bpar[top] == N) top = N;
+    }
+    __syncwarp();
+    return top;
 }
 
-// Event (d) on lane 0: inner blossom B shatters (tops are set by the caller).
-__device__ __noinline__ void isl_shatter(Isl &I, int B) {
-    const int m = I.cl[B - IN], cb = I.cb[B - IN];
-    const int P = I.tpar[B], Cn = I.mate[B];
-    const int xp = isl_child_of(I, B, I.tps[B]), xc = isl_child_of(I, B, I.ms[B]);
-    int ip = -1, ic = -1;
-#pragma unroll 1
-    for (int j = 0; j < m; j++) {
-        if (I.cn[cb + j] == xp) ip = j;
-        if (I.cn[cb + j] == xc) ic = j;
+// Event (d): inner blossom B shatters.  Returns the event's top node (I.err on
+// an inconsistent state).  One warp.
+__device__ __noinline__ int isl_shatter(Isl &I, int B, int n, int lane) {
+    int top = lane;
+    if (lane < n) {
+        top = I.top(lane);
+        if (top == B) top = isl_child_of(I, B, lane);
     }
-    if (ip < 0 || ic < 0 || Cn < 0) { I.err = 1; return; }
+    __syncwarp();
+    if (lane == 0) {
+        const int m = I.cl[B - IN], cb = I.cb[B - IN];
+        const int P = I.tpar[B], Cn = I.mate[B];
+        const int xp = isl_child_of(I, B, I.tps[B]), xc = isl_child_of(I, B, I.ms[B]);
+        int ip = -1, ic = -1;
 #pragma unroll 1
-    for (int j = 0; j < m; j++) I.bpar[I.cn[cb + j]] = -1;
-    auto wrap = [&](int j) { j %= m; return j < 0 ? j + m : j; };
-    const int fwd = wrap(ic - ip), dir = (fwd % 2 == 0) ? 1 : -1, Ln = dir > 0 ? fwd : m - fwd;
-    int prev = -1;
-#pragma unroll 1
-    for (int j = 0; j <= Ln; j++) {
-        const int idx = wrap(ip + dir * j), q = I.cn[cb + idx];
-        I.lab[q] = (j % 2 == 0) ? -1 : 1;
-        I.root[q] = I.root[B];
-        if (j == 0) {
-            I.tpar[q] = (signed char)P; I.tps[q] = I.tps[B]; I.tpo[q] = I.tpo[B];
-        } else {
-            const int pidx = wrap(ip + dir * (j - 1));
-            const int self = dir > 0 ? I.co[cb + pidx] : I.cs[cb + idx], other = dir > 0 ? I.cs[cb + pidx] : I.co[cb + idx];
-            I.tpar[q] = (signed char)prev; I.tps[q] = (signed char)self; I.tpo[q] = (signed char)other;
-            if (j % 2 == 1) {
-                I.mate[q] = (signed char)prev; I.ms[q] = (signed char)self; I.mo[q] = (signed char)other;
-                I.mate[prev] = (signed char)q; I.ms[prev] = (signed char)other; I.mo[prev] = (signed char)self;
-            }
+        for (int j = 0; j < m; j++) {
+            if (I.cn[cb + j] == xp) ip = j;
+            if (I.cn[cb + j] == xc) ic = j;
         }
-        prev = q;
-    }
-    I.mate[prev] = (signed char)Cn; I.ms[prev] = I.ms[B]; I.mo[prev] = I.mo[B];
-    I.mate[Cn] = (signed char)prev; I.tpar[Cn] = (signed char)prev;
+        if (ip < 0 || ic < 0 || Cn < 0) {
+            I.err = 1;
+        } else {
 #pragma unroll 1
-    for (int j = 1; j <= m - 1 - Ln; j += 2) {
-        const int i1 = wrap(ic + dir * j), i2 = wrap(ic + dir * (j + 1));
-        const int x = I.cn[cb + i1], z = I.cn[cb + i2];
-        const int lx = dir > 0 ? I.cs[cb + i1] : I.co[cb + i2], lz = dir > 0 ? I.co[cb + i1] : I.cs[cb + i2];
-        I.lab[x] = 0; I.lab[z] = 0;
-        I.tpar[x] = -1; I.tpar[z] = -1;
-        I.root[x] = -1; I.root[z] = -1;
-        I.mate[x] = (signed char)z; I.ms[x] = (signed char)lx; I.mo[x] = (signed char)lz;
-        I.mate[z] = (signed char)x; I.ms[z] = (signed char)lz; I.mo[z] = (signed char)lx;
+            for (int j = 0; j < m; j++) I.bpar[I.cn[cb + j]] = -1;
+            auto wrap = [&](int j) { j %= m; return j < 0 ? j + m : j; };
+            const int fwd = wrap(ic - ip), dir = (fwd % 2 == 0) ? 1 : -1, Ln = dir > 0 ? fwd : m - fwd;
+            int prev = -1;
+#pragma unroll 1
+            for (int j = 0; j <= Ln; j++) {
+                const int idx = wrap(ip + dir * j), q = I.cn[cb + idx];
+                I.lab[q] = (j % 2 == 0) ? -1 : 1;
+                I.root[q] = I.root[B];
+                if (j == 0) {
+                    I.tpar[q] = (signed char)P; I.tps[q] = I.tps[B]; I.tpo[q] = I.tpo[B];
+                } else {
+                    const int pidx = wrap(ip + dir * (j - 1));
+                    const int self = dir > 0 ? I.co[cb + pidx] : I.cs[cb + idx];
+                    const int other = dir > 0 ? I.cs[cb + pidx] : I.co[cb + idx];
+                    I.tpar[q] = (signed char)prev; I.tps[q] = (signed char)self; I.tpo[q] = (signed char)other;
+                    if (j % 2 == 1) {
+                        I.mate[q] = (signed char)prev; I.ms[q] = (signed char)self; I.mo[q] = (signed char)other;
+                        I.mate[prev] = (signed char)q; I.ms[prev] = (signed char)other; I.mo[prev] = (signed char)self;
+                    }
+                }
+                prev = q;
+            }
+            I.mate[prev] = (signed char)Cn; I.ms[prev] = I.ms[B]; I.mo[prev] = I.mo[B];
+            I.mate[Cn] = (signed char)prev; I.tpar[Cn] = (signed char)prev;
+#pragma unroll 1
+            for (int j = 1; j <= m - 1 - Ln; j += 2) {
+                const int i1 = wrap(ic + dir * j), i2 = wrap(ic + dir * (j + 1));
+                const int x = I.cn[cb + i1], z = I.cn[cb + i2];
+                const int lx = dir > 0 ? I.cs[cb + i1] : I.co[cb + i2], lz = dir > 0 ? I.co[cb + i1] : I.cs[cb + i2];
+                I.lab[x] = 0; I.lab[z] = 0;
+                I.tpar[x] = -1; I.tpar[z] = -1;
+                I.root[x] = -1; I.root[z] = -1;
+                I.mate[x] = (signed char)z; I.ms[x] = (signed char)lx; I.mo[x] = (signed char)lz;
+                I.mate[z] = (signed char)x; I.ms[z] = (signed char)lz; I.mo[z] = (signed char)lx;
+            }
+            I.lab[B] = 0; I.y[B] = 0;
+        }
     }
-    I.lab[B] = 0; I.y[B] = 0;
+    __syncwarp();
+    return top;
 }
 
 // Distance of two matched events of an island (as tight_dist).
 __device__ __forceinline__ int isl_dist(const Isl &I, int a, int b) {
-    int d = I.rad[a] + I.rad[b];
+    int d = (I.pk[a] >> 8) + (I.pk[b] >> 8);
 #pragma unroll 1
     for (int B = I.bpar[a]; B >= 0; B = I.bpar[B]) {
         int x = I.bpar[b];
@@ -2336,31 +2414,48 @@ __device__ __forceinline__ int isl_dist(const Isl &I, int a, int b) {
 }
 
 // A matched pair of the shot (b = -1: boundary) at distance d, for the path walks.
-__device__ __forceinline__ void put_path(const Slab &S, int *cnt, int a, int b, int d) {
-    const int k = atomicAdd(cnt, 1);   // at most one per event
-    S.tmpa[k] = a; S.tmpb[k] = b; S.cst2[k] = d;
+__device__ __forceinline__ void put_path(Fast &X, int a, int b, int d) {
+    const int k = atomicAdd(&X.cnt[F_NPATH], 1);   // at most one per event
+    X.pa[k] = a; X.pb[k] = b; X.pd[k] = d;
 }
 
-// The matched pairs inside blossom `node` whose leaf ext is matched outside, and so on down (lane 0).
-__device__ __noinline__ void isl_expand(Isl &I, const Slab &S, int *cnt, int node, int ext) {
-    int sp = 0;
-    I.ta[sp] = (signed char)node; I.tb[sp++] = (signed char)ext;
+// The matched pairs of a finished island.  One warp.
+__device__ __noinline__ void isl_paths(Fast &X, Isl &I, int n, unsigned bal, int lane) {
 #pragma unroll 1
-    while (sp > 0) {
-        const int v = I.ta[--sp], e = I.tb[sp];
-        if (v < IN) continue;
-        const int m = I.cl[v - IN], cb = I.cb[v - IN], c0 = isl_child_of(I, v, e);
-        int i0 = 0;
+    for (int h = 0; h < 2; h++) {
+        const int v = lane + h * IN;
+        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+        if (I.bpar[v] >= 0) continue;
+        const int mt = I.mate[v], s = I.ms[v];
+        if (mt == MATE_BOUNDARY) put_path(X, I.ev[s], -1, I.bd[s]);
+        else if (v < mt) put_path(X, I.ev[s], I.ev[I.mo[v]], isl_dist(I, s, I.mo[v]));
+    }
+    if (lane != 0) return;
+    // inside blossoms: the child holding the externally matched leaf keeps that
+    // match, the other children pair up along the cycle
 #pragma unroll 1
-        for (int j = 0; j < m; j++) if (I.cn[cb + j] == c0) i0 = j;
-        I.ta[sp] = (signed char)c0; I.tb[sp++] = (signed char)e;
+    for (unsigned m = bal; m; m &= m - 1) {
+        int sp = 0;
+        const int b = IN + __ffs(m) - 1;
+        if (I.bpar[b] >= 0) continue;
+        I.ta[sp] = (signed char)b; I.tb[sp++] = I.ms[b];
 #pragma unroll 1
-        for (int j = 1; j < m; j += 2) {
-            const int i1 = (i0 + j) % m, i2 = (i0 + j + 1) % m;
-            const int lx = I.cs[cb + i1], lz = I.co[cb + i1];
-            put_path(S, cnt, I.ev[lx], I.ev[lz], isl_dist(I, lx, lz));
-            I.ta[sp] = (signed char)I.cn[cb + i1]; I.tb[sp++] = (signed char)lx;
-            I.ta[sp] = (signed char)I.cn[cb + i2]; I.tb[sp++] = (signed char)lz;
+        while (sp > 0) {
+            const int v = I.ta[--sp], e = I.tb[sp];
+            if (v < IN) continue;
+            const int len = I.cl[v - IN], cb = I.cb[v - IN], c0 = isl_child_of(I, v, e);
+            int i0 = 0;
+#pragma unroll 1
+            for (int j = 0; j < len; j++) if (I.cn[cb + j] == c0) i0 = j;
+            I.ta[sp] = (signed char)c0; I.tb[sp++] = (signed char)e;
+#pragma unroll 1
+            for (int j = 1; j < len; j += 2) {
+                const int i1 = (i0 + j) % len, i2 = (i0 + j + 1) % len;
+                const int lx = I.cs[cb + i1], lz = I.co[cb + i1];
+                put_path(X, I.ev[lx], I.ev[lz], isl_dist(I, lx, lz));
+                I.ta[sp] = (signed char)I.cn[cb + i1]; I.tb[sp++] = (signed char)lx;
+                I.ta[sp] = (signed char)I.cn[cb + i2]; I.tb[sp++] = (signed char)lz;
+            }
         }
     }
 }
@@ -2371,10 +2466,10 @@ __device__ __noinline__ void isl_expand(Isl &I, const Slab &S, int *cnt, int nod
 // shorter than brad, so the event is in the list of one of those y.  Lane j gets
 // the j-th event found (rank f, exact distance d); returns their number, or -1
 // when a list is not complete or more than 32 are found.  One warp.
-__device__ __noinline__ int far_events(const Slab &S, const Shot &C, int v, int q, int lane, int &f, int &d) {
-    const DGraph &g = C.g;
+__device__ __noinline__ int far_events(const Fast &X, int v, int q, int lane, int &f, int &d) {
+    const DGraph &g = *X.g;
     const int4 h = __ldg(g.bhdr + v);
-    const int n = h.z + max(h.w, 0), r = q - g.brad + g.wmax;
+    const int n = h.z + max(h.w, 0), r = q - g.brad + g.wmax, brad = g.brad, wmax = g.wmax;
     int found = 0;
     f = -1;
     d = INT_MAX;
@@ -2385,7 +2480,7 @@ __device__ __noinline__ int far_events(const Slab &S, const Shot &C, int v, int 
         bool use = false;
         if (k + lane < n) {
             e = __ldg(g.ball + (unsigned)h.x + k + lane);
-            use = e.y > r - g.wmax && e.y <= r;
+            use = e.y > r - wmax && e.y <= r;
             if (use) he = __ldg(g.bhdr + e.x);
         }
         if (__any_sync(FULL, he.w < 0)) return -1;
@@ -2406,14 +2501,14 @@ __device__ __noinline__ int far_events(const Slab &S, const Shot &C, int v, int 
                 }
 #pragma unroll
                 for (int u = 0; u < 4; u++)
-                    if (dy + x[u].y > g.brad && dy + x[u].y <= q && x[u].x != v && is_defect(C, x[u].x)) hit |= 1u << u;
+                    if (dy + x[u].y > brad && dy + x[u].y <= q && x[u].x != v && X.defect(x[u].x)) hit |= 1u << u;
                 if (!__any_sync(FULL, hit)) continue;
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
 #pragma unroll 1
                     for (unsigned mh = __ballot_sync(FULL, (hit >> u) & 1u); mh; mh &= mh - 1) {
                         const int o = __ffs(mh) - 1;
-                        const int ro = rank_of(S, C, __shfl_sync(FULL, x[u].x, o)), dr = dy + __shfl_sync(FULL, x[u].y, o);
+                        const int ro = X.rank(__shfl_sync(FULL, x[u].x, o)), dr = dy + __shfl_sync(FULL, x[u].y, o);
                         const unsigned same = __ballot_sync(FULL, f == ro);
                         if (!same) {
                             if (found == WS) return -1;
@@ -2430,279 +2525,287 @@ __device__ __noinline__ int far_events(const Slab &S, const Shot &C, int v, int 
     return found;
 }
 
+// EXTEND in the island of c (as extend_due): the events that its due regions
+// can touch until they fall due again are read off the ball table and recorded
+// among the shot's pairs, those of the island itself also in I.pair.  Returns
+// the island's pairs, -1 outside the limits, -2 beyond the table.  One warp.
+__device__ __noinline__ int isl_extend(Fast &X, Isl &I, int c, int n, int np, int lane) {
+    const DGraph &g = *X.g;
+    const int b1 = g.b1, brad = g.brad, wmax = g.wmax;
+    const int *const comp = X.comp(), *const st = X.st(), *const px = X.px();
+    int ev = 0, sR = -1, R = 0, q = 0;
+    bool scan = false, far = false;
+    if (lane < n) {
+        const int p = I.pk[lane], rad = p >> 8, xt = I.xt[lane];
+        if ((p & (3 * LAB1)) == 2 * LAB1 && xt <= rad) {
+            ev = I.ev[lane];
+            sR = xt + X.L - 1;   // explored radius, -1: never
+            R = max(sR + X.band, rad + X.L + X.band);
+            q = X.reach(b1, R);
+            scan = sR >= 0 || q > b1;
+            if (!scan) I.xt[lane] = R - X.L + 1;
+            far = scan && (q > 2 * brad - 2 * wmax || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[ev]).w < 0);
+        }
+    }
+    if (__any_sync(FULL, far)) return -2;
+#pragma unroll 1
+    for (unsigned m = __ballot_sync(FULL, scan); m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        const int s = __shfl_sync(FULL, ev, l), ql = __shfl_sync(FULL, q, l), sRl = __shfl_sync(FULL, sR, l);
+        const int q0 = sRl < 0 ? b1 : max(b1, X.reach(b1, sRl));
+        const int v = X.svtx()[s];
+        const int4 h = __ldg(g.bhdr + v);
+        const int len = h.z + h.w;
+        bool more = false;
+        // the list's own events, then those beyond it
+        int nfar = 0, ff = 0, fd = 0;
+        if (ql > brad) nfar = far_events(X, v, ql, lane, ff, fd);
+        if (nfar < 0) return -1;
+#pragma unroll 1
+        for (int k = 0; k < len + (nfar ? WS : 0); k += WS) {
+            bool hit = false;
+            int f = 0, d = 0;
+            if (k < len) {
+                if (k + lane < len) {
+                    const int2 e = __ldg(g.ball + (unsigned)h.x + k + lane);
+                    more |= e.y > sRl;
+                    hit = e.y > q0 && e.y <= ql && X.defect(e.x);
+                    d = e.y;
+                    if (hit) f = X.rank(e.x);
+                }
+            } else {
+                hit = lane < nfar && fd > q0;
+                f = ff;
+                d = fd;
+            }
+            const unsigned mh = __ballot_sync(FULL, hit);
+            if (!mh) continue;
+            const bool in = hit && comp[f] == c;
+            // a level-1 cluster stands still unless it is touched
+            const int mt = __reduce_min_sync(FULL, hit && !in && st[f] != MATE_NONE ? d - px[f] : INT_MAX);
+            if (lane == l) I.meet[l] = min(I.meet[l], mt);
+            int b = 0;
+            if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(mh));
+            b = __shfl_sync(FULL, b, 0) + __popc(mh & ((1u << lane) - 1u));
+            if (hit && b < X.pcap) X.pr[b] = pk_pair(min(s, f), max(s, f), d);
+            const unsigned mi = __ballot_sync(FULL, in);
+            const int j = np + __popc(mi & ((1u << lane) - 1u));
+            if (in && j < IP) {
+                const int k2 = (int)X.cw()[f];
+                I.pair[j] = make_int2(d, min(l, k2) | max(l, k2) << 8);
+            }
+            np += __popc(mi);
+            if (np > IP || __any_sync(FULL, hit && b >= X.pcap)) return -1;
+        }
+        more = __any_sync(FULL, more);
+        if (lane == l) I.xt[l] = sRl >= 0 && !more ? INT_MAX : R - X.L + 1;
+    }
+    __syncwarp();
+    return np;
+}
+
 // Run the island of the component with lowest event c and `size` events from t
 // = 0 (SI S1, events as in run_matcher): growing roots and, in an island that
 // was joined with level-1 clusters, their events frozen as level 1 left them.
-// One warp.  np0: pairs within b_1.  tcut as in Shot.  level1: a level-1 cluster (its
-// bands are counted here; the top level's aged bands are collected in xR, since
-// regions due at the same time share one).  paths: the matched pairs are wanted.
-// Returns ISL_FAIL when the island is outside the limits, ISL_STOP when a region
-// touched a level-1 cluster outside or outgrew the ball table (the radii so far
-// are in px, cw[c] is ISL_ALONE).
-__device__ __forceinline__ int run_island(const Slab &S, const Shot &C, const Fast &F, Isl &I, int c, int size, int np0,
-                                           int tcut, bool level1, bool paths, int lane, IslRec &rec) {
-    const DGraph &g = C.g;
+// level1: a level-1 cluster (its bands are counted here; the top level's aged
+// bands are collected, since regions due at the same time share one).  One
+// warp.  The result is left in I.rec.  Returns ISL_FAIL when the island is
+// outside the limits, ISL_STOP when a region touched a level-1 cluster outside
+// or outgrew the ball table (the radii so far are in px, cw[c] is ISL_ALONE).
+__device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool level1, int lane) {
     if (size > IN) return ISL_FAIL;
-    // members in rank order: the first is c, the others are near it
-    int n = 0;
+    const int n = size;
+    {
+        // members in rank order: the first is c, the others are near it
+        const int *const comp = X.comp();
+        unsigned *const cw = X.cw();
+        const int K = X.K;
+        int k = 0;
 #pragma unroll 1
-    for (int base = c; base < C.K && n < size; base += WS) {
-        const int s = base + lane;
-        const bool in = s < C.K && F.comp[s] == c;
-        const unsigned m = __ballot_sync(FULL, in);
-        if (in) {
-            const int k = n + __popc(m & ((1u << lane) - 1u));
-            I.ev[k] = s;
-            F.cw[s] = (unsigned)k;   // its lane
+        for (int base = c; base < K && k < n; base += WS) {
+            const int s = base + lane;
+            const bool in = s < K && comp[s] == c;
+            const unsigned m = __ballot_sync(FULL, in);
+            if (in) {
+                const int j = k + __popc(m & ((1u << lane) - 1u));
+                I.ev[j] = s;
+                cw[s] = (unsigned)j;   // its lane
+            }
+            k += __popc(m);
         }
-        n += __popc(m);
     }
     __syncwarp();
-    n = size;
-    int ev = 0, bd = INT_MAX, sR = -1, mrad = 0;
-    int meet = INT_MAX;   // radius at which this region touches a level-1 cluster
-    bool exh = false, bad = false;
+    int rad = 0, top = lane;
+    bool bad = false;
+    I.lab[lane] = 0;
     if (lane < n) {
-        ev = I.ev[lane];
-        bd = F.bd[ev];
-        const int st = level1 ? MATE_NONE : F.st[ev];
+        const int ev = I.ev[lane], bd = X.bd()[ev];
+        const int st = level1 ? (int)MATE_NONE : X.st()[ev];
         const bool frozen = st != MATE_NONE;
-        if (st == ST_RUN) bad = true;
-        mrad = st == MATE_BOUNDARY ? bd : 0;   // of a frozen pair: set with its pair below
-        sR = frozen ? -1 : C.L + C.band;   // first extension, due at t = 0: within the listed pairs
-        I.rad[lane] = mrad; I.y[lane] = mrad;
+        bad = st == ST_RUN;
+        if (st == MATE_BOUNDARY) rad = bd;   // (a frozen pair's radius: with its pair below)
+        I.bd[lane] = bd;
+        // explored radius after the first extension, due at t = 0, which the listed pairs cover
+        I.xt[lane] = frozen ? -X.L : X.band + 1;
+        I.meet[lane] = INT_MAX;
+        I.pk[lane] = rad << 8 | lane;
         I.lab[lane] = frozen ? 0 : 1; I.bpar[lane] = -1; I.tpar[lane] = -1;
         I.mate[lane] = frozen ? MATE_BOUNDARY : MATE_NONE; I.ms[lane] = (signed char)lane; I.mo[lane] = -1;
-        I.root[lane] = frozen ? -1 : (signed char)lane; I.minl[lane] = (signed char)lane; I.top[lane] = (signed char)lane;
+        I.root[lane] = frozen ? -1 : (signed char)lane; I.minl[lane] = (signed char)lane;
     }
+    if (lane == 0) { I.nc = 0; I.err = 0; }
     if (__any_sync(FULL, bad)) return ISL_FAIL;
     __syncwarp();
-    if (lane == 0) { I.nc = 0; I.err = 0; }
     int np = 0;
+    {
+        const unsigned long long *const pr = X.pr;
+        const int *const comp = X.comp(), np0 = X.np0;
 #pragma unroll 1
-    for (int base = 0; base < np0; base += WS) {
-        const int i = base + lane;
-        unsigned long long p = 0;
-        bool in = false;
-        if (i < np0) {
-            p = F.pr[i];
-            in = F.comp[pr_lo(p)] == c;
-        }
-        const unsigned m = __ballot_sync(FULL, in);
-        if (!m) continue;
-        const int k = np + __popc(m & ((1u << lane) - 1u));
-        if (in && k < IP) {
-            const int a = (int)F.cw[pr_lo(p)], b = (int)F.cw[pr_hi(p)], d = pr_val(p);
-            I.pa[k] = (unsigned char)a;
-            I.pb[k] = (unsigned char)b;
-            I.pd[k] = d;
-            if (!level1 && F.st[pr_lo(p)] == pr_hi(p)) {   // a level-1 pair: frozen, matched at d / 2
-                I.rad[a] = I.rad[b] = I.y[a] = I.y[b] = d / 2;
-                I.mate[a] = (signed char)b; I.mo[a] = (signed char)b;
-                I.mate[b] = (signed char)a; I.mo[b] = (signed char)a;
+        for (int base = 0; base < np0; base += WS) {
+            const int i = base + lane;
+            unsigned long long p = 0;
+            bool in = false;
+            if (i < np0) {
+                p = pr[i];
+                in = comp[pr_lo(p)] == c;
             }
+            const unsigned m = __ballot_sync(FULL, in);
+            if (!m) continue;
+            const int k = np + __popc(m & ((1u << lane) - 1u));
+            if (in && k < IP) {
+                const int a = (int)X.cw()[pr_lo(p)], b = (int)X.cw()[pr_hi(p)], d = pr_val(p);
+                I.pair[k] = make_int2(d, a | b << 8);
+                if (!level1 && X.st()[pr_lo(p)] == pr_hi(p)) {   // a level-1 pair: frozen, matched at d / 2
+                    I.pk[a] = d / 2 << 8 | a;
+                    I.pk[b] = d / 2 << 8 | b;
+                    I.mate[a] = (signed char)b; I.mo[a] = (signed char)b;
+                    I.mate[b] = (signed char)a; I.mo[b] = (signed char)a;
+                }
+            }
+            np += __popc(m);
         }
-        np += __popc(m);
     }
     if (np > IP) return ISL_FAIL;
     __syncwarp();
-    if (lane < n) mrad = I.rad[lane];
-    unsigned bal = 0;   // blossoms alive
-    auto stop = [&]() {
-        if (lane < n) F.px[ev] = mrad;
-        if (lane == 0) { F.cw[c] = ISL_ALONE; atomicAdd(&F.cnt[F_STOP], 1); }
-        __syncwarp();
-        return ISL_STOP;
-    };
+    if (lane < n) rad = I.pk[lane] >> 8;
+    int yl = rad, mrad = rad;   // the leaf's dual, the largest radius so far
+    unsigned bal = 0;           // blossoms alive
     int t = 0, nm = 0, ncut = 0, tlast = 0, nx = level1 ? 1 : 0;
 #pragma unroll 1
     for (int it = 0;; it++) {
-        if (it > 200 * n) return ISL_FAIL;   // far below the shot's event budget
-        // next event: key dt << 12 | kind << 10 | lo << 5 | hi, dt < 2^20
-        unsigned key = ~0u;
-        bool grows = false;
-        auto cand = [&](int dt, int kind, int lo, int hi) {
-            bad |= dt < 0;
-            key = min(key, dt >= 0xfffff ? ~1u : ((unsigned)dt << 12) | (unsigned)(kind << 10 | lo << 5 | hi));
-        };
-        int lab = 0, rad = 0;
+        if (it > 200 * n || t >= (1 << 22)) return ISL_FAIL;   // far below the shot's event budget
+        int lab = 0;
         if (lane < n) {
-            lab = I.lab[I.top[lane]];
-            rad = I.rad[lane];
-            if (lab == 1) {
-                grows = true;
-                if (!exh) cand(max(0, sR - C.L + 1 - rad), EV_EXTEND, lane, 0);
-                if (bd != INT_MAX) cand(bd - rad, EV_BOUNDARY, lane, 0);
-            }
+            lab = I.lab[top];
+            I.pk[lane] = rad << 8 | (lab + 1) << 6 | top;
+        }
+        if (!__any_sync(FULL, lab == 1)) break;
+        __syncwarp();
+        // next event: key dt << 12 | kind << 10 | lo << 5 | hi, dt < 2^20 - 1;
+        // touching a level-1 cluster outside is kind EXTEND with hi = 1
+        unsigned key = ~0u;
+        auto cand = [&](int dt, int code) {
+            if ((unsigned)dt < 0xfffffu) key = min(key, ((unsigned)dt << 12) | (unsigned)code);
+        };
+        if (lab == 1) {
+            const int bd = I.bd[lane];
+            bad = bd < rad;
+            cand(max(0, I.xt[lane] - rad), EV_EXTEND << 10 | lane << 5);
+            cand(max(0, I.meet[lane] - rad), EV_EXTEND << 10 | lane << 5 | 1);
+            cand(bd - rad, EV_BOUNDARY << 10 | lane << 5);
         }
 #pragma unroll 1
         for (int p = lane; p < np; p += WS) {
-            const int a = I.pa[p], b = I.pb[p], A = I.top[a], B = I.top[b];
-            const int r = I.lab[A] + I.lab[B];
-            if (A == B || r <= 0) continue;
-            const int gap = I.pd[p] - I.rad[a] - I.rad[b];
-            bad |= (gap & (r - 1)) != 0;
-            cand(r == 2 ? gap >> 1 : gap, EV_COLLIDE, min(a, b), max(a, b));
+            const int2 pq = I.pair[p];
+            const int a = pq.y & 255, b = pq.y >> 8;
+            const int ka = I.pk[a], kb = I.pk[b];
+            const int r = ((ka >> 6) & 3) + ((kb >> 6) & 3) - 2;
+            if (((ka ^ kb) & (LAB1 - 1)) == 0 || r <= 0) continue;
+            const int gap = pq.x - (ka >> 8) - (kb >> 8);
+            bad |= gap < 0 || (gap & (r - 1)) != 0;
+            cand(gap >> (r - 1), EV_COLLIDE << 10 | a << 5 | b);
         }
         if ((bal >> lane) & 1u) {
             const int v = IN + lane;
-            if (I.bpar[v] < 0 && I.lab[v] == -1) cand(I.y[v], EV_IMPLODE, I.minl[v], 0);
+            if (I.bpar[v] < 0 && I.lab[v] == -1) cand(I.y[v], EV_IMPLODE << 10 | I.minl[v] << 5);
         }
         if (__any_sync(FULL, bad)) return ISL_FAIL;
-        if (!__any_sync(FULL, grows)) break;
         key = __reduce_min_sync(FULL, key);
-        if (key >= ~1u) return ISL_FAIL;   // no event left (no solution), or far away
+        if (key == ~0u) return ISL_FAIL;   // no event left (no solution), or far away
         const int dt = (int)(key >> 12), kind = (int)(key >> 10) & 3, lo = (int)(key >> 5) & 31, hi = (int)key & 31;
         t += dt;
-        if (t >= (1 << 25)) return ISL_FAIL;
-        if (__any_sync(FULL, lab == 1 && meet <= rad + dt)) {
-            mrad = max(mrad, rad + lab * dt);
-            return stop();
-        }
         if (dt > 0) {
-            if (lane < n) {
-                rad += lab * dt;
-                I.rad[lane] = rad;
-                mrad = max(mrad, rad);
-                if (I.top[lane] == lane) I.y[lane] += lab * dt;
-            }
+            rad += lab * dt;
+            mrad = max(mrad, rad);
+            if (top == lane) yl += lab * dt;
             if ((bal >> lane) & 1u) {
                 const int v = IN + lane;
                 if (I.bpar[v] < 0) I.y[v] += I.lab[v] * dt;
             }
         }
-        __syncwarp();
         if (kind == EV_EXTEND) {
-            // regions that came within L of their explored radius
-            const bool due = lab == 1 && !exh && sR - C.L + 1 - rad <= 0;
-            int R = 0, q = 0;
-            bool scan = false, far = false;
-            if (due) {
-                R = max(sR + C.band, rad + C.L + C.band);
-                q = reach_of(C, R);
-                scan = sR >= 0 || q > g.b1;
-                if (!scan) sR = R;
-                far = scan && (q > 2 * g.brad - 2 * g.wmax || sR > g.brad - g.wmax || __ldg(g.bhdr + F.svtx[ev]).w < 0);
+            int r = -2;
+            if (!hi) {
+                if (lane < n) I.pk[lane] = rad << 8 | (lab + 1) << 6 | top;
+                __syncwarp();
+                r = isl_extend(X, I, c, n, np, lane);
+                if (r == -1) return ISL_FAIL;
             }
-            if (__any_sync(FULL, far)) return stop();
-#pragma unroll 1
-            for (unsigned m = __ballot_sync(FULL, scan); m; m &= m - 1) {
-                const int l = __ffs(m) - 1;
-                const int s = __shfl_sync(FULL, ev, l), ql = __shfl_sync(FULL, q, l), sRl = __shfl_sync(FULL, sR, l);
-                const int q0 = sRl < 0 ? g.b1 : max(g.b1, reach_of(C, sRl));
-                const int4 h = __ldg(g.bhdr + F.svtx[s]);
-                const int len = h.z + h.w;
-                bool more = false;
-                // the list's own events, then those beyond it
-                int nfar = 0, ff = 0, fd = 0;
-                if (ql > g.brad) nfar = far_events(S, C, F.svtx[s], ql, lane, ff, fd);
-                if (nfar < 0) return ISL_FAIL;
-#pragma unroll 1
-                for (int k = 0; k < len + (nfar ? WS : 0); k += WS) {
-                    bool hit = false;
-                    int f = 0, d = 0;
-                    if (k < len) {
-                        if (k + lane < len) {
-                            const int2 e = __ldg(g.ball + (unsigned)h.x + k + lane);
-                            more |= e.y > sRl;
-                            hit = e.y > q0 && e.y <= ql && is_defect(C, e.x);
-                            d = e.y;
-                            if (hit) f = rank_of(S, C, e.x);
-                        }
-                    } else {
-                        hit = lane < nfar && fd > q0;
-                        f = ff;
-                        d = fd;
-                    }
-                    const unsigned mh = __ballot_sync(FULL, hit);
-                    if (!mh) continue;
-                    const bool in = hit && F.comp[f] == c;
-                    // a level-1 cluster stands still unless it is touched
-                    const int mt = hit && !in && F.st[f] != MATE_NONE ? d - F.px[f] : INT_MAX;
-                    const int ml = __reduce_min_sync(FULL, mt);
-                    if (lane == l) meet = min(meet, ml);
-                    int b = 0;
-                    if (lane == 0) b = atomicAdd(&F.cnt[F_NP], __popc(mh));
-                    b = __shfl_sync(FULL, b, 0) + __popc(mh & ((1u << lane) - 1u));
-                    if (hit && b < F.pcap) F.pr[b] = pk_pair(min(s, f), max(s, f), d);
-                    const unsigned mi = __ballot_sync(FULL, in);
-                    const int j = np + __popc(mi & ((1u << lane) - 1u));
-                    if (in && j < IP) { I.pa[j] = (unsigned char)l; I.pb[j] = (unsigned char)F.cw[f]; I.pd[j] = d; }
-                    np += __popc(mi);
-                    if (np > IP || __any_sync(FULL, hit && b >= F.pcap)) return ISL_FAIL;
-                }
-                more = __any_sync(FULL, more);
-                if (lane == l) { exh = sR >= 0 && !more; sR = R; }
+            if (r == -2) {
+                if (lane < n) X.px()[I.ev[lane]] = mrad;
+                if (lane == 0) { X.cw()[c] = ISL_ALONE; atomicAdd(&X.cnt[F_STOP], 1); }
+                __syncwarp();
+                return ISL_STOP;
             }
+            np = r;
             // a band: counted at once, except that at the top level regions of
             // several islands coming of age at one time share it
             if (level1 || dt == 0) {
                 nx++;
             } else if (lane == 0) {
-                const int k = atomicAdd(&F.cnt[F_AGED], 1);
-                if (k < C.K) { S.xR[k] = t; S.sbeg[k] = c; S.scnt[k] = n; }
+                const int k = atomicAdd(&X.cnt[F_AGED], 1);
+                if (k < X.K) { X.aged_t[k] = t; X.aged_c[k] = c; X.aged_n[k] = n; }
             }
-            __syncwarp();
             continue;
         }
         nm++;
-        if (t <= tcut) ncut++;
+        if (t <= X.tcut) ncut++;
         tlast = t;
         if (kind == EV_IMPLODE) {
-            const int B = I.top[lo];
-            if (lane < n && I.top[lane] == B) I.top[lane] = (signed char)isl_child_of(I, B, lane);
-            __syncwarp();
-            if (lane == 0) isl_shatter(I, B);
+            const int B = I.top(lo);
+            top = isl_shatter(I, B, n, lane);
             bal &= ~(1u << (B - IN));
-            __syncwarp();
             if (I.err) return ISL_FAIL;
             continue;
         }
-        int a = lo, b = hi, A = I.top[a], B = -1;
+        int a = lo, b = hi, A = I.top(a), B = -1;
         if (kind == EV_COLLIDE) {
-            B = I.top[b];
+            B = I.top(b);
             if (I.lab[A] != 1) { int x = A; A = B; B = x; x = a; a = b; b = x; }
         }
-        const int lb = B >= 0 ? I.lab[B] : 0, mb = B >= 0 ? I.mate[B] : MATE_BOUNDARY;
+        const int lb = B >= 0 ? I.lab[B] : 0, mb = B >= 0 ? (int)I.mate[B] : (int)MATE_BOUNDARY;
         const int rA = I.root[A], rB = lb == 1 ? I.root[B] : -3;
         __syncwarp();
         if (lb == 1 && rA == rB) {
-            // blossom
             if (bal == ~0u) return ISL_FAIL;
             const int N = IN + __ffs(~bal) - 1;
-            int ok = 0;
-            if (lane == 0) ok = isl_blossom(I, N, A, a, B, b);
-            if (!__shfl_sync(FULL, ok, 0)) return ISL_FAIL;
-            __syncwarp();
-            const int L0 = I.cn[I.cb[N - IN]];   // its root becomes N's
-#pragma unroll 1
-            for (int h = 0; h < 2; h++) {
-                const int v = lane + h * IN;
-                if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
-                if (I.bpar[v] >= 0) continue;
-                const int tp = I.tpar[v], mt = I.mate[v];
-                if (tp >= 0 && I.bpar[tp] == N) I.tpar[v] = (signed char)N;
-                if (mt >= 0 && I.bpar[mt] == N) I.mate[v] = (signed char)N;
-                if (I.root[v] == L0) I.root[v] = (signed char)N;
-            }
-            if (lane < n) {
-                const int tp = I.top[lane];
-                if (I.bpar[tp] == N) I.top[lane] = (signed char)N;
-            }
+            top = isl_blossom(I, N, A, a, B, b, n, bal, lane);
+            if (top < 0) return ISL_FAIL;
             bal |= 1u << (N - IN);
         } else if (lb == 1 || mb == MATE_BOUNDARY) {
             // augment: the trees' nodes leave them while lane 0 rematches
             // along the tree paths
-#pragma unroll 1
-            for (int h = 0; h < 2; h++) {
-                const int v = lane + h * IN;
-                if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+            if (lane < n && I.bpar[lane] < 0 && I.lab[lane] != 0 && (I.root[lane] == rA || I.root[lane] == rB)) {
+                I.lab[lane] = 0; I.root[lane] = -1;
+            }
+            if ((bal >> lane) & 1u) {
+                const int v = IN + lane;
                 if (I.bpar[v] < 0 && I.lab[v] != 0 && (I.root[v] == rA || I.root[v] == rB)) { I.lab[v] = 0; I.root[v] = -1; }
             }
             if (lane == 0) {
                 isl_flip(I, A);
-                if (lb == 1) isl_flip(I, B);
                 if (B >= 0) {
+                    if (lb == 1) isl_flip(I, B);
                     I.mate[A] = (signed char)B; I.ms[A] = (signed char)a; I.mo[A] = (signed char)b;
                     I.mate[B] = (signed char)A; I.ms[B] = (signed char)b; I.mo[B] = (signed char)a;
                 } else {
@@ -2725,32 +2828,22 @@ __device__ __forceinline__ int run_island(const Slab &S, const Shot &C, const Fa
     int w = 0;
     unsigned long long o = 0;
     if (lane < n) {
-        w = I.y[lane];
-        F.px[ev] = mrad;
+        w = yl;
+        X.px()[I.ev[lane]] = mrad;
+        if (I.bpar[lane] < 0 && I.mate[lane] == MATE_BOUNDARY) o = __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[lane]]]);
     }
-    if ((bal >> lane) & 1u) w += I.y[IN + lane];
-    for (int h = 0; h < 2; h++) {
-        const int v = lane + h * IN;
-        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
-        if (I.bpar[v] >= 0) continue;
-        const int mt = I.mate[v];
-        if (mt == MATE_BOUNDARY) {
-            const int s = I.ev[I.ms[v]];
-            o ^= __ldg(g.eobs + (unsigned)(__ldg(g.vbnd + F.svtx[s]) & 0xffffffffu));
-            if (paths) put_path(S, &F.cnt[F_NPATH], s, -1, F.bd[s]);
-        } else if (paths && v < mt) {
-            put_path(S, &F.cnt[F_NPATH], I.ev[I.ms[v]], I.ev[I.mo[v]], isl_dist(I, I.ms[v], I.mo[v]));
-        }
+    if ((bal >> lane) & 1u) {
+        const int v = IN + lane;
+        w += I.y[v];
+        if (I.bpar[v] < 0 && I.mate[v] == MATE_BOUNDARY) o ^= __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[v]]]);
     }
-    if (paths) {
-        for (unsigned m = bal; m; m &= m - 1) {
-            const int v = IN + __ffs(m) - 1;
-            if (lane == 0 && I.bpar[v] < 0) isl_expand(I, S, &F.cnt[F_NPATH], v, I.ms[v]);
-        }
+    if (X.paths) {
+        __syncwarp();
+        isl_paths(X, I, n, bal, lane);
     }
-    rec.w = (int)__reduce_add_sync(FULL, (unsigned)w);
-    rec.o = ((unsigned long long)__reduce_xor_sync(FULL, (unsigned)(o >> 32)) << 32) | __reduce_xor_sync(FULL, (unsigned)o);
-    rec.size = n; rec.nm = nm; rec.ncut = ncut; rec.tlast = tlast; rec.nx = nx;
+    w = (int)__reduce_add_sync(FULL, (unsigned)w);
+    o = ((unsigned long long)__reduce_xor_sync(FULL, (unsigned)(o >> 32)) << 32) | __reduce_xor_sync(FULL, (unsigned)o);
+    if (lane == 0) I.rec = IslRec{o, w, n, nm, ncut, tlast, nx};
     __syncwarp();
     return ISL_OK;
 }
@@ -2759,10 +2852,9 @@ __device__ __forceinline__ int run_island(const Slab &S, const Shot &C, const Fa
 // counts before each word into S.wcum; returns their number.  Every thread of
 // the team calls; ends with a barrier.
 template <int NW>
-__device__ __forceinline__ int load_events(const Slab &S, const DGraph &g, const unsigned *row, int *svtx, int cap,
-                                           Team<NW> &T) {
+__device__ __forceinline__ int load_events(int *wcum, const DGraph &g, const unsigned *row, int *svtx, int cap, Team<NW> &T) {
     int K = 0;
-    const int nvec = g.words >> 2;
+    const int nvec = g.words >> 2, n = g.n;
     const uint4 *rv = reinterpret_cast<const uint4 *>(row);
 #pragma unroll 1
     for (int base = 0; base < nvec; base += T.NT) {
@@ -2770,18 +2862,18 @@ __device__ __forceinline__ int load_events(const Slab &S, const DGraph &g, const
         uint4 v = make_uint4(0, 0, 0, 0);
         if (i < nvec) v = __ldg(rv + i);
         unsigned wv[4] = {v.x, v.y, v.z, v.w};
-        if (i * 128 + 128 > g.n) {   // drop padding bits beyond n
+        if (i * 128 + 128 > n) {   // drop padding bits beyond n
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const int bit0 = (i * 4 + q) * 32;
-                if (bit0 >= g.n) wv[q] = 0;
-                else if (bit0 + 32 > g.n) wv[q] &= (1u << (g.n - bit0)) - 1u;
+                if (bit0 >= n) wv[q] = 0;
+                else if (bit0 + 32 > n) wv[q] &= (1u << (n - bit0)) - 1u;
             }
         }
         const int c0 = __popc(wv[0]), c1 = c0 + __popc(wv[1]), c2 = c1 + __popc(wv[2]), c = c2 + __popc(wv[3]);
         int total;
         int pos = K + T.excl_scan(c, total);
-        if (i < nvec) reinterpret_cast<int4 *>(S.wcum)[i] = make_int4(pos, pos + c0, pos + c1, pos + c2);
+        if (i < nvec) reinterpret_cast<int4 *>(wcum)[i] = make_int4(pos, pos + c0, pos + c1, pos + c2);
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             unsigned bits = wv[q];
@@ -2799,31 +2891,104 @@ __device__ __forceinline__ int load_events(const Slab &S, const DGraph &g, const
     return K;
 }
 
-constexpr int USE_GENERAL = -3;   // the shot is outside the fast path's limits
-
-// Decode one shot by level 1 and islands.  Same results and diagnostics as the
-// general path below, which takes what is outside the limits (USE_GENERAL).
-constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
+// Per-event arrays of the shot and its pairs within b_1 (as near_pairs: from
+// their lower ends, off the ball table; half a warp per event, since most lists
+// have 12 entries).  Returns false when an event's list is not complete or
+// longer than level 1 takes.  Every thread of the team calls; ends with a
+// barrier.
+template <int NW>
+__device__ __forceinline__ bool fast_pairs(Fast &X, Team<NW> &T) {
+    const DGraph &g = *X.g;
+    const int lane = T.lane, K = X.K, half = lane >> 4, sub = lane & 15;
+    int *const svtx = X.svtx(), *const bd = X.bd(), *const comp = X.comp(), *const st = X.st();
+    unsigned *const cw = X.cw();
+    const unsigned *const row = X.row;
+    const int *const wcum = X.wcum;
+    unsigned long long *const pr = X.pr;
+    const int pcap = X.pcap;
+    const int2 *const ball = g.ball;
+    const int most = g.hop2 ? INT_MAX : LB_CAP - 1;
+    bool odd = false;
+    int np = 0;
+#pragma unroll 1
+    for (int base = T.warp() * WS; base < K; base += T.NT) {
+        const int s = base + lane;
+        int beg = 0, len = 0;
+        if (s < K) {
+            const int v = svtx[s];
+            const int4 h = __ldg(g.bhdr + v);
+            const unsigned long long vb = __ldg(g.vbnd + v);
+            bd[s] = vb == EMPTY64 ? INT_MAX : (int)(vb >> 32);
+            comp[s] = s;
+            cw[s] = 0;
+            st[s] = MATE_NONE;
+            odd |= h.z < 0 || h.z > most;
+            beg = h.x;
+            len = h.z < 0 ? 0 : h.y;
+        }
+#pragma unroll 2
+        for (int e0 = 0; e0 < WS && base + e0 < K; e0 += 2) {
+            const unsigned eb = (unsigned)__shfl_sync(FULL, beg, e0 + half);
+            const int el = __shfl_sync(FULL, len, e0 + half);
+            const int em = max(el, __shfl_xor_sync(FULL, el, 16));
+#pragma unroll 1
+            for (int k = 0; k < em; k += 16) {
+                bool hit = false;
+                int2 e = make_int2(0, 0);
+                unsigned word = 0;
+                if (k + sub < el) {
+                    e = __ldg(ball + eb + k + sub);
+                    word = __ldg(row + (e.x >> 5));
+                    hit = (word >> (e.x & 31)) & 1u;
+                }
+                const unsigned m = __ballot_sync(FULL, hit);
+                if (!m) continue;
+                int b;
+                if constexpr (NW == 1) {
+                    b = np;
+                    np += __popc(m);
+                } else {
+                    b = 0;
+                    if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(m));
+                    b = __shfl_sync(FULL, b, 0);
+                }
+                if (hit) {
+                    const int j = b + __popc(m & ((1u << lane) - 1u));
+                    const int f = wcum[e.x >> 5] + __popc(word & ((1u << (e.x & 31)) - 1u));
+                    if (j < pcap) pr[j] = pk_pair(base + e0 + half, f, e.y);
+                }
+            }
+        }
+    }
+    if constexpr (NW == 1)
+        if (lane == 0) X.cnt[F_NP] = np;
+    odd = T.any(odd);
+    T.sync();
+    return !odd;
+}
 
 // Components of the events by min-label propagation with shortcuts over the
 // pairs within b_1, [0, np0), and those marked MET in [np0, np1); labels start
 // as they are.  Every thread of the team calls; ends with a barrier.
 template <int NW>
-__device__ __forceinline__ void fast_components(const Fast &F, int np0, int np1, int K, Team<NW> &T) {
-    volatile int *comp = F.comp;
+__device__ __forceinline__ void fast_components(Fast &X, int np1, Team<NW> &T) {
+    int *const compw = X.comp();
+    volatile int *const comp = compw;
+    const unsigned long long *const pr = X.pr;
+    const int np0 = X.np0, K = X.K;
 #pragma unroll 1
     for (int round = 0; round <= K; round++) {
         bool changed = false;
 #pragma unroll 1
         for (int i = T.tid(); i < np1; i += T.NT) {
-            const unsigned long long p = F.pr[i];
+            const unsigned long long p = pr[i];
             if (i >= np0 && !(p & MET)) continue;
             const int a = pr_lo(p), b = pr_hi(p), la = comp[a], lb = comp[b];
             if (la != lb) {
                 const int m = min(la, lb), h = max(la, lb);
-                atomicMin(&F.comp[a], m);
-                atomicMin(&F.comp[b], m);
-                atomicMin(&F.comp[h], m);
+                atomicMin(&compw[a], m);
+                atomicMin(&compw[b], m);
+                atomicMin(&compw[h], m);
                 changed = true;
             }
         }
@@ -2836,343 +3001,389 @@ __device__ __forceinline__ void fast_components(const Fast &F, int np0, int np1,
         }
         T.sync();
     }
+    T.sync();
 }
 
-template <bool WIN, int NW>
-__device__ __forceinline__ int decode_fast(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
-                                           Team<NW> &T, FastShared<NW> &M, long long &w_out, unsigned long long &o_out,
-                                           int *dg) {
-    Shot C;
-    C.g = g;
-    C.row = row;
-    C.band = max(g.wmax, 1) * max(A.band_factor, 1);
-    C.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
-    C.real = 0;
-    C.paths = 0;
-    // level 1 present, lists complete, first extensions within the listed pairs
-    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (1 << 27) || reach_of(C, C.L + C.band) > g.b1 ||
-        g.words > A.caps.wcap)
-        return USE_GENERAL;
-    Fast F;
-    F.cnt = M.cnt;
-    F.svtx = M.svtx; F.bd = M.bd; F.comp = M.comp; F.px = M.px; F.st = M.st; F.cw = M.cw;
-    F.pr = M.pr;
-    F.pcap = M.PS;
-    int K = load_events(S, g, row, M.svtx, M.KS, T);
-    C.K = K;
-    if (K == 0) {
-        w_out = 0; o_out = 0;
-        if (dg && T.tid() < QEC_DIAG_FIELDS) dg[T.tid()] = 0;   // no detection event: E_ideal = 0
-        if constexpr (WIN)
-#pragma unroll 1
-            for (int w = T.tid(); w < g.words; w += T.NT) A.carry[(row - A.syn) + w] = 0u;
-        return QEC_SHOT_OK;
+// Level 1 of the shot: sizes, contacts and pairs within d_1 of the components,
+// then clusters in closed form (their weight and observable added to w and o).
+// The other clusters (from the front of X.list) and the islands (from its back)
+// are listed by their lowest event.  Per-thread: t1 the last stopping time, ncl
+// the clusters, nres their events.  Every thread of the team calls; ends with a
+// barrier.
+struct Level1 {
+    long long w;
+    unsigned long long o;
+    int t1, ncl, nres;
+};
+__device__ __forceinline__ void add_closed(Fast &X, int s, int st, int d, long long &w, unsigned long long &o) {
+    if (st == MATE_BOUNDARY) {
+        const int bd = X.bd()[s];
+        w += bd;
+        o ^= __ldg(X.g->vobs + X.svtx()[s]);
+        if (X.paths) put_path(X, s, -1, bd);
+    } else {
+        w += d / 2;
+        if (X.paths && s < st) put_path(X, s, st, d);
     }
-    if (K > A.caps.kc || K > 4000) return USE_GENERAL;
-    const bool paths = WIN || g.internal_obs;
-    int np0 = 0;
-#pragma unroll 1
-    for (bool small = K <= M.KS;; small = false) {
-        if (!small) {   // per-event arrays in the slab
-            F.svtx = S.svtx; F.bd = S.cst0; F.comp = S.comp; F.px = S.xcur; F.st = S.xidx;
-            F.cw = reinterpret_cast<unsigned *>(S.cst1);
-            F.pr = S.tl;
-            F.pcap = A.caps.ec;
-            load_events(S, g, row, S.svtx, A.caps.kc, T);
-        }
-        if (T.tid() < 8) M.cnt[T.tid()] = 0;
-        T.sync();
-        // pairs within b_1 (as near_pairs)
-        int flags = 0, np = 0;
-        const int lane = T.lane;
-#pragma unroll 1
-        for (int base = T.warp() * WS; base < K; base += T.NT) {
-            const int s = base + lane;
-            int beg = 0, len = 0;
-            if (s < K) {
-                const int v = F.svtx[s];
-                const int4 h = __ldg(g.bhdr + v);
-                const unsigned long long vb = __ldg(g.vbnd + v);
-                F.bd[s] = vb == EMPTY64 ? INT_MAX : (int)(vb >> 32);
-                F.comp[s] = s;
-                F.cw[s] = 0;
-                F.st[s] = MATE_NONE;
-                if (h.z < 0 || (!g.hop2 && h.z >= LB_CAP)) flags |= 1;
-                beg = h.x;
-                len = h.z < 0 ? 0 : h.y;
-            }
-            int incl = len;
-#pragma unroll
-            for (int o = 1; o < WS; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int total = __shfl_sync(FULL, incl, WS - 1);
-            const int excl = incl - len;
-#pragma unroll 1
-            for (int t0 = 0; t0 < total; t0 += WS) {
-                const int t = t0 + lane;
-                int ow = 0;   // owner: the last lane whose first entry number is <= t
-#pragma unroll
-                for (int step = WS / 2; step > 0; step >>= 1) {
-                    const int e = __shfl_sync(FULL, excl, ow + step);
-                    if (e <= t) ow += step;
-                }
-                const unsigned oj = (unsigned)__shfl_sync(FULL, beg - excl, ow) + (unsigned)t;
-                bool hit = false;
-                int2 e = make_int2(0, 0);
-                unsigned word = 0;
-                if (t < total) {
-                    e = __ldg(g.ball + oj);
-                    word = __ldg(row + (e.x >> 5));
-                    hit = (word >> (e.x & 31)) & 1u;
-                }
-                const unsigned m = __ballot_sync(FULL, hit);
-                if (!m) continue;
-                int b;
-                if constexpr (NW == 1) {
-                    b = np;
-                    np += __popc(m);
-                } else {
-                    b = 0;
-                    if (lane == 0) b = atomicAdd(&M.cnt[F_NP], __popc(m));
-                    b = __shfl_sync(FULL, b, 0);
-                }
-                if (hit) {
-                    const int j = b + __popc(m & ((1u << lane) - 1u));
-                    const int f = S.wcum[e.x >> 5] + __popc(word & ((1u << (e.x & 31)) - 1u));
-                    if (j < F.pcap) F.pr[j] = pk_pair(base + ow, f, e.y);
-                }
-            }
-        }
-        if constexpr (NW == 1)
-            if (lane == 0) M.cnt[F_NP] = np;
-        flags = T.template red32<2>(flags);
-        if constexpr (NW == 1) T.sync();
-        if (flags) return USE_GENERAL;
-        np0 = M.cnt[F_NP];
-        if (np0 <= F.pcap && np0 < (1 << 18)) break;
-        if (!small) return USE_GENERAL;
-        T.sync();
-    }
-    fast_components(F, np0, np0, K, T);
+}
+template <int NW>
+__device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, Team<NW> &T) {
+    const DGraph &g = *X.g;
+    const int K = X.K, np0 = X.np0, b1 = g.b1, d1 = g.d1;
+    const int *const comp = X.comp(), *const bdv = X.bd();
+    int *const px = X.px(), *const stv = X.st();
+    unsigned *const cwv = X.cw();
+    const unsigned long long *const pr = X.pr;
+    int *const list = X.list;
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
-        const int r = F.comp[s];
-        atomicAdd(&F.cw[r], 1u);
-        if (2LL * F.bd[s] <= (long long)g.b1) atomicOr(&F.cw[r], 1u << 31);
+        const int r = comp[s];
+        atomicAdd(&cwv[r], 1u);
+        if (2LL * bdv[s] <= (long long)b1) atomicOr(&cwv[r], 1u << 31);
     }
     // pairs within d_1, each noted at its two events: the pair of an accepted
     // two-event cluster
 #pragma unroll 1
     for (int i = T.tid(); i < np0; i += T.NT) {
-        const unsigned long long p = F.pr[i];
-        if (pr_val(p) > g.d1) continue;
-        atomicAdd(&F.cw[F.comp[pr_lo(p)]], 1u << 12);
-        F.px[pr_lo(p)] = i;
-        F.px[pr_hi(p)] = i;
+        const unsigned long long p = pr[i];
+        if (pr_val(p) > d1) continue;
+        const int a = pr_lo(p), b = pr_hi(p);
+        atomicAdd(&cwv[comp[a]], 1u << 12);
+        px[a] = i;
+        px[b] = i;
     }
     T.sync();
-    // level-1 clusters in closed form; the other clusters (from the front of
-    // xsrc) and the islands (from its back) are listed by their lowest event
-    long long wsum = 0;
-    unsigned long long osum = 0;
-    IslRec *const recs = reinterpret_cast<IslRec *>(S.wl0);   // of the islands, by their lowest event
-    // of the level-1 clusters run (lane 0 of each warp)
-    long long lw = 0;
-    unsigned long long lo = 0;
-    int lnm = 0, lmax = 0, ltlast = 0, lnx = 0;
-    // what a closed form adds to the result
-    auto closed = [&](int s, int st, int d) {
-        if (st == MATE_BOUNDARY) {
-            wsum += F.bd[s];
-            osum ^= __ldg(g.eobs + (unsigned)(__ldg(g.vbnd + F.svtx[s]) & 0xffffffffu));
-            if (paths) put_path(S, &M.cnt[F_NPATH], s, -1, F.bd[s]);
-        } else {
-            wsum += d / 2;
-            if (paths && s < st) put_path(S, &M.cnt[F_NPATH], s, st, d);
-        }
-    };
-    int t1 = 0, ncl1 = 0, nres1 = 0;
+    Level1 L{0, 0, 0, 0, 0};
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
-        const int r = F.comp[s];
-        const unsigned cw = F.cw[r];
+        const int r = comp[s];
+        const unsigned cw = cwv[r];
         const int size = (int)(cw & 4095u), prs = (int)(cw >> 12) & 0x7ffff;
         const bool ok = prs == size * (size - 1) / 2 && ((cw >> 31) || size % 2 == 0);
         if (ok && size <= 2) {
-            int st = MATE_BOUNDARY, rad = F.bd[s], d = 0;   // one boundary event at time bd
+            int st = MATE_BOUNDARY, rad = bdv[s], d = 0;   // one boundary event at time bd
             bool fine = true;
             if (size == 2) {
-                const unsigned long long p = F.pr[F.px[s]];
+                const unsigned long long p = pr[px[s]];
                 st = pr_lo(p) == s ? pr_hi(p) : pr_lo(p);
                 d = pr_val(p);
                 rad = d / 2;   // one collision at time d/2
-                fine = rad <= F.bd[s] && rad <= F.bd[st];
+                fine = rad <= bdv[s] && rad <= bdv[st];
             }
             if (fine) {
-                F.st[s] = st;
-                F.px[s] = rad;
-                t1 = max(t1, rad); nres1++;
-                if (s == r) ncl1++;
-                closed(s, st, d);
+                stv[s] = st;
+                px[s] = rad;
+                L.t1 = max(L.t1, rad);
+                L.nres++;
+                if (s == r) L.ncl++;
+                add_closed(X, s, st, d, L.w, L.o);
                 continue;
             }
         }
-        if (ok) F.st[s] = ST_RUN;
+        if (ok) stv[s] = ST_RUN;
         if (s == r) {
-            if (ok) { S.xsrc[atomicAdd(&M.cnt[F_N1], 1)] = s; nres1 += size; ncl1++; }
-            else S.xsrc[K - 1 - atomicAdd(&M.cnt[F_N2], 1)] = s;
+            if (ok) { list[atomicAdd(&X.cnt[F_N1], 1)] = s; L.nres += size; L.ncl++; }
+            else list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
         }
     }
     T.sync();
-    const int n1 = M.cnt[F_N1];
-    if (dg) t1 = T.maxi(t1);
-    // the remaining level-1 clusters
-    int fail = 0;
+    out = L;
+}
+
+// What islands met, after they have run: marks the pairs in [np0, np1) whose
+// regions meet, joins their components and lists what has to run (in X.list,
+// from its back) and all islands (in X.all); w, o: what is left of the closed
+// forms.  Returns 0 when nothing met, 1 when something was joined, 2 when the
+// shot is outside the limits.  Every thread of the team calls; ends with a
+// barrier.
+template <int NW>
+__device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int round, Team<NW> T, long long &w,
+                                      unsigned long long &o) {
+    int *const list = X.list, *const all = X.all;
+    const int K = X.K, np0 = X.np0, nstop = X.cnt[F_STOP];
+    int *const comp = X.comp(), *const px = X.px(), *const st = X.st();
+    unsigned *const cw = X.cw();
+    int flags = 0;   // 1: something met, 2: outside the limits
+#pragma unroll 1
+    for (int i = np0 + T.tid(); i < np1; i += T.NT) {
+        const unsigned long long p = X.pr[i];
+        const int a = pr_lo(p), b = pr_hi(p);
+        if (comp[a] != comp[b] && px[a] + px[b] >= pr_val(p)) {
+            flags |= 1;
+            if (st[a] == ST_RUN || st[b] == ST_RUN) flags |= 2;
+            X.pr[i] = p | MET;
+            cw[comp[a]] = 0;
+            cw[comp[b]] = 0;
+        }
+    }
+    T.sync();
+    // an island that stopped but met nothing needs explored balls
+#pragma unroll 1
+    for (int i = nstop ? T.tid() : n2; i < n2; i += T.NT)
+        if (cw[list[K - 1 - i]] == ISL_ALONE) flags |= 2;
+    flags = T.template red32<2>(flags);
+    if ((flags & 2) || ((flags & 1) && (round >= 32 || (X.paths && n1)))) {
+        T.sync();
+        return 2;
+    }
+    if (!(flags & 1)) {
+        T.sync();
+        return 0;
+    }
+    // run what was joined (with paths: everything, since their list starts over)
+    T.sync();
+    fast_components(X, np1, T);
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) {
+        cw[s] = 0;
+        if (round == 0 && st[s] != MATE_NONE) X.recs[s].size = 0;   // not an island so far
+    }
+    if (T.tid() == 0) {
+        X.cnt[F_NP] = np0; X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_NPATH] = 0; X.cnt[F_STOP] = 0;
+    }
+    T.sync();
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) atomicAdd(&cw[comp[s]], 1u);
+    T.sync();
+    w = 0;
+    o = 0;
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) {
+        const int c = comp[s], size = (int)cw[c];
+        if ((st[s] == MATE_BOUNDARY && size == 1) || (st[s] >= 0 && size == 2)) {
+            add_closed(X, s, st[s], 2 * px[s], w, o);
+        } else if (s == c && st[s] != ST_RUN) {
+            all[atomicAdd(&X.cnt[F_NALL], 1)] = s;
+            if (X.paths || X.recs[s].size != size) list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
+        }
+    }
+    T.sync();
+    return 1;
+}
+
+constexpr int USE_GENERAL = -3;   // the shot is outside the fast path's limits
+constexpr int HAS_ISLANDS = -4;   // begun: its islands are listed
+
+// What the warps of a block that decode a shot each share: the islands of all
+// their shots, taken by whichever warp is free.
+struct Pool {
+    int n[32], next;
+};
+
+// A shot between the phases of the fast path (per thread).
+struct FastShot {
+    Level1 L;
+    IslRec lev;   // level-1 clusters run (lane 0 of each warp)
+    int lmax, K, np0, n1, n2;
+};
+
+// First phase: events, pairs, level 1.  Returns QEC_SHOT_OK for a shot without
+// events (everything written), HAS_ISLANDS or USE_GENERAL.
+template <bool WIN, int NW>
+__device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
+                                          Team<NW> &T, FastShared<NW> &M, FastShot &Q, int *dg) {
+    // level 1 present, lists complete, first extensions within the listed pairs
+    const int band = max(g.wmax, 1) * max(A.band_factor, 1);
+    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (int)MET ||
+        band + max(band, (g.b1 + 1) >> 1) > g.b1 || g.words > A.caps.wcap)
+        return USE_GENERAL;
+    Fast &X = M.f;
+    bool small = true;
+    int K = 0;
+#pragma unroll 1
+    for (;;) {
+        if (T.tid() == 0) {
+            X.g = &g;
+            X.row = row;
+            X.wcum = S.wcum;
+            X.ev = small ? M.ev : reinterpret_cast<int *>(S.wl1);   // 48 K words of 8 bytes
+            X.pr = small ? M.pr : S.tl;
+            X.stride = small ? M.KS : A.caps.kc;
+            X.pcap = small ? M.PS : A.caps.ec;
+            X.recs = reinterpret_cast<IslRec *>(S.wl0);
+            X.list = S.xsrc; X.all = S.xcnt;
+            X.aged_t = S.xR; X.aged_c = S.sbeg; X.aged_n = S.scnt;
+            X.pa = S.tmpa; X.pb = S.tmpb; X.pd = S.cst2;
+            X.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
+            X.band = band;
+            X.paths = WIN || g.internal_obs;
+            X.tcut = 0;
+        }
+        if (T.tid() < F_TOTAL) X.cnt[T.tid()] = 0;
+        T.sync();
+        K = load_events(S.wcum, g, row, X.ev, X.stride, T);
+        if (K == 0) {
+            if (dg && T.tid() < QEC_DIAG_FIELDS) dg[T.tid()] = 0;   // no detection event: E_ideal = 0
+            if constexpr (WIN)
+                for (int w = T.tid(); w < g.words; w += T.NT) A.carry[(row - A.syn) + w] = 0u;
+            return QEC_SHOT_OK;
+        }
+        if (K > A.caps.kc || K > 4000) return USE_GENERAL;
+        if (K <= X.stride) {
+            if (T.tid() == 0) X.K = K;
+            T.sync();
+            if (!fast_pairs(X, T)) return USE_GENERAL;
+            Q.np0 = X.cnt[F_NP];
+            if (Q.np0 <= X.pcap && Q.np0 < (1 << 18)) break;
+            if (!small) return USE_GENERAL;
+        }
+        T.sync();
+        small = false;
+    }
+    if (T.tid() == 0) X.np0 = Q.np0;
+    T.sync();
+    fast_components(X, Q.np0, T);
+    fast_level1(X, Q.L, T);
+    Q.K = K;
+    Q.n1 = X.cnt[F_N1];
+    Q.n2 = X.cnt[F_N2];
+    Q.lev = IslRec{0, 0, 0, 0, 0, 0, 0};
+    Q.lmax = 0;
+    if (dg) {
+        Q.L.t1 = T.maxi(Q.L.t1);
+        T.sync();
+        if (T.tid() == 0) X.tcut = Q.L.t1;
+        T.sync();
+    }
+    return HAS_ISLANDS;
+}
+
+// Second phase: the islands, and what remains of level 1 before them.  POOL: the
+// warps of the block have a shot each and share their islands (phases of the
+// warps in step keep the instruction cache warm, and no warp waits for the
+// largest shot alone); `busy`: this warp has one.  Then the shot's own pairs
+// recorded by extensions, which join different islands or clusters when the
+// radii reach their distance.  Returns QEC_SHOT_OK or USE_GENERAL.
+template <bool WIN, int NW, bool POOL>
+__device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool &P, FastShot &Q, bool busy, int *dg) {
     Isl &I = M.isl[T.warp()];
-    int n2 = M.cnt[F_N2], nall = n2, naged = 0;
-    const int *all = S.xsrc + (K - n2);   // the islands
+    const int lane = T.lane, K = Q.K;
+    // stage 0: level-1 clusters; 1: islands; 2: islands joined since
+    int stage = busy && Q.n1 > 0 ? 0 : 1, round = 0, i = T.warp(), status = QEC_SHOT_OK, pooled = 0;
+    int incl = 0;   // islands of the block's shots up to this lane's
 #pragma unroll 1
-    for (int round = 0;; round++) {
-        if (round == 0 && n1 > 0) {
-#pragma unroll 1
-            for (int i = T.warp(); i < n1 && !fail; i += NW) {
-                const int c = S.xsrc[i];
-                IslRec r;
-                fail = run_island(S, C, F, I, c, (int)(F.cw[c] & 4095u), np0, 0, true, paths, T.lane, r) != ISL_OK;
-                if (T.lane == 0 && !fail) {
-                    lw += r.w; lo ^= r.o;
-                    lnm += r.nm; lmax = max(lmax, r.nm); ltlast = max(ltlast, r.tlast); lnx += r.nx;
+    for (;;) {
+        // the next cluster or island
+        int c = -1;
+        Fast *X = &M.f;
+        if (stage == 1 && POOL) {
+            if (!pooled) {
+                if (lane == 0) P.n[threadIdx.x >> 5] = busy && status == QEC_SHOT_OK ? Q.n2 : 0;
+                __syncthreads();
+                incl = lane < (int)(blockDim.x >> 5) ? P.n[lane] : 0;
+#pragma unroll
+                for (int o = 1; o < WS; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                pooled = __shfl_sync(FULL, incl, WS - 1) + 1;
+            }
+            int k = 0;
+            if (lane == 0) k = atomicAdd(&P.next, 1);
+            k = __shfl_sync(FULL, k, 0);
+            if (k < pooled - 1) {
+                const int w = __popc(__ballot_sync(FULL, incl <= k));   // whose island it is
+                const int before = __shfl_sync(FULL, incl, max(w - 1, 0));
+                X = &(&M - (threadIdx.x >> 5) + w)->f;
+                c = X->list[X->K - 1 - (k - (w ? before : 0))];
+            }
+        } else if (i < (stage ? Q.n2 : Q.n1) && status == QEC_SHOT_OK) {
+            c = M.f.list[stage ? K - 1 - i : i];
+            i += NW;
+        }
+        if (c >= 0) {
+            const int r = run_island(*X, I, c, (int)(X->cw()[c] & 4095u), stage == 0, lane);
+            if (lane == 0) {
+                if (r == ISL_OK && stage == 0) {
+                    Q.lev.w += I.rec.w; Q.lev.o ^= I.rec.o; Q.lev.nm += I.rec.nm; Q.lev.nx += I.rec.nx;
+                    Q.lev.tlast = max(Q.lev.tlast, I.rec.tlast);
+                    Q.lmax = max(Q.lmax, I.rec.nm);
+                } else if (r == ISL_OK) {
+                    X->recs[c] = I.rec;
+                } else {
+                    if (r == ISL_FAIL || stage == 0) X->cnt[F_FAIL] = 1;
+                    X->recs[c].size = -1;
                 }
             }
-            if (dg) t1 = max(t1, T.maxi(ltlast));
+            __syncwarp();
+            continue;
         }
-#pragma unroll 1
-        for (int i = T.warp(); i < n2 && !fail; i += NW) {
-            const int c = S.xsrc[K - 1 - i];
-            IslRec r;
-            r.size = -1;
-            fail = run_island(S, C, F, I, c, (int)(F.cw[c] & 4095u), np0, t1, false, paths, T.lane, r) == ISL_FAIL;
-            if (T.lane == 0) recs[c] = r;
+        // the end of a stage
+        if (stage == 1 && POOL) {
+            __syncthreads();
+            if (threadIdx.x == 0) P.next = 0;
+            if (!busy) return QEC_SHOT_OK;
         }
-        fail = T.template red32<2>(fail);
-        if constexpr (NW == 1) T.sync();
-        if (fail) return USE_GENERAL;
-        // pairs recorded by extensions join different islands or clusters when
-        // the radii reach their distance
-        const int np1 = M.cnt[F_NP];
-        naged = M.cnt[F_AGED];
-        if (naged > K) return USE_GENERAL;
-        const int nstop = M.cnt[F_STOP];
-        if (np1 == np0) {
-            if (nstop) return USE_GENERAL;
-            break;
-        }
-        bool met = false;
-#pragma unroll 1
-        for (int i = np0 + T.tid(); i < np1; i += T.NT) {
-            const unsigned long long p = F.pr[i];
-            const int a = pr_lo(p), b = pr_hi(p);
-            if (F.comp[a] != F.comp[b] && F.px[a] + F.px[b] >= pr_val(p)) {
-                met = true;
-                if (F.st[a] == ST_RUN || F.st[b] == ST_RUN) fail = 1;
-                F.pr[i] = p | MET;
-                F.cw[F.comp[a]] = 0;
-                F.cw[F.comp[b]] = 0;
+        T.sync();
+        i = T.warp();
+        if (M.f.cnt[F_FAIL] || M.f.cnt[F_AGED] > K) status = USE_GENERAL;
+        if (stage == 0) {
+            stage = 1;
+            if (dg) {
+                Q.L.t1 = max(Q.L.t1, T.maxi(Q.lev.tlast));
+                T.sync();
+                if (T.tid() == 0) M.f.tcut = Q.L.t1;
+                T.sync();
             }
+            continue;
         }
-        T.sync();
-        // a stopped island that met nothing needs explored balls
-#pragma unroll 1
-        for (int i = nstop ? T.tid() : n2; i < n2; i += T.NT)
-            if (F.cw[S.xsrc[K - 1 - i]] == ISL_ALONE) fail = 1;
-        if (T.any(fail != 0)) return USE_GENERAL;
-        if (!T.any(met)) break;
-        if (round == 32) return USE_GENERAL;
-        // join what met and run what was joined (with paths: everything, since
-        // their list starts over)
-        if (paths && n1) return USE_GENERAL;
-        fast_components(F, np0, np1, K, T);
-#pragma unroll 1
-        for (int s = T.tid(); s < K; s += T.NT) {
-            F.cw[s] = 0;
-            if (round == 0 && F.st[s] != MATE_NONE) recs[s].size = 0;   // not an island so far
-        }
-        if (T.tid() == 0) {
-            M.cnt[F_NP] = np0; M.cnt[F_N2] = 0; M.cnt[F_NALL] = 0; M.cnt[F_NPATH] = 0; M.cnt[F_STOP] = 0;
-        }
-        T.sync();
-#pragma unroll 1
-        for (int s = T.tid(); s < K; s += T.NT) atomicAdd(&F.cw[F.comp[s]], 1u);
-        T.sync();
-        wsum = 0;
-        osum = 0;
-#pragma unroll 1
-        for (int s = T.tid(); s < K; s += T.NT) {
-            const int c = F.comp[s], size = (int)F.cw[c], st = F.st[s];
-            if ((st == MATE_BOUNDARY && size == 1) || (st >= 0 && size == 2)) {
-                closed(s, st, 2 * F.px[s]);
-            } else if (s == c && st != ST_RUN) {
-                S.xcnt[atomicAdd(&M.cnt[F_NALL], 1)] = s;
-                if (paths || recs[s].size != size) S.xsrc[K - 1 - atomicAdd(&M.cnt[F_N2], 1)] = s;
-            }
-        }
-        T.sync();
-        n2 = M.cnt[F_N2];
-        nall = M.cnt[F_NALL];
-        all = S.xcnt;
+        if (status != QEC_SHOT_OK) return status;
+        const int np1 = M.f.cnt[F_NP];
+        if (np1 == Q.np0) return M.f.cnt[F_STOP] ? USE_GENERAL : QEC_SHOT_OK;   // (stopped, having met nothing)
+        const int j = fast_join(M.f, np1, Q.n1, Q.n2, round++, T, Q.L.w, Q.L.o);
+        if (j != 1) return j == 2 ? USE_GENERAL : QEC_SHOT_OK;
+        Q.n2 = M.f.cnt[F_N2];
+        stage = 2;
     }
+}
+
+// Last phase: the shot's result and diagnostics.
+template <bool WIN, int NW>
+__device__ __forceinline__ int fast_end(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
+                                        Team<NW> &T, FastShared<NW> &M, FastShot &Q, long long &w_out,
+                                        unsigned long long &o_out, int *dg) {
+    Fast &X = M.f;
+    const int K = Q.K, n1 = Q.n1;
     // the islands together
+    const int joined = X.cnt[F_NALL], nall = joined ? joined : X.cnt[F_N2];
+    const int *const all = joined ? X.all : X.list + (K - nall);
     int ntop = 0, ncut = 0, tlast = 0, tnx = 0;
 #pragma unroll 1
     for (int i = T.tid(); i < nall; i += T.NT) {
-        const IslRec r = recs[all[i]];
-        wsum += r.w;
-        osum ^= r.o;
+        const IslRec r = X.recs[all[i]];
+        Q.L.w += r.w;
+        Q.L.o ^= r.o;
         ntop += r.nm; ncut += r.ncut; tlast = max(tlast, r.tlast); tnx += r.nx;
     }
-    const long long budget = min(A.max_events, 256LL * K + 4096);
-    if (budget < 256LL * K + 4096) {   // a budget set lower: the run over everything counts exactly
-        if ((long long)T.add(lnm + lnx + ntop + tnx) + naged + n1 + 2 > budget) return USE_GENERAL;
+    const int naged = X.cnt[F_AGED];
+    if (A.max_events < 256LL * K + 4096) {   // a budget set lower: the run over everything counts exactly
+        if ((long long)T.add(Q.lev.nm + Q.lev.nx + ntop + tnx) + naged + n1 + 2 > A.max_events) return USE_GENERAL;
     }
-    int aged = 0;
-    if (dg) {   // bands: one per time at which regions of the top level came of age
+    w_out = T.sum64(Q.L.w + Q.lev.w) / 2;
+    o_out = T.xor64(Q.L.o ^ Q.lev.o);
+    if (dg) {
+        // parallel event count over level 1 and the top level (Methods,
+        // "Numerical evaluation").  Bands: one per time at which regions of the
+        // top level came of age (entries of islands joined since don't count)
+        int aged = 0;
 #pragma unroll 1
         for (int i = T.tid(); i < naged; i += T.NT) {
-            // (entries of islands that were joined since don't count)
-            auto live = [&](int k) { return F.comp[S.sbeg[k]] == S.sbeg[k] && recs[S.sbeg[k]].size == S.scnt[k]; };
-            const int x = S.xR[i];
+            auto live = [&](int k) { const int c = X.aged_c[k]; return X.comp()[c] == c && X.recs[c].size == X.aged_n[k]; };
+            const int x = X.aged_t[i];
             int first = live(i);
 #pragma unroll 1
-            for (int j = 0; j < i && first; j++) first = !(S.xR[j] == x && live(j));
+            for (int j = 0; j < i && first; j++) first = !(X.aged_t[j] == x && live(j));
             aged += first;
         }
         aged = T.add(aged);
-    }
-    const long long wint = T.sum64(wsum + lw);
-    unsigned long long ob = T.xor64(osum ^ lo);
-    if (paths) {
-        const unsigned long long po = walk_paths<WIN>(A, S, C, T, F.svtx, M.cnt[F_NPATH], 1,
-                                                      WIN ? A.carry + (row - A.syn) : nullptr);
-        const int err = T.bcast(ldr(&S.ctr[C_ERR]));
-        if (C.paths) release_tables(S, C, T, err != 0);
-        if (err) return USE_GENERAL;
-        ob = WIN ? po : ob ^ po;
-    }
-    w_out = wint / 2;
-    o_out = ob;
-    if (dg) {
-        // parallel event count over level 1 and the top level (Methods,
-        // "Numerical evaluation")
-        const int ncl = T.add(ncl1), nres = T.add(nres1);
-        lnm = T.add(lnm); lnx = T.add(lnx); lmax = T.maxi(lmax);
+        const int ncl = T.add(Q.L.ncl), nres = T.add(Q.L.nres);
+        const int lnm = T.add(Q.lev.nm), lnx = T.add(Q.lev.nx), lmax = T.maxi(Q.lmax);
         ntop = T.add(ntop); ncut = T.add(ncut); tnx = T.add(tnx); tlast = T.maxi(tlast);
         // closed forms have one event each
         const int e1 = max(lmax, ncl > n1 ? 1 : 0), ntot = (ncl - n1) + lnm;
         if (T.tid() == 0) {
             dg[QEC_DIAG_E_IDEAL] = ntop > 0 ? max(e1, ncut) + ntop - ncut : e1;
-            dg[QEC_DIAG_T_IDEAL] = ntop > 0 ? max(t1, tlast) : t1;
+            dg[QEC_DIAG_T_IDEAL] = ntop > 0 ? max(Q.L.t1, tlast) : Q.L.t1;
             dg[QEC_DIAG_EVENTS] = ntot + ntop;
             dg[QEC_DIAG_L1_CLUSTERS] = ncl;
             dg[QEC_DIAG_L1_DEFECTS] = nres;
@@ -3180,6 +3391,22 @@ __device__ __forceinline__ int decode_fast(const BatchArgs &A, const Slab &S, co
             dg[QEC_DIAG_BANDS] = lnx + tnx + aged + (nall > 0 ? 1 : 0);
             dg[QEC_DIAG_DEFECTS] = K;
         }
+    }
+    if (WIN || g.internal_obs) {
+        Shot C;
+        C.g = g;
+        C.row = row;
+        C.K = K;
+        C.L = X.L;
+        C.band = X.band;
+        C.real = 0;
+        C.paths = 0;
+        const unsigned long long po = walk_paths<WIN>(A, S, C, T, X.ev, X.cnt[F_NPATH], 1,
+                                                      WIN ? A.carry + (row - A.syn) : nullptr);
+        const int err = T.bcast(ldr(&S.ctr[C_ERR]));
+        if (C.paths) release_tables(S, C, T, err != 0);
+        if (err) return USE_GENERAL;
+        o_out = WIN ? po : o_out ^ po;
     }
     return QEC_SHOT_OK;
 }
@@ -3208,26 +3435,78 @@ __device__ __noinline__ int decode_general(const BatchArgs &A, const Slab &S, co
     return status;
 }
 
-template <bool WIN, int NW>
-__device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, Team<NW> &T, FastShared<NW> &M,
-                            unsigned long long deadline) {
+// One shot's place in the batch.
+struct ShotRef {
+    const DGraph *g;
+    const unsigned *row;
+    long long shot, off;
+    int *dg;
+};
+__device__ __forceinline__ ShotRef shot_ref(const BatchArgs &A, long long shot) {
     int gi = A.graph_of_shot ? A.graph_of_shot[shot] : 0;
     if (gi < 0 || gi >= A.num_graphs) gi = 0;
-    const DGraph &g = A.g[gi];
-    const long long off = A.syn_off ? A.syn_off[shot] : shot * (long long)g.words;
-    const unsigned *row = A.syn + off;
+    ShotRef r;
+    r.g = &A.g[gi];
+    r.shot = shot;
+    r.off = A.syn_off ? A.syn_off[shot] : shot * (long long)r.g->words;
+    r.row = A.syn + r.off;
+    r.dg = A.diag_out ? A.diag_out + shot * QEC_DIAG_FIELDS : nullptr;
+    return r;
+}
+
+// Write a shot's outputs (status < 0: it did not fit its slab).
+template <bool WIN, int NW>
+__device__ __forceinline__ void finish_shot(const BatchArgs &A, const ShotRef &r, Team<NW> &T, int status, long long w,
+                                            unsigned long long o) {
+    const bool retried = status < 0 && A.pass == 0 && A.single_shot < 0;   // goes to the overflow pass
+    if (status < 0) {
+        status = QEC_SHOT_CAPACITY;
+        if (retried && T.tid() == 0) {
+            const unsigned long long idx = atomicAdd(&A.queue[1], 1ull);
+            A.overflow[idx] = (int)r.shot;
+        }
+        w = 0;
+        o = 0;
+    }
+    if (r.dg && status != QEC_SHOT_OK && T.tid() < QEC_DIAG_FIELDS) r.dg[T.tid()] = 0;
+    if constexpr (WIN) {
+        // sliding window: nothing is committed by a failed shot
+        if (status != QEC_SHOT_OK)
+            for (int i = T.tid(); i < r.g->words; i += T.NT) A.carry[r.off + i] = 0u;
+        if (T.tid() == 0) {
+            if (status == QEC_SHOT_OK) A.cobs[r.shot] ^= o;
+            else if (!retried) A.st_out[r.shot] = status;
+        }
+    } else if (T.tid() == 0) {
+        A.w_out[r.shot] = w;
+        A.obs_out[r.shot] = o;
+        A.st_out[r.shot] = status;
+        if (A.done && !retried) {
+            // the results reach the host before the flag that publishes them
+            __threadfence_system();
+            asm volatile("st.release.sys.global.b32 [%0], %1;" :: "l"(A.done + r.shot), "r"(1) : "memory");
+        }
+    }
+    T.sync();
+}
+
+// Decode one shot by a team.  POOL (NW = 1): every warp of the block calls at
+// the same time, those without a shot with busy = false.
+template <bool WIN, int NW, bool POOL>
+__device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, const ShotRef &r, bool busy, Team<NW> &T,
+                                            FastShared<NW> &M, Pool &P, unsigned long long deadline) {
     if constexpr (NW > 1) {
         // a shot below the split threshold goes to the team's first warp
         // alone (a team's barriers cost more than its lanes save there)
-        if (A.team_split > 0) {
+        if (A.team_split > 1) {
             int K = 0;
-            if (T.warp() == 0) K = count_defects(g, row, T.lane);
+            if (T.warp() == 0) K = count_defects(*r.g, r.row, T.lane);
             K = T.bcast(K);
             if (K < A.team_split) {
                 if (T.warp() == 0) {
                     Team<1> T1;
                     T1.lane = T.lane;
-                    decode_shot<WIN, 1>(A, S, shot, T1, reinterpret_cast<FastShared<1> &>(M), deadline);
+                    decode_shot<WIN, 1, false>(A, S, r, true, T1, reinterpret_cast<FastShared<1> &>(M), P, deadline);
                 }
                 T.sync();
                 return;
@@ -3236,50 +3515,30 @@ __device__ void decode_shot(const BatchArgs &A, const Slab &S, long long shot, T
     }
     long long w = 0;
     unsigned long long o = 0;
-    int *dg = A.diag_out ? A.diag_out + shot * QEC_DIAG_FIELDS : nullptr;
-    int status = decode_fast<WIN, NW>(A, S, g, row, T, M, w, o, dg);
+    FastShot Q;
+    Q.n1 = Q.n2 = Q.K = 0;
+    int status = QEC_SHOT_OK;
+    if (busy) status = fast_begin<WIN, NW>(A, S, *r.g, r.row, T, M, Q, r.dg);
+    if (POOL || status == HAS_ISLANDS) {
+        const bool has = busy && status == HAS_ISLANDS;
+        const int st = fast_islands<WIN, NW, POOL>(T, M, P, Q, has, r.dg);
+        if (has) status = st == QEC_SHOT_OK ? fast_end<WIN, NW>(A, S, *r.g, r.row, T, M, Q, w, o, r.dg) : st;
+    }
+    if (!busy) return;
     if (status == USE_GENERAL) {
         T.sync();
-        status = decode_general<WIN, NW>(A, S, g, row, T, deadline, w, o, dg);
+        status = decode_general<WIN, NW>(A, S, *r.g, r.row, T, deadline, w, o, r.dg);
     }
-    const bool retried = status < 0 && A.pass == 0 && A.single_shot < 0;   // goes to the overflow pass
-    if (status < 0) {
-        status = QEC_SHOT_CAPACITY;
-        if (retried && T.tid() == 0) {
-            const unsigned long long idx = atomicAdd(&A.queue[1], 1ull);
-            A.overflow[idx] = (int)shot;
-        }
-        w = 0;
-        o = 0;
-    }
-    if (dg && status != QEC_SHOT_OK && T.tid() < QEC_DIAG_FIELDS) dg[T.tid()] = 0;
-    if constexpr (WIN) {
-        // sliding window: nothing is committed by a failed shot
-        if (status != QEC_SHOT_OK)
-            for (int i = T.tid(); i < g.words; i += T.NT) A.carry[off + i] = 0u;
-        if (T.tid() == 0) {
-            if (status == QEC_SHOT_OK) A.cobs[shot] ^= o;
-            else if (!retried) A.st_out[shot] = status;
-        }
-    } else if (T.tid() == 0) {
-        A.w_out[shot] = w;
-        A.obs_out[shot] = o;
-        A.st_out[shot] = status;
-        if (A.done && !retried) {
-            // the results reach the host before the flag that publishes them
-            __threadfence_system();
-            asm volatile("st.release.sys.global.b32 [%0], %1;" :: "l"(A.done + shot), "r"(1) : "memory");
-        }
-    }
-    T.sync();
+    finish_shot<WIN, NW>(A, r, T, status, w, o);
 }
 
 // One team per warp (NW = 1, any block size that is a multiple of 32) or one
 // team per block (NW > 1, blocks of exactly 32 NW threads).
 template <bool WIN, int NW>
-__global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW, NW == 1 ? QEC_MIN_BLOCKS : (NW == 4 ? 4 : 1))
+__global__ void __launch_bounds__(NW == 1 ? 32 * QEC_MAX_WARPS : 32 * NW, NW == 1 ? 24 / QEC_MAX_WARPS : (NW == 4 ? 4 : 1))
 batch_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(16) char dyn[];   // one FastShared per team
+    __shared__ Pool pool;
     Team<NW> T;
     T.lane = threadIdx.x & 31;
     FastShared<NW> &M = reinterpret_cast<FastShared<NW> *>(dyn)[NW == 1 ? threadIdx.x >> 5 : 0];
@@ -3298,20 +3557,28 @@ batch_kernel(const __grid_constant__ BatchArgs a) {
         unsigned long long t0 = T.tid() == 0 ? now_ns() : 0;
         deadline = T.bcast64(t0) + (unsigned long long)a.watchdog_ns;
     }
-    if (a.single_shot >= 0) {
-        if (wid == 0) decode_shot<WIN, NW>(a, S, a.single_shot, T, M, deadline);
-        return;
-    }
+    if (NW == 1 && threadIdx.x == 0) pool.next = 0;
+    __syncthreads();
+    // a single shot is the work of the first team; otherwise team t starts with
+    // item (its place in the block) x blocks + block, so that a small batch
+    // spreads over the SMs, and goes on with whatever is next
+    const bool one = a.single_shot >= 0;
     unsigned long long *counter = a.queue + (a.pass == 0 ? 0 : 2);
-    const long long limit = a.pass == 0 ? a.num_shots : (long long)min(a.queue[1], (unsigned long long)a.num_shots);
-    for (long long it = 0; it < a.num_shots + 1; it++) {
-        unsigned long long item = 0;
-        if (T.tid() == 0) item = atomicAdd(counter, 1ull);
-        item = T.bcast64(item);
-        if ((long long)item >= limit) break;
-        const long long shot = a.pass == 0 ? (a.order ? (long long)a.order[item] : (long long)item)
-                                           : (long long)a.overflow[item];
-        decode_shot<WIN, NW>(a, S, shot, T, M, deadline);
+    const long long teams = NW == 1 ? (long long)gridDim.x * (blockDim.x >> 5) : (long long)gridDim.x;
+    const long long limit = one ? 1 : (a.pass == 0 ? a.num_shots : (long long)min(a.queue[1], (unsigned long long)a.num_shots));
+    long long item = NW == 1 ? (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x : (long long)blockIdx.x;
+    for (long long it = 0; it < limit + 1; it++) {
+        const bool busy = item < limit;
+        if (NW == 1 ? !__syncthreads_or(busy) : !busy) break;
+        ShotRef r{a.g, a.syn, 0, 0, nullptr};
+        unsigned long long next = 0;
+        if (busy) {
+            r = shot_ref(a, one ? a.single_shot
+                                : (a.pass == 0 ? (a.order ? (long long)a.order[item] : item) : (long long)a.overflow[item]));
+            if (T.tid() == 0 && !one) next = atomicAdd(counter, 1ull);
+        }
+        decode_shot<WIN, NW, NW == 1>(a, S, r, busy, T, M, pool, deadline);
+        item = busy && !one ? (long long)T.bcast64(next) + teams : limit;
     }
 }
 
@@ -3390,27 +3657,39 @@ SlabCaps caps_for_kcap(int kcap, int table_factor) {
 
 namespace {
 
-// Launch one instantiation with its teams' shared memory (above 48 KB a kernel
-// needs the attribute, set on every launch of the current device: it is per
-// device, and a microsecond).
+// Shared memory of a block, and the attribute that a kernel needs above 48 KB
+// (set once per device, for the largest block).
+template <int NW>
+constexpr int smem_of(int block) { return (int)sizeof(FastShared<NW>) * (NW == 1 ? block / 32 : 1); }
+
+template <bool WIN, int NW>
+cudaError_t allow_smem() {
+    static std::atomic<unsigned long long> ready{0};   // bit per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (ready.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(batch_kernel<WIN, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             smem_of<NW>(32 * QEC_MAX_WARPS));
+    if (e == cudaSuccess) ready.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+
 template <bool WIN, int NW>
 cudaError_t launch_as(const BatchArgs &a, int grid, int block, cudaStream_t s) {
-    const int smem = (int)sizeof(FastShared<NW>) * (NW == 1 ? block / 32 : 1);
-    if (smem + (int)sizeof(TeamShared) > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(batch_kernel<WIN, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
-    batch_kernel<WIN, NW><<<grid, NW == 1 ? block : 32 * NW, smem, s>>>(a);
+    const cudaError_t e = allow_smem<WIN, NW>();
+    if (e != cudaSuccess) return e;
+    batch_kernel<WIN, NW><<<grid, NW == 1 ? block : 32 * NW, smem_of<NW>(block), s>>>(a);
     return cudaGetLastError();
 }
 
 template <int NW>
 int blocks_per_sm(int block) {
-    const int smem = (int)sizeof(FastShared<NW>) * (NW == 1 ? block / 32 : 1);
     int nb = 0;
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel<false, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem<false, NW>();
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, NW>, block, (size_t)smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<false, NW>, block, (size_t)smem_of<NW>(block));
     return e == cudaSuccess && nb > 0 ? nb : 1;
 }
 

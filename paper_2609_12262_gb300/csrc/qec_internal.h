@@ -39,6 +39,7 @@ struct DGraph {
     // boundary vertex << 32 | lowest merged id among the boundary edges at that
     // distance; all ones when no boundary is reachable
     const unsigned long long *vbnd;
+    const unsigned long long *vobs;   // [n]: observable mask of that edge (0 when there is none)
     // ball table (balls.cu): header {first entry, higher detectors within b1,
     // detectors within b1 (-1: list not complete), detectors beyond b1 within
     // brad (-1: not complete)} of every detector, entries {detector, distance}
@@ -89,7 +90,7 @@ struct BatchArgs {
     unsigned long long *cobs;
     unsigned *carry;
     // multi-warp teams: a shot with fewer detection events than this is
-    // decoded by the team's first warp alone (0: always by the whole team)
+    // decoded by the team's first warp alone (0 or 1: always by the whole team)
     int team_split;
     // serving: per-shot completion flags in host memory mapped into the
     // device (obs_out / w_out / st_out then point there too); set to 1, after
