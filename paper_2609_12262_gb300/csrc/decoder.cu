@@ -80,7 +80,10 @@
 #define QEC_HT_FACTOR 64   // explored-table slots per detection event (rounded up to a power of two)
 #endif
 #ifndef QEC_MAX_WARPS
-#define QEC_MAX_WARPS 8   // warps of a block that decode a shot each; 24 of them fit an SM
+#define QEC_MAX_WARPS 4   // warps of a block that decode a shot each
+#endif
+#ifndef QEC_SM_WARPS
+#define QEC_SM_WARPS 20   // such warps per SM that the register budget must allow
 #endif
 
 namespace qec {
@@ -201,16 +204,15 @@ __device__ __forceinline__ unsigned long long warp_min64_redux(unsigned long lon
     return ((unsigned long long)mh << 32) | ml;
 }
 
+// 64-bit sums and XORs with the 32-bit reduction unit (values below 2^51: 26
+// low bits and the rest apart, so that 32 of either stay below 2^31).
 __device__ __forceinline__ long long warp_sum64(long long v) {
-#pragma unroll
-    for (int o = WS / 2; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    return v;
+    const long long lo = __reduce_add_sync(FULL, (unsigned)v & 0x3ffffffu);
+    return lo + ((long long)(int)__reduce_add_sync(FULL, (unsigned)(v >> 26)) << 26);
 }
 
 __device__ __forceinline__ unsigned long long warp_xor64(unsigned long long v) {
-#pragma unroll
-    for (int o = WS / 2; o; o >>= 1) v ^= __shfl_xor_sync(FULL, v, o);
-    return v;
+    return ((unsigned long long)__reduce_xor_sync(FULL, (unsigned)(v >> 32)) << 32) | __reduce_xor_sync(FULL, (unsigned)v);
 }
 
 // ------------------------------------------------------------------ teams --
@@ -2185,7 +2187,10 @@ struct __align__(16) Isl {
     __device__ __forceinline__ int top(int e) const { return pk[e] & (LAB1 - 1); }
 };
 
-enum { ST_RUN = -3 };
+enum { ST_RUN = -3, ST_ONE = -4, ST_TWO = -5 };
+constexpr unsigned CW_OPEN = 1u << 30, CW_SIDE = 1u << 31;
+// frozen at the start of the top level
+__device__ __forceinline__ bool st_frozen(int st) { return st >= 0 || st == MATE_BOUNDARY || st == ST_RUN; }
 enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2 };
 constexpr unsigned ISL_ALONE = 1u << 31;
 constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
@@ -2195,12 +2200,15 @@ enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL
 // shared memory or, for shots with more events than it holds, in the slab:
 //   svtx  vertex                      bd  boundary distance (INT_MAX: none)
 //   comp  lowest event of the component
-//   px    a pair within d_1, later the largest radius
+//   px    nearest event: distance << 12 | event (all ones: none within b_1),
+//         later the largest radius
 //   st    level-1 state: the partner or MATE_BOUNDARY in a closed form,
-//         MATE_NONE: a growing root of the top level, ST_RUN: in a level-1
-//         cluster that was run
-//   cw    at a component's lowest event: size | pairs within d_1 << 12 |
-//         boundary contact << 31; in an island, the event's lane
+//         ST_RUN: in a level-1 cluster of more events; a growing root of the
+//         top level: MATE_NONE, or ST_ONE / ST_TWO in an island solved in
+//         closed form (ST_TWO: the higher event of a pair)
+//   cw    at a component's lowest event: size | pairs within d_1 << 12 | not
+//         in closed form << 30 | boundary contact << 31; in an island, the
+//         event's lane
 // and the pairs, lo << 46 | hi << 28 | distance.
 struct __align__(16) Fast {
     const DGraph *g;
@@ -2582,7 +2590,7 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl &I, int c, int n, int np, in
             if (!mh) continue;
             const bool in = hit && comp[f] == c;
             // a level-1 cluster stands still unless it is touched
-            const int mt = __reduce_min_sync(FULL, hit && !in && st[f] != MATE_NONE ? d - px[f] : INT_MAX);
+            const int mt = __reduce_min_sync(FULL, hit && !in && st_frozen(st[f]) ? d - px[f] : INT_MAX);
             if (lane == l) I.meet[l] = min(I.meet[l], mt);
             int b = 0;
             if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(mh));
@@ -2641,7 +2649,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
     if (lane < n) {
         const int ev = I.ev[lane], bd = X.bd()[ev];
         const int st = level1 ? (int)MATE_NONE : X.st()[ev];
-        const bool frozen = st != MATE_NONE;
+        const bool frozen = st_frozen(st);
         bad = st == ST_RUN;
         if (st == MATE_BOUNDARY) rad = bd;   // (a frozen pair's radius: with its pair below)
         I.bd[lane] = bd;
@@ -2892,22 +2900,23 @@ __device__ __forceinline__ int load_events(int *wcum, const DGraph &g, const uns
 }
 
 // Per-event arrays of the shot and its pairs within b_1 (as near_pairs: from
-// their lower ends, off the ball table; half a warp per event, since most lists
-// have 12 entries).  Returns false when an event's list is not complete or
-// longer than level 1 takes.  Every thread of the team calls; ends with a
-// barrier.
+// their lower ends, off the ball table; eight lanes per event and two entries
+// per lane, since most lists have 12 entries).  Pairs are first noted with the
+// other event's vertex and get its rank afterwards, every lane busy.  Returns
+// false when an event's list is not complete or longer than level 1 takes.
+// Every thread of the team calls; ends with a barrier.
 template <int NW>
 __device__ __forceinline__ bool fast_pairs(Fast &X, Team<NW> &T) {
     const DGraph &g = *X.g;
-    const int lane = T.lane, K = X.K, half = lane >> 4, sub = lane & 15;
-    int *const svtx = X.svtx(), *const bd = X.bd(), *const comp = X.comp(), *const st = X.st();
+    const int lane = T.lane, K = X.K, sub = 2 * (lane & 7);
+    int *const svtx = X.svtx(), *const bd = X.bd(), *const comp = X.comp(), *const px = X.px();
     unsigned *const cw = X.cw();
     const unsigned *const row = X.row;
-    const int *const wcum = X.wcum;
     unsigned long long *const pr = X.pr;
     const int pcap = X.pcap;
     const int2 *const ball = g.ball;
     const int most = g.hop2 ? INT_MAX : LB_CAP - 1;
+    const unsigned lt = (1u << lane) - 1u;
     bool odd = false;
     int np = 0;
 #pragma unroll 1
@@ -2921,48 +2930,54 @@ __device__ __forceinline__ bool fast_pairs(Fast &X, Team<NW> &T) {
             bd[s] = vb == EMPTY64 ? INT_MAX : (int)(vb >> 32);
             comp[s] = s;
             cw[s] = 0;
-            st[s] = MATE_NONE;
+            px[s] = -1;
             odd |= h.z < 0 || h.z > most;
             beg = h.x;
             len = h.z < 0 ? 0 : h.y;
         }
-#pragma unroll 2
-        for (int e0 = 0; e0 < WS && base + e0 < K; e0 += 2) {
-            const unsigned eb = (unsigned)__shfl_sync(FULL, beg, e0 + half);
-            const int el = __shfl_sync(FULL, len, e0 + half);
-            const int em = max(el, __shfl_xor_sync(FULL, el, 16));
+        const int longest = __reduce_max_sync(FULL, len);
 #pragma unroll 1
-            for (int k = 0; k < em; k += 16) {
-                bool hit = false;
-                int2 e = make_int2(0, 0);
-                unsigned word = 0;
-                if (k + sub < el) {
-                    e = __ldg(ball + eb + k + sub);
-                    word = __ldg(row + (e.x >> 5));
-                    hit = (word >> (e.x & 31)) & 1u;
+        for (int e0 = lane >> 3; __any_sync(FULL, e0 < WS && base + e0 < K); e0 += 4) {
+            const unsigned eb = (unsigned)__shfl_sync(FULL, beg, e0);
+            const int el = __shfl_sync(FULL, len, e0);
+#pragma unroll 1
+            for (int k = sub; __any_sync(FULL, k - sub < longest); k += 16) {
+                bool h0 = false, h1 = false;
+                int4 e = make_int4(0, 0, 0, 0);
+                if (k < el) {
+                    e = __ldg(reinterpret_cast<const int4 *>(ball + eb + k));   // lists start on 128-byte lines
+                    h0 = (__ldg(row + (e.x >> 5)) >> (e.x & 31)) & 1u;
+                    h1 = k + 1 < el && ((__ldg(row + (e.z >> 5)) >> (e.z & 31)) & 1u);
                 }
-                const unsigned m = __ballot_sync(FULL, hit);
-                if (!m) continue;
+                const unsigned m0 = __ballot_sync(FULL, h0), m1 = __ballot_sync(FULL, h1);
+                if (!(m0 | m1)) continue;
+                const int c0 = __popc(m0), c = c0 + __popc(m1);
                 int b;
                 if constexpr (NW == 1) {
                     b = np;
-                    np += __popc(m);
+                    np += c;
                 } else {
                     b = 0;
-                    if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(m));
+                    if (lane == 0) b = atomicAdd(&X.cnt[F_NP], c);
                     b = __shfl_sync(FULL, b, 0);
                 }
-                if (hit) {
-                    const int j = b + __popc(m & ((1u << lane) - 1u));
-                    const int f = wcum[e.x >> 5] + __popc(word & ((1u << (e.x & 31)) - 1u));
-                    if (j < pcap) pr[j] = pk_pair(base + e0 + half, f, e.y);
-                }
+                const unsigned long long self = (unsigned long long)(unsigned)(base + e0) << 52;
+                const int j0 = b + __popc(m0 & lt), j1 = b + c0 + __popc(m1 & lt);
+                if (h0 && j0 < pcap) pr[j0] = self | ((unsigned long long)(unsigned)e.x << 26) | (unsigned)e.y;
+                if (h1 && j1 < pcap) pr[j1] = self | ((unsigned long long)(unsigned)e.z << 26) | (unsigned)e.w;
             }
         }
     }
     if constexpr (NW == 1)
         if (lane == 0) X.cnt[F_NP] = np;
     odd = T.any(odd);
+    if constexpr (NW == 1) T.sync();
+    const int n = min(X.cnt[F_NP], pcap);
+#pragma unroll 1
+    for (int i = T.tid(); i < n; i += T.NT) {
+        const unsigned long long p = pr[i];
+        pr[i] = pk_pair((int)(p >> 52), X.rank((int)(p >> 26) & 0x3ffffff), (int)p & 0x3ffffff);
+    }
     T.sync();
     return !odd;
 }
@@ -3005,82 +3020,114 @@ __device__ __forceinline__ void fast_components(Fast &X, int np1, Team<NW> &T) {
 }
 
 // Level 1 of the shot: sizes, contacts and pairs within d_1 of the components,
-// then clusters in closed form (their weight and observable added to w and o).
+// then what has a closed form (its weight and observable added to w and o):
+// level-1 clusters of one or two events, and with `quick` every cluster or
+// island in which each event either meets the event nearest to it, which
+// has no nearer one itself (at half their distance), or the boundary first, and
+// no other pair can touch before both its events have stopped.  Those are 60 %
+// of the islands (two or three pairs near each other).  A pair that could be
+// tight at the very time its events stop leaves the island open: the order of
+// simultaneous events decides there.  Without `quick` (diagnostics are wanted)
+// islands still take the closed form, level-1 clusters of more events run.
 // The other clusters (from the front of X.list) and the islands (from its back)
 // are listed by their lowest event.  Per-thread: t1 the last stopping time, ncl
 // the clusters, nres their events.  Every thread of the team calls; ends with a
 // barrier.
 struct Level1 {
-    long long w;
-    unsigned long long o;
+    long long w, wr;   // wr, ro: of clusters that nothing reopens
+    unsigned long long o, ro;
     int t1, ncl, nres;
 };
-__device__ __forceinline__ void add_closed(Fast &X, int s, int st, int d, long long &w, unsigned long long &o) {
-    if (st == MATE_BOUNDARY) {
+__device__ __forceinline__ void add_closed(Fast &X, int s, int partner, int d, long long &w, unsigned long long &o) {
+    if (partner < 0) {
         const int bd = X.bd()[s];
         w += bd;
         o ^= __ldg(X.g->vobs + X.svtx()[s]);
         if (X.paths) put_path(X, s, -1, bd);
     } else {
         w += d / 2;
-        if (X.paths && s < st) put_path(X, s, st, d);
+        if (X.paths && s < partner) put_path(X, s, partner, d);
     }
 }
 template <int NW>
-__device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, Team<NW> &T) {
+__device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, bool quick, Team<NW> &T) {
     const DGraph &g = *X.g;
-    const int K = X.K, np0 = X.np0, b1 = g.b1, d1 = g.d1;
+    const int K = X.K, np0 = X.np0, b1 = g.b1, d1 = g.d1, band = X.band;
     const int *const comp = X.comp(), *const bdv = X.bd();
     int *const px = X.px(), *const stv = X.st();
     unsigned *const cwv = X.cw();
     const unsigned long long *const pr = X.pr;
     int *const list = X.list;
+    const bool pack = b1 < (1 << 19);   // distances fit beside the event
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
         const int r = comp[s];
         atomicAdd(&cwv[r], 1u);
-        if (2LL * bdv[s] <= (long long)b1) atomicOr(&cwv[r], 1u << 31);
+        if (2LL * bdv[s] <= (long long)b1) atomicOr(&cwv[r], CW_SIDE);
     }
-    // pairs within d_1, each noted at its two events: the pair of an accepted
-    // two-event cluster
 #pragma unroll 1
     for (int i = T.tid(); i < np0; i += T.NT) {
         const unsigned long long p = pr[i];
-        if (pr_val(p) > d1) continue;
-        const int a = pr_lo(p), b = pr_hi(p);
-        atomicAdd(&cwv[comp[a]], 1u << 12);
-        px[a] = i;
-        px[b] = i;
+        const int a = pr_lo(p), b = pr_hi(p), d = pr_val(p);
+        if (d <= d1) atomicAdd(&cwv[comp[a]], 1u << 12);
+        atomicMin(reinterpret_cast<unsigned *>(px) + a, (unsigned)d << 12 | (unsigned)b);
+        atomicMin(reinterpret_cast<unsigned *>(px) + b, (unsigned)d << 12 | (unsigned)a);
     }
     T.sync();
-    Level1 L{0, 0, 0, 0, 0};
+    // when each event would stop (st: 2 x time, + 1 at the boundary)
+#pragma unroll 1
+    for (int s = T.tid(); s < K; s += T.NT) {
+        const unsigned near = (unsigned)px[s];
+        const int bd = bdv[s], d = near == ~0u ? INT_MAX : (int)(near >> 12);
+        bool ok = pack;
+        int t = d >> 1;
+        if (bd < t) {
+            t = bd;
+            stv[s] = 2 * min(t, 1 << 29) + 1;
+        } else {
+            const unsigned back = near == ~0u ? 0u : (unsigned)px[near & 4095u];
+            ok &= near != ~0u && (back & 4095u) == (unsigned)s && bdv[near & 4095u] >= t;
+            stv[s] = 2 * min(t, 1 << 29);
+        }
+        if (!ok || t > band) atomicOr(&cwv[comp[s]], CW_OPEN);
+    }
+    T.sync();
+#pragma unroll 1
+    for (int i = T.tid(); i < np0; i += T.NT) {
+        const unsigned long long p = pr[i];
+        const int a = pr_lo(p), b = pr_hi(p), d = pr_val(p), sa = stv[a], sb = stv[b];
+        const bool matched = (px[a] & 4095) == b && !(sa & 1) && (px[b] & 4095) == a;
+        if (!matched && d <= (sa >> 1) + (sb >> 1)) atomicOr(&cwv[comp[a]], CW_OPEN);
+    }
+    T.sync();
+    Level1 L{0, 0, 0, 0, 0, 0, 0};
+    const bool whole = quick && !X.paths;   // clusters of more events too
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
         const int r = comp[s];
         const unsigned cw = cwv[r];
-        const int size = (int)(cw & 4095u), prs = (int)(cw >> 12) & 0x7ffff;
-        const bool ok = prs == size * (size - 1) / 2 && ((cw >> 31) || size % 2 == 0);
-        if (ok && size <= 2) {
-            int st = MATE_BOUNDARY, rad = bdv[s], d = 0;   // one boundary event at time bd
-            bool fine = true;
-            if (size == 2) {
-                const unsigned long long p = pr[px[s]];
-                st = pr_lo(p) == s ? pr_hi(p) : pr_lo(p);
-                d = pr_val(p);
-                rad = d / 2;   // one collision at time d/2
-                fine = rad <= bdv[s] && rad <= bdv[st];
-            }
-            if (fine) {
-                stv[s] = st;
-                px[s] = rad;
+        const int size = (int)(cw & 4095u), prs = (int)(cw >> 12) & 0x3ffff;
+        const bool ok = prs == size * (size - 1) / 2 && ((cw & CW_SIDE) || size % 2 == 0);
+        const int near = (int)((unsigned)px[s] >> 12), other = px[s] & 4095;
+        // a cluster of one or two events: one boundary event, or one collision
+        // when no boundary is nearer
+        const bool small = ok && pack && (size == 1 || (size == 2 && near / 2 <= bdv[s] && near / 2 <= bdv[other]));
+        if (small || (!(cw & CW_OPEN) && (!ok || whole))) {
+            const bool side = small ? size == 1 : (stv[s] & 1) != 0;
+            const int rad = side ? bdv[s] : near / 2;
+            stv[s] = small ? (side ? (int)MATE_BOUNDARY : other)
+                           : (ok ? (int)ST_RUN : (side || s < other ? (int)ST_ONE : (int)ST_TWO));
+            if (ok && !small) add_closed(X, s, side ? -1 : other, near, L.wr, L.ro);
+            else add_closed(X, s, side ? -1 : other, near, L.w, L.o);
+            px[s] = rad;
+            if (ok) {
                 L.t1 = max(L.t1, rad);
                 L.nres++;
                 if (s == r) L.ncl++;
-                add_closed(X, s, st, d, L.w, L.o);
-                continue;
             }
+            continue;
         }
-        if (ok) stv[s] = ST_RUN;
+        stv[s] = ok ? (int)ST_RUN : (int)MATE_NONE;
         if (s == r) {
             if (ok) { list[atomicAdd(&X.cnt[F_N1], 1)] = s; L.nres += size; L.ncl++; }
             else list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
@@ -3136,7 +3183,8 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int roun
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
         cw[s] = 0;
-        if (round == 0 && st[s] != MATE_NONE) X.recs[s].size = 0;   // not an island so far
+        if (round == 0 && st[s] != MATE_NONE) X.recs[s].size = 0;   // not run so far
+        if (st[s] == ST_ONE || st[s] == ST_TWO) st[s] = MATE_NONE;   // run from now on
     }
     if (T.tid() == 0) {
         X.cnt[F_NP] = np0; X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_NPATH] = 0; X.cnt[F_STOP] = 0;
@@ -3151,8 +3199,10 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int roun
     for (int s = T.tid(); s < K; s += T.NT) {
         const int c = comp[s], size = (int)cw[c];
         if ((st[s] == MATE_BOUNDARY && size == 1) || (st[s] >= 0 && size == 2)) {
-            add_closed(X, s, st[s], 2 * px[s], w, o);
-        } else if (s == c && st[s] != ST_RUN) {
+            add_closed(X, s, st[s], 2 * px[s], w, o);   // (MATE_BOUNDARY is negative)
+        } else if (st[s] == ST_RUN) {
+            // (unchanged: nothing joined it)
+        } else if (s == c) {
             all[atomicAdd(&X.cnt[F_NALL], 1)] = s;
             if (X.paths || X.recs[s].size != size) list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
         }
@@ -3170,6 +3220,25 @@ struct Pool {
     int n[32], next;
 };
 
+// The fields of a team's Fast that stay the same from shot to shot.  One thread.
+template <int NW>
+__device__ __forceinline__ void fast_small(FastShared<NW> &M) {
+    M.f.ev = M.ev;
+    M.f.pr = M.pr;
+    M.f.stride = M.KS;
+    M.f.pcap = M.PS;
+}
+template <int NW>
+__device__ __forceinline__ void fast_setup(const Slab &S, FastShared<NW> &M) {
+    Fast &X = M.f;
+    X.wcum = S.wcum;
+    X.recs = reinterpret_cast<IslRec *>(S.wl0);
+    X.list = S.xsrc; X.all = S.xcnt;
+    X.aged_t = S.xR; X.aged_c = S.sbeg; X.aged_n = S.scnt;
+    X.pa = S.tmpa; X.pb = S.tmpb; X.pd = S.cst2;
+    fast_small(M);
+}
+
 // A shot between the phases of the fast path (per thread).
 struct FastShot {
     Level1 L;
@@ -3184,7 +3253,7 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
                                           Team<NW> &T, FastShared<NW> &M, FastShot &Q, int *dg) {
     // level 1 present, lists complete, first extensions within the listed pairs
     const int band = max(g.wmax, 1) * max(A.band_factor, 1);
-    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (int)MET ||
+    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (1 << 26) ||
         band + max(band, (g.b1 + 1) >> 1) > g.b1 || g.words > A.caps.wcap)
         return USE_GENERAL;
     Fast &X = M.f;
@@ -3195,19 +3264,18 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
         if (T.tid() == 0) {
             X.g = &g;
             X.row = row;
-            X.wcum = S.wcum;
-            X.ev = small ? M.ev : reinterpret_cast<int *>(S.wl1);   // 48 K words of 8 bytes
-            X.pr = small ? M.pr : S.tl;
-            X.stride = small ? M.KS : A.caps.kc;
-            X.pcap = small ? M.PS : A.caps.ec;
-            X.recs = reinterpret_cast<IslRec *>(S.wl0);
-            X.list = S.xsrc; X.all = S.xcnt;
-            X.aged_t = S.xR; X.aged_c = S.sbeg; X.aged_n = S.scnt;
-            X.pa = S.tmpa; X.pb = S.tmpb; X.pd = S.cst2;
             X.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
             X.band = band;
             X.paths = WIN || g.internal_obs;
             X.tcut = 0;
+            if (!small) {
+                X.ev = reinterpret_cast<int *>(S.wl1);   // 48 K words of 8 bytes
+                X.pr = S.tl;
+                X.stride = A.caps.kc;
+                X.pcap = A.caps.ec;
+            } else if (X.stride != M.KS) {
+                fast_small(M);
+            }
         }
         if (T.tid() < F_TOTAL) X.cnt[T.tid()] = 0;
         T.sync();
@@ -3233,7 +3301,7 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
     if (T.tid() == 0) X.np0 = Q.np0;
     T.sync();
     fast_components(X, Q.np0, T);
-    fast_level1(X, Q.L, T);
+    fast_level1(X, Q.L, !dg, T);
     Q.K = K;
     Q.n1 = X.cnt[F_N1];
     Q.n2 = X.cnt[F_N2];
@@ -3355,12 +3423,23 @@ __device__ __forceinline__ int fast_end(const BatchArgs &A, const Slab &S, const
         Q.L.o ^= r.o;
         ntop += r.nm; ncut += r.ncut; tlast = max(tlast, r.tlast); tnx += r.nx;
     }
+    int closed = 0;   // islands in closed form: their events
+    if (dg) {
+#pragma unroll 1
+        for (int s = T.tid(); s < K; s += T.NT) {
+            const int st = X.st()[s], t = X.px()[s];
+            if (st != ST_ONE && st != ST_TWO) continue;
+            if (st == ST_ONE) { ntop++; ncut += t <= X.tcut; }
+            tlast = max(tlast, t);
+            closed = 1;
+        }
+    }
     const int naged = X.cnt[F_AGED];
     if (A.max_events < 256LL * K + 4096) {   // a budget set lower: the run over everything counts exactly
-        if ((long long)T.add(Q.lev.nm + Q.lev.nx + ntop + tnx) + naged + n1 + 2 > A.max_events) return USE_GENERAL;
+        if ((long long)T.add(Q.lev.nm + Q.lev.nx + ntop + tnx) + naged + n1 + K + 2 > A.max_events) return USE_GENERAL;
     }
-    w_out = T.sum64(Q.L.w + Q.lev.w) / 2;
-    o_out = T.xor64(Q.L.o ^ Q.lev.o);
+    w_out = T.sum64(Q.L.w + Q.L.wr + Q.lev.w) / 2;
+    o_out = T.xor64(Q.L.o ^ Q.L.ro ^ Q.lev.o);
     if (dg) {
         // parallel event count over level 1 and the top level (Methods,
         // "Numerical evaluation").  Bands: one per time at which regions of the
@@ -3376,6 +3455,7 @@ __device__ __forceinline__ int fast_end(const BatchArgs &A, const Slab &S, const
             aged += first;
         }
         aged = T.add(aged);
+        closed = T.any(closed != 0);
         const int ncl = T.add(Q.L.ncl), nres = T.add(Q.L.nres);
         const int lnm = T.add(Q.lev.nm), lnx = T.add(Q.lev.nx), lmax = T.maxi(Q.lmax);
         ntop = T.add(ntop); ncut = T.add(ncut); tnx = T.add(tnx); tlast = T.maxi(tlast);
@@ -3388,7 +3468,7 @@ __device__ __forceinline__ int fast_end(const BatchArgs &A, const Slab &S, const
             dg[QEC_DIAG_L1_CLUSTERS] = ncl;
             dg[QEC_DIAG_L1_DEFECTS] = nres;
             dg[QEC_DIAG_TOP_EVENTS] = ntop;
-            dg[QEC_DIAG_BANDS] = lnx + tnx + aged + (nall > 0 ? 1 : 0);
+            dg[QEC_DIAG_BANDS] = lnx + tnx + aged + (nall > 0 || closed ? 1 : 0);
             dg[QEC_DIAG_DEFECTS] = K;
         }
     }
@@ -3506,7 +3586,11 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
                 if (T.warp() == 0) {
                     Team<1> T1;
                     T1.lane = T.lane;
-                    decode_shot<WIN, 1, false>(A, S, r, true, T1, reinterpret_cast<FastShared<1> &>(M), P, deadline);
+                    FastShared<1> &M1 = reinterpret_cast<FastShared<1> &>(M);
+                    if (T.lane == 0) fast_setup(S, M1);
+                    __syncwarp();
+                    decode_shot<WIN, 1, false>(A, S, r, true, T1, M1, P, deadline);
+                    if (T.lane == 0) fast_setup(S, M);
                 }
                 T.sync();
                 return;
@@ -3535,7 +3619,7 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
 // One team per warp (NW = 1, any block size that is a multiple of 32) or one
 // team per block (NW > 1, blocks of exactly 32 NW threads).
 template <bool WIN, int NW>
-__global__ void __launch_bounds__(NW == 1 ? 32 * QEC_MAX_WARPS : 32 * NW, NW == 1 ? 24 / QEC_MAX_WARPS : (NW == 4 ? 4 : 1))
+__global__ void __launch_bounds__(NW == 1 ? 32 * QEC_MAX_WARPS : 32 * NW, NW == 1 ? QEC_SM_WARPS / QEC_MAX_WARPS : (NW == 4 ? 4 : 1))
 batch_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(16) char dyn[];   // one FastShared per team
     __shared__ Pool pool;
@@ -3558,6 +3642,7 @@ batch_kernel(const __grid_constant__ BatchArgs a) {
         deadline = T.bcast64(t0) + (unsigned long long)a.watchdog_ns;
     }
     if (NW == 1 && threadIdx.x == 0) pool.next = 0;
+    if (T.tid() == 0) fast_setup(S, M);
     __syncthreads();
     // a single shot is the work of the first team; otherwise team t starts with
     // item (its place in the block) x blocks + block, so that a small batch
