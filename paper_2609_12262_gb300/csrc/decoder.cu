@@ -2159,10 +2159,7 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
 // what they share lies in shared memory: with everything inlined and unrolled
 // the million-shot batch was 40 % slower, waiting for instructions and spilled
 // registers.
-constexpr int IN = 32;    // events of an island (one lane each); blossoms are nodes IN .. 2 IN - 1
-constexpr int IP = 64;    // pairs
-constexpr int IC = 96;    // blossom cycle entries
-constexpr int LAB1 = 1 << 6;
+constexpr int TOP_BITS = 7, TOP_MASK = (1 << TOP_BITS) - 1, RAD_SHIFT = TOP_BITS + 2;
 
 // What one island, or several, add to the shot (w: internal units).
 struct __align__(16) IslRec {
@@ -2171,10 +2168,18 @@ struct __align__(16) IslRec {
     int nm, ncut, tlast, nx;   // matcher events, those at times <= tcut, time of the last, bands counted here
 };
 
+// An island: E events per lane.  E = 1 lies in shared memory; E = 2, for the few
+// islands that need it (0.1 % of circuit-level d = 13 shots, 1 % of d = 51
+// windows at p = 0.005), in the slab.
+template <int E>
 struct __align__(16) Isl {
+    static constexpr int IN = 32 * E;    // events; blossoms are nodes IN .. 2 IN - 1
+    static constexpr int IP = 128 * E;   // pairs
+    static constexpr int IC = 96 * E;    // blossom cycle entries
+    static constexpr int LB = 4 + E;     // bits of an event in a key
     int2 pair[IP];        // distance, lower event | higher event << 8
-    int pk[IN];           // per event: radius << 8 | (label of its top node + 1) << 6 | top node
-    int y[2 * IN];        // duals (leaves: written at the end)
+    int pk[IN];           // per event: radius << 9 | (label of its top node + 1) << 7 | top node
+    int y[2 * IN];        // duals of the blossoms
     int ev[IN], bd[IN];   // event of the shot, boundary distance
     int xt[IN];           // radius at which the explored radius falls due (INT_MAX: ball exhausted)
     int meet[IN];         // radius at which the region touches a level-1 cluster outside
@@ -2184,14 +2189,16 @@ struct __align__(16) Isl {
     unsigned char cn[IC], cs[IC], co[IC], cb[IN], cl[IN];   // cycles: child, its leaf, the next child's leaf
     signed char ta[2 * IN], tb[2 * IN];                     // tree paths / expansion stack
     int nc, err;
-    __device__ __forceinline__ int top(int e) const { return pk[e] & (LAB1 - 1); }
+    __device__ __forceinline__ int top(int e) const { return pk[e] & TOP_MASK; }
+    __device__ __forceinline__ int rad(int e) const { return pk[e] >> RAD_SHIFT; }
+    __device__ __forceinline__ void set_top(int e, int v) { pk[e] = (pk[e] & ~TOP_MASK) | v; }
 };
 
 enum { ST_RUN = -3, ST_ONE = -4, ST_TWO = -5 };
 constexpr unsigned CW_OPEN = 1u << 30, CW_SIDE = 1u << 31;
 // frozen at the start of the top level
 __device__ __forceinline__ bool st_frozen(int st) { return st >= 0 || st == MATE_BOUNDARY || st == ST_RUN; }
-enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2 };
+enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2, ISL_BIG = 3 };
 constexpr unsigned ISL_ALONE = 1u << 31;
 constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
 enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6, F_FAIL = 7, F_TOTAL = 8 };   // Fast::cnt
@@ -2220,6 +2227,8 @@ struct __align__(16) Fast {
     int *list, *all;                   // clusters and islands to run; all islands once some were joined
     int *aged_t, *aged_c, *aged_n;     // bands of regions that came of age: time, island, its size
     int *pa, *pb, *pd;                 // matched pairs for the path walks
+    char *spare;                       // room for larger islands, nspare bytes
+    int nspare, nlist;                 // nlist: room in the lists above
     int stride, pcap, K, np0, tcut, L, band, paths;
     int cnt[F_TOTAL];
     __device__ __forceinline__ int *svtx() const { return ev; }
@@ -2240,11 +2249,11 @@ struct __align__(16) Fast {
 // events, and one island per warp.
 template <int NW>
 struct __align__(16) FastShared {
-    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + KS / 4;
+    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + (NW == 1 ? KS / 2 : KS / 4);
     Fast f;
     unsigned long long pr[PS];
     int ev[6 * KS];
-    Isl isl[NW];
+    Isl<1> isl[NW];
 };
 
 __device__ __forceinline__ unsigned long long pk_pair(int a, int b, int d) {
@@ -2254,7 +2263,8 @@ __device__ __forceinline__ int pr_lo(unsigned long long p) { return (int)(p >> 4
 __device__ __forceinline__ int pr_hi(unsigned long long p) { return (int)(p >> 28) & 0x3ffff; }
 __device__ __forceinline__ int pr_val(unsigned long long p) { return (int)(p & (MET - 1)); }
 
-__device__ __forceinline__ int isl_child_of(const Isl &I, int B, int leaf) {
+template <int E>
+__device__ __forceinline__ int isl_child_of(const Isl<E> &I, int B, int leaf) {
     int v = leaf;
 #pragma unroll 1
     while (v >= 0 && I.bpar[v] != B) v = I.bpar[v];
@@ -2262,7 +2272,8 @@ __device__ __forceinline__ int isl_child_of(const Isl &I, int B, int leaf) {
 }
 
 // flip matches along the tree path from outer A to its root (lane 0)
-__device__ __forceinline__ void isl_flip(Isl &I, int A) {
+template <int E>
+__device__ __forceinline__ void isl_flip(Isl<E> &I, int A) {
     int v = A;
 #pragma unroll 1
     while (I.tpar[v] >= 0) {
@@ -2274,9 +2285,11 @@ __device__ __forceinline__ void isl_flip(Isl &I, int A) {
 }
 
 // Event (c): the new blossom N over outer A, B of one tree.  `bal`: blossoms
-// alive before.  Returns the event's top node, or -1 when the cycle pool is
-// full.  One warp.
-__device__ __noinline__ int isl_blossom(Isl &I, int N, int A, int a, int B, int b, int n, unsigned bal, int lane) {
+// alive before.  Returns false when the cycle pool is full.  One warp.
+template <int E>
+__device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, int b, int n, const unsigned (&bal)[E],
+                                         int lane) {
+    constexpr int IN = Isl<E>::IN, IC = Isl<E>::IC;
     int ok = 1;
     if (lane == 0) {
         int na = 0, nb = 0;
@@ -2316,36 +2329,33 @@ __device__ __noinline__ int isl_blossom(Isl &I, int N, int A, int a, int B, int 
             I.cb[N - IN] = (unsigned char)cb; I.cl[N - IN] = (unsigned char)m;
         }
     }
-    if (!__shfl_sync(FULL, ok, 0)) return -1;
+    if (!__shfl_sync(FULL, ok, 0)) return false;
     __syncwarp();
     const int L0 = I.cn[I.cb[N - IN]];   // if it was its tree's root, N is now
 #pragma unroll 1
-    for (int h = 0; h < 2; h++) {
-        const int v = lane + h * IN;
-        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+    for (int h = 0; h < 2 * E; h++) {
+        const int v = lane + h * WS;
+        if (h < E ? v >= n : !((bal[h - E] >> lane) & 1u)) continue;
         if (I.bpar[v] >= 0) continue;
         const int tp = I.tpar[v], mt = I.mate[v];
         if (tp >= 0 && I.bpar[tp] == N) I.tpar[v] = (signed char)N;
         if (mt >= 0 && I.bpar[mt] == N) I.mate[v] = (signed char)N;
         if (I.root[v] == L0) I.root[v] = (signed char)N;
     }
-    int top = lane;
-    if (lane < n) {
-        top = I.top(lane);
-        if (I.bpar[top] == N) top = N;
-    }
+#pragma unroll 1
+    for (int e = lane; e < n; e += WS)
+        if (I.bpar[I.top(e)] == N) I.set_top(e, N);
     __syncwarp();
-    return top;
+    return true;
 }
 
-// Event (d): inner blossom B shatters.  Returns the event's top node (I.err on
-// an inconsistent state).  One warp.
-__device__ __noinline__ int isl_shatter(Isl &I, int B, int n, int lane) {
-    int top = lane;
-    if (lane < n) {
-        top = I.top(lane);
-        if (top == B) top = isl_child_of(I, B, lane);
-    }
+// Event (d): inner blossom B shatters (I.err on an inconsistent state).  One warp.
+template <int E>
+__device__ __noinline__ void isl_shatter(Isl<E> &I, int B, int n, int lane) {
+    constexpr int IN = Isl<E>::IN;
+#pragma unroll 1
+    for (int e = lane; e < n; e += WS)
+        if (I.top(e) == B) I.set_top(e, max(0, isl_child_of(I, B, e)));
     __syncwarp();
     if (lane == 0) {
         const int m = I.cl[B - IN], cb = I.cb[B - IN];
@@ -2401,12 +2411,12 @@ __device__ __noinline__ int isl_shatter(Isl &I, int B, int n, int lane) {
         }
     }
     __syncwarp();
-    return top;
 }
 
 // Distance of two matched events of an island (as tight_dist).
-__device__ __forceinline__ int isl_dist(const Isl &I, int a, int b) {
-    int d = (I.pk[a] >> 8) + (I.pk[b] >> 8);
+template <int E>
+__device__ __forceinline__ int isl_dist(const Isl<E> &I, int a, int b) {
+    int d = I.rad(a) + I.rad(b);
 #pragma unroll 1
     for (int B = I.bpar[a]; B >= 0; B = I.bpar[B]) {
         int x = I.bpar[b];
@@ -2428,11 +2438,13 @@ __device__ __forceinline__ void put_path(Fast &X, int a, int b, int d) {
 }
 
 // The matched pairs of a finished island.  One warp.
-__device__ __noinline__ void isl_paths(Fast &X, Isl &I, int n, unsigned bal, int lane) {
+template <int E>
+__device__ __noinline__ void isl_paths(Fast &X, Isl<E> &I, int n, const unsigned (&bal)[E], int lane) {
+    constexpr int IN = Isl<E>::IN;
 #pragma unroll 1
-    for (int h = 0; h < 2; h++) {
-        const int v = lane + h * IN;
-        if (h ? !((bal >> lane) & 1u) : lane >= n) continue;
+    for (int h = 0; h < 2 * E; h++) {
+        const int v = lane + h * WS;
+        if (h < E ? v >= n : !((bal[h - E] >> lane) & 1u)) continue;
         if (I.bpar[v] >= 0) continue;
         const int mt = I.mate[v], s = I.ms[v];
         if (mt == MATE_BOUNDARY) put_path(X, I.ev[s], -1, I.bd[s]);
@@ -2442,10 +2454,9 @@ __device__ __noinline__ void isl_paths(Fast &X, Isl &I, int n, unsigned bal, int
     // inside blossoms: the child holding the externally matched leaf keeps that
     // match, the other children pair up along the cycle
 #pragma unroll 1
-    for (unsigned m = bal; m; m &= m - 1) {
+    for (int b = IN; b < 2 * IN; b++) {
         int sp = 0;
-        const int b = IN + __ffs(m) - 1;
-        if (I.bpar[b] >= 0) continue;
+        if (!((bal[(b - IN) >> 5] >> (b & 31)) & 1u) || I.bpar[b] >= 0) continue;
         I.ta[sp] = (signed char)b; I.tb[sp++] = I.ms[b];
 #pragma unroll 1
         while (sp > 0) {
@@ -2537,29 +2548,36 @@ __device__ __noinline__ int far_events(const Fast &X, int v, int q, int lane, in
 // can touch until they fall due again are read off the ball table and recorded
 // among the shot's pairs, those of the island itself also in I.pair.  Returns
 // the island's pairs, -1 outside the limits, -2 beyond the table.  One warp.
-__device__ __noinline__ int isl_extend(Fast &X, Isl &I, int c, int n, int np, int lane) {
+template <int E>
+__device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np, int lane) {
+    constexpr int IP = Isl<E>::IP;
     const DGraph &g = *X.g;
     const int b1 = g.b1, brad = g.brad, wmax = g.wmax;
     const int *const comp = X.comp(), *const st = X.st(), *const px = X.px();
-    int ev = 0, sR = -1, R = 0, q = 0;
-    bool scan = false, far = false;
-    if (lane < n) {
-        const int p = I.pk[lane], rad = p >> 8, xt = I.xt[lane];
-        if ((p & (3 * LAB1)) == 2 * LAB1 && xt <= rad) {
-            ev = I.ev[lane];
-            sR = xt + X.L - 1;   // explored radius, -1: never
-            R = max(sR + X.band, rad + X.L + X.band);
-            q = X.reach(b1, R);
-            scan = sR >= 0 || q > b1;
-            if (!scan) I.xt[lane] = R - X.L + 1;
-            far = scan && (q > 2 * brad - 2 * wmax || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[ev]).w < 0);
+    unsigned scan[E];
+    bool far = false;
+#pragma unroll
+    for (int h = 0; h < E; h++) {
+        const int e = lane + h * WS;
+        bool sc = false;
+        if (e < n) {
+            const int p = I.pk[e], rad = p >> RAD_SHIFT, xt = I.xt[e];
+            if (((p >> TOP_BITS) & 3) == 2 && xt <= rad) {
+                const int sR = xt + X.L - 1;   // explored radius, -1: never
+                const int R = max(sR + X.band, rad + X.L + X.band), q = X.reach(b1, R);
+                sc = sR >= 0 || q > b1;
+                if (!sc) I.xt[e] = R - X.L + 1;
+                far |= sc && (q > 2 * brad - 2 * wmax || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[I.ev[e]]).w < 0);
+            }
         }
+        scan[h] = __ballot_sync(FULL, sc);
     }
     if (__any_sync(FULL, far)) return -2;
 #pragma unroll 1
-    for (unsigned m = __ballot_sync(FULL, scan); m; m &= m - 1) {
-        const int l = __ffs(m) - 1;
-        const int s = __shfl_sync(FULL, ev, l), ql = __shfl_sync(FULL, q, l), sRl = __shfl_sync(FULL, sR, l);
+    for (int i = 0; i < Isl<E>::IN; i++) {
+        if (!((scan[i >> 5] >> (i & 31)) & 1u)) continue;
+        const int s = I.ev[i], sRl = I.xt[i] + X.L - 1;
+        const int R = max(sRl + X.band, I.rad(i) + X.L + X.band), ql = X.reach(b1, R);
         const int q0 = sRl < 0 ? b1 : max(b1, X.reach(b1, sRl));
         const int v = X.svtx()[s];
         const int4 h = __ldg(g.bhdr + v);
@@ -2591,22 +2609,23 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl &I, int c, int n, int np, in
             const bool in = hit && comp[f] == c;
             // a level-1 cluster stands still unless it is touched
             const int mt = __reduce_min_sync(FULL, hit && !in && st_frozen(st[f]) ? d - px[f] : INT_MAX);
-            if (lane == l) I.meet[l] = min(I.meet[l], mt);
+            if (lane == 0) I.meet[i] = min(I.meet[i], mt);
             int b = 0;
             if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(mh));
             b = __shfl_sync(FULL, b, 0) + __popc(mh & ((1u << lane) - 1u));
             if (hit && b < X.pcap) X.pr[b] = pk_pair(min(s, f), max(s, f), d);
-            const unsigned mi = __ballot_sync(FULL, in);
+            // inside the island: unless the other event has it recorded
+            const int k2 = in ? (int)X.cw()[f] : 0;
+            const bool add = in && (I.xt[k2] != INT_MAX && d > max(b1, X.reach(b1, I.xt[k2] + X.L - 1)));
+            const unsigned mi = __ballot_sync(FULL, add);
             const int j = np + __popc(mi & ((1u << lane) - 1u));
-            if (in && j < IP) {
-                const int k2 = (int)X.cw()[f];
-                I.pair[j] = make_int2(d, min(l, k2) | max(l, k2) << 8);
-            }
+            if (add && j < IP) I.pair[j] = make_int2(d, min(i, k2) | max(i, k2) << 8);
             np += __popc(mi);
             if (np > IP || __any_sync(FULL, hit && b >= X.pcap)) return -1;
         }
         more = __any_sync(FULL, more);
-        if (lane == l) I.xt[l] = sRl >= 0 && !more ? INT_MAX : R - X.L + 1;
+        if (lane == 0) I.xt[i] = sRl >= 0 && !more ? INT_MAX : R - X.L + 1;
+        __syncwarp();
     }
     __syncwarp();
     return np;
@@ -2618,10 +2637,14 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl &I, int c, int n, int np, in
 // level1: a level-1 cluster (its bands are counted here; the top level's aged
 // bands are collected, since regions due at the same time share one).  One
 // warp.  The result is left in I.rec.  Returns ISL_FAIL when the island is
-// outside the limits, ISL_STOP when a region touched a level-1 cluster outside
-// or outgrew the ball table (the radii so far are in px, cw[c] is ISL_ALONE).
-__device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool level1, int lane) {
-    if (size > IN) return ISL_FAIL;
+// outside the limits, ISL_BIG when a larger E has room, ISL_STOP when a region
+// touched a level-1 cluster outside or outgrew the ball table (the radii so far
+// are in px, cw[c] is ISL_ALONE).
+template <int E>
+__device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, bool level1, int lane) {
+    constexpr int IN = Isl<E>::IN, IP = Isl<E>::IP, LB = Isl<E>::LB;
+    constexpr unsigned DT_END = (1u << (30 - 2 * LB)) - 1u;
+    if (size > IN) return ISL_BIG;
     const int n = size;
     {
         // members in rank order: the first is c, the others are near it
@@ -2637,29 +2660,34 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
             if (in) {
                 const int j = k + __popc(m & ((1u << lane) - 1u));
                 I.ev[j] = s;
-                cw[s] = (unsigned)j;   // its lane
+                cw[s] = (unsigned)j;   // its place
             }
             k += __popc(m);
         }
     }
     __syncwarp();
-    int rad = 0, top = lane;
+    int rad[E], top[E];
     bool bad = false;
-    I.lab[lane] = 0;
-    if (lane < n) {
-        const int ev = I.ev[lane], bd = X.bd()[ev];
-        const int st = level1 ? (int)MATE_NONE : X.st()[ev];
-        const bool frozen = st_frozen(st);
-        bad = st == ST_RUN;
-        if (st == MATE_BOUNDARY) rad = bd;   // (a frozen pair's radius: with its pair below)
-        I.bd[lane] = bd;
-        // explored radius after the first extension, due at t = 0, which the listed pairs cover
-        I.xt[lane] = frozen ? -X.L : X.band + 1;
-        I.meet[lane] = INT_MAX;
-        I.pk[lane] = rad << 8 | lane;
-        I.lab[lane] = frozen ? 0 : 1; I.bpar[lane] = -1; I.tpar[lane] = -1;
-        I.mate[lane] = frozen ? MATE_BOUNDARY : MATE_NONE; I.ms[lane] = (signed char)lane; I.mo[lane] = -1;
-        I.root[lane] = frozen ? -1 : (signed char)lane; I.minl[lane] = (signed char)lane;
+#pragma unroll
+    for (int h = 0; h < E; h++) {
+        const int e = lane + h * WS;
+        rad[h] = 0;
+        top[h] = e;
+        if (e < n) {
+            const int ev = I.ev[e], bd = X.bd()[ev];
+            const int st = level1 ? (int)MATE_NONE : X.st()[ev];
+            const bool frozen = st_frozen(st);
+            bad |= st == ST_RUN;
+            if (st == MATE_BOUNDARY) rad[h] = bd;   // (a frozen pair's radius: with its pair below)
+            I.bd[e] = bd;
+            // explored radius after the first extension, due at t = 0, which the listed pairs cover
+            I.xt[e] = frozen ? -X.L : X.band + 1;
+            I.meet[e] = INT_MAX;
+            I.pk[e] = rad[h] << RAD_SHIFT | e;
+            I.lab[e] = frozen ? 0 : 1; I.bpar[e] = -1; I.tpar[e] = -1;
+            I.mate[e] = frozen ? MATE_BOUNDARY : MATE_NONE; I.ms[e] = (signed char)e; I.mo[e] = -1;
+            I.root[e] = frozen ? -1 : (signed char)e; I.minl[e] = (signed char)e;
+        }
     }
     if (lane == 0) { I.nc = 0; I.err = 0; }
     if (__any_sync(FULL, bad)) return ISL_FAIL;
@@ -2684,8 +2712,8 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
                 const int a = (int)X.cw()[pr_lo(p)], b = (int)X.cw()[pr_hi(p)], d = pr_val(p);
                 I.pair[k] = make_int2(d, a | b << 8);
                 if (!level1 && X.st()[pr_lo(p)] == pr_hi(p)) {   // a level-1 pair: frozen, matched at d / 2
-                    I.pk[a] = d / 2 << 8 | a;
-                    I.pk[b] = d / 2 << 8 | b;
+                    I.pk[a] = d / 2 << RAD_SHIFT | a;
+                    I.pk[b] = d / 2 << RAD_SHIFT | b;
                     I.mate[a] = (signed char)b; I.mo[a] = (signed char)b;
                     I.mate[b] = (signed char)a; I.mo[b] = (signed char)a;
                 }
@@ -2693,74 +2721,99 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
             np += __popc(m);
         }
     }
-    if (np > IP) return ISL_FAIL;
+    if (np > IP) return ISL_BIG;
     __syncwarp();
-    if (lane < n) rad = I.pk[lane] >> 8;
-    int yl = rad, mrad = rad;   // the leaf's dual, the largest radius so far
-    unsigned bal = 0;           // blossoms alive
+    int yl[E], mrad[E], lab[E];   // the leaf's dual, the largest radius so far, the label of its top node
+    unsigned bal[E];              // blossoms alive
+#pragma unroll
+    for (int h = 0; h < E; h++) {
+        if (lane + h * WS < n) rad[h] = I.rad(lane + h * WS);
+        yl[h] = mrad[h] = rad[h];
+        bal[h] = 0;
+    }
     int t = 0, nm = 0, ncut = 0, tlast = 0, nx = level1 ? 1 : 0;
 #pragma unroll 1
     for (int it = 0;; it++) {
-        if (it > 200 * n || t >= (1 << 22)) return ISL_FAIL;   // far below the shot's event budget
-        int lab = 0;
-        if (lane < n) {
-            lab = I.lab[top];
-            I.pk[lane] = rad << 8 | (lab + 1) << 6 | top;
+        if (it > 200 * n || t >= (1 << 21)) return ISL_FAIL;   // far below the shot's event budget
+        bool grows = false;
+#pragma unroll
+        for (int h = 0; h < E; h++) {
+            const int e = lane + h * WS;
+            lab[h] = 0;
+            if (e < n) {
+                lab[h] = I.lab[top[h]];
+                I.pk[e] = rad[h] << RAD_SHIFT | (lab[h] + 1) << TOP_BITS | top[h];
+            }
+            grows |= lab[h] == 1;
         }
-        if (!__any_sync(FULL, lab == 1)) break;
+        if (!__any_sync(FULL, grows)) break;
         __syncwarp();
-        // next event: key dt << 12 | kind << 10 | lo << 5 | hi, dt < 2^20 - 1;
-        // touching a level-1 cluster outside is kind EXTEND with hi = 1
+        // next event: key dt | kind | lo | hi; touching a level-1 cluster
+        // outside is kind EXTEND with hi = 1
         unsigned key = ~0u;
-        auto cand = [&](int dt, int code) {
-            if ((unsigned)dt < 0xfffffu) key = min(key, ((unsigned)dt << 12) | (unsigned)code);
+        auto cand = [&](int dt, int kind, int lo, int hi) {
+            if ((unsigned)dt < DT_END) key = min(key, ((unsigned)dt << (2 + 2 * LB)) | (unsigned)(kind << (2 * LB) | lo << LB | hi));
         };
-        if (lab == 1) {
-            const int bd = I.bd[lane];
-            bad = bd < rad;
-            cand(max(0, I.xt[lane] - rad), EV_EXTEND << 10 | lane << 5);
-            cand(max(0, I.meet[lane] - rad), EV_EXTEND << 10 | lane << 5 | 1);
-            cand(bd - rad, EV_BOUNDARY << 10 | lane << 5);
+#pragma unroll
+        for (int h = 0; h < E; h++) {
+            const int e = lane + h * WS;
+            if (lab[h] == 1) {
+                const int bd = I.bd[e];
+                bad |= bd < rad[h];
+                cand(max(0, I.xt[e] - rad[h]), EV_EXTEND, e, 0);
+                cand(max(0, I.meet[e] - rad[h]), EV_EXTEND, e, 1);
+                cand(bd - rad[h], EV_BOUNDARY, e, 0);
+            }
         }
 #pragma unroll 1
         for (int p = lane; p < np; p += WS) {
             const int2 pq = I.pair[p];
             const int a = pq.y & 255, b = pq.y >> 8;
             const int ka = I.pk[a], kb = I.pk[b];
-            const int r = ((ka >> 6) & 3) + ((kb >> 6) & 3) - 2;
-            if (((ka ^ kb) & (LAB1 - 1)) == 0 || r <= 0) continue;
-            const int gap = pq.x - (ka >> 8) - (kb >> 8);
+            const int r = ((ka >> TOP_BITS) & 3) + ((kb >> TOP_BITS) & 3) - 2;
+            if (((ka ^ kb) & TOP_MASK) == 0 || r <= 0) continue;
+            const int gap = pq.x - (ka >> RAD_SHIFT) - (kb >> RAD_SHIFT);
             bad |= gap < 0 || (gap & (r - 1)) != 0;
-            cand(gap >> (r - 1), EV_COLLIDE << 10 | a << 5 | b);
+            cand(gap >> (r - 1), EV_COLLIDE, a, b);
         }
-        if ((bal >> lane) & 1u) {
-            const int v = IN + lane;
-            if (I.bpar[v] < 0 && I.lab[v] == -1) cand(I.y[v], EV_IMPLODE << 10 | I.minl[v] << 5);
-        }
+#pragma unroll
+        for (int h = 0; h < E; h++)
+            if ((bal[h] >> lane) & 1u) {
+                const int v = IN + lane + h * WS;
+                if (I.bpar[v] < 0 && I.lab[v] == -1) cand(I.y[v], EV_IMPLODE, I.minl[v], 0);
+            }
         if (__any_sync(FULL, bad)) return ISL_FAIL;
         key = __reduce_min_sync(FULL, key);
         if (key == ~0u) return ISL_FAIL;   // no event left (no solution), or far away
-        const int dt = (int)(key >> 12), kind = (int)(key >> 10) & 3, lo = (int)(key >> 5) & 31, hi = (int)key & 31;
+        const int dt = (int)(key >> (2 + 2 * LB)), kind = (int)(key >> (2 * LB)) & 3;
+        const int lo = (int)(key >> LB) & (IN - 1), hi = (int)key & (IN - 1);
         t += dt;
         if (dt > 0) {
-            rad += lab * dt;
-            mrad = max(mrad, rad);
-            if (top == lane) yl += lab * dt;
-            if ((bal >> lane) & 1u) {
-                const int v = IN + lane;
-                if (I.bpar[v] < 0) I.y[v] += I.lab[v] * dt;
+#pragma unroll
+            for (int h = 0; h < E; h++) {
+                rad[h] += lab[h] * dt;
+                mrad[h] = max(mrad[h], rad[h]);
+                if (top[h] == lane + h * WS) yl[h] += lab[h] * dt;
+                if ((bal[h] >> lane) & 1u) {
+                    const int v = IN + lane + h * WS;
+                    if (I.bpar[v] < 0) I.y[v] += I.lab[v] * dt;
+                }
             }
         }
         if (kind == EV_EXTEND) {
             int r = -2;
             if (!hi) {
-                if (lane < n) I.pk[lane] = rad << 8 | (lab + 1) << 6 | top;
+#pragma unroll
+                for (int h = 0; h < E; h++)
+                    if (lane + h * WS < n) I.pk[lane + h * WS] = rad[h] << RAD_SHIFT | (lab[h] + 1) << TOP_BITS | top[h];
                 __syncwarp();
                 r = isl_extend(X, I, c, n, np, lane);
-                if (r == -1) return ISL_FAIL;
+                if (r == -1) return ISL_BIG;
             }
             if (r == -2) {
-                if (lane < n) X.px()[I.ev[lane]] = mrad;
+#pragma unroll
+                for (int h = 0; h < E; h++)
+                    if (lane + h * WS < n) X.px()[I.ev[lane + h * WS]] = mrad[h];
                 if (lane == 0) { X.cw()[c] = ISL_ALONE; atomicAdd(&X.cnt[F_STOP], 1); }
                 __syncwarp();
                 return ISL_STOP;
@@ -2772,78 +2825,93 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
                 nx++;
             } else if (lane == 0) {
                 const int k = atomicAdd(&X.cnt[F_AGED], 1);
-                if (k < X.K) { X.aged_t[k] = t; X.aged_c[k] = c; X.aged_n[k] = n; }
+                if (k < X.nlist) { X.aged_t[k] = t; X.aged_c[k] = c; X.aged_n[k] = n; }
             }
             continue;
         }
         nm++;
         if (t <= X.tcut) ncut++;
         tlast = t;
+        bool tops = false;   // the events' top nodes changed
         if (kind == EV_IMPLODE) {
             const int B = I.top(lo);
-            top = isl_shatter(I, B, n, lane);
-            bal &= ~(1u << (B - IN));
+            isl_shatter(I, B, n, lane);
+#pragma unroll
+            for (int h = 0; h < E; h++)
+                if (((B - IN) >> 5) == h) bal[h] &= ~(1u << (B & 31));
             if (I.err) return ISL_FAIL;
-            continue;
-        }
-        int a = lo, b = hi, A = I.top(a), B = -1;
-        if (kind == EV_COLLIDE) {
-            B = I.top(b);
-            if (I.lab[A] != 1) { int x = A; A = B; B = x; x = a; a = b; b = x; }
-        }
-        const int lb = B >= 0 ? I.lab[B] : 0, mb = B >= 0 ? (int)I.mate[B] : (int)MATE_BOUNDARY;
-        const int rA = I.root[A], rB = lb == 1 ? I.root[B] : -3;
-        __syncwarp();
-        if (lb == 1 && rA == rB) {
-            if (bal == ~0u) return ISL_FAIL;
-            const int N = IN + __ffs(~bal) - 1;
-            top = isl_blossom(I, N, A, a, B, b, n, bal, lane);
-            if (top < 0) return ISL_FAIL;
-            bal |= 1u << (N - IN);
-        } else if (lb == 1 || mb == MATE_BOUNDARY) {
-            // augment: the trees' nodes leave them while lane 0 rematches
-            // along the tree paths
-            if (lane < n && I.bpar[lane] < 0 && I.lab[lane] != 0 && (I.root[lane] == rA || I.root[lane] == rB)) {
-                I.lab[lane] = 0; I.root[lane] = -1;
-            }
-            if ((bal >> lane) & 1u) {
-                const int v = IN + lane;
-                if (I.bpar[v] < 0 && I.lab[v] != 0 && (I.root[v] == rA || I.root[v] == rB)) { I.lab[v] = 0; I.root[v] = -1; }
-            }
-            if (lane == 0) {
-                isl_flip(I, A);
-                if (B >= 0) {
-                    if (lb == 1) isl_flip(I, B);
-                    I.mate[A] = (signed char)B; I.ms[A] = (signed char)a; I.mo[A] = (signed char)b;
-                    I.mate[B] = (signed char)A; I.ms[B] = (signed char)b; I.mo[B] = (signed char)a;
-                } else {
-                    I.mate[A] = MATE_BOUNDARY; I.ms[A] = (signed char)a; I.mo[A] = -1;
-                }
-            }
-        } else if (lb == 0 && mb >= 0) {
-            if (lane == 0) {   // grow
-                I.lab[B] = -1; I.tpar[B] = (signed char)A; I.tps[B] = (signed char)b; I.tpo[B] = (signed char)a;
-                I.root[B] = (signed char)rA;
-                I.lab[mb] = 1; I.tpar[mb] = (signed char)B; I.tps[mb] = I.ms[mb]; I.tpo[mb] = I.mo[mb];
-                I.root[mb] = (signed char)rA;
-            }
+            tops = true;
         } else {
-            return ISL_FAIL;
+            int a = lo, b = hi, A = I.top(a), B = -1;
+            if (kind == EV_COLLIDE) {
+                B = I.top(b);
+                if (I.lab[A] != 1) { int x = A; A = B; B = x; x = a; a = b; b = x; }
+            }
+            const int lb = B >= 0 ? I.lab[B] : 0, mb = B >= 0 ? (int)I.mate[B] : (int)MATE_BOUNDARY;
+            const int rA = I.root[A], rB = lb == 1 ? I.root[B] : -3;
+            __syncwarp();
+            if (lb == 1 && rA == rB) {
+                int N = -1;
+#pragma unroll
+                for (int h = 0; h < E; h++)
+                    if (N < 0 && bal[h] != ~0u) N = IN + h * WS + __ffs(~bal[h]) - 1;
+                if (N < 0 || !isl_blossom(I, N, A, a, B, b, n, bal, lane)) return ISL_BIG;
+#pragma unroll
+                for (int h = 0; h < E; h++)
+                    if (((N - IN) >> 5) == h) bal[h] |= 1u << (N & 31);
+                tops = true;
+            } else if (lb == 1 || mb == MATE_BOUNDARY) {
+                // augment: the trees' nodes leave them while lane 0 rematches
+                // along the tree paths
+#pragma unroll
+                for (int h = 0; h < 2 * E; h++) {
+                    const int v = lane + h * WS;
+                    if (h < E ? v >= n : !((bal[h < E ? 0 : h - E] >> lane) & 1u)) continue;
+                    if (I.bpar[v] < 0 && I.lab[v] != 0 && (I.root[v] == rA || I.root[v] == rB)) { I.lab[v] = 0; I.root[v] = -1; }
+                }
+                if (lane == 0) {
+                    isl_flip(I, A);
+                    if (B >= 0) {
+                        if (lb == 1) isl_flip(I, B);
+                        I.mate[A] = (signed char)B; I.ms[A] = (signed char)a; I.mo[A] = (signed char)b;
+                        I.mate[B] = (signed char)A; I.ms[B] = (signed char)b; I.mo[B] = (signed char)a;
+                    } else {
+                        I.mate[A] = MATE_BOUNDARY; I.ms[A] = (signed char)a; I.mo[A] = -1;
+                    }
+                }
+            } else if (lb == 0 && mb >= 0) {
+                if (lane == 0) {   // grow
+                    I.lab[B] = -1; I.tpar[B] = (signed char)A; I.tps[B] = (signed char)b; I.tpo[B] = (signed char)a;
+                    I.root[B] = (signed char)rA;
+                    I.lab[mb] = 1; I.tpar[mb] = (signed char)B; I.tps[mb] = I.ms[mb]; I.tpo[mb] = I.mo[mb];
+                    I.root[mb] = (signed char)rA;
+                }
+            } else {
+                return ISL_FAIL;
+            }
         }
         __syncwarp();
+        if (tops) {
+#pragma unroll
+            for (int h = 0; h < E; h++)
+                if (lane + h * WS < n) top[h] = I.top(lane + h * WS);
+        }
     }
     // result: the duals' sum, the boundary matches' observables, largest radii
     int w = 0;
     unsigned long long o = 0;
-    if (lane < n) {
-        w = yl;
-        X.px()[I.ev[lane]] = mrad;
-        if (I.bpar[lane] < 0 && I.mate[lane] == MATE_BOUNDARY) o = __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[lane]]]);
-    }
-    if ((bal >> lane) & 1u) {
-        const int v = IN + lane;
-        w += I.y[v];
-        if (I.bpar[v] < 0 && I.mate[v] == MATE_BOUNDARY) o ^= __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[v]]]);
+#pragma unroll
+    for (int h = 0; h < E; h++) {
+        const int e = lane + h * WS, v = IN + e;
+        if (e < n) {
+            w += yl[h];
+            X.px()[I.ev[e]] = mrad[h];
+            if (I.bpar[e] < 0 && I.mate[e] == MATE_BOUNDARY) o ^= __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[e]]]);
+        }
+        if ((bal[h] >> lane) & 1u) {
+            w += I.y[v];
+            if (I.bpar[v] < 0 && I.mate[v] == MATE_BOUNDARY) o ^= __ldg(X.g->vobs + X.svtx()[I.ev[I.ms[v]]]);
+        }
     }
     if (X.paths) {
         __syncwarp();
@@ -2854,6 +2922,10 @@ __device__ __forceinline__ int run_island(Fast &X, Isl &I, int c, int size, bool
     if (lane == 0) I.rec = IslRec{o, w, n, nm, ncut, tlast, nx};
     __syncwarp();
     return ISL_OK;
+}
+
+__device__ __noinline__ int run_island_big(Fast &X, Isl<2> &I, int c, int size, bool level1, int lane) {
+    return run_island<2>(X, I, c, size, level1, lane);
 }
 
 // Detection events of the row into svtx (those past cap dropped) and their
@@ -3229,10 +3301,13 @@ __device__ __forceinline__ void fast_small(FastShared<NW> &M) {
     M.f.pcap = M.PS;
 }
 template <int NW>
-__device__ __forceinline__ void fast_setup(const Slab &S, FastShared<NW> &M) {
+__device__ __forceinline__ void fast_setup(const Slab &S, const SlabCaps &caps, FastShared<NW> &M) {
     Fast &X = M.f;
     X.wcum = S.wcum;
     X.recs = reinterpret_cast<IslRec *>(S.wl0);
+    X.spare = reinterpret_cast<char *>(X.recs + caps.kc);
+    X.nspare = caps.wc * 8 - caps.kc * (int)sizeof(IslRec);
+    X.nlist = caps.kc;
     X.list = S.xsrc; X.all = S.xcnt;
     X.aged_t = S.xR; X.aged_c = S.sbeg; X.aged_n = S.scnt;
     X.pa = S.tmpa; X.pb = S.tmpb; X.pd = S.cst2;
@@ -3324,7 +3399,7 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
 // radii reach their distance.  Returns QEC_SHOT_OK or USE_GENERAL.
 template <bool WIN, int NW, bool POOL>
 __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool &P, FastShot &Q, bool busy, int *dg) {
-    Isl &I = M.isl[T.warp()];
+    Isl<1> &I = M.isl[T.warp()];
     const int lane = T.lane, K = Q.K;
     // stage 0: level-1 clusters; 1: islands; 2: islands joined since
     int stage = busy && Q.n1 > 0 ? 0 : 1, round = 0, i = T.warp(), status = QEC_SHOT_OK, pooled = 0;
@@ -3360,14 +3435,27 @@ __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool
             i += NW;
         }
         if (c >= 0) {
-            const int r = run_island(*X, I, c, (int)(X->cw()[c] & 4095u), stage == 0, lane);
+            const int size = (int)(X->cw()[c] & 4095u);
+            int r = run_island<1>(*X, I, c, size, stage == 0, lane);
+            const IslRec *rec = &I.rec;
+            if (r == ISL_BIG) {
+                r = ISL_FAIL;
+                // spare list room of this team's slab, which holds one per warp
+                // in all but the smallest slabs of block-wide teams
+                Isl<2> *const big = reinterpret_cast<Isl<2> *>(M.f.spare) + T.warp();
+                if (reinterpret_cast<char *>(big + 1) <= M.f.spare + M.f.nspare) {
+                    r = run_island_big(*X, *big, c, size, stage == 0, lane);
+                    if (r == ISL_BIG) r = ISL_FAIL;
+                    rec = &big->rec;
+                }
+            }
             if (lane == 0) {
                 if (r == ISL_OK && stage == 0) {
-                    Q.lev.w += I.rec.w; Q.lev.o ^= I.rec.o; Q.lev.nm += I.rec.nm; Q.lev.nx += I.rec.nx;
-                    Q.lev.tlast = max(Q.lev.tlast, I.rec.tlast);
-                    Q.lmax = max(Q.lmax, I.rec.nm);
+                    Q.lev.w += rec->w; Q.lev.o ^= rec->o; Q.lev.nm += rec->nm; Q.lev.nx += rec->nx;
+                    Q.lev.tlast = max(Q.lev.tlast, rec->tlast);
+                    Q.lmax = max(Q.lmax, rec->nm);
                 } else if (r == ISL_OK) {
-                    X->recs[c] = I.rec;
+                    X->recs[c] = *rec;
                 } else {
                     if (r == ISL_FAIL || stage == 0) X->cnt[F_FAIL] = 1;
                     X->recs[c].size = -1;
@@ -3384,7 +3472,7 @@ __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool
         }
         T.sync();
         i = T.warp();
-        if (M.f.cnt[F_FAIL] || M.f.cnt[F_AGED] > K) status = USE_GENERAL;
+        if (M.f.cnt[F_FAIL] || M.f.cnt[F_AGED] > M.f.nlist) status = USE_GENERAL;
         if (stage == 0) {
             stage = 1;
             if (dg) {
@@ -3397,6 +3485,7 @@ __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool
         }
         if (status != QEC_SHOT_OK) return status;
         const int np1 = M.f.cnt[F_NP];
+        if (np1 > M.f.pcap) return USE_GENERAL;
         if (np1 == Q.np0) return M.f.cnt[F_STOP] ? USE_GENERAL : QEC_SHOT_OK;   // (stopped, having met nothing)
         const int j = fast_join(M.f, np1, Q.n1, Q.n2, round++, T, Q.L.w, Q.L.o);
         if (j != 1) return j == 2 ? USE_GENERAL : QEC_SHOT_OK;
@@ -3587,10 +3676,10 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
                     Team<1> T1;
                     T1.lane = T.lane;
                     FastShared<1> &M1 = reinterpret_cast<FastShared<1> &>(M);
-                    if (T.lane == 0) fast_setup(S, M1);
+                    if (T.lane == 0) fast_setup(S, A.caps, M1);
                     __syncwarp();
                     decode_shot<WIN, 1, false>(A, S, r, true, T1, M1, P, deadline);
-                    if (T.lane == 0) fast_setup(S, M);
+                    if (T.lane == 0) fast_setup(S, A.caps, M);
                 }
                 T.sync();
                 return;
@@ -3642,7 +3731,7 @@ batch_kernel(const __grid_constant__ BatchArgs a) {
         deadline = T.bcast64(t0) + (unsigned long long)a.watchdog_ns;
     }
     if (NW == 1 && threadIdx.x == 0) pool.next = 0;
-    if (T.tid() == 0) fast_setup(S, M);
+    if (T.tid() == 0) fast_setup(S, a.caps, M);
     __syncthreads();
     // a single shot is the work of the first team; otherwise team t starts with
     // item (its place in the block) x blocks + block, so that a small batch
