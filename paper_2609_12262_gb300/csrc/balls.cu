@@ -26,8 +26,8 @@ namespace qec {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int CAP = 512;     // entries of one ball; a larger one is stored to b_1 only, or not at all
-constexpr int HS = 1024;     // hash slots per warp, at most half full (plus one entry per lane)
+constexpr int CAP = 1024;    // entries of one ball; a larger one is stored to b_1 only, or not at all
+constexpr int HS = 2048;     // hash slots per warp, at most half full (plus one entry per lane)
 constexpr int WPB = 4;       // warps per block, one ball at a time each
 constexpr int ALIGN = 16;    // lists start on 128-byte lines
 
@@ -46,8 +46,8 @@ __device__ int grow(const DGraph &g, Ball &B, int v, int R, int lane) {
     for (int i = lane; i < HS; i += 32) { B.key[i] = -1; B.dist[i] = INT_MAX; }
     for (int i = lane; i < HS / 32; i += 32) B.queued[i] = 0;
     __syncwarp();
-    auto home = [](int x) { return ((unsigned)x * 2654435761u) >> 22; };   // HS = 2^10
-    static_assert(HS == 1024, "home slot");
+    auto home = [](int x) { return ((unsigned)x * 2654435761u) >> 21; };   // HS = 2^11
+    static_assert(HS == 2048, "home slot");
     if (lane == 0) {
         const unsigned h = home(v);
         B.key[h] = v;
@@ -105,10 +105,13 @@ __device__ int grow(const DGraph &g, Ball &B, int v, int R, int lane) {
     return -1;
 }
 
-// One warp per detector.  out == NULL: add every list's room to *cursor; else
+// One warp per detector.  out == NULL: add every list's room to *cursor, or with
+// `whole`, once some ball of radius R is too large, only mark cursor[1]; else
 // write the lists and their headers, each list where *cursor stands.
-__global__ void __launch_bounds__(32 * WPB) ball_kernel(DGraph g, int R, unsigned long long *cursor, int4 *hdr, int2 *out) {
-    __shared__ Ball ball[WPB];
+__global__ void __launch_bounds__(32 * WPB) ball_kernel(DGraph g, int R, bool whole, unsigned long long *cursor, int4 *hdr,
+                                                        int2 *out) {
+    extern __shared__ __align__(16) char dyn[];
+    Ball *const ball = reinterpret_cast<Ball *>(dyn);
     const int lane = threadIdx.x & 31;
     Ball &B = ball[threadIdx.x >> 5];
     const int nw = gridDim.x * WPB;
@@ -116,6 +119,11 @@ __global__ void __launch_bounds__(32 * WPB) ball_kernel(DGraph g, int R, unsigne
     for (int v = blockIdx.x * WPB + (threadIdx.x >> 5); v < g.n; v += nw) {
         bool far = true;
         int n = R > g.b1 ? grow(g, B, v, R, lane) : -1;
+        if (n < 0 && whole && R > g.b1) {
+            if (lane == 0) *(volatile unsigned long long *)(cursor + 1) = 1;
+            return;
+        }
+        if (whole && *(volatile unsigned long long *)(cursor + 1)) return;
         if (n < 0) {   // too many entries: b_1 only
             far = R <= g.b1;
             __syncwarp();
@@ -176,32 +184,40 @@ int grid_for(int n, int wpb) { return (int)std::min<long long>(((long long)n + w
 
 }  // namespace
 
-cudaError_t build_ball_table(DGraph &g, int4 **hdr, int2 **ball) {
+cudaError_t build_ball_table(DGraph &g, bool wide, int4 **hdr, int2 **ball) {
     *hdr = nullptr;
     *ball = nullptr;
-    unsigned long long *cursor = nullptr, total = 0;
+    unsigned long long *cursor = nullptr, total[2] = {0, 0};
     cudaError_t e = cudaMalloc(hdr, sizeof(int4) * (size_t)g.n);
     if (e == cudaSuccess) e = cudaMalloc(&cursor, sizeof(total));
-    // regions of up to two edges' radius stay within four largest weights of
-    // each other; the table's far part is left out where it would be large
-    constexpr unsigned long long FAR_LIMIT = 1ull << 26, LIMIT = (1ull << 31) - 1;   // entries of 8 bytes
-    int R = (int)std::min<long long>(std::max<long long>(g.b1, 4LL * g.wmax + 4), INT_MAX / 4);
+    const int smem = (int)sizeof(Ball) * WPB;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ball_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // Radius: six largest weights (a region of up to four edges' radius and
+    // smaller ones stay within it of each other), for windows of a sliding decode
+    // eight (an event at an open end has no boundary near), where every ball fits
+    // and the table stays below 128 MB; else four, with single balls that are too
+    // large stored to b_1 only; else b_1.  Six instead of four: 3,000 d = 31
+    // windows 0.52 -> 0.37 ms, 1,024 circuit-level d = 13 shots 0.19 -> 0.12 ms.
+    constexpr unsigned long long WIDE_LIMIT = 1ull << 24, FAR_LIMIT = 1ull << 26, LIMIT = (1ull << 31) - 1;   // entries
     const int grid = grid_for(g.n, WPB);
-    for (;;) {
+    int R = g.b1;
+    for (int k : {8, 6, 4, 0}) {
+        if (k == 8 && !wide) continue;
+        if (k > 4 && (unsigned long long)g.n * 256 > WIDE_LIMIT) continue;
+        R = (int)std::min<long long>(std::max<long long>(g.b1, (long long)k * g.wmax + 4), INT_MAX / 4);
         if (e == cudaSuccess) e = cudaMemset(cursor, 0, sizeof(total));
         if (e != cudaSuccess) break;
-        ball_kernel<<<grid, 32 * WPB>>>(g, R, cursor, *hdr, nullptr);
-        e = cudaMemcpy(&total, cursor, sizeof(total), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess || R <= g.b1 || total <= FAR_LIMIT) break;
-        R = g.b1;
+        ball_kernel<<<grid, 32 * WPB, smem>>>(g, R, k > 4, cursor, *hdr, nullptr);
+        e = cudaMemcpy(total, cursor, sizeof(total), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess || (!total[1] && total[0] <= (k > 4 ? WIDE_LIMIT : FAR_LIMIT))) break;
     }
-    if (e == cudaSuccess && total <= LIMIT) {
-        e = cudaMalloc(ball, sizeof(int2) * (size_t)(total + 1));
+    if (e == cudaSuccess && total[0] <= LIMIT) {
+        e = cudaMalloc(ball, sizeof(int2) * (size_t)(total[0] + 1));
         if (e != cudaSuccess) { (void)cudaGetLastError(); *ball = nullptr; e = cudaSuccess; }
     }
     if (e == cudaSuccess && *ball) {
         e = cudaMemset(cursor, 0, sizeof(total));
-        if (e == cudaSuccess) ball_kernel<<<grid, 32 * WPB>>>(g, R, cursor, *hdr, *ball);
+        if (e == cudaSuccess) ball_kernel<<<grid, 32 * WPB, smem>>>(g, R, false, cursor, *hdr, *ball);
     } else if (e == cudaSuccess) {
         e = cudaMemset(*hdr, 0xff, sizeof(int4) * (size_t)g.n);   // no room: no list is complete
     }

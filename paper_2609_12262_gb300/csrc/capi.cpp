@@ -553,7 +553,7 @@ int qec_schedule(int32_t wmax_internal, const qec_params *params, int64_t *d_k, 
     return lev >= 1 ? lev : fail(QEC_EINVAL, "no admissible level-1 parameters");
 }
 
-int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) {
+static int graph_create(const qec_graph_desc *desc, bool window, qec_graph **out) {
     if (!out) return fail(QEC_EINVAL, "out is NULL");
     *out = nullptr;
     if (!desc) return fail(QEC_EINVAL, "desc is NULL");
@@ -700,12 +700,14 @@ int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) {
         ce = cudaMemcpy(g->d_vbnd, vb.data(), sizeof(unsigned long long) * vb.size(), cudaMemcpyHostToDevice);
     d.vbnd = g->d_vbnd;
     d.vobs = g->d_vbnd + n;
-    if (ce == cudaSuccess) ce = qec::build_ball_table(d, &g->d_bhdr, &g->d_ball);
+    if (ce == cudaSuccess) ce = qec::build_ball_table(d, window, &g->d_bhdr, &g->d_ball);
     if (ce == cudaErrorMemoryAllocation) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
     if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "graph tables"); }
     *out = g;
     return QEC_OK;
 }
+
+int qec_graph_create(const qec_graph_desc *desc, qec_graph **out) { return graph_create(desc, false, out); }
 
 int qec_graph_create_window(const qec_graph *stream, int32_t first_detector, int32_t num_detectors,
                             const qec_params *params, qec_graph **out) {
@@ -738,7 +740,7 @@ int qec_graph_create_window(const qec_graph *stream, int32_t first_detector, int
     d.w = w.data();
     d.obs = o.data();
     d.params = params ? params : (stream->has_params ? &stream->params : nullptr);
-    return qec_graph_create(&d, out);
+    return graph_create(&d, true, out);
 }
 
 int qec_graph_destroy(qec_graph *g) {

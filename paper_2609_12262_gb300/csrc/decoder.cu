@@ -1443,7 +1443,7 @@ template <bool COMMIT>
 __device__ unsigned long long walk_table(const Slab &S, const DGraph &g, int src, int4 h, int x, int dx, int lane,
                                          unsigned *carry) {
     unsigned long long o = 0;
-    const int n = h.z + max(h.w, 0);
+    const int n = dx <= g.b1 ? h.z : h.z + max(h.w, 0);   // (nothing on the path is farther than dx)
     int cur = x, dcur = dx;
     for (int step = 0; step < 1 << 22 && cur != src; step++) {
         const int r0 = __ldg(g.row + cur), deg = __ldg(g.row + cur + 1) - r0;
@@ -2174,7 +2174,7 @@ struct __align__(16) IslRec {
 template <int E>
 struct __align__(16) Isl {
     static constexpr int IN = 32 * E;    // events; blossoms are nodes IN .. 2 IN - 1
-    static constexpr int IP = 128 * E;   // pairs
+    static constexpr int IP = E == 1 ? 64 : 256;   // pairs
     static constexpr int IC = 96 * E;    // blossom cycle entries
     static constexpr int LB = 4 + E;     // bits of an event in a key
     int2 pair[IP];        // distance, lower event | higher event << 8
@@ -2201,7 +2201,7 @@ __device__ __forceinline__ bool st_frozen(int st) { return st >= 0 || st == MATE
 enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2, ISL_BIG = 3 };
 constexpr unsigned ISL_ALONE = 1u << 31;
 constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
-enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6, F_FAIL = 7, F_TOTAL = 8 };   // Fast::cnt
+enum { F_NP = 0, F_N1 = 1, F_N2 = 2, F_AGED = 3, F_NPATH = 4, F_STOP = 5, F_NALL = 6, F_FAIL = 7, F_WIDE = 8, F_TOTAL = 12 };   // Fast::cnt
 
 // The shot being decoded by a team.  Per-event arrays, `stride` ints each, in
 // shared memory or, for shots with more events than it holds, in the slab:
@@ -2229,7 +2229,9 @@ struct __align__(16) Fast {
     int *pa, *pb, *pd;                 // matched pairs for the path walks
     char *spare;                       // room for larger islands, nspare bytes
     int nspare, nlist;                 // nlist: room in the lists above
-    int stride, pcap, K, np0, tcut, L, band, paths;
+    int path0, path1;                  // matched pairs of the level-1 clusters run
+    int late;                          // every island has run once: px holds radii
+    int stride, pcap, K, np0, tcut, L, band, cap, paths;
     int cnt[F_TOTAL];
     __device__ __forceinline__ int *svtx() const { return ev; }
     __device__ __forceinline__ int *bd() const { return ev + stride; }
@@ -2241,15 +2243,17 @@ struct __align__(16) Fast {
     __device__ __forceinline__ int rank(int v) const {
         return wcum[v >> 5] + __popc(__ldg(row + (v >> 5)) & ((1u << (v & 31)) - 1u));
     }
-    // as reach_of
-    __device__ __forceinline__ int reach(int b1, int R) const { return R - L + max(R - L, (b1 + 1) >> 1); }
+    // Radius within which the other events have to be known once a ball has
+    // radius R, as reach_of, but taking no other region to be larger than `cap`;
+    // pairs of regions that are both larger are checked at the end (wide_apart).
+    __device__ __forceinline__ int reach(int b1, int R) const { return R - L + min(max(R - L, (b1 + 1) >> 1), cap); }
 };
 
 // Shared memory of a team: the shot, per-event arrays of shots with at most KS
 // events, and one island per warp.
 template <int NW>
 struct __align__(16) FastShared {
-    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + (NW == 1 ? KS / 2 : KS / 4);
+    static constexpr int KS = NW == 1 ? 128 : (NW == TEAM_MID ? 1280 : 2048), PS = KS + KS / 4;
     Fast f;
     unsigned long long pr[PS];
     int ev[6 * KS];
@@ -2287,7 +2291,7 @@ __device__ __forceinline__ void isl_flip(Isl<E> &I, int A) {
 // Event (c): the new blossom N over outer A, B of one tree.  `bal`: blossoms
 // alive before.  Returns false when the cycle pool is full.  One warp.
 template <int E>
-__device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, int b, int n, const unsigned (&bal)[E],
+__device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, int b, int n, unsigned long long bal,
                                          int lane) {
     constexpr int IN = Isl<E>::IN, IC = Isl<E>::IC;
     int ok = 1;
@@ -2335,7 +2339,7 @@ __device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, 
 #pragma unroll 1
     for (int h = 0; h < 2 * E; h++) {
         const int v = lane + h * WS;
-        if (h < E ? v >= n : !((bal[h - E] >> lane) & 1u)) continue;
+        if (h < E ? v >= n : !((bal >> (v - IN)) & 1ull)) continue;
         if (I.bpar[v] >= 0) continue;
         const int tp = I.tpar[v], mt = I.mate[v];
         if (tp >= 0 && I.bpar[tp] == N) I.tpar[v] = (signed char)N;
@@ -2439,12 +2443,12 @@ __device__ __forceinline__ void put_path(Fast &X, int a, int b, int d) {
 
 // The matched pairs of a finished island.  One warp.
 template <int E>
-__device__ __noinline__ void isl_paths(Fast &X, Isl<E> &I, int n, const unsigned (&bal)[E], int lane) {
+__device__ __noinline__ void isl_paths(Fast &X, Isl<E> &I, int n, unsigned long long bal, int lane) {
     constexpr int IN = Isl<E>::IN;
 #pragma unroll 1
     for (int h = 0; h < 2 * E; h++) {
         const int v = lane + h * WS;
-        if (h < E ? v >= n : !((bal[h - E] >> lane) & 1u)) continue;
+        if (h < E ? v >= n : !((bal >> (v - IN)) & 1ull)) continue;
         if (I.bpar[v] >= 0) continue;
         const int mt = I.mate[v], s = I.ms[v];
         if (mt == MATE_BOUNDARY) put_path(X, I.ev[s], -1, I.bd[s]);
@@ -2456,7 +2460,7 @@ __device__ __noinline__ void isl_paths(Fast &X, Isl<E> &I, int n, const unsigned
 #pragma unroll 1
     for (int b = IN; b < 2 * IN; b++) {
         int sp = 0;
-        if (!((bal[(b - IN) >> 5] >> (b & 31)) & 1u) || I.bpar[b] >= 0) continue;
+        if (!((bal >> (b - IN)) & 1ull) || I.bpar[b] >= 0) continue;
         I.ta[sp] = (signed char)b; I.tb[sp++] = I.ms[b];
 #pragma unroll 1
         while (sp > 0) {
@@ -2566,8 +2570,9 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
                 const int sR = xt + X.L - 1;   // explored radius, -1: never
                 const int R = max(sR + X.band, rad + X.L + X.band), q = X.reach(b1, R);
                 sc = sR >= 0 || q > b1;
+                if (R - X.L > X.cap) X.cnt[F_WIDE] = 1;
                 if (!sc) I.xt[e] = R - X.L + 1;
-                far |= sc && (q > 2 * brad - 2 * wmax || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[I.ev[e]]).w < 0);
+                far |= sc && (q > max(brad, min(2 * brad - 2 * wmax, 6 * wmax + 8)) || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[I.ev[e]]).w < 0);
             }
         }
         scan[h] = __ballot_sync(FULL, sc);
@@ -2607,8 +2612,9 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             const unsigned mh = __ballot_sync(FULL, hit);
             if (!mh) continue;
             const bool in = hit && comp[f] == c;
-            // a level-1 cluster stands still unless it is touched
-            const int mt = __reduce_min_sync(FULL, hit && !in && st_frozen(st[f]) ? d - px[f] : INT_MAX);
+            // a level-1 cluster stands still unless it is touched; once every
+            // island has run, their radii then are as good a guess
+            const int mt = __reduce_min_sync(FULL, hit && !in && (X.late || st_frozen(st[f])) ? d - px[f] : INT_MAX);
             if (lane == 0) I.meet[i] = min(I.meet[i], mt);
             int b = 0;
             if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(mh));
@@ -2731,6 +2737,8 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
         yl[h] = mrad[h] = rad[h];
         bal[h] = 0;
     }
+    // (by value to the functions out of line: a reference would put it in memory)
+    auto alive = [&]() { return E == 1 ? (unsigned long long)bal[0] : bal[0] | (unsigned long long)bal[E - 1] << 32; };
     int t = 0, nm = 0, ncut = 0, tlast = 0, nx = level1 ? 1 : 0;
 #pragma unroll 1
     for (int it = 0;; it++) {
@@ -2855,7 +2863,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
 #pragma unroll
                 for (int h = 0; h < E; h++)
                     if (N < 0 && bal[h] != ~0u) N = IN + h * WS + __ffs(~bal[h]) - 1;
-                if (N < 0 || !isl_blossom(I, N, A, a, B, b, n, bal, lane)) return ISL_BIG;
+                if (N < 0 || !isl_blossom(I, N, A, a, B, b, n, alive(), lane)) return ISL_BIG;
 #pragma unroll
                 for (int h = 0; h < E; h++)
                     if (((N - IN) >> 5) == h) bal[h] |= 1u << (N & 31);
@@ -2915,7 +2923,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
     }
     if (X.paths) {
         __syncwarp();
-        isl_paths(X, I, n, bal, lane);
+        isl_paths(X, I, n, alive(), lane);
     }
     w = (int)__reduce_add_sync(FULL, (unsigned)w);
     o = ((unsigned long long)__reduce_xor_sync(FULL, (unsigned)(o >> 32)) << 32) | __reduce_xor_sync(FULL, (unsigned)o);
@@ -3216,7 +3224,7 @@ __device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, bool quick, Te
 // shot is outside the limits.  Every thread of the team calls; ends with a
 // barrier.
 template <int NW>
-__device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int round, Team<NW> T, long long &w,
+__device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<NW> T, long long &w,
                                       unsigned long long &o) {
     int *const list = X.list, *const all = X.all;
     const int K = X.K, np0 = X.np0, nstop = X.cnt[F_STOP];
@@ -3241,7 +3249,7 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int roun
     for (int i = nstop ? T.tid() : n2; i < n2; i += T.NT)
         if (cw[list[K - 1 - i]] == ISL_ALONE) flags |= 2;
     flags = T.template red32<2>(flags);
-    if ((flags & 2) || ((flags & 1) && (round >= 32 || (X.paths && n1)))) {
+    if ((flags & 2) || ((flags & 1) && round >= 32)) {
         T.sync();
         return 2;
     }
@@ -3259,7 +3267,14 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int roun
         if (st[s] == ST_ONE || st[s] == ST_TWO) st[s] = MATE_NONE;   // run from now on
     }
     if (T.tid() == 0) {
-        X.cnt[F_NP] = np0; X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_NPATH] = 0; X.cnt[F_STOP] = 0;
+        X.cnt[F_NP] = np0; X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_STOP] = 0;
+        X.late = 1;
+        // the path list keeps the pairs of the level-1 clusters run
+        int k = 0;
+#pragma unroll 1
+        for (int i = X.path0; i < X.path1; i++, k++) { X.pa[k] = X.pa[i]; X.pb[k] = X.pb[i]; X.pd[k] = X.pd[i]; }
+        X.path0 = 0;
+        X.path1 = X.cnt[F_NPATH] = k;
     }
     T.sync();
 #pragma unroll 1
@@ -3281,6 +3296,39 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n1, int n2, int roun
     }
     T.sync();
     return 1;
+}
+
+// Whether every two regions past the cap of Fast::reach are known to each other
+// or stayed apart: the larger one's reach held the other's event, or their
+// distance (in the ball table of one of them, or beyond it) exceeds the sum of
+// their radii.  One warp.
+__device__ __noinline__ bool wide_apart(Fast &X, int lane) {
+    const DGraph &g = *X.g;
+    const int K = X.K, cap = X.cap, brad = g.brad;
+    const int *const px = X.px(), *const svtx = X.svtx();
+    int mine = -1, n = 0;   // lane j: the j-th wide event
+#pragma unroll 1
+    for (int base = 0; base < K; base += WS) {
+        const bool wide = base + lane < K && px[base + lane] > cap;
+#pragma unroll 1
+        for (unsigned m = __ballot_sync(FULL, wide); m; m &= m - 1, n++)
+            if (lane == n) mine = base + __ffs(m) - 1;
+    }
+    if (n > WS) return false;
+    bool ok = true;
+#pragma unroll 1
+    for (int i = 0; i + 1 < n; i++) {
+        const int a = __shfl_sync(FULL, mine, i), ra = px[a];
+        const int4 h = __ldg(g.bhdr + svtx[a]);
+        const int v = lane > i && lane < n ? svtx[mine] : -1, rb = v < 0 ? 0 : px[mine];
+        if (h.w < 0 || __any_sync(FULL, v >= 0 && ra + rb > brad)) return false;
+#pragma unroll 1
+        for (int k = 0; k < h.z + h.w; k++) {   // one entry for all lanes
+            const int2 e = __ldg(g.ball + (unsigned)h.x + k);
+            if (e.x == v && e.y <= ra + rb && e.y > max(ra, rb) + cap) ok = false;
+        }
+    }
+    return !__any_sync(FULL, !ok);
 }
 
 constexpr int USE_GENERAL = -3;   // the shot is outside the fast path's limits
@@ -3341,8 +3389,10 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
             X.row = row;
             X.L = max(g.wmax, (g.b1 + 1) / 2) + 1;
             X.band = band;
+            X.cap = max(2 * g.wmax + 1, (g.b1 + 1) >> 1);
             X.paths = WIN || g.internal_obs;
             X.tcut = 0;
+            X.late = X.path0 = X.path1 = 0;
             if (!small) {
                 X.ev = reinterpret_cast<int *>(S.wl1);   // 48 K words of 8 bytes
                 X.pr = S.tl;
@@ -3382,6 +3432,10 @@ __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, con
     Q.n2 = X.cnt[F_N2];
     Q.lev = IslRec{0, 0, 0, 0, 0, 0, 0};
     Q.lmax = 0;
+    if (WIN || g.internal_obs) {
+        if (T.tid() == 0) X.path0 = X.path1 = X.cnt[F_NPATH];
+        T.sync();
+    }
     if (dg) {
         Q.L.t1 = T.maxi(Q.L.t1);
         T.sync();
@@ -3474,6 +3528,8 @@ __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool
         i = T.warp();
         if (M.f.cnt[F_FAIL] || M.f.cnt[F_AGED] > M.f.nlist) status = USE_GENERAL;
         if (stage == 0) {
+            if (T.tid() == 0) M.f.path1 = M.f.cnt[F_NPATH];
+            T.sync();
             stage = 1;
             if (dg) {
                 Q.L.t1 = max(Q.L.t1, T.maxi(Q.lev.tlast));
@@ -3486,9 +3542,15 @@ __device__ __forceinline__ int fast_islands(Team<NW> &T, FastShared<NW> &M, Pool
         if (status != QEC_SHOT_OK) return status;
         const int np1 = M.f.cnt[F_NP];
         if (np1 > M.f.pcap) return USE_GENERAL;
-        if (np1 == Q.np0) return M.f.cnt[F_STOP] ? USE_GENERAL : QEC_SHOT_OK;   // (stopped, having met nothing)
-        const int j = fast_join(M.f, np1, Q.n1, Q.n2, round++, T, Q.L.w, Q.L.o);
-        if (j != 1) return j == 2 ? USE_GENERAL : QEC_SHOT_OK;
+        auto stands = [&]() -> int {
+            if (!M.f.cnt[F_WIDE]) return QEC_SHOT_OK;
+            bool ok = true;
+            if (T.warp() == 0) ok = wide_apart(M.f, lane);
+            return T.any(!ok) ? USE_GENERAL : QEC_SHOT_OK;
+        };
+        if (np1 == Q.np0) return M.f.cnt[F_STOP] ? USE_GENERAL : stands();   // (stopped, having met nothing)
+        const int j = fast_join(M.f, np1, Q.n2, round++, T, Q.L.w, Q.L.o);
+        if (j != 1) return j == 2 ? USE_GENERAL : stands();
         Q.n2 = M.f.cnt[F_N2];
         stage = 2;
     }

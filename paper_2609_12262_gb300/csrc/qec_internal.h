@@ -101,7 +101,8 @@ struct BatchArgs {
 // Build the ball table of g (row, slot, n, b1, wmax set) on the current device
 // and set g's bhdr, ball and brad; the arrays are the caller's to free, also
 // after an error.  Detectors whose ball is too large get an incomplete header.
-cudaError_t build_ball_table(DGraph &g, int4 **hdr, int2 **ball);
+// wide: a window of a sliding decode, which takes a larger radius.
+cudaError_t build_ball_table(DGraph &g, bool wide, int4 **hdr, int2 **ball);
 // Seam distances of a commit region (device bitmap) into seam[n].
 cudaError_t build_seam(const DGraph &g, const unsigned *commit, int *seam);
 
