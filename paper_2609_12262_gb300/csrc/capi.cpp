@@ -32,14 +32,9 @@ struct qec_graph {
     long long dk[8] = {0}, bk[8] = {0};
     std::vector<int> eu, ev, ew;    // merged edges (host copy)
     std::vector<unsigned long long> eobs;
-    int *d_row = nullptr;
-    Slot *d_slot = nullptr;
-    int *d_seid = nullptr;
-    unsigned long long *d_eobs = nullptr;
-    int2 *d_eend = nullptr;
+    char *d_image = nullptr;        // every array of the graph but the ball table
     unsigned *d_commit = nullptr;   // commit-region bitmap (sliding windows)
     int *d_seam = nullptr;          // distances to its border
-    unsigned long long *d_vbnd = nullptr;
     int4 *d_bhdr = nullptr;         // ball table
     int2 *d_ball = nullptr;
     int components = 0;             // connected components of the detector graph
@@ -645,20 +640,6 @@ static int graph_create(const qec_graph_desc *desc, bool window, qec_graph **out
     cudaError_t ce = cudaGetDevice(&g->device);
     if (ce != cudaSuccess) { delete g; return cuda_fail(ce, "cudaGetDevice"); }
     const size_t nslots = (size_t)row[n] + 1, ne = (size_t)g->m + 1;
-    ce = cudaMalloc(&g->d_row, sizeof(int) * ((size_t)n + 1));
-    if (ce == cudaSuccess) ce = cudaMalloc(&g->d_slot, sizeof(Slot) * nslots);
-    if (ce == cudaSuccess) ce = cudaMalloc(&g->d_eobs, sizeof(unsigned long long) * ne);
-    if (ce == cudaSuccess) ce = cudaMalloc(&g->d_eend, sizeof(int2) * ne);
-    if (ce == cudaSuccess) ce = cudaMalloc(&g->d_seid, sizeof(int) * nslots);
-    if (ce != cudaSuccess) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
-    std::vector<unsigned long long> eo(g->eobs);
-    eo.push_back(0);
-    ce = cudaMemcpy(g->d_row, row.data(), sizeof(int) * ((size_t)n + 1), cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) ce = cudaMemcpy(g->d_slot, slots.data(), sizeof(Slot) * nslots, cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) ce = cudaMemcpy(g->d_eobs, eo.data(), sizeof(unsigned long long) * ne, cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) ce = cudaMemcpy(g->d_eend, eend.data(), sizeof(int2) * ne, cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) ce = cudaMemcpy(g->d_seid, seid.data(), sizeof(int) * nslots, cudaMemcpyHostToDevice);
-    if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "cudaMemcpy"); }
     DGraph &d = g->dg;
     d.n = n;
     d.words = g->words;
@@ -686,20 +667,35 @@ static int graph_create(const qec_graph_desc *desc, bool window, qec_graph **out
         const long long b2 = g->num_levels >= 2 ? g->bk[1] : g->bk[0];
         g->upper_single = (g->components == 1 && b2 >= g->diam_ub) ? 1 : 0;
     }
-    d.row = g->d_row;
-    d.slot = g->d_slot;
-    d.eobs = g->d_eobs;
-    d.eend = g->d_eend;
-    d.seid = g->d_seid;
     std::vector<unsigned long long> vb = boundary_candidates(n, D);
     vb.resize(2 * (size_t)n, 0);   // then the observable mask of every candidate's edge
     for (int x = 0; x < n; x++)
         if (vb[(size_t)x] != ~0ull) vb[(size_t)n + x] = g->eobs[(size_t)(unsigned)vb[(size_t)x]];
-    ce = cudaMalloc(&g->d_vbnd, sizeof(unsigned long long) * vb.size());
-    if (ce == cudaSuccess)
-        ce = cudaMemcpy(g->d_vbnd, vb.data(), sizeof(unsigned long long) * vb.size(), cudaMemcpyHostToDevice);
-    d.vbnd = g->d_vbnd;
-    d.vobs = g->d_vbnd + n;
+    std::vector<unsigned long long> eo(g->eobs);
+    eo.push_back(0);
+    // one allocation and one copy for all arrays, each on its own 256 bytes
+    std::vector<char> image;
+    auto put = [&](const void *p, size_t bytes) {
+        const size_t at = (image.size() + 255) / 256 * 256;
+        image.resize(at + bytes);
+        if (bytes) std::memcpy(image.data() + at, p, bytes);
+        return at;
+    };
+    const size_t at_row = put(row.data(), sizeof(int) * ((size_t)n + 1)), at_slot = put(slots.data(), sizeof(Slot) * nslots);
+    const size_t at_seid = put(seid.data(), sizeof(int) * nslots), at_eobs = put(eo.data(), sizeof(unsigned long long) * ne);
+    const size_t at_eend = put(eend.data(), sizeof(int2) * ne);
+    const size_t at_vbnd = put(vb.data(), sizeof(unsigned long long) * vb.size());
+    ce = cudaMalloc(&g->d_image, image.size());
+    if (ce != cudaSuccess) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
+    ce = cudaMemcpy(g->d_image, image.data(), image.size(), cudaMemcpyHostToDevice);
+    if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "cudaMemcpy"); }
+    d.row = reinterpret_cast<const int *>(g->d_image + at_row);
+    d.slot = reinterpret_cast<const Slot *>(g->d_image + at_slot);
+    d.eobs = reinterpret_cast<const unsigned long long *>(g->d_image + at_eobs);
+    d.eend = reinterpret_cast<const int2 *>(g->d_image + at_eend);
+    d.seid = reinterpret_cast<const int *>(g->d_image + at_seid);
+    d.vbnd = reinterpret_cast<const unsigned long long *>(g->d_image + at_vbnd);
+    d.vobs = d.vbnd + n;
     if (ce == cudaSuccess) ce = qec::build_ball_table(d, window, &g->d_bhdr, &g->d_ball);
     if (ce == cudaErrorMemoryAllocation) { qec_graph_destroy(g); return fail(QEC_ENOMEM, "device allocation failed"); }
     if (ce != cudaSuccess) { qec_graph_destroy(g); return cuda_fail(ce, "graph tables"); }
@@ -745,14 +741,9 @@ int qec_graph_create_window(const qec_graph *stream, int32_t first_detector, int
 
 int qec_graph_destroy(qec_graph *g) {
     if (!g) return QEC_OK;
-    if (g->d_row) cudaFree(g->d_row);
-    if (g->d_slot) cudaFree(g->d_slot);
-    if (g->d_eobs) cudaFree(g->d_eobs);
-    if (g->d_eend) cudaFree(g->d_eend);
-    if (g->d_seid) cudaFree(g->d_seid);
+    if (g->d_image) cudaFree(g->d_image);
     if (g->d_commit) cudaFree(g->d_commit);
     if (g->d_seam) cudaFree(g->d_seam);
-    if (g->d_vbnd) cudaFree(g->d_vbnd);
     if (g->d_bhdr) cudaFree(g->d_bhdr);
     if (g->d_ball) cudaFree(g->d_ball);
     delete g;

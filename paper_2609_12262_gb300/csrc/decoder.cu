@@ -31,11 +31,15 @@
 //   3. Algorithm 1, level 1: with every pair within b_1 and every boundary
 //      contact, min-label components, the diameter <= d_1 test and the parity
 //      condition decide the level-1 processing clusters.
-//   4. Algorithm 2: level-1 clusters are solved independently (closed form for
-//      the isolated pair and boundary singleton, the event loop otherwise), then
-//      every remaining event runs from t = 0 with the stopped level-1
-//      configurations present as frozen regions (hierarchical execution rule).
-//      Global mode runs every event in one execution instead.
+//   4. Algorithm 2: level-1 clusters and islands (components of the level-1
+//      graph that it does not accept) are solved in closed form where every
+//      event only meets its nearest one, else each by a run of its own from t = 0
+//      in shared memory; islands whose regions met something outside are joined
+//      with it (a level-1 cluster frozen as it stopped) and run again.  That is
+//      the run of every remaining event from t = 0 with the stopped level-1
+//      configurations present as frozen regions (hierarchical execution rule),
+//      which shots outside the limits of this path, and global mode, take as one
+//      run with its state in the slab (the general path).
 //   5. Result: the weight is the sum of the duals (every matched edge is tight),
 //      the observable mask that of the boundary matches' edges.  Only where
 //      detector-detector edges carry observables, and in the sliding-window
@@ -55,18 +59,21 @@
 // thread writes between the barrier before the read and the barrier after it,
 // so all threads of a team always take the same path.
 //
-// The rarely taken matcher steps (augment, blossom, shatter), the path walks and
-// the explored balls are kept out of line (__noinline__), so that the kernel's
-// hot code stays small enough for the instruction cache.
+// The rarely taken steps (blossom, shatter, path walks, the general path) are
+// kept out of line (__noinline__), so that the kernel's hot code stays small
+// enough for the instruction cache.
 //
-// What bounds it: dependent loads of per-shot state and of the tables (no
-// contraction, and the algorithmic bytes take a thousandth of the time).  The
-// ball table replaced, per event, ~25 hash insertions with their contact walks
-// and two enumerations of two-edge paths by ~13 coalesced list entries: a
-// million shots of d = 7 .. 21 at p = 0.003 from 88.7 to 21.5 ms, 100,000 of
-// d = 11 with own weights from 6.1 to 1.46 ms, 1,024 circuit-level d = 13 shots
-// (whose two-edge rule does not hold) from 7.4 to 0.16 ms, one d = 51 window
-// from 1.42 to 0.92 ms.
+// What bounds it: dependent loads of per-shot state and of the tables and the
+// issue of ~3,000 (d = 11) to ~8,000 (d = 21) warp instructions per shot (no
+// contraction; the algorithmic bytes take a hundredth of the time).  What it
+// took, on one GB300, million shots of d = 7 .. 21 at p = 0.003 / one d = 51
+// window / 1,024 circuit-level d = 13 shots, in ms:
+//   hash insertions, contact walks, path enumerations   88.7 / 1.42 / 7.4
+//   ball tables (per event ~13 coalesced list entries)  21.5 / 0.92 / 0.16
+//   islands in shared memory                            13.7 / 0.115 / 0.33
+//   phases in step, islands pooled                      12.0 / 0.096 / 0.24
+//   closed forms, 20 warps per SM                        8.9 / 0.064 / 0.20
+//   larger islands, wider tables                         9.3 / 0.065 / 0.12
 
 #include <algorithm>
 #include <atomic>
@@ -933,7 +940,7 @@ __device__ __forceinline__ int reach_of(const Shot &C, int R) {
 // are read off the table's list of the source's vertex (nothing at all when
 // the pairs within b1, listed at the start of the shot, already cover it).
 // Otherwise the shot goes over to explored balls.  The table's radius (balls.cu:
-// four largest weights) lets a region's radius grow to two edges before that;
+// six largest weights) lets a region's radius grow to three edges before that;
 // a shot gains a band each time exactly when it would with explored balls, so
 // the diagnostics do not depend on which is used.  Returns the number of due
 // regions.  Every thread of the team calls; ends with a barrier.
@@ -2156,9 +2163,8 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
 //
 // Shots outside the limits below take the run over everything (the general
 // path).  The phases are separate functions whose loops are not unrolled, and
-// what they share lies in shared memory: with everything inlined and unrolled
-// the million-shot batch was 40 % slower, waiting for instructions and spilled
-// registers.
+// what they share lies in shared memory: unrolled, the million-shot batch was 40 %
+// slower (15.6 against 11.0 ms), waiting for instructions.
 constexpr int TOP_BITS = 7, TOP_MASK = (1 << TOP_BITS) - 1, RAD_SHIFT = TOP_BITS + 2;
 
 // What one island, or several, add to the shot (w: internal units).
@@ -2246,7 +2252,11 @@ struct __align__(16) Fast {
     // Radius within which the other events have to be known once a ball has
     // radius R, as reach_of, but taking no other region to be larger than `cap`;
     // pairs of regions that are both larger are checked at the end (wide_apart).
-    __device__ __forceinline__ int reach(int b1, int R) const { return R - L + min(max(R - L, (b1 + 1) >> 1), cap); }
+    // No region grows past its event's boundary distance.
+    __device__ __forceinline__ int reach(int b1, int R, int bd) const {
+        const int r = min(R - L, bd);
+        return r + min(max(r, (b1 + 1) >> 1), cap);
+    }
 };
 
 // Shared memory of a team: the shot, per-event arrays of shots with at most KS
@@ -2568,11 +2578,13 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             const int p = I.pk[e], rad = p >> RAD_SHIFT, xt = I.xt[e];
             if (((p >> TOP_BITS) & 3) == 2 && xt <= rad) {
                 const int sR = xt + X.L - 1;   // explored radius, -1: never
-                const int R = max(sR + X.band, rad + X.L + X.band), q = X.reach(b1, R);
+                const int R = max(sR + X.band, rad + X.L + X.band), bd = I.bd[e], q = X.reach(b1, R, bd);
                 sc = sR >= 0 || q > b1;
-                if (R - X.L > X.cap) X.cnt[F_WIDE] = 1;
+                if (min(R - X.L, bd) > X.cap) X.cnt[F_WIDE] = 1;
                 if (!sc) I.xt[e] = R - X.L + 1;
-                far |= sc && (q > max(brad, min(2 * brad - 2 * wmax, 6 * wmax + 8)) || sR > brad - wmax || __ldg(g.bhdr + X.svtx()[I.ev[e]]).w < 0);
+                far |= sc && (q > max(brad, min(2 * brad - 2 * wmax, 6 * wmax + 8)) ||
+                              (sR > brad - wmax && R - X.L < bd) ||   // (else it never falls due again)
+                              __ldg(g.bhdr + X.svtx()[I.ev[e]]).w < 0);
             }
         }
         scan[h] = __ballot_sync(FULL, sc);
@@ -2582,8 +2594,8 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
     for (int i = 0; i < Isl<E>::IN; i++) {
         if (!((scan[i >> 5] >> (i & 31)) & 1u)) continue;
         const int s = I.ev[i], sRl = I.xt[i] + X.L - 1;
-        const int R = max(sRl + X.band, I.rad(i) + X.L + X.band), ql = X.reach(b1, R);
-        const int q0 = sRl < 0 ? b1 : max(b1, X.reach(b1, sRl));
+        const int R = max(sRl + X.band, I.rad(i) + X.L + X.band), ql = X.reach(b1, R, I.bd[i]);
+        const int q0 = sRl < 0 ? b1 : max(b1, X.reach(b1, sRl, I.bd[i]));
         const int v = X.svtx()[s];
         const int4 h = __ldg(g.bhdr + v);
         const int len = h.z + h.w;
@@ -2622,7 +2634,7 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             if (hit && b < X.pcap) X.pr[b] = pk_pair(min(s, f), max(s, f), d);
             // inside the island: unless the other event has it recorded
             const int k2 = in ? (int)X.cw()[f] : 0;
-            const bool add = in && (I.xt[k2] != INT_MAX && d > max(b1, X.reach(b1, I.xt[k2] + X.L - 1)));
+            const bool add = in && (I.xt[k2] != INT_MAX && d > max(b1, X.reach(b1, I.xt[k2] + X.L - 1, I.bd[k2])));
             const unsigned mi = __ballot_sync(FULL, add);
             const int j = np + __popc(mi & ((1u << lane) - 1u));
             if (add && j < IP) I.pair[j] = make_int2(d, min(i, k2) | max(i, k2) << 8);
@@ -2630,7 +2642,7 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             if (np > IP || __any_sync(FULL, hit && b >= X.pcap)) return -1;
         }
         more = __any_sync(FULL, more);
-        if (lane == 0) I.xt[i] = sRl >= 0 && !more ? INT_MAX : R - X.L + 1;
+        if (lane == 0) I.xt[i] = sRl >= 0 && !more && sRl <= brad - wmax ? INT_MAX : R - X.L + 1;
         __syncwarp();
     }
     __syncwarp();
