@@ -1012,6 +1012,7 @@ static int decode_common(const qec_graph *const *graphs, int32_t num_graphs, con
         a.slab_bytes = w.slab_bytes;
         a.caps = w.caps;
         a.pass = 0;
+        a.defer = team == 1;
         if (team > 1) ce = qec::launch_batch(a, (int)nteams, 32 * team, s, team);
         else ce = qec::launch_batch(a, (int)(nwarps / wpb), 32 * wpb, s);
         if (ce != cudaSuccess) return cuda_fail(ce, "kernel launch");
@@ -1019,7 +1020,8 @@ static int decode_common(const qec_graph *const *graphs, int32_t num_graphs, con
         a.slab_bytes = w.slab_bytes2;
         a.caps = w.caps2;
         a.pass = 1;
-        ce = qec::launch_batch(a, (int)nwarps2, team > 1 ? 32 * team : 32, s, team);
+        const int team2 = team > 1 ? team : qec::TEAM_BIG;
+        ce = qec::launch_batch(a, (int)std::min<long long>(nwarps2, num_shots), 32 * team2, s, team2);
         if (ce != cudaSuccess) return cuda_fail(ce, "kernel launch");
     }
     if (!capturing) {

@@ -3772,7 +3772,9 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
         if (has) status = st == QEC_SHOT_OK ? fast_end<WIN, NW>(A, S, *r.g, r.row, T, M, Q, w, o, r.dg) : st;
     }
     if (!busy) return;
-    if (status == USE_GENERAL) {
+    if (status == USE_GENERAL && NW == 1 && A.defer && A.pass == 0) {
+        status = -1;   // left to the blocks of the overflow pass
+    } else if (status == USE_GENERAL) {
         T.sync();
         status = decode_general<WIN, NW>(A, S, *r.g, r.row, T, deadline, w, o, r.dg);
     }

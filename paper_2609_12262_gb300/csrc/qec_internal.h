@@ -89,6 +89,11 @@ struct BatchArgs {
     // change to a failure, and obs_out / w_out are not written
     unsigned long long *cobs;
     unsigned *carry;
+    // one-warp main pass: shots outside the fast path's limits go to the
+    // overflow pass, which the caller launches with TEAM_BIG warps per shot (one
+    // of them takes a warp about a millisecond, in which the rest of the batch is
+    // long done)
+    int defer;
     // multi-warp teams: a shot with fewer detection events than this is
     // decoded by the team's first warp alone (0 or 1: always by the whole team)
     int team_split;

@@ -193,13 +193,15 @@ cudaError_t launch_slot(qec_stream *st, Slot &s) {
         const int wpb = 4;
         int warps = std::min(st->nwarps, (s.n + 0));
         warps = (warps + wpb - 1) / wpb * wpb;
+        a.defer = 1;
         if ((e = qec::launch_batch(a, warps / wpb, 32 * wpb, s.cs))) return e;
     }
     a.slabs = s.slabs2;
     a.slab_bytes = st->sb2;
     a.caps = st->caps2;
     a.pass = 1;
-    if ((e = qec::launch_batch(a, st->nwarps2, team > 1 ? 32 * team : 32, s.cs, team))) return e;
+    const int team2 = team > 1 ? team : qec::TEAM_BIG;
+    if ((e = qec::launch_batch(a, std::min(s.n, st->nwarps2), 32 * team2, s.cs, team2))) return e;
     return cudaEventRecord(s.ev, s.cs);
 }
 

@@ -1,6 +1,6 @@
-"""The decoder's ball table at the edges of its range, against the oracle:
-events far apart (regions that grow past the table's radius, so that the shot
-goes over to explored balls), level-1 radii below, at and beyond what a list
+"""The decoder's ball table and islands at the edges of their range, against the
+oracle: events far apart (regions that grow past the table's radius, so that the
+shot goes over to explored balls), islands past one and two events per lane, level-1 radii below, at and beyond what a list
 holds, circuit-level weights, and both execution modes, for every team size.
 Results are whole numbers and must be equal.  Needs a GB300."""
 
@@ -30,6 +30,10 @@ CASES = [
     ("d13_p01", rotated_surface_code(13, 13, 0.01), None, "sampled"),
     ("circuit_d9", rotated_surface_code_circuit(9, 9, 0.002), None, "sampled"),
     ("circuit_d7_far", rotated_surface_code_circuit(7, 7, 0.001), None, "far"),
+    # islands of more events than a warp has lanes, of more than two per lane,
+    # and batches whose other shots leave them to the overflow pass
+    ("circuit_d13_dense", rotated_surface_code_circuit(13, 13, 0.0025), None, "sampled"),
+    ("d15_dense", rotated_surface_code(15, 15, 0.012), None, "sampled"),
     # 3 and 6 edges: more vertices within b_1 than a first level-1 ball was
     # ever enumerated for; 9 edges: more than a list of the table holds
     ("b1_3_edges", rotated_surface_code(13, 13, 0.001), (1, 3), "sampled"),
