@@ -395,7 +395,8 @@ typedef struct {
 /* Create a serving stream on the current device.  device_budget_bytes bounds
  * the device memory of the stream's in-flight slots (each slot: scratch for
  * 2 warps per SM with room for 512 detection events per window, an overflow
- * pass for larger windows, and window/result buffers); it must hold at least
+ * pass for larger windows and those that need the general path, and
+ * window/result buffers); it must hold at least
  * two slots (QEC_ENOMEM otherwise) and at most eight are used.  max_inflight
  * (>= 1) bounds the windows admitted (queued or on the GPU) at once.
  * Errors: QEC_EINVAL, QEC_ENOMEM, QEC_ECUDA. */

@@ -64,3 +64,29 @@ def test_ball_table_edges(qd, team, name, pg, level1, kind):  # noqa: F811
                     assert tuple(int(D[i, COL[f]]) for f in FIELDS) == tuple(int(r[f]) for f in FIELDS), (name, mode, i)
     finally:
         qd.set_tuning(team_warps=-1)
+
+
+# windows of a sliding decode at rates where events at the open end stand alone,
+# with boundaries within (d = 13) and beyond (d = 21) the table's reach
+WINDOWS = [("d13", 13, 26, 13, dict(p=0.003)), ("d15", 15, 30, 15, dict(p=0.003)), ("d15_short", 15, 18, 9, dict(p=0.001)),
+           ("d21", 21, 42, 21, dict(p=0.001)), ("d17_weights", 17, 34, 17, dict(p_range=(0.001, 0.004), p_seed=3))]
+
+
+@pytest.mark.parametrize("team", [1, 16])
+@pytest.mark.parametrize("name,d,W,C,kw", WINDOWS, ids=[c[0] for c in WINDOWS])
+def test_window_tables(qd, team, name, d, W, C, kw):  # noqa: F811
+    import torch
+    from oracle.window import sliding_window_decode
+    from paper_2609_12262_gb300.window import SlidingWindow
+    pg = rotated_surface_code(d, W + C, **kw)
+    shots = 10
+    syn = sample_shots(pg, shots, 9)[0]
+    qd.set_tuning(team_warps=team)
+    try:
+        dec = SlidingWindow(qd.Graph.from_phys(pg), pg.nz, W, C)
+        obs, st = dec.decode(torch.from_numpy(syn.view(np.int32).reshape(-1)).cuda(), shots)
+        torch.cuda.synchronize()
+        ro, rs = sliding_window_decode(pg, syn, W, C)
+        assert np.array_equal(st.cpu().numpy(), rs) and np.array_equal(qd.to_uint64(obs), ro)
+    finally:
+        qd.set_tuning(team_warps=-1)
