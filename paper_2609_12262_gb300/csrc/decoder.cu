@@ -2855,6 +2855,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
         bool tops = false;   // the events' top nodes changed
         if (kind == EV_IMPLODE) {
             const int B = I.top(lo);
+            __syncwarp();   // every lane has read it before the shatter moves the event to another node
             isl_shatter(I, B, n, lane);
 #pragma unroll
             for (int h = 0; h < E; h++)

@@ -1,0 +1,32 @@
+"""The kernels on the host emulation of tests/emulation.py (no GPU), against the oracle.
+
+The lanes of a warp run in any order between two warp wide operations there: results that need a wait that is not
+written down differ, fault or never end.  Results are whole numbers and must be equal."""
+
+import pytest
+
+from tests import emulation
+
+DECODE = """
+import numpy as np, torch
+from oracle import OracleGraph
+from synth import *
+from tests import emulation
+q = emulation.load(order=%(order)d)
+def check(pg, shots, mode, team, split=1, seed=5, **kw):
+    g, og = q.Graph.from_phys(pg, **kw), OracleGraph.from_phys(pg, **kw)
+    syn, _ = sample_shots(pg, shots, seed)
+    q.set_tuning(team_warps=team, team_split_events=split)
+    o, w, s, _ = q.decode_batch_ex([g], torch.from_numpy(syn.view(np.int32).reshape(-1)), mode=mode, diag=False,
+                                   stream=emulation.STREAM)
+    rw, ro, rs = og.decode_bitmaps(syn, mode)
+    assert np.array_equal(s.numpy(), rs) and np.array_equal(w.numpy(), rw) and np.array_equal(q.to_uint64(o), ro)
+"""
+
+
+@pytest.mark.parametrize("order", [0, 1, 2], ids=["ascending", "descending", "random"])
+def test_islands_with_blossoms_in_any_lane_order(order):
+    emulation.run(DECODE % {"order": order} + """
+check(rotated_surface_code(11, 11, 0.01), 60, "hier", 1)
+check(rotated_surface_code(9, 9, p_range=(0.001, 0.02), p_seed=1), 60, "hier", 4)
+""", timeout=300)
