@@ -1387,7 +1387,7 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
             // the blossom is read by every thread before any thread's shatter
             // loop rewrites the stop pointers
             const int B = S.src[lo].stop;
-            if constexpr (NW > 1) T.sync();
+            T.sync();
             ev_shatter(S, C, B, T);
         } else if (kind == EV_BOUNDARY) {
             ev_augment(S, C, S.src[lo].stop, lo, -1, -1, T, nhi);
@@ -1403,7 +1403,7 @@ __device__ int run_matcher(const Slab &S, Shot &C, Team<NW> &T, int &nhi) {
             else if (lb == 0 && S.mate[B] >= 0) act = 2;
             // every thread has read the state it dispatches on before any
             // thread changes it
-            if constexpr (NW > 1) T.sync();
+            T.sync();
             if (act == 0) ev_blossom(S, C, A, a, B, b, T, nhi);
             else if (act == 1) ev_augment(S, C, A, a, B, b, T, nhi);
             else if (act == 2) {

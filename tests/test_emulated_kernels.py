@@ -30,3 +30,12 @@ def test_islands_with_blossoms_in_any_lane_order(order):
 check(rotated_surface_code(11, 11, 0.01), 60, "hier", 1)
 check(rotated_surface_code(9, 9, p_range=(0.001, 0.02), p_seed=1), 60, "hier", 4)
 """, timeout=300)
+
+
+@pytest.mark.parametrize("order", [0, 1, 2], ids=["ascending", "descending", "random"])
+def test_general_path_of_one_warp_in_any_lane_order(order):
+    emulation.run(DECODE % {"order": order} + """
+check(rotated_surface_code(7, 7, 0.01), 40, "global", 1)
+check(rotated_surface_code(9, 9, p_range=(0.001, 0.02), p_seed=1), 20, "global", 1)
+check(rotated_surface_code(7, 7, 0.01), 20, "global", 16, split=20)   # the first warp of a block
+""", timeout=300)
