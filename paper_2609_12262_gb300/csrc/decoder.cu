@@ -2281,17 +2281,19 @@ template <int E>
 __device__ __forceinline__ int isl_child_of(const Isl<E> &I, int B, int leaf) {
     int v = leaf;
 #pragma unroll 1
-    while (v >= 0 && I.bpar[v] != B) v = I.bpar[v];
+    for (int k = 0; k < I.IN && v >= 0 && I.bpar[v] != B; k++) v = I.bpar[v];
     return v;
 }
 
-// flip matches along the tree path from outer A to its root (lane 0)
+// flip matches along the tree path from outer A to its root (lane 0; I.err when
+// the path is no tree path)
 template <int E>
 __device__ __forceinline__ void isl_flip(Isl<E> &I, int A) {
     int v = A;
 #pragma unroll 1
-    while (I.tpar[v] >= 0) {
+    for (int k = 0; I.tpar[v] >= 0; k++) {
         const int i = I.tpar[v], o = I.tpar[i];
+        if (o < 0 || k >= I.IN) { I.err = 1; return; }
         I.mate[i] = (signed char)o; I.ms[i] = I.tps[i]; I.mo[i] = I.tpo[i];
         I.mate[o] = (signed char)i; I.ms[o] = I.tpo[i]; I.mo[o] = I.tps[i];
         v = o;
@@ -2299,7 +2301,8 @@ __device__ __forceinline__ void isl_flip(Isl<E> &I, int A) {
 }
 
 // Event (c): the new blossom N over outer A, B of one tree.  `bal`: blossoms
-// alive before.  Returns false when the cycle pool is full.  One warp.
+// alive before.  Returns false when the cycle pool is full or the paths do not
+// meet.  One warp.
 template <int E>
 __device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, int b, int n, unsigned long long bal,
                                          int lane) {
@@ -2308,13 +2311,13 @@ __device__ __noinline__ bool isl_blossom(Isl<E> &I, int N, int A, int a, int B, 
     if (lane == 0) {
         int na = 0, nb = 0;
 #pragma unroll 1
-        for (int v = A; v >= 0; v = I.tpar[v]) I.ta[na++] = (signed char)v;
+        for (int v = A; v >= 0 && na < 2 * IN; v = I.tpar[v]) I.ta[na++] = (signed char)v;
 #pragma unroll 1
-        for (int v = B; v >= 0; v = I.tpar[v]) I.tb[nb++] = (signed char)v;
+        for (int v = B; v >= 0 && nb < 2 * IN; v = I.tpar[v]) I.tb[nb++] = (signed char)v;
 #pragma unroll 1
         while (na > 1 && nb > 1 && I.ta[na - 2] == I.tb[nb - 2]) { na--; nb--; }
         const int Lc = I.ta[na - 1], m = na + nb - 1, cb = I.nc;
-        if (cb + m > IC) {
+        if (cb + m > IC || Lc != I.tb[nb - 1]) {
             ok = 0;
         } else {
             I.nc = cb + m;
@@ -2431,17 +2434,12 @@ __device__ __noinline__ void isl_shatter(Isl<E> &I, int B, int n, int lane) {
 template <int E>
 __device__ __forceinline__ int isl_dist(const Isl<E> &I, int a, int b) {
     int d = I.rad(a) + I.rad(b);
+    int B = I.bpar[a];
 #pragma unroll 1
-    for (int B = I.bpar[a]; B >= 0; B = I.bpar[B]) {
-        int x = I.bpar[b];
+    for (int k = 0; k < I.IN && B >= 0; k++, B = I.bpar[B])   // at most IN blossoms hold an event
+        if (isl_child_of(I, B, b) >= 0) break;
 #pragma unroll 1
-        while (x >= 0 && x != B) x = I.bpar[x];
-        if (x == B) {
-#pragma unroll 1
-            for (; B >= 0; B = I.bpar[B]) d -= 2 * I.y[B];
-            break;
-        }
-    }
+    for (int k = 0; k < I.IN && B >= 0; k++, B = I.bpar[B]) d -= 2 * I.y[B];
     return d;
 }
 
@@ -2473,10 +2471,11 @@ __device__ __noinline__ void isl_paths(Fast &X, Isl<E> &I, int n, unsigned long 
         if (!((bal >> (b - IN)) & 1ull) || I.bpar[b] >= 0) continue;
         I.ta[sp] = (signed char)b; I.tb[sp++] = I.ms[b];
 #pragma unroll 1
-        while (sp > 0) {
+        for (int k = 0; k < 2 * IN && sp > 0; k++) {   // each node of the blossom once
             const int v = I.ta[--sp], e = I.tb[sp];
             if (v < IN) continue;
             const int len = I.cl[v - IN], cb = I.cb[v - IN], c0 = isl_child_of(I, v, e);
+            if (sp + len > 2 * IN) break;
             int i0 = 0;
 #pragma unroll 1
             for (int j = 0; j < len; j++) if (I.cn[cb + j] == c0) i0 = j;
@@ -2860,7 +2859,6 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
 #pragma unroll
             for (int h = 0; h < E; h++)
                 if (((B - IN) >> 5) == h) bal[h] &= ~(1u << (B & 31));
-            if (I.err) return ISL_FAIL;
             tops = true;
         } else {
             int a = lo, b = hi, A = I.top(a), B = -1;
@@ -2912,6 +2910,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
             }
         }
         __syncwarp();
+        if (I.err) return ISL_FAIL;
         if (tops) {
 #pragma unroll
             for (int h = 0; h < E; h++)

@@ -7,6 +7,7 @@ import os
 import re
 import subprocess
 import sys
+import tempfile
 import types
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -88,6 +89,19 @@ def build(csrc=CSRC, out=None, flags=()):
     for o in objs:
         os.remove(o)
     return lib
+
+
+def program(code, timeout=60):
+    """Compile a C++ program around the translated decoder.cu (its internal names are in reach) and run it."""
+    with open(os.path.join(CSRC, "decoder.cu")) as r:
+        text = _translate(r.read())
+    with tempfile.TemporaryDirectory() as tmp:
+        src, exe = os.path.join(tmp, "program.cpp"), os.path.join(tmp, "program")
+        with open(src, "w") as w:
+            w.write(text + code)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-U_FORTIFY_SOURCE", "-I", HOST, "-I", CSRC, src,
+                        os.path.join(HOST, "runtime.cpp"), "-o", exe, "-lpthread"], check=True)
+        return subprocess.run([exe], timeout=timeout, check=True, capture_output=True, text=True).stdout
 
 
 def load(path=None, order=0, seed=1, sms=1):

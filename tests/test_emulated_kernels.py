@@ -39,3 +39,37 @@ check(rotated_surface_code(7, 7, 0.01), 40, "global", 1)
 check(rotated_surface_code(9, 9, p_range=(0.001, 0.02), p_seed=1), 20, "global", 1)
 check(rotated_surface_code(7, 7, 0.01), 20, "global", 16, split=20)   # the first warp of a block
 """, timeout=300)
+
+
+def test_walks_over_an_island_end_on_a_broken_tree():
+    # two nodes that are each other's tree parent (or blossom), which no event leaves behind: the walk gives up
+    emulation.program("""
+#include <cstdio>
+using namespace qec;
+static Isl<1> I;
+static void clear() {
+    memset(&I, 0, sizeof I);
+    memset(I.tpar, -1, sizeof I.tpar);
+    memset(I.bpar, -1, sizeof I.bpar);
+}
+int main() {
+    clear();
+    I.tpar[0] = 1; I.tpar[1] = 2; I.tpar[2] = 1;
+    isl_flip(I, 0);
+    if (!I.err) return 1;
+    clear();
+    I.bpar[3] = 40; I.bpar[40] = 41; I.bpar[41] = 40; I.bpar[5] = 41;
+    isl_child_of(I, 50, 3);
+    isl_dist(I, 3, 5);
+    clear();
+    I.tpar[0] = 1; I.tpar[1] = 0; I.tpar[6] = 7; I.tpar[7] = 6;
+    static int ok[32];
+    emu::launch(1, 32, [&] { ok[threadIdx.x] = isl_blossom(I, 32, 0, 0, 6, 6, 8, 0, threadIdx.x); });
+    for (int l = 0; l < 32; l++) if (ok[l]) return 2;
+    // and the ordinary case still works: 0 -> inner 1 -> root 2
+    clear();
+    I.tpar[0] = 1; I.tpar[1] = 2; I.tps[1] = 1; I.tpo[1] = 2; I.tps[0] = 0; I.tpo[0] = 1;
+    isl_flip(I, 0);
+    return I.err || I.mate[1] != 2 || I.mate[2] != 1;
+}
+""")
