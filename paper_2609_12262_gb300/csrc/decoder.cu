@@ -2154,7 +2154,11 @@ __device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g
 // the whole state in shared memory, and afterwards every recorded pair that
 // joins two of them is checked: where the largest radii reach its distance, the
 // two are joined (an accepted cluster's events frozen as level 1 left them) and
-// run again.  A pair that can become tight is always recorded: see reach_of.
+// run again.  A pair whose regions meet is always recorded: within b_1 it is
+// listed from the start, beyond it the extensions of the larger of the two
+// regions reach the other's event (Fast::reach) unless both are past
+// Fast::cap, which wide_apart checks.  Since the smaller region need not have it,
+// a record is kept for as long as the island that made it stands.
 //
 // A run over everything costs a scan of all events and pairs per event: a d =
 // 51 window at p = 0.003 (1,170 events, 250 matcher events in 88 islands of at
@@ -3231,8 +3235,8 @@ __device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, bool quick, Te
 
 // What islands met, after they have run: marks the pairs in [np0, np1) whose
 // regions meet, joins their components and lists what has to run (in X.list,
-// from its back) and all islands (in X.all); w, o: what is left of the closed
-// forms.  Returns 0 when nothing met, 1 when something was joined, 2 when the
+// from its back) and all islands (in X.all); of the pairs those that what has to
+// run would not record again are kept.  w, o: what is left of the closed forms.  Returns 0 when nothing met, 1 when something was joined, 2 when the
 // shot is outside the limits.  Every thread of the team calls; ends with a
 // barrier.
 template <int NW>
@@ -3279,7 +3283,7 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<
         if (st[s] == ST_ONE || st[s] == ST_TWO) st[s] = MATE_NONE;   // run from now on
     }
     if (T.tid() == 0) {
-        X.cnt[F_NP] = np0; X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_STOP] = 0;
+        X.cnt[F_N2] = 0; X.cnt[F_NALL] = 0; X.cnt[F_STOP] = 0;
         X.late = 1;
         // the path list keeps the pairs of the level-1 clusters run
         int k = 0;
@@ -3294,17 +3298,42 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<
     T.sync();
     w = 0;
     o = 0;
+    // what an event is part of: 0 a level-1 cluster on its own, 1 an island that
+    // stands as it ran, 2 an island to run
+    auto part = [&](int s) {
+        const int c = comp[s], size = (int)cw[c];
+        if ((st[s] == MATE_BOUNDARY && size == 1) || (st[s] >= 0 && size == 2) || st[s] == ST_RUN) return 0;
+        return X.paths || X.recs[c].size != size ? 2 : 1;
+    };
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
-        const int c = comp[s], size = (int)cw[c];
-        if ((st[s] == MATE_BOUNDARY && size == 1) || (st[s] >= 0 && size == 2)) {
-            add_closed(X, s, st[s], 2 * px[s], w, o);   // (MATE_BOUNDARY is negative)
-        } else if (st[s] == ST_RUN) {
-            // (unchanged: nothing joined it)
-        } else if (s == c) {
+        const int p = part(s);
+        if (p == 0) {
+            if (st[s] != ST_RUN) add_closed(X, s, st[s], 2 * px[s], w, o);   // (MATE_BOUNDARY is negative)
+        } else if (s == comp[s]) {
             all[atomicAdd(&X.cnt[F_NALL], 1)] = s;
-            if (X.paths || X.recs[s].size != size) list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
+            if (p == 2) list[K - 1 - atomicAdd(&X.cnt[F_N2], 1)] = s;
         }
+    }
+    // pairs recorded by what stands stay: the region that recorded one does not
+    // come back to it, and the other, the smaller of the two, may not reach as far.
+    // What runs records its own again.
+    if (T.warp() == 0) {
+        int np = np0;
+#pragma unroll 1
+        for (int base = np0; base < np1; base += WS) {
+            unsigned long long p = 0;
+            bool keep = false;
+            if (base + T.lane < np1) {
+                p = X.pr[base + T.lane];
+                keep = part(pr_lo(p)) != 2 || part(pr_hi(p)) != 2;
+            }
+            const unsigned m = __ballot_sync(FULL, keep);   // (read before any is moved)
+            if (keep) X.pr[np + __popc(m & ((1u << T.lane) - 1u))] = p;
+            np += __popc(m);
+            __syncwarp();
+        }
+        if (T.lane == 0) X.cnt[F_NP] = np;
     }
     T.sync();
     return 1;

@@ -101,7 +101,7 @@ using std::max;
 using std::min;
 
 // ---- runtime calls: one device, every call done when it returns
-enum cudaError_t { cudaSuccess = 0, cudaErrorMemoryAllocation = 2, cudaErrorNotReady = 600 };
+enum cudaError_t { cudaSuccess = 0, cudaErrorInvalidValue = 1, cudaErrorMemoryAllocation = 2, cudaErrorNotReady = 600 };
 typedef void *cudaStream_t;
 typedef void *cudaEvent_t;
 enum cudaStreamCaptureStatus { cudaStreamCaptureStatusNone = 0 };

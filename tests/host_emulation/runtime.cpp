@@ -1,7 +1,6 @@
 // Fibers, warp and block wide operations and launches of the host emulation.
 #include <setjmp.h>
 #include <stdio.h>
-#include <time.h>
 #include <ucontext.h>
 
 #include <algorithm>
@@ -39,7 +38,6 @@ Fiber *self = nullptr;
 jmp_buf sched;
 const std::function<void()> *body = nullptr;
 int order = 0, nthreads = 0, block_here = 0, block_alive = 0, block_acc = 0, block_out = 0;
-long long executed = 0;
 std::mt19937 rng(1);
 std::mutex one;
 
@@ -120,18 +118,13 @@ void run_block() {
 
 char *dynamic_shared() { return reinterpret_cast<char *>(dyn.data()); }
 
-unsigned long long now_ns() {
-    timespec t;
-    clock_gettime(CLOCK_MONOTONIC, &t);
-    return (unsigned long long)t.tv_sec * 1000000000ull + (unsigned long long)t.tv_nsec;
-}
+unsigned long long now_ns() { return 1; }   // (the emulation is slow: no shot runs out of time)
 
 int lane() { return self->tid & 31; }
 
 const unsigned long long *exchange(unsigned mask, unsigned long long v) {
     static unsigned long long alone[32];
     const int l = self->tid & 31;
-    executed++;
     if (mask == 1u << l) {
         alone[l] = v;
         return alone;

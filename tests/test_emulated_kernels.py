@@ -73,3 +73,43 @@ int main() {
     return I.err || I.mate[1] != 2 || I.mate[2] != 1;
 }
 """)
+
+
+# (user weights of the edges between boundary, the named events and boundary; weight and observable of the matching):
+# an island that stands met nothing while its neighbour was small, and is met once that one has been joined and grown
+JOINS = [([[100, 100], [100, 100, 10], [100], [100, 100, 100, 20], [100, 100, 50]], 530, 0),
+         ([[50, 50], [50, 50, 5], [50], [50, 50, 50, 10], [50, 50, 25]], 265, 0),
+         ([[40, 40, 40, 45], [50, 50, 50], [50], [40, 40, 40, 35], [40, 40, 30]], 305, 0)]
+
+JOIN_CODE = """
+def decode(g, events, mode, diag):
+    row = pack_defects(np.asarray(events), g.num_detectors)
+    o, w, s, _ = q.decode_batch_ex([g], torch.from_numpy(row.view(np.int32)), mode=mode, diag=diag, num_shots=1,
+                                   stream=emulation.STREAM)
+    return int(w[0]), int(q.to_uint64(o)[0]), int(s[0])
+pg = rotated_surface_code(13, 13, p_range=(0.001, 0.02), p_seed=1)
+surface = q.Graph.from_phys(pg)
+for team in (1, 4, 16):
+    q.set_tuning(team_warps=team)
+    for diag in (False, True):
+        for segments, weight, obs in %r:
+            u, v, w, o, named, at, n = [], [], [], [], [], -1, sum(map(len, segments)) - 1
+            for segment in segments:
+                for x in segment:
+                    u.append(max(at, 0)), v.append(-1 if at < 0 or at == n - 1 else at + 1)
+                    if at < 0: o.append(1)
+                    else: o.append(0)
+                    w.append(x)
+                    at += 1
+                named.append(at)
+            g = q.Graph(n, u, v, w, o)
+            for mode in ("hier", "global"):
+                got = decode(g, named[:-1], mode, diag)
+                assert got == (weight, obs, 0), (team, diag, mode, segments, got)
+        for events, weight in (([409, 552, 559, 625], 587), ([551, 731, 736, 754], 502), ([55, 115, 139, 157], 541)):
+            assert decode(surface, events, "hier", diag) == (weight, 0, 0), (team, diag, events)
+"""
+
+
+def test_an_island_that_stands_is_met_by_a_joined_one():
+    emulation.run(DECODE % {"order": 0} + JOIN_CODE % (JOINS,))
