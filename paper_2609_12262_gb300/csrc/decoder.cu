@@ -3415,11 +3415,8 @@ struct FastShot {
 template <bool WIN, int NW>
 __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
                                           Team<NW> &T, FastShared<NW> &M, FastShot &Q, int *dg) {
-    // level 1 present, lists complete, first extensions within the listed pairs
+    if (!fast_path_takes(g, A.mode, A.band_factor) || g.words > A.caps.wcap) return USE_GENERAL;
     const int band = max(g.wmax, 1) * max(A.band_factor, 1);
-    if (A.mode != QEC_MODE_HIERARCHICAL || !g.ball || g.brad >= (1 << 26) ||
-        band + max(band, (g.b1 + 1) >> 1) > g.b1 || g.words > A.caps.wcap)
-        return USE_GENERAL;
     Fast &X = M.f;
     bool small = true;
     int K = 0;
@@ -3801,7 +3798,7 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
         if (has) status = st == QEC_SHOT_OK ? fast_end<WIN, NW>(A, S, *r.g, r.row, T, M, Q, w, o, r.dg) : st;
     }
     if (!busy) return;
-    if (status == USE_GENERAL && NW == 1 && A.defer && A.pass == 0) {
+    if (status == USE_GENERAL && NW == 1 && A.defer && A.pass == 0 && fast_path_takes(*r.g, A.mode, A.band_factor)) {
         status = -1;   // left to the blocks of the overflow pass
     } else if (status == USE_GENERAL) {
         T.sync();

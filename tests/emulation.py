@@ -67,7 +67,7 @@ def build(csrc=CSRC, out=None, flags=()):
         return lib
     os.makedirs(out, exist_ok=True)
     tag = ".%d" % os.getpid()
-    jobs, objs = [], []
+    jobs, objs, made = [], [], []
     for f in names + ["runtime.cpp"]:
         src = os.path.join(HOST if f == "runtime.cpp" else csrc, f)
         if f.endswith(".cu"):
@@ -76,6 +76,7 @@ def build(csrc=CSRC, out=None, flags=()):
             src = os.path.join(out, f + tag + ".cpp")
             with open(src, "w") as w:
                 w.write(text)
+            made.append(src)
         objs.append(os.path.join(out, f + tag + ".o"))
         cmd = ["g++", "-std=c++17", "-O1", "-fPIC", "-w", "-U_FORTIFY_SOURCE", "-I", HOST, "-I", csrc, *flags,
                "-c", src, "-o", objs[-1]]
@@ -86,8 +87,8 @@ def build(csrc=CSRC, out=None, flags=()):
             raise RuntimeError(" ".join(cmd) + "\n" + err.decode(errors="replace")[:4000])
     subprocess.run(["g++", "-shared", "-o", lib + tag, *objs, *flags, "-lpthread"], check=True)
     os.replace(lib + tag, lib)
-    for o in objs:
-        os.remove(o)
+    for f in objs + made:
+        os.remove(f)
     return lib
 
 
@@ -112,6 +113,7 @@ def load(path=None, order=0, seed=1, sms=1):
     L.emu_order.argtypes = [ctypes.c_int, ctypes.c_uint]
     L.emu_order(order, seed)
     L.emu_sms(sms)
+    L.emu_barriers.restype = ctypes.c_longlong
     return q
 
 

@@ -37,6 +37,7 @@ std::vector<unsigned long long> dyn;
 Fiber *self = nullptr;
 jmp_buf sched;
 const std::function<void()> *body = nullptr;
+long long barriers = 0;   // block wide barriers passed
 int order = 0, nthreads = 0, block_here = 0, block_alive = 0, block_acc = 0, block_out = 0;
 std::mt19937 rng(1);
 std::mutex one;
@@ -55,6 +56,7 @@ void warp_done(Warp &w, int first) {
 
 void block_done() {
     if (!block_here || block_here != block_alive) return;
+    barriers++;
     block_out = block_acc;
     block_acc = block_here = 0;
     for (int i = 0; i < nthreads; i++) fibers[(size_t)i]->waits = false;
@@ -96,7 +98,9 @@ void run_block() {
     block_alive = nthreads;
     block_here = block_acc = 0;
     std::vector<int> turn((size_t)nthreads);
-    for (int i = 0; i < nthreads; i++) turn[(size_t)i] = order == 1 ? nthreads - 1 - i : i;
+    const bool back = order == 1 || order == 4;
+    const int last_lane = back ? 0 : 31;
+    for (int i = 0; i < nthreads; i++) turn[(size_t)i] = back ? nthreads - 1 - i : i;
     while (block_alive > 0) {
         if (order == 2) std::shuffle(turn.begin(), turn.end(), rng);
         bool ran = false;
@@ -105,6 +109,8 @@ void run_block() {
             if (f->ended || f->waits) continue;
             resume(f);
             ran = true;
+            // one warp at a time: back to the first once a warp's lanes have had their turn
+            if (order >= 3 && (i & 31) == last_lane) break;
         }
         if (!ran) {
             fprintf(stderr, "emulation: block %u waits for ever (%d of %d threads at a barrier)\n", block_idx.x, block_here, block_alive);
@@ -168,10 +174,12 @@ void launch(long long grid, int block, size_t smem, const std::function<void()> 
 }  // namespace emu
 
 extern "C" {
-// 0: lanes in order, 1: last lane first, 2: any order (seeded)
+// 0: lanes in order, 1: last lane first, 2: any order (seeded), 3 and 4: one warp
+// as far as it gets before the next, first or last warp first
 void emu_order(int order, unsigned seed) {
     emu::order = order;
     emu::rng.seed(seed);
 }
 void emu_sms(int n) { emu::sms = n; }
+long long emu_barriers() { return emu::barriers; }
 }

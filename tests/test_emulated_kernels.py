@@ -113,3 +113,20 @@ for team in (1, 4, 16):
 
 def test_an_island_that_stands_is_met_by_a_joined_one():
     emulation.run(DECODE % {"order": 0} + JOIN_CODE % (JOINS,))
+
+
+def test_batches_outside_the_fast_path_stay_with_their_warps():
+    # one block takes what a warp leaves to the second pass, with some hundred barriers per shot; a batch whose every
+    # shot is outside the fast path's limits (by its mode or band) keeps its warps
+    emulation.run(DECODE % {"order": 0} + """
+def barriers(*a, **kw):
+    before = q.lib().emu_barriers()
+    check(*a, **kw)
+    return q.lib().emu_barriers() - before
+pg, shots = rotated_surface_code(7, 7, 0.01), 60
+few = barriers(pg, shots, "hier", 1)
+assert few < 10 * shots, few
+assert barriers(pg, shots, "global", 1) < 10 * shots
+q.set_tuning(band_factor=2)
+assert barriers(pg, shots, "hier", 1) < 10 * shots
+""")
