@@ -2237,10 +2237,11 @@ struct __align__(16) Fast {
     int *list, *all;                   // clusters and islands to run; all islands once some were joined
     int *aged_t, *aged_c, *aged_n;     // bands of regions that came of age: time, island, its size
     int *pa, *pb, *pd;                 // matched pairs for the path walks
+    int *was;                          // after a join: radii of what stands, -1: what runs again
     char *spare;                       // room for larger islands, nspare bytes
     int nspare, nlist;                 // nlist: room in the lists above
     int path0, path1;                  // matched pairs of the level-1 clusters run
-    int late;                          // every island has run once: px holds radii
+    int late;                          // every island has run once, see `was`
     int stride, pcap, K, np0, tcut, L, band, cap, paths;
     int cnt[F_TOTAL];
     __device__ __forceinline__ int *svtx() const { return ev; }
@@ -2566,7 +2567,7 @@ __device__ __noinline__ int far_events(const Fast &X, int v, int q, int lane, in
 // among the shot's pairs, those of the island itself also in I.pair.  Returns
 // the island's pairs, -1 outside the limits, -2 beyond the table.  One warp.
 template <int E>
-__device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np, int lane) {
+__device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np, bool level1, int lane) {
     constexpr int IP = Isl<E>::IP;
     const DGraph &g = *X.g;
     const int b1 = g.b1, brad = g.brad, wmax = g.wmax;
@@ -2627,9 +2628,16 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             const unsigned mh = __ballot_sync(FULL, hit);
             if (!mh) continue;
             const bool in = hit && comp[f] == c;
-            // a level-1 cluster stands still unless it is touched; once every
-            // island has run, their radii then are as good a guess
-            const int mt = __reduce_min_sync(FULL, hit && !in && (X.late || st_frozen(st[f])) ? d - px[f] : INT_MAX);
+            // a level-1 cluster stands still unless it is touched, and so does,
+            // once every island has run, one that does not run again.  (Others'
+            // radii are being written now: they would stop this island, or not, as
+            // the warps happen to be timed.)
+            int rf = -1;
+            if (hit && !in) {
+                if (X.late) rf = X.was[f];
+                else if (st_frozen(st[f]) && !(level1 && st[f] == ST_RUN)) rf = px[f];
+            }
+            const int mt = __reduce_min_sync(FULL, rf >= 0 ? d - rf : INT_MAX);
             if (lane == 0) I.meet[i] = min(I.meet[i], mt);
             int b = 0;
             if (lane == 0) b = atomicAdd(&X.cnt[F_NP], __popc(mh));
@@ -2830,7 +2838,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
                 for (int h = 0; h < E; h++)
                     if (lane + h * WS < n) I.pk[lane + h * WS] = rad[h] << RAD_SHIFT | (lab[h] + 1) << TOP_BITS | top[h];
                 __syncwarp();
-                r = isl_extend(X, I, c, n, np, lane);
+                r = isl_extend(X, I, c, n, np, level1, lane);
                 if (r == -1) return ISL_BIG;
             }
             if (r == -2) {
@@ -3308,6 +3316,7 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<
 #pragma unroll 1
     for (int s = T.tid(); s < K; s += T.NT) {
         const int p = part(s);
+        X.was[s] = p == 2 ? -1 : px[s];
         if (p == 0) {
             if (st[s] != ST_RUN) add_closed(X, s, st[s], 2 * px[s], w, o);   // (MATE_BOUNDARY is negative)
         } else if (s == comp[s]) {
@@ -3400,6 +3409,7 @@ __device__ __forceinline__ void fast_setup(const Slab &S, const SlabCaps &caps, 
     X.list = S.xsrc; X.all = S.xcnt;
     X.aged_t = S.xR; X.aged_c = S.sbeg; X.aged_n = S.scnt;
     X.pa = S.tmpa; X.pb = S.tmpb; X.pd = S.cst2;
+    X.was = S.xcur;
     fast_small(M);
 }
 

@@ -130,3 +130,34 @@ assert barriers(pg, shots, "global", 1) < 10 * shots
 q.set_tuning(band_factor=2)
 assert barriers(pg, shots, "hier", 1) < 10 * shots
 """)
+
+
+def test_the_route_of_a_joined_shot_does_not_depend_on_the_order_of_lanes_or_warps():
+    # b reached its boundary, is joined with x and ends smaller; a is joined with the pair c, d at the same time and
+    # would stop where b's first radius was
+    emulation.run(DECODE % {"order": 0} + """
+u, v, w, o, place = [], [], [], [], {}
+def detector(name=None):
+    if name not in place or name is None:
+        place[name if name else len(place)] = len(place)
+    return place[name] if name else len(place) - 1
+for a, b, length in (("a", "d", 150), ("d", "c", 50), ("c", None, 35), ("a", None, 200), ("a", "b", 230),
+                     ("b", None, 100), ("b", "x", 150), ("x", None, 80)):
+    at, end = detector(a), detector(b) if b else -1
+    while length > 0:
+        nxt = end if length <= 50 else detector()
+        u.append(at), v.append(nxt), w.append(min(length, 50)), o.append(0)
+        at, length = nxt, length - 50
+g = q.Graph(len(place), u, v, w, o)
+row = torch.from_numpy(pack_defects(sorted(place[k] for k in "abcdx"), len(place)).view(np.int32))
+for team in (1, 4, 16):
+    q.set_tuning(team_warps=team)
+    barriers = set()
+    for order in range(5):
+        q.lib().emu_order(order, 7)
+        before = q.lib().emu_barriers()
+        _, weight, status = q.decode_batch([g], row, num_shots=1, stream=emulation.STREAM)
+        barriers.add(q.lib().emu_barriers() - before)
+        assert (int(weight[0]), int(status[0])) == (335, 0), (team, order, weight, status)
+    assert len(barriers) == 1 and max(barriers) < 60, (team, barriers)
+""")
