@@ -258,8 +258,8 @@ int qec_decode_batch_ex(const qec_graph *const *graphs, int32_t num_graphs,
 
 /* Mark the detectors of g's commit region: detector_bitmap is a host array of
  * words_per_shot(g) uint32 words (bit i = detector i), copied before return;
- * NULL removes the region (and waits for the device to be idle).  Errors:
- * QEC_EINVAL, QEC_ENOMEM, QEC_ECUDA. */
+ * NULL removes the region.  Replacing or removing a region waits for the device
+ * to be idle.  Errors: QEC_EINVAL, QEC_ENOMEM, QEC_ECUDA. */
 int qec_graph_set_commit_region(qec_graph *g, const uint32_t *detector_bitmap);
 
 /* Decode one window of a batch of streams (Alg. 1 + Alg. 2, as

@@ -770,7 +770,12 @@ int qec_graph_set_commit_region(qec_graph *g, const uint32_t *detector_bitmap) {
     for (int i = 0; i < g->words; i++) bits[(size_t)i] = detector_bitmap[i];
     if (g->n % 32) bits[(size_t)(g->n / 32)] &= (1u << (g->n % 32)) - 1u;   // detectors only
     for (int i = g->n / 32 + (g->n % 32 ? 1 : 0); i < g->words; i++) bits[(size_t)i] = 0u;
-    if (!g->d_commit) {
+    if (g->d_commit) {
+        // the region and the distances to its border are replaced in place (a
+        // captured decode reads them there): no decode may still be reading either
+        ce = cudaDeviceSynchronize();
+        if (ce != cudaSuccess) return cuda_fail(ce, "cudaDeviceSynchronize");
+    } else {
         ce = cudaMalloc(&g->d_commit, sizeof(unsigned) * (size_t)g->words);
         if (ce != cudaSuccess) { g->d_commit = nullptr; return fail(QEC_ENOMEM, "cudaMalloc"); }
     }

@@ -35,7 +35,7 @@ inline uint4 make_uint4(unsigned x, unsigned y, unsigned z, unsigned w) { return
 
 namespace emu {
 extern dim3 thread_idx, block_idx, block_dim, grid_dim;
-extern int sms;
+extern int sms, syncs;
 char *dynamic_shared();
 unsigned long long now_ns();
 // warp wide: every lane's value, once all lanes of the mask are here
@@ -126,7 +126,7 @@ template <class T> cudaError_t cudaGetSymbolAddress(void **p, T &s) { *p = (void
 inline cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 inline cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 inline cudaError_t cudaDeviceGetAttribute(int *v, int, int) { *v = emu::sms; return cudaSuccess; }
-inline cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+inline cudaError_t cudaDeviceSynchronize() { emu::syncs++; return cudaSuccess; }
 inline cudaError_t cudaGetLastError() { return cudaSuccess; }
 inline const char *cudaGetErrorString(cudaError_t) { return "error"; }
 inline cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = nullptr; return cudaSuccess; }

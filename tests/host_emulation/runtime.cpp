@@ -13,7 +13,7 @@
 namespace emu {
 
 dim3 thread_idx, block_idx, block_dim, grid_dim;
-int sms = 1;
+int sms = 1, syncs = 0;
 
 namespace {
 
@@ -181,5 +181,6 @@ void emu_order(int order, unsigned seed) {
     emu::rng.seed(seed);
 }
 void emu_sms(int n) { emu::sms = n; }
+int emu_syncs() { return emu::syncs; }   // waits for the whole device
 long long emu_barriers() { return emu::barriers; }
 }

@@ -161,3 +161,15 @@ for team in (1, 4, 16):
         assert (int(weight[0]), int(status[0])) == (335, 0), (team, order, weight, status)
     assert len(barriers) == 1 and max(barriers) < 60, (team, barriers)
 """)
+
+
+def test_replacing_a_commit_region_waits_for_the_device():
+    emulation.run(DECODE % {"order": 0} + """
+g = q.Graph.from_phys(rotated_surface_code(5, 5, 0.003))
+region = np.full(g.words, 0xffff, np.uint32)
+g.set_commit_region(region)
+for new in (region * 3, None):
+    before = q.lib().emu_syncs()
+    g.set_commit_region(new)
+    assert q.lib().emu_syncs() == before + 1
+""")
