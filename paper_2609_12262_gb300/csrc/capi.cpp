@@ -882,7 +882,7 @@ static int decode_common(const qec_graph *const *graphs, int32_t num_graphs, con
     for (int i = 0; i < num_graphs; i++) {
         if (!graphs[i]) return fail(QEC_EINVAL, "NULL graph");
         if (graphs[i]->device != dev) return fail(QEC_EINVAL, "graph lives on another device");
-        if (window && !graphs[i]->d_commit) return fail(QEC_EINVAL, "graph has no commit region");
+        if (window && !graphs[i]->dg.commit) return fail(QEC_EINVAL, "graph has no commit region");
         nmax = std::max(nmax, graphs[i]->n);
     }
     qec_tuning tune;

@@ -35,7 +35,7 @@ inline uint4 make_uint4(unsigned x, unsigned y, unsigned z, unsigned w) { return
 
 namespace emu {
 extern dim3 thread_idx, block_idx, block_dim, grid_dim;
-extern int sms, syncs;
+extern int sms, syncs, fail_alloc;
 char *dynamic_shared();
 unsigned long long now_ns();
 // warp wide: every lane's value, once all lanes of the mask are here
@@ -109,6 +109,7 @@ enum { cudaMemcpyHostToDevice, cudaMemcpyDeviceToHost, cudaHostAllocDefault, cud
        cudaStreamNonBlocking, cudaDevAttrMultiProcessorCount, cudaFuncAttributeMaxDynamicSharedMemorySize };
 struct cudaFuncAttributes { int maxThreadsPerBlock; };
 template <class T> cudaError_t cudaMalloc(T **p, size_t n) {
+    if (emu::fail_alloc > 0 && --emu::fail_alloc == 0) return cudaErrorMemoryAllocation;
     *p = (T *)aligned_alloc(256, (n + 256) / 256 * 256);
     if (!*p) return cudaErrorMemoryAllocation;
     if (n < (1u << 20)) memset(*p, 0xa5, n);

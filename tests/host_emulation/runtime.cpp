@@ -13,7 +13,7 @@
 namespace emu {
 
 dim3 thread_idx, block_idx, block_dim, grid_dim;
-int sms = 1, syncs = 0;
+int sms = 1, syncs = 0, fail_alloc = 0;
 
 namespace {
 
@@ -181,6 +181,7 @@ void emu_order(int order, unsigned seed) {
     emu::rng.seed(seed);
 }
 void emu_sms(int n) { emu::sms = n; }
+void emu_fail_alloc(int n) { emu::fail_alloc = n; }   // the n-th allocation from now on fails
 int emu_syncs() { return emu::syncs; }   // waits for the whole device
 long long emu_barriers() { return emu::barriers; }
 }

@@ -173,3 +173,25 @@ for new in (region * 3, None):
     g.set_commit_region(new)
     assert q.lib().emu_syncs() == before + 1
 """)
+
+
+def test_a_commit_region_that_could_not_be_made_is_none():
+    emulation.run(DECODE % {"order": 0} + """
+g = q.Graph.from_phys(rotated_surface_code(5, 5, 0.003))
+region = np.full(g.words, 0xffff, np.uint32)
+rows = torch.ones(g.words, dtype=torch.int32)
+def decode():
+    obs, carry, status = torch.zeros(1, dtype=torch.int64), torch.empty_like(rows), torch.zeros(1, dtype=torch.int32)
+    q.decode_window_batch([g], rows, obs, carry, status, num_shots=1, stream=emulation.STREAM)
+    assert int(status[0]) == 0
+for n in (1, 2):
+    q.lib().emu_fail_alloc(n)
+    for call in (lambda: g.set_commit_region(region), decode):
+        try:
+            call()
+        except q.QecError:
+            continue
+        raise AssertionError(n)
+g.set_commit_region(region)
+decode()
+""")
