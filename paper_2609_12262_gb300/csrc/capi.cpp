@@ -202,16 +202,20 @@ struct PhysKey {
 // Exact distances over detector-detector slots (boundary vertices are leaves,
 // so no path passes through them) from a set of start distances.  Weights are
 // bounded, so the queue is a ring of buckets, one per distance modulo
-// (largest weight + 1); a heap where that ring would be large.
+// (largest weight + 1), with a bit per bucket in use: a run over a long chain of
+// heavy edges passes up to 2^30 distances, 64 empty ones at a time.  A heap where
+// that ring would be large.
 struct Distances {
     const std::vector<int> &row;
     const std::vector<Slot> &slots;
     const int wmax;
     std::vector<std::vector<int>> ring;
+    std::vector<unsigned long long> used;   // bit per bucket
     std::vector<int> order;   // vertices settled by the last run, by distance
 
     Distances(const std::vector<int> &r, const std::vector<Slot> &s, int w) : row(r), slots(s), wmax(w) {
         if (wmax < (1 << 16)) ring.resize((size_t)wmax + 1);
+        used.resize((ring.size() + 63) / 64);
     }
 
     // dist: start distances (LLONG_MAX: none) in, distances out; starts: the
@@ -250,20 +254,41 @@ struct Distances {
         const long long C = (long long)ring.size();
         size_t next = 0, held = 0;
         long long d = 0;
+        auto put = [&](long long nd, int y) {
+            const size_t r = (size_t)(nd % C);
+            ring[r].push_back(y);
+            used[r >> 6] |= 1ull << (r & 63);
+            held++;
+        };
         while (held || next < wait.size()) {
-            if (!held) d = first[next];
+            const long long start = next < wait.size() ? first[next] : LLONG_MAX;
+            d = held ? std::min(start, ahead(d)) : start;
             for (; next < wait.size() && first[next] == d; next++)
-                if (dist[(size_t)wait[next]] == d) { ring[(size_t)(d % C)].push_back(wait[next]); held++; }
-            auto &b = ring[(size_t)(d % C)];
+                if (dist[(size_t)wait[next]] == d) put(d, wait[next]);
+            const size_t r = (size_t)(d % C);
+            auto &b = ring[r];
             for (size_t i = 0; i < b.size(); i++) {   // positive weights: no push into this bucket
                 const int x = b[i];
                 if (dist[(size_t)x] != d) continue;
-                relax(dist, x, [&](long long nd, int y) { ring[(size_t)(nd % C)].push_back(y); held++; });
+                relax(dist, x, put);
             }
             held -= b.size();
             b.clear();
-            d++;
+            used[r >> 6] &= ~(1ull << (r & 63));
         }
+    }
+
+    // the first distance from d on whose bucket is in use (one is)
+    long long ahead(long long d) const {
+        const size_t C = ring.size(), r = (size_t)(d % (long long)C);
+        size_t word = r >> 6;
+        unsigned long long bits = used[word] & (~0ull << (r & 63));
+        for (size_t n = 0; !bits && n <= used.size(); n++) {
+            word = word + 1 < used.size() ? word + 1 : 0;
+            bits = used[word];
+        }
+        const size_t at = word * 64 + (size_t)__builtin_ctzll(bits);
+        return d + (long long)(at >= r ? at - r : at + C - r);
     }
 
     void run_heap(std::vector<long long> &dist, const std::vector<int> &starts) {

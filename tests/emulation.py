@@ -92,16 +92,17 @@ def build(csrc=CSRC, out=None, flags=()):
     return lib
 
 
-def program(code, timeout=60):
-    """Compile a C++ program around the translated decoder.cu (its internal names are in reach) and run it."""
-    with open(os.path.join(CSRC, "decoder.cu")) as r:
+def program(code, source="decoder.cu", timeout=60):
+    """Compile a C++ program around a translated source (its internal names are in reach) and run it."""
+    lib = build()
+    with open(os.path.join(CSRC, source)) as r:
         text = _translate(r.read())
     with tempfile.TemporaryDirectory() as tmp:
         src, exe = os.path.join(tmp, "program.cpp"), os.path.join(tmp, "program")
         with open(src, "w") as w:
             w.write(text + code)
-        subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-U_FORTIFY_SOURCE", "-I", HOST, "-I", CSRC, src,
-                        os.path.join(HOST, "runtime.cpp"), "-o", exe, "-lpthread"], check=True)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-U_FORTIFY_SOURCE", "-I", HOST, "-I", CSRC, src, lib,
+                        "-Wl,-rpath," + os.path.dirname(lib), "-o", exe, "-lpthread"], check=True)
         return subprocess.run([exe], timeout=timeout, check=True, capture_output=True, text=True).stdout
 
 

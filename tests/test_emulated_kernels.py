@@ -195,3 +195,55 @@ for n in (1, 2):
 g.set_commit_region(region)
 decode()
 """)
+
+
+def test_distances_along_chains_of_heavy_edges():
+    # equal to a heap's on random graphs, from one start and from several, and quick where distances are long
+    emulation.program("""
+#include <chrono>
+#include <random>
+static void graph(int n, const std::vector<std::array<int, 3>> &edges, std::vector<int> &row, std::vector<Slot> &slots) {
+    row.assign((size_t)n + 1, 0);
+    for (auto &e : edges) { row[(size_t)e[0] + 1]++; row[(size_t)e[1] + 1]++; }
+    for (int x = 0; x < n; x++) row[(size_t)x + 1] += row[(size_t)x];
+    slots.resize(2 * edges.size() + 1);
+    std::vector<int> at(row);
+    for (auto &e : edges) {
+        slots[(size_t)at[(size_t)e[0]]++] = Slot{e[1], e[2]};
+        slots[(size_t)at[(size_t)e[1]]++] = Slot{e[0], e[2]};
+    }
+}
+int main() {
+    std::mt19937 rng(1);
+    std::vector<int> row;
+    std::vector<Slot> slots;
+    for (int trial = 0; trial < 300; trial++) {
+        const int n = 2 + (int)(rng() % 200), w = 1 + (int)(rng() % (trial % 3 ? 100 : 65535));
+        std::vector<std::array<int, 3>> edges;
+        for (int i = 0; i < n * (int)(1 + rng() % 3); i++) {
+            const int a = (int)(rng() % (unsigned)n), b = (int)(rng() % (unsigned)n);
+            if (a != b) edges.push_back({a, b, 1 + (int)(rng() % (unsigned)w)});
+        }
+        graph(n, edges, row, slots);
+        Distances ring(row, slots, w), heap(row, slots, 1 << 16);
+        std::vector<long long> a((size_t)n, LLONG_MAX), b;
+        std::vector<int> starts;
+        for (int x = 0; x < n; x++)
+            if (rng() % 8 == 0 || x == 0) { a[(size_t)x] = (long long)(rng() % 100000u); starts.push_back(x); }
+        b = a;
+        ring.run(a, starts);
+        heap.run(b, starts);
+        if (a != b) return 1;
+    }
+    const int n = 16000, w = 65534;
+    std::vector<std::array<int, 3>> edges;
+    for (int i = 0; i + 1 < n; i++) edges.push_back({i, i + 1, w});
+    graph(n, edges, row, slots);
+    Distances D(row, slots, w);
+    std::vector<long long> dist((size_t)n);
+    const auto t = std::chrono::steady_clock::now();
+    D.from(0, dist);
+    if (dist[(size_t)n - 1] != (long long)w * (n - 1)) return 2;
+    return std::chrono::duration<double>(std::chrono::steady_clock::now() - t).count() < 0.5 ? 0 : 3;
+}
+""".replace("#include <chrono>", "#include <array>\n#include <chrono>"), source="capi.cpp")
