@@ -3634,8 +3634,12 @@ __device__ __forceinline__ int fast_end(const BatchArgs &A, const Slab &S, const
         }
     }
     const int naged = X.cnt[F_AGED];
-    if (A.max_events < 256LL * K + 4096) {   // a budget set lower: the run over everything counts exactly
-        if ((long long)T.add(Q.lev.nm + Q.lev.nx + ntop + tnx) + naged + n1 + K + 2 > A.max_events) return USE_GENERAL;
+    if (A.max_events < 256LL * K + 4096) {
+        // a budget set lower: unless the events are surely within it, the run over
+        // everything counts exactly.  Each of its runs adds one step that finds no
+        // event; a closed form of n > 1 events stands for at most n events, and as
+        // a level-1 cluster for an extension and that step besides.
+        if ((long long)T.add(Q.lev.nm + Q.lev.nx + ntop + tnx) + naged + n1 + 2 * K + 2 > A.max_events) return USE_GENERAL;
     }
     w_out = T.sum64(Q.L.w + Q.L.wr + Q.lev.w) / 2;
     o_out = T.xor64(Q.L.o ^ Q.L.ro ^ Q.lev.o);

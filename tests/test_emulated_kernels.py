@@ -247,3 +247,22 @@ int main() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - t).count() < 0.5 ? 0 : 3;
 }
 """.replace("#include <chrono>", "#include <array>\n#include <chrono>"), source="capi.cpp")
+
+
+def test_the_event_budget_of_closed_forms():
+    # six level-1 clusters of three events that all reach the boundary: each budget gives the status that the run over
+    # everything gives, which counts 5 steps per cluster and one at the end
+    emulation.run(DECODE % {"order": 0} + """
+u, v, w, o = [], [], [], []
+for c in range(6):
+    for x, y, weight in ((0, 1, 50), (1, 2, 50), (0, 2, 50), (0, None, 10), (1, None, 11), (2, None, 12)):
+        u.append(3 * c + x), v.append(-1 if y is None else 3 * c + y), w.append(weight), o.append(0)
+g = q.Graph(18, u, v, w, o)
+row = torch.from_numpy(pack_defects(list(range(18)), 18).view(np.int32))
+q.set_tuning(team_warps=1)
+for budget in range(1, 70):
+    q.set_tuning(max_events=budget)
+    for diag in (False, True):
+        _, weight, status, _ = q.decode_batch_ex([g], row, num_shots=1, diag=diag, stream=emulation.STREAM)
+        assert int(status[0]) == (q.SHOT_OK if budget >= 31 else q.SHOT_BUDGET_EXCEEDED), (budget, diag)
+""")
