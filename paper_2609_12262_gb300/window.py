@@ -43,11 +43,19 @@ class SlidingWindow:
         self.nz = int(layer_size)
         self.W, self.C = W, C
         self.windows = []
+        u, v, w, o = stream.merged_edges()
+        made = {}   # windows with the same edges and commit region share one graph and its tables
         for a, nl, last in plan(n // self.nz, W, C):
-            g = Graph.window(stream, a * self.nz, nl * self.nz)
-            bits = np.zeros(g.words * 32, np.uint8)
-            bits[:(g.num_detectors if last else C * self.nz)] = 1
-            g.set_commit_region(np.packbits(bits, bitorder="little").view(np.uint32))
+            first, count = a * self.nz, nl * self.nz
+            inside = (u >= first) & (u < first + count) & ((v < 0) | ((v >= first) & (v < first + count)))
+            key = (count, last, (u[inside] - first).tobytes(), np.where(v[inside] < 0, -1, v[inside] - first).tobytes(),
+                   w[inside].tobytes(), o[inside].tobytes())
+            g = made.get(key)
+            if g is None:
+                g = made[key] = Graph.window(stream, first, count)
+                bits = np.zeros(g.words * 32, np.uint8)
+                bits[:(g.num_detectors if last else C * self.nz)] = 1
+                g.set_commit_region(np.packbits(bits, bitorder="little").view(np.uint32))
             self.windows.append((a, nl, last, g))
 
     def decode(self, syndromes, num_streams: int, stream=None):

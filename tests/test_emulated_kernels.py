@@ -266,3 +266,20 @@ for budget in range(1, 70):
         _, weight, status, _ = q.decode_batch_ex([g], row, num_shots=1, diag=diag, stream=emulation.STREAM)
         assert int(status[0]) == (q.SHOT_OK if budget >= 31 else q.SHOT_BUDGET_EXCEEDED), (budget, diag)
 """)
+
+
+def test_equal_windows_share_one_graph():
+    # eight windows: all but the last, which has another commit region, are equal where the
+    # edges have one weight, and all differ where each edge has its own
+    emulation.run(DECODE % {"order": 0} + """
+from oracle.window import sliding_window_decode
+from paper_2609_12262_gb300.window import SlidingWindow
+for kw, graphs in (({"p": 0.01}, 2), ({"p_range": (0.005, 0.02), "p_seed": 2}, 8)):
+    pg = rotated_surface_code(5, 44, **kw)
+    syn, _ = sample_shots(pg, 8, 3)
+    dec = SlidingWindow(q.Graph.from_phys(pg), pg.nz, 10, 5)
+    assert len(dec.windows) == 8 and len({id(x[3]) for x in dec.windows}) == graphs
+    obs, status = dec.decode(torch.from_numpy(syn.view(np.int32).reshape(-1)), 8, stream=emulation.STREAM)
+    ro, rs = sliding_window_decode(pg, syn, 10, 5)
+    assert np.array_equal(status.numpy(), rs) and np.array_equal(q.to_uint64(obs), ro)
+""")
