@@ -3383,6 +3383,7 @@ __device__ __noinline__ bool wide_apart(Fast &X, int lane) {
 
 constexpr int USE_GENERAL = -3;   // the shot is outside the fast path's limits
 constexpr int HAS_ISLANDS = -4;   // begun: its islands are listed
+constexpr int NOT_FAST = -5;      // the fast path takes no shot of this graph and mode
 
 // What the warps of a block that decode a shot each share: the islands of all
 // their shots, taken by whichever warp is free.
@@ -3421,11 +3422,12 @@ struct FastShot {
 };
 
 // First phase: events, pairs, level 1.  Returns QEC_SHOT_OK for a shot without
-// events (everything written), HAS_ISLANDS or USE_GENERAL.
+// events (everything written), HAS_ISLANDS, USE_GENERAL or NOT_FAST.
 template <bool WIN, int NW>
 __device__ __forceinline__ int fast_begin(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
                                           Team<NW> &T, FastShared<NW> &M, FastShot &Q, int *dg) {
-    if (!fast_path_takes(g, A.mode, A.band_factor) || g.words > A.caps.wcap) return USE_GENERAL;
+    if (!fast_path_takes(g, A.mode, A.band_factor)) return NOT_FAST;
+    if (g.words > A.caps.wcap) return USE_GENERAL;
     const int band = max(g.wmax, 1) * max(A.band_factor, 1);
     Fast &X = M.f;
     bool small = true;
@@ -3812,9 +3814,9 @@ __device__ __forceinline__ void decode_shot(const BatchArgs &A, const Slab &S, c
         if (has) status = st == QEC_SHOT_OK ? fast_end<WIN, NW>(A, S, *r.g, r.row, T, M, Q, w, o, r.dg) : st;
     }
     if (!busy) return;
-    if (status == USE_GENERAL && NW == 1 && A.defer && A.pass == 0 && fast_path_takes(*r.g, A.mode, A.band_factor)) {
+    if (status == USE_GENERAL && NW == 1 && A.defer && A.pass == 0) {
         status = -1;   // left to the blocks of the overflow pass
-    } else if (status == USE_GENERAL) {
+    } else if (status == USE_GENERAL || status == NOT_FAST) {
         T.sync();
         status = decode_general<WIN, NW>(A, S, *r.g, r.row, T, deadline, w, o, r.dg);
     }

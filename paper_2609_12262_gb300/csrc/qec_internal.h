@@ -117,8 +117,8 @@ cudaError_t build_seam(const DGraph &g, const unsigned *commit, int *seam);
 // Whether the fast path (decoder.cu) takes shots of g at all: level 1 is
 // present, and the first extensions stay within the listed pairs.
 __host__ __device__ inline bool fast_path_takes(const DGraph &g, int mode, int band_factor) {
-    const long long band = (long long)(g.wmax > 1 ? g.wmax : 1) * (band_factor > 1 ? band_factor : 1);
-    const long long half = (g.b1 + 1) >> 1;
+    const int band = (g.wmax > 1 ? g.wmax : 1) * (band_factor > 1 ? band_factor : 1);   // (at most 2^21 x 64)
+    const int half = (g.b1 + 1) >> 1;
     return mode == QEC_MODE_HIERARCHICAL && g.ball && g.brad < (1 << 26) && band + (band > half ? band : half) <= g.b1;
 }
 
