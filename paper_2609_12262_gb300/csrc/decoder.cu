@@ -2191,8 +2191,8 @@ struct __align__(16) Isl {
     int pk[IN];           // per event: radius << 9 | (label of its top node + 1) << 7 | top node
     int y[2 * IN];        // duals of the blossoms
     int ev[IN], bd[IN];   // event of the shot, boundary distance
-    int xt[IN];           // radius at which the explored radius falls due (INT_MAX: ball exhausted)
-    int meet[IN];         // radius at which the region touches a level-1 cluster outside
+    int xt[IN];           // radius at which the explored radius falls due (NEVER: ball exhausted)
+    int meet[IN];         // radius at which the region touches what stands outside (NEVER: nothing so far)
     IslRec rec;           // result
     signed char lab[2 * IN], bpar[2 * IN], tpar[2 * IN], tps[2 * IN], tpo[2 * IN];
     signed char mate[2 * IN], ms[2 * IN], mo[2 * IN], root[2 * IN], minl[2 * IN];
@@ -2208,6 +2208,7 @@ enum { ST_RUN = -3, ST_ONE = -4, ST_TWO = -5 };
 constexpr unsigned CW_OPEN = 1u << 30, CW_SIDE = 1u << 31;
 // frozen at the start of the top level
 __device__ __forceinline__ bool st_frozen(int st) { return st >= 0 || st == MATE_BOUNDARY || st == ST_RUN; }
+constexpr int NEVER = 1 << 30;   // past every radius
 enum { ISL_FAIL = 0, ISL_OK = 1, ISL_STOP = 2, ISL_BIG = 3 };
 constexpr unsigned ISL_ALONE = 1u << 31;
 constexpr unsigned long long MET = 1ull << 27;   // in a pair: its events' regions meet
@@ -2645,7 +2646,7 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             if (hit && b < X.pcap) X.pr[b] = pk_pair(min(s, f), max(s, f), d);
             // inside the island: unless the other event has it recorded
             const int k2 = in ? (int)X.cw()[f] : 0;
-            const bool add = in && (I.xt[k2] != INT_MAX && d > max(b1, X.reach(b1, I.xt[k2] + X.L - 1, I.bd[k2])));
+            const bool add = in && (I.xt[k2] != NEVER && d > max(b1, X.reach(b1, I.xt[k2] + X.L - 1, I.bd[k2])));
             const unsigned mi = __ballot_sync(FULL, add);
             const int j = np + __popc(mi & ((1u << lane) - 1u));
             if (add && j < IP) I.pair[j] = make_int2(d, min(i, k2) | max(i, k2) << 8);
@@ -2653,7 +2654,7 @@ __device__ __noinline__ int isl_extend(Fast &X, Isl<E> &I, int c, int n, int np,
             if (np > IP || __any_sync(FULL, hit && b >= X.pcap)) return -1;
         }
         more = __any_sync(FULL, more);
-        if (lane == 0) I.xt[i] = sRl >= 0 && !more && sRl <= brad - wmax ? INT_MAX : R - X.L + 1;
+        if (lane == 0) I.xt[i] = sRl >= 0 && !more && sRl <= brad - wmax ? NEVER : R - X.L + 1;
         __syncwarp();
     }
     __syncwarp();
@@ -2711,7 +2712,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
             I.bd[e] = bd;
             // explored radius after the first extension, due at t = 0, which the listed pairs cover
             I.xt[e] = frozen ? -X.L : X.band + 1;
-            I.meet[e] = INT_MAX;
+            I.meet[e] = NEVER;
             I.pk[e] = rad[h] << RAD_SHIFT | e;
             I.lab[e] = frozen ? 0 : 1; I.bpar[e] = -1; I.tpar[e] = -1;
             I.mate[e] = frozen ? MATE_BOUNDARY : MATE_NONE; I.ms[e] = (signed char)e; I.mo[e] = -1;
@@ -2788,6 +2789,7 @@ __device__ __forceinline__ int run_island(Fast &X, Isl<E> &I, int c, int size, b
 #pragma unroll
         for (int h = 0; h < E; h++) {
             const int e = lane + h * WS;
+            bad |= rad[h] < 0;   // two regions past Fast::cap have met without knowing each other
             if (lab[h] == 1) {
                 const int bd = I.bd[e];
                 bad |= bd < rad[h];

@@ -13,6 +13,7 @@ import types
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2609_12262_gb300", "csrc")
 HOST = os.path.join(ROOT, "tests", "host_emulation")
+OUT = os.path.join(ROOT, "tests", "_build")
 STREAM = types.SimpleNamespace(cuda_stream=0)
 
 
@@ -58,7 +59,7 @@ def _translate(src):
 
 def build(csrc=CSRC, out=None, flags=()):
     """Compile the sources of `csrc` (default: this repository's) and return the library's path."""
-    out = out or os.path.join(ROOT, "tests", "_build")
+    out = out or OUT
     lib = os.path.join(out, "libqec_host.so")
     names = sorted(f for f in os.listdir(csrc) if f.endswith((".cu", ".cpp")))
     deps = [os.path.join(csrc, f) for f in os.listdir(csrc)] + [os.path.join(HOST, f) for f in os.listdir(HOST)] + \

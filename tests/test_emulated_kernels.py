@@ -283,3 +283,20 @@ for kw, graphs in (({"p": 0.01}, 2), ({"p_range": (0.005, 0.02), "p_seed": 2}, 8
     ro, rs = sliding_window_decode(pg, syn, 10, 5)
     assert np.array_equal(status.numpy(), rs) and np.array_equal(q.to_uint64(obs), ro)
 """)
+
+
+def test_a_radius_below_zero_ends_the_island():
+    # two regions past the reach meet unnoticed, and an inner region between them shrinks below zero: the shot goes to
+    # the run over everything at once, without steps on a state that no shot can be in (its times overflow)
+    lib = emulation.build(out=emulation.OUT + "/checked",
+                          flags=("-fsanitize=signed-integer-overflow", "-fno-sanitize-recover=all"))
+    emulation.run((DECODE % {"order": 0}).replace("load(", "load(%r, " % lib) + """
+pg = rotated_surface_code(11, 11, p_range=(0.001, 0.004), p_seed=3)
+row = pack_defects([38, 162, 232, 237, 238, 412, 417], pg.num_detectors)[None, :]
+g, og = q.Graph.from_phys(pg), OracleGraph.from_phys(pg)
+for team in (1, 4, 16):
+    q.set_tuning(team_warps=team)
+    o, w, s = q.decode_batch([g], torch.from_numpy(row.view(np.int32)), num_shots=1, stream=emulation.STREAM)
+    rw, ro, rs = og.decode_bitmaps(row, "hier")
+    assert (int(w[0]), int(q.to_uint64(o)[0]), int(s[0])) == (rw[0], ro[0], rs[0])
+""")
