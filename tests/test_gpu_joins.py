@@ -50,3 +50,65 @@ def test_joined_islands_equal_global_mode(qd, team, shots):  # noqa: F811
             assert np.array_equal(x, y), np.nonzero(x != y)[0][:5]
     finally:
         qd.set_tuning(team_warps=-1)
+
+
+def chain(rng, n):
+    """A path between two boundaries, with a boundary edge at some detectors in between."""
+    u, v = list(range(n - 1)) + [0, n - 1], list(range(1, n)) + [-1, -1]
+    side = rng.choice(n, size=int(rng.integers(0, 4)), replace=False).tolist()
+    return n, u + side, v + [-1] * len(side)
+
+
+def tree(rng, n):
+    u = list(range(1, n))
+    v = [int(rng.integers(max(0, i - 5), i)) for i in u]
+    side = rng.choice(n, size=int(rng.integers(1, 5)), replace=False).tolist()
+    return n, u + side, v + [-1] * len(side)
+
+
+def grid(rng, n):
+    a = int(rng.integers(3, 7))
+    b = n // a
+    at = np.arange(a * b).reshape(a, b)
+    u = np.concatenate([at[:-1].ravel(), at[:, :-1].ravel(), at[:, 0], at[:, -1]]).tolist()
+    v = np.concatenate([at[1:].ravel(), at[:, 1:].ravel(), np.full(2 * a, -1)]).tolist()
+    return a * b, u, v
+
+
+@pytest.mark.parametrize("team", [1, 4, 16])
+@pytest.mark.parametrize("kind", [chain, tree, grid], ids=["chain", "tree", "grid"])
+def test_sparse_shots_of_small_graphs_equal_the_oracle(qd, kind, team):  # noqa: F811
+    """Without diagnostics, where clusters of more events have closed forms too."""
+    import torch
+    from oracle import OracleGraph
+    from synth import pack_defects
+    rng = np.random.default_rng(team)
+    qd.set_tuning(team_warps=team)
+    try:
+        for wmax in (1, 5, 30, 100) * 2:
+            n, u, v = kind(rng, int(rng.integers(30, 60)))
+            w = rng.integers(max(1, wmax // 3), wmax + 1, len(u))
+            o = [0 if b >= 0 else 1 << (i % 2) for i, b in enumerate(v)]
+            near = [[] for _ in range(n)]
+            for a, b in zip(u, v):
+                if b >= 0:
+                    near[a].append(b)
+                    near[b].append(a)
+            rows = []
+            for _ in range(1000):
+                x, events = int(rng.integers(0, n)), set()
+                for _ in range(int(rng.integers(2, 8))):
+                    events ^= {x}
+                    for _ in range(int(rng.integers(1, 6))):
+                        x = int(rng.choice(near[x]))
+                rows.append(pack_defects(np.array(sorted(events), int), n))
+            rows = np.stack(rows)
+            g, og = qd.Graph(n, u, v, w, o, num_observables=2), OracleGraph(n, u, v, w, o)
+            obs, weight, status = qd.decode_batch([g], torch.from_numpy(rows.view(np.int32).reshape(-1)).cuda())
+            torch.cuda.synchronize()
+            rw, ro, rs = og.decode_bitmaps(rows, "hier")
+            got = status.cpu().numpy(), weight.cpu().numpy(), qd.to_uint64(obs)
+            for x, y in zip(got, (rs, rw, ro)):
+                assert np.array_equal(x, y), (wmax, np.nonzero(x != y)[0][:5])
+    finally:
+        qd.set_tuning(team_warps=-1)
