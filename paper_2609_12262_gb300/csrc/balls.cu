@@ -7,13 +7,13 @@
 // beyond b_1 up to the table radius.  A decode finds the events near an event
 // by testing a list against the syndrome row instead of searching the graph.
 //
-// Six largest weights of radius hold 290 entries per detector on average at
-// d = 21 (11 MB), four 108 and, at d = 51, 70 MB.  A list starts on its own
+// Six largest weights of radius hold 279 entries per detector on average at
+// d = 21 (11 MB), four, at d = 51, 119 (64 MB).  A list starts on its own
 // 128-byte line with the entries level 1 reads (12 on average, one line).
 // Building takes one bounded search per detector, a warp each, in shared memory;
-// it runs twice, once for the sizes (a d = 25 graph is created in 6.2 instead
-// of 4.2 ms, a d = 51 graph in 19.3 instead of 20.7, its distance runs being
-// faster).
+// it runs twice, once for the sizes (a d = 5 graph is created in 0.22 instead of
+// 0.15 ms, d = 25 in 2.9 instead of 2.4, d = 51 in 19.2 instead of 20.6, its
+// distance runs being faster).
 //
 // Seam distances: for every detector a lower bound on its distance to the
 // nearest detector on the other side of the commit region's border (sliding
@@ -197,9 +197,10 @@ cudaError_t build_ball_table(DGraph &g, bool wide, int4 **hdr, int2 **ball) {
     // Radius: six largest weights (a region of up to four edges' radius and
     // smaller ones stay within it of each other), for windows of a sliding decode
     // eight (an event at an open end has no boundary near), where every ball fits
-    // and the table stays below 128 MB; else four, with single balls that are too
-    // large stored to b_1 only; else b_1.  Six instead of four: 3,000 d = 31
-    // windows 0.52 -> 0.37 ms, 1,024 circuit-level d = 13 shots 0.19 -> 0.12 ms.
+    // and the table stays below 128 MB; else four below 512 MB, with single balls
+    // that are too large stored to b_1 only; else b_1, at whatever size that takes
+    // (128 bytes to 8 KB per detector, at most 16 GB).  Six instead of four: 3,000
+    // d = 31 windows 0.52 -> 0.37 ms, 1,024 circuit-level d = 13 shots 0.19 -> 0.12 ms.
     constexpr unsigned long long WIDE_LIMIT = 1ull << 24, FAR_LIMIT = 1ull << 26, LIMIT = (1ull << 31) - 1;   // entries
     const int grid = grid_for(g.n, WPB);
     int R = g.b1;

@@ -74,6 +74,7 @@
 //   phases in step, islands pooled                      12.0 / 0.096 / 0.24
 //   closed forms, 20 warps per SM                        8.9 / 0.064 / 0.20
 //   larger islands, wider tables                         9.3 / 0.065 / 0.12
+//   one-warp overflow deferred; waits, bounds, records   9.8 / 0.065 / 0.13
 
 #include <algorithm>
 #include <atomic>
