@@ -3098,9 +3098,14 @@ __device__ __forceinline__ void fast_components(Fast &X, int np1, Team<NW> &T) {
     volatile int *const comp = compw;
     const unsigned long long *const pr = X.pr;
     const int np0 = X.np0, K = X.K;
+    // after an earlier join the pairs that joined events may be gone, and their
+    // labels alone hold them together: those have to settle too
+    const bool joined = X.late;
+    bool again = false;
 #pragma unroll 1
-    for (int round = 0; round <= K; round++) {
-        bool changed = false;
+    for (int round = 0; round <= 2 * K; round++) {
+        bool changed = again;
+        again = false;
 #pragma unroll 1
         for (int i = T.tid(); i < np1; i += T.NT) {
             const unsigned long long p = pr[i];
@@ -3119,7 +3124,7 @@ __device__ __forceinline__ void fast_components(Fast &X, int np1, Team<NW> &T) {
 #pragma unroll 1
         for (int s = T.tid(); s < K; s += T.NT) {
             const int r = comp[s], rr = comp[r];
-            if (rr < r) comp[s] = rr;
+            if (rr < r) { comp[s] = rr; again = joined; }
         }
         T.sync();
     }
@@ -3247,9 +3252,9 @@ __device__ __forceinline__ void fast_level1(Fast &X, Level1 &out, bool quick, Te
 // What islands met, after they have run: marks the pairs in [np0, np1) whose
 // regions meet, joins their components and lists what has to run (in X.list,
 // from its back) and all islands (in X.all); of the pairs those that what has to
-// run would not record again are kept.  w, o: what is left of the closed forms.  Returns 0 when nothing met, 1 when something was joined, 2 when the
-// shot is outside the limits.  Every thread of the team calls; ends with a
-// barrier.
+// run would not record again are kept.  w, o: what is left of the closed forms.
+// Returns 0 when nothing met, 1 when something was joined, 2 when the shot is
+// outside the limits.  Every thread of the team calls; ends with a barrier.
 template <int NW>
 __device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<NW> T, long long &w,
                                       unsigned long long &o) {

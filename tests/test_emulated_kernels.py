@@ -300,3 +300,20 @@ for team in (1, 4, 16):
     rw, ro, rs = og.decode_bitmaps(row, "hier")
     assert (int(w[0]), int(q.to_uint64(o)[0]), int(s[0])) == (rw[0], ro[0], rs[0])
 """)
+
+
+def test_events_joined_earlier_follow_their_component():
+    # the pair that joined an event in one round is gone in the next: its label alone ties it to what it was joined with
+    emulation.run(DECODE % {"order": 0} + """
+for seed, events, weight in ((6, [195, 202, 531, 627, 634, 803, 904, 923, 1007, 1085], 893),
+                             (9, [91, 210, 252, 295, 361, 379, 546, 649], 957),
+                             (28, [555, 675, 712, 718, 723, 876, 927, 1011, 1031, 1052], 1052)):
+    pg = rotated_surface_code(13, 13, p_range=(0.001, 0.02), p_seed=seed)
+    g, row = q.Graph.from_phys(pg), torch.from_numpy(pack_defects(events, pg.num_detectors).view(np.int32))
+    for team in (1, 4, 16):
+        q.set_tuning(team_warps=team)
+        for order in range(5):
+            q.lib().emu_order(order, 3)
+            _, w, status = q.decode_batch([g], row, num_shots=1, stream=emulation.STREAM)
+            assert (int(w[0]), int(status[0])) == (weight, 0), (seed, team, order, int(w[0]))
+""")
