@@ -1889,12 +1889,18 @@ __device__ __forceinline__ int near_pairs(const Slab &S, const Shot &C, Team<NW>
     return flags;
 }
 
-// Decode one shot with hash tables scaled by `scale`; returns QEC_SHOT_* or -1
-// when the working set overflowed (retry with a larger scale).
+constexpr int LEVEL1_OVERLAP = -6;
+
+// Decode one shot with hash tables scaled by `scale`; returns QEC_SHOT_*, -1
+// when the working set overflowed (retry with a larger scale), or
+// LEVEL1_OVERLAP when two accepted level-1 clusters have grown into each other.
+// (A cluster of odd size stops as late as its nearest boundary contact plus its
+// diameter, which can pass the b_1 / 2 that keeps clusters apart.  Their duals
+// together are then no solution, and the shot is decoded without level 1.)
 // WIN: sliding-window mode (BatchArgs::carry set), compiled as its own kernel so
 // that the ordinary kernel carries none of its code.
 template <bool WIN, int NW>
-__device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
+__device__ int decode_attempt_body(const BatchArgs &A, int mode, const Slab &S, const DGraph &g, const unsigned *row,
                                    Team<NW> &T, unsigned scale, unsigned long long deadline, long long &w_out,
                                    unsigned long long &o_out, int *dg, Shot &C) {
     C.g = g;
@@ -1949,7 +1955,7 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     const int odd = T.template red32<2>(near_pairs(S, C, T));
     const int Rbig = max(g.b1, C.band);   // level-1 ball of an event with many vertices within b_1
     if ((odd & 1) || ((odd & 2) && reach_of(C, Rbig) > g.b1)) go_real(S, C, T);
-    if (A.mode == QEC_MODE_HIERARCHICAL) {
+    if (mode == QEC_MODE_HIERARCHICAL) {
         // ---- Algorithm 1, level 1.  An event with more than LB_CAP vertices
         // within b_1 gets its first ball here
         if (odd) {
@@ -1973,7 +1979,7 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
         const int err = T.bcast(ldr(&S.ctr[C_ERR]));
         if (err) return (err & ERR_INTERNAL) ? QEC_SHOT_INTERNAL : -1;
     }
-    if (A.mode == QEC_MODE_HIERARCHICAL) {
+    if (mode == QEC_MODE_HIERARCHICAL) {
         const int npairs = T.bcast(ldr(&S.ctr[C_NPAIRS]));
         // connected components of pairs within b_1: min-label propagation
         for (int s = T.tid(); s < K; s += T.NT) { S.comp[s] = s; S.cst0[s] = 0; S.cst1[s] = 0; S.cst2[s] = 0; }
@@ -2062,9 +2068,21 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
     // from t = 0 with the stopped level-1 configurations present as frozen
     // regions (global mode: every event, from an empty state).  One call site
     // of the event loop serves both, which keeps the kernel's hot code small.
+    bool ran = false;
     for (int guard = 0; guard <= K + 1; guard++) {
         while (gr < K && (S.comp[gr] != gr || !(S.cst1[gr] & 2))) gr++;
         const bool top = gr >= K;
+        if (top && ran) {
+            // (the larger of two regions has recorded the pair, see reach_of)
+            const int np = T.bcast(ldr(&S.ctr[C_NPAIRS]));
+            bool overlap = false;
+            for (int i = T.tid(); i < np; i += T.NT) {
+                const int4 pq = ld_pr(&S.pr[i]);
+                const int a = pq.x, b = pq.y;
+                if (a >= 0 && S.comp[a] != S.comp[b]) overlap |= S.src[a].srad + S.src[b].srad > pq.z;
+            }
+            if (T.any(overlap)) return LEVEL1_OVERLAP;
+        }
         if (top) {
             for (int s = T.tid(); s < K; s += T.NT) {
                 if (S.nd[s].alive || S.src[s].stop != s) S.src[s].inplay = 1;   // stopped level-1 configuration
@@ -2086,6 +2104,7 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
                    : st == RUN_BUDGET ? QEC_SHOT_BUDGET_EXCEEDED : QEC_SHOT_INTERNAL;
         }
         if (top) break;
+        ran = true;
         for (int s = T.tid(); s < K; s += T.NT)
             if (S.comp[s] == gr) S.src[s].inplay = 0;
         T.sync();
@@ -2131,13 +2150,13 @@ __device__ int decode_attempt_body(const BatchArgs &A, const Slab &S, const DGra
 // in the band lists and the pair list are reset, after anything else the
 // whole region the attempt could have used.
 template <bool WIN, int NW>
-__device__ int decode_attempt(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row, Team<NW> &T,
+__device__ int decode_attempt(const BatchArgs &A, int mode, const Slab &S, const DGraph &g, const unsigned *row, Team<NW> &T,
                               unsigned scale, unsigned long long deadline, long long &w_out,
                               unsigned long long &o_out, int *dg) {
     Shot C;
     C.real = 0;
     C.paths = 0;
-    const int st = decode_attempt_body<WIN, NW>(A, S, g, row, T, scale, deadline, w_out, o_out, dg, C);
+    const int st = decode_attempt_body<WIN, NW>(A, mode, S, g, row, T, scale, deadline, w_out, o_out, dg, C);
     // (the tables are used by explored balls only)
     if (C.real || C.paths) release_tables(S, C, T, st != QEC_SHOT_OK);
     return st;
@@ -3722,9 +3741,16 @@ template <bool WIN, int NW>
 __device__ __noinline__ int decode_general(const BatchArgs &A, const Slab &S, const DGraph &g, const unsigned *row,
                                            Team<NW> T, unsigned long long deadline, long long &w,
                                            unsigned long long &o, int *dg) {
-    int status = -1;
-    for (unsigned scale = 1; scale <= 64 && status == -1; scale *= 4)
-        status = decode_attempt<WIN, NW>(A, S, g, row, T, scale, deadline, w, o, dg);
+    int status = -1, mode = A.mode;
+    for (unsigned scale = 1; scale <= 64 && status == -1;) {
+        status = decode_attempt<WIN, NW>(A, mode, S, g, row, T, scale, deadline, w, o, dg);
+        if (status == LEVEL1_OVERLAP) {
+            status = -1;
+            mode = QEC_MODE_GLOBAL;
+        } else {
+            scale *= 4;
+        }
+    }
     return status;
 }
 

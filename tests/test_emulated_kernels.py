@@ -317,3 +317,20 @@ for seed, events, weight in ((6, [195, 202, 531, 627, 634, 803, 904, 923, 1007, 
             _, w, status = q.decode_batch([g], row, num_shots=1, stream=emulation.STREAM)
             assert (int(w[0]), int(status[0])) == (weight, 0), (seed, team, order, int(w[0]))
 """)
+
+
+def test_level1_clusters_that_grow_into_each_other():
+    # a cluster of three reaches its boundary later than b_1 / 2 and covers part of the next cluster's region
+    emulation.run(DECODE % {"order": 0} + """
+for pg, events in ((rotated_surface_code(9, 9, p_range=(0.0005, 0.1), p_seed=5), [77, 229, 232, 237]),
+                   (rotated_surface_code(17, 17, p_range=(0.001, 0.05), p_seed=2), [1343, 1590, 1599, 1606]),
+                   (rotated_surface_code(17, 17, p_range=(0.001, 0.05), p_seed=5), [928, 1337, 1344, 1353])):
+    g, og, row = q.Graph.from_phys(pg), OracleGraph.from_phys(pg), pack_defects(events, pg.num_detectors)
+    for team in (1, 4, 16):
+        q.set_tuning(team_warps=team)
+        for diag in (False, True):
+            o, w, s, _ = q.decode_batch_ex([g], torch.from_numpy(row.view(np.int32)), num_shots=1, diag=diag,
+                                           stream=emulation.STREAM)
+            r = og.decode(events, "hier")
+            assert r.touch_violations and (int(w[0]), int(q.to_uint64(o)[0]), int(s[0])) == (r.weight, r.obs, r.status)
+""")
