@@ -3375,10 +3375,11 @@ __device__ __noinline__ int fast_join(Fast &X, int np1, int n2, int round, Team<
     return 1;
 }
 
-// Whether every two regions past the cap of Fast::reach are known to each other
-// or stayed apart: the larger one's reach held the other's event, or their
-// distance (in the ball table of one of them, or beyond it) exceeds the sum of
-// their radii.  One warp.
+// Whether every two regions past the cap of Fast::reach knew each other when they
+// met, or stayed apart: they are at most two caps apart (where they meet, the
+// larger one has half the distance, and its reach holds the rest; farther ones may
+// be recorded too late), or their distance (in the ball table of one of them, or
+// beyond it) exceeds the sum of their radii.  One warp.
 __device__ __noinline__ bool wide_apart(Fast &X, int lane) {
     const DGraph &g = *X.g;
     const int K = X.K, cap = X.cap, brad = g.brad;
@@ -3402,7 +3403,7 @@ __device__ __noinline__ bool wide_apart(Fast &X, int lane) {
 #pragma unroll 1
         for (int k = 0; k < h.z + h.w; k++) {   // one entry for all lanes
             const int2 e = __ldg(g.ball + (unsigned)h.x + k);
-            if (e.x == v && e.y <= ra + rb && e.y > max(ra, rb) + cap) ok = false;
+            if (e.x == v && e.y <= ra + rb && e.y > 2 * cap) ok = false;
         }
     }
     return !__any_sync(FULL, !ok);

@@ -334,3 +334,18 @@ for pg, events in ((rotated_surface_code(9, 9, p_range=(0.0005, 0.1), p_seed=5),
             r = og.decode(events, "hier")
             assert r.touch_violations and (int(w[0]), int(q.to_uint64(o)[0]), int(s[0])) == (r.weight, r.obs, r.status)
 """)
+
+
+def test_two_wide_regions_that_know_each_other_too_late():
+    # both are past the reach's cap where they meet, and one records the other only after that
+    emulation.run(DECODE % {"order": 0} + """
+for seed, events in ((3, [38, 98, 102, 114, 338, 502, 513, 573]), (4, [227, 299, 332, 432, 443, 503]),
+                     (5, [23, 99, 154, 159, 202, 287, 332, 337]), (7, [136, 251, 311, 328, 334, 372, 388, 512])):
+    pg = rotated_surface_code(11, 11, p_range=(0.002, 0.006), p_seed=seed)
+    g, row = q.Graph.from_phys(pg), pack_defects(events, pg.num_detectors)[None, :]
+    rw, ro, rs = OracleGraph.from_phys(pg).decode_bitmaps(row, "hier")
+    for team in (1, 4, 16):
+        q.set_tuning(team_warps=team)
+        o, w, s = q.decode_batch([g], torch.from_numpy(row.view(np.int32)), num_shots=1, stream=emulation.STREAM)
+        assert (int(w[0]), int(q.to_uint64(o)[0]), int(s[0])) == (rw[0], ro[0], rs[0]), (seed, team)
+""")
